@@ -152,4 +152,11 @@ def work(case):
 
 
 def tolerance(case):
-    return {"rel": 1e-2,"max":0.1} if case["out"]=="bf16" else {"rel":1e-4}
+    """About four times what the results differ by from the same formulas in 64 bits: over the listed cases and fifty more
+    float32 results by 8e-7 and 1.9e-5 (large logits: the tensor cores' float32 sums), bfloat16 ones by 1.7e-3 and
+    4.8e-3 (one rounding), attention by 2.4e-3 and 1.3e-2 (weights and result both rounded)."""
+    if case["out"] == "f32":
+        return {"rel": 4e-6, "max": 8e-5}
+    if case["op"] == "attention":
+        return {"rel": 1e-2, "max": 5e-2}
+    return {"rel": 7e-3, "max": 2e-2}
