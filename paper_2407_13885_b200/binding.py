@@ -1,4 +1,5 @@
-"""ctypes binding of ``libattnw.so`` - argument marshalling only.
+"""Binding of ``libattnw.so`` - argument marshalling only, by ctypes and, for the calls on CUDA tensors, by the extension
+module ``_attnw_torch`` (csrc/torch_calls.cpp).
 
 Every operation runs in the library's CUDA kernels; nothing here computes.  If the compiled
 library is missing the import of this module raises: there is no fallback.  PyTorch is used
@@ -63,6 +64,17 @@ class AttnwError(RuntimeError):
     def __init__(self, code: int, where: str):
         self.code = code
         super().__init__(f"{where}: attnw status {code}: {strerror(code)}")
+
+
+def _load_native():
+    if not os.path.exists(_build.EXT_PATH):
+        raise ImportError(f"{_build.EXT_PATH} is missing: build it with `python -m paper_2407_13885_b200.build`.")
+    from . import _attnw_torch
+    _attnw_torch.set_error(AttnwError)
+    return _attnw_torch
+
+
+_native = _load_native()
 
 
 def strerror(code: int) -> str:
@@ -132,43 +144,14 @@ def attnw_fused(Q: torch.Tensor, K: torch.Tensor, scale: float, P: torch.Tensor 
 
     ``Q, K``: CUDA bfloat16 ``[B, H, N, d]``; returns ``P [B, H, N, N]`` (bfloat16 or float32).
     Asynchronous on ``stream`` (default: torch's current stream)."""
-    _require_cuda(Q, "Q", torch.bfloat16)
-    _require_cuda(K, "K", torch.bfloat16)
-    if Q.dim() != 4 or Q.shape != K.shape:
-        raise ValueError("Q and K must both be [B, H, N, d]")
-    B, H, N, d = Q.shape
-    if P is None:
-        P = torch.empty((B, H, N, N), dtype=out_dtype, device=Q.device)
-    else:
-        _require_cuda(P, "P", P.dtype)
-        if tuple(P.shape) != (B, H, N, N) or P.dtype not in (torch.bfloat16, torch.float32):
-            raise ValueError("P must be [B, H, N, N] in bfloat16 or float32")
-    fn = lib.attnw_fused if P.dtype == torch.bfloat16 else lib.attnw_fused_f32
-    with torch.cuda.device(Q.device):
-        _check(fn(Q.data_ptr(), K.data_ptr(), P.data_ptr(), B, H, N, d, float(scale), _stream_ptr(stream)),
-               "attnw_fused")
-    return P
+    return _native.attnw_fused(Q, K, scale, P, out_dtype, None if stream is None else _stream_ptr(stream))
 
 
 def attn_fused(Q: torch.Tensor, K: torch.Tensor, V: torch.Tensor, scale: float, O: torch.Tensor | None = None,
                stream=None) -> torch.Tensor:
     """``O = Softmax(scale * Q K^T) V`` in one fused kernel; ``Q, K, V, O``: CUDA bfloat16 ``[B, H, N, d]``.
     Asynchronous on ``stream`` (default: torch's current stream)."""
-    for t, name in ((Q, "Q"), (K, "K"), (V, "V")):
-        _require_cuda(t, name, torch.bfloat16)
-    if Q.dim() != 4 or Q.shape != K.shape or Q.shape != V.shape:
-        raise ValueError("Q, K and V must all be [B, H, N, d]")
-    B, H, N, d = Q.shape
-    if O is None:
-        O = torch.empty((B, H, N, d), dtype=torch.bfloat16, device=Q.device)
-    else:
-        _require_cuda(O, "O", torch.bfloat16)
-        if tuple(O.shape) != (B, H, N, d):
-            raise ValueError("O must be [B, H, N, d]")
-    with torch.cuda.device(Q.device):
-        _check(lib.attn_fused(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), B, H, N, d, float(scale),
-                              _stream_ptr(stream)), "attn_fused")
-    return O
+    return _native.attn_fused(Q, K, V, scale, O, None if stream is None else _stream_ptr(stream))
 
 
 def project_qk(X: torch.Tensor, Wq: torch.Tensor, Wk: torch.Tensor, Q: torch.Tensor | None = None,
@@ -176,44 +159,13 @@ def project_qk(X: torch.Tensor, Wq: torch.Tensor, Wk: torch.Tensor, Q: torch.Ten
     """Queries and keys from the inputs: ``Q[b,h] = X[b] Wq[h]^T``, ``K[b,h] = X[b] Wk[h]^T`` for CUDA bfloat16
     ``X [B, N, d_model]`` and ``Wq, Wk [H, d, d_model]`` -> ``Q, K [B, H, N, d]`` (bfloat16), the layout
     ``attnw_fused`` and ``attn_fused`` read.  Asynchronous on ``stream`` (default: torch's current stream)."""
-    for t, name in ((X, "X"), (Wq, "Wq"), (Wk, "Wk")):
-        _require_cuda(t, name, torch.bfloat16)
-    if X.dim() != 3 or Wq.dim() != 3 or Wq.shape != Wk.shape or Wq.shape[2] != X.shape[2]:
-        raise ValueError("X must be [B, N, d_model] and Wq, Wk [H, d, d_model]")
-    B, N, d_model = X.shape
-    H, d, _ = Wq.shape
-    outs = []
-    for t, name in ((Q, "Q"), (K, "K")):
-        if t is None:
-            t = torch.empty((B, H, N, d), dtype=torch.bfloat16, device=X.device)
-        else:
-            _require_cuda(t, name, torch.bfloat16)
-            if tuple(t.shape) != (B, H, N, d):
-                raise ValueError(f"{name} must be [B, H, N, d]")
-        outs.append(t)
-    with torch.cuda.device(X.device):
-        _check(lib.attnw_project_qk(X.data_ptr(), Wq.data_ptr(), Wk.data_ptr(), outs[0].data_ptr(), outs[1].data_ptr(), B, N,
-                                    d_model, H, d, _stream_ptr(stream)), "attnw_project_qk")
-    return outs[0], outs[1]
+    return _native.project_qk(X, Wq, Wk, Q, K, None if stream is None else _stream_ptr(stream))
 
 
 def softmax_rows(S: torch.Tensor, P: torch.Tensor | None = None, out_dtype: torch.dtype = torch.bfloat16,
                  stream=None) -> torch.Tensor:
     """Row-wise Softmax of float32 scores ``S [rows, cols]`` -> ``P`` (bfloat16 or float32)."""
-    _require_cuda(S, "S", torch.float32)
-    if S.dim() != 2:
-        raise ValueError("S must be [rows, cols]")
-    rows, cols = S.shape
-    if P is None:
-        P = torch.empty((rows, cols), dtype=out_dtype, device=S.device)
-    else:
-        _require_cuda(P, "P", P.dtype)
-        if tuple(P.shape) != (rows, cols) or P.dtype not in (torch.bfloat16, torch.float32):
-            raise ValueError("P must be [rows, cols] in bfloat16 or float32")
-    fn = lib.softmax_rows if P.dtype == torch.bfloat16 else lib.softmax_rows_f32
-    with torch.cuda.device(S.device):
-        _check(fn(S.data_ptr(), P.data_ptr(), rows, cols, _stream_ptr(stream)), "softmax_rows")
-    return P
+    return _native.softmax_rows(S, P, out_dtype, None if stream is None else _stream_ptr(stream))
 
 
 def _require_host(t: torch.Tensor, name: str, dtype) -> None:

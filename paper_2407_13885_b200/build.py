@@ -1,9 +1,11 @@
-"""Builds ``libattnw.so`` in-tree with nvcc for sm_100a (no JIT cache, no torch extension)."""
+"""Builds, in-tree and without a JIT cache, ``libattnw.so`` (nvcc, sm_100a) and ``_attnw_torch`` (host compiler): the
+extension module that takes torch tensors to the library's C ABI without Python in between."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
+import sysconfig
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _CSRC = os.path.join(_PKG, "csrc")
@@ -11,6 +13,9 @@ LIB_PATH = os.path.join(_PKG, "libattnw.so")
 SOURCES = [os.path.join(_CSRC, "attnw_api.cu")]
 _DEPS = [os.path.join(_CSRC, f) for f in sorted(os.listdir(_CSRC))] + [
     os.path.join(os.path.dirname(_PKG), "include", "attnw.h")]
+EXT_PATH = os.path.join(_PKG, "_attnw_torch.so")
+EXT_SOURCE = os.path.join(_CSRC, "torch_calls.cpp")
+_DEPS.remove(EXT_SOURCE)
 
 
 def nvcc_path() -> str:
@@ -30,11 +35,40 @@ def nvcc_command(out: str, verbose_ptxas: bool = False, defines: tuple[str, ...]
     return cmd
 
 
+def ext_command(out: str) -> list[str]:
+    import torch
+    from torch.utils import cpp_extension
+    torch_lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cuda_home = os.path.dirname(os.path.dirname(nvcc_path()))
+    includes = [sysconfig.get_paths()["include"], *cpp_extension.include_paths(), os.path.join(cuda_home, "include")]
+    return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *["-isystem" + i for i in includes],
+            "-o", out, EXT_SOURCE, "-L" + _PKG, "-l:" + os.path.basename(LIB_PATH), "-L" + torch_lib, "-ltorch_python",
+            "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN"]
+
+
+def _older(target: str, deps: list[str]) -> bool:
+    return not os.path.exists(target) or any(os.path.getmtime(d) > os.path.getmtime(target) for d in deps)
+
+
 def is_stale() -> bool:
-    if not os.path.exists(LIB_PATH):
-        return True
-    built = os.path.getmtime(LIB_PATH)
-    return any(os.path.getmtime(d) > built for d in _DEPS)
+    return _older(LIB_PATH, _DEPS)
+
+
+def _compile(cmd: list[str], tmp: str, target: str) -> str:
+    proc = subprocess.run(cmd, capture_output=True, text=True)
+    if proc.returncode != 0:
+        raise RuntimeError(f"{cmd[0]} failed:\n" + proc.stdout + proc.stderr)
+    os.replace(tmp, target)
+    return proc.stderr
+
+
+def build_extension(force: bool = False) -> str:
+    """Compile ``_attnw_torch`` if it is missing or older than its source or the C header; returns its path."""
+    if force or _older(EXT_PATH, [EXT_SOURCE, os.path.join(os.path.dirname(_PKG), "include", "attnw.h")]):
+        tmp = EXT_PATH + f".tmp{os.getpid()}"
+        _compile(ext_command(tmp), tmp, EXT_PATH)
+    return EXT_PATH
 
 
 def build_library(force: bool = False, verbose_ptxas: bool = False, defines: tuple[str, ...] = (),
@@ -44,15 +78,13 @@ def build_library(force: bool = False, verbose_ptxas: bool = False, defines: tup
     target = out or LIB_PATH
     if defines and out is None:
         raise ValueError("a build with extra definitions needs its own output path")
-    if not force and out is None and not is_stale():
-        return LIB_PATH
-    tmp = target + f".tmp{os.getpid()}"
-    proc = subprocess.run(nvcc_command(tmp, verbose_ptxas, defines), capture_output=True, text=True)
-    if proc.returncode != 0:
-        raise RuntimeError("nvcc failed:\n" + proc.stdout + proc.stderr)
-    os.replace(tmp, target)
-    if verbose_ptxas:
-        print(proc.stderr)
+    if force or out is not None or is_stale():
+        tmp = target + f".tmp{os.getpid()}"
+        messages = _compile(nvcc_command(tmp, verbose_ptxas, defines), tmp, target)
+        if verbose_ptxas:
+            print(messages)
+    if out is None:
+        build_extension(force)
     return target
 
 

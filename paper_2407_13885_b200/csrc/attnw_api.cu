@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/attnw.h"
+#include "launch.cuh"
 #include "attnw_fused.cuh"
 #include "attn_fused.cuh"
 #include "attn_onepass.cuh"
@@ -25,7 +26,6 @@ namespace {
 
 using namespace attnw;
 
-constexpr int kMaxDevices = 64;
 // Consecutive launches of the grid-row kernel use different exchange areas in turn: the last CTAs of one launch may still
 // be reading the pairs of their last row block when the next launch (which starts as soon as its whole grid fits) posts.
 constexpr int kGridrowAreas = 4;
@@ -70,7 +70,7 @@ constexpr double kTwoPassPerSm = 0.9;  // measured: per-SM throughput of the two
 std::mutex g_mutex;
 
 struct DeviceInfo {
-    bool ready = false;
+    std::atomic<bool> ready{false};  // cc_major and sm_count are valid
     int cc_major = 0;
     int sm_count = 0;
     int fused_pairs[2][2] = {};  // [d == 128][float32 P]: co-resident two-CTA clusters of the two-pass kernel, 0 = not asked yet
@@ -93,7 +93,7 @@ DeviceInfo g_devices[kMaxDevices];
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn g_encode_tiled = nullptr;
+std::atomic<EncodeTiledFn> g_encode_tiled{nullptr};
 
 // Current device's cached properties; returns an attnw_status.
 int current_device(DeviceInfo** out) {
@@ -102,23 +102,22 @@ int current_device(DeviceInfo** out) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
     }
-    std::lock_guard<std::mutex> lock(g_mutex);
     DeviceInfo& d = g_devices[dev];
-    if (!d.ready) {
+    if (!d.ready.load(std::memory_order_acquire)) {
+        std::lock_guard<std::mutex> lock(g_mutex);
         if (cudaDeviceGetAttribute(&d.cc_major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&d.sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
             (void)cudaGetLastError();
             return ATTNW_ERR_CUDA;
         }
-        d.ready = true;
+        d.ready.store(true, std::memory_order_release);
     }
     *out = &d;
     return d.cc_major == 10 ? ATTNW_OK : ATTNW_ERR_UNSUPPORTED;
 }
 
 int load_encoder() {
-    std::lock_guard<std::mutex> lock(g_mutex);
-    if (g_encode_tiled) return ATTNW_OK;
+    if (g_encode_tiled.load(std::memory_order_relaxed)) return ATTNW_OK;
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult qres;
     if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess ||
@@ -126,7 +125,7 @@ int load_encoder() {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
     }
-    g_encode_tiled = reinterpret_cast<EncodeTiledFn>(fn);
+    g_encode_tiled.store(reinterpret_cast<EncodeTiledFn>(fn), std::memory_order_relaxed);
     return ATTNW_OK;
 }
 
@@ -137,7 +136,7 @@ int encode_3d(CUtensorMap* map, CUtensorMapDataType dtype, size_t esize, const v
     const cuuint64_t strides[2] = {dim0 * esize, dim0 * dim1 * esize};
     const cuuint32_t box[3] = {box0, box1, 1};
     const cuuint32_t elem_strides[3] = {1, 1, 1};
-    CUresult r = g_encode_tiled(map, dtype, 3, const_cast<void*>(base), dims, strides, box, elem_strides,
+    CUresult r = g_encode_tiled.load(std::memory_order_relaxed)(map, dtype, 3, const_cast<void*>(base), dims, strides, box, elem_strides,
                                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? ATTNW_OK : ATTNW_ERR_CUDA;
@@ -186,8 +185,7 @@ int launch_fused(DeviceInfo* dev, const void* Q, const void* K, void* P, int BH,
             rc = encode_3d(&tm_p, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, P, N, N, BH, 32, kTile);
     }
     if (rc != ATTNW_OK) return rc;
-    // The attribute is per device and per kernel; set it on every launch path's first use.
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kDynamicBytes) != cudaSuccess) {
+    if (allow_smem<attnw_fused_kernel<D, OutT>>(L::kDynamicBytes) != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
     }
@@ -259,8 +257,7 @@ int resident_max_clusters_impl(DeviceInfo* dev, int cluster_ctas) {  // (both ex
     if (cached != 0) return cached;
     using L = ResidentSmem<D, CMAX>;
     auto kernel = attnw_resident_kernel<D, CMAX, false>;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kDynamicBytes) != cudaSuccess ||
-        (CMAX > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+    if (allow_smem<attnw_resident_kernel<D, CMAX, false>>(L::kDynamicBytes, CMAX > 8) != cudaSuccess) {
         (void)cudaGetLastError();
         return cached = -1;
     }
@@ -301,8 +298,7 @@ int launch_resident_impl(DeviceInfo* dev, const void* Q, const void* K, void* P,
     if (rc == ATTNW_OK) rc = encode_3d(&tm_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, D, N, BH, 64, kTile);
     if (rc == ATTNW_OK) rc = encode_3d(&tm_p, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, P, N, N, BH, 64, kTile);
     if (rc != ATTNW_OK) return rc;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kDynamicBytes) != cudaSuccess ||
-        (CMAX > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+    if (allow_smem<attnw_resident_kernel<D, CMAX, OWNER>>(L::kDynamicBytes, CMAX > 8) != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
     }
@@ -358,7 +354,7 @@ int launch_gridrow(DeviceInfo* dev, const void* Q, const void* K, void* P, int B
     if (rc == ATTNW_OK) rc = encode_3d(&tm_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, D, N, BH, 64, kTile);
     if (rc == ATTNW_OK) rc = encode_3d(&tm_p, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, P, N, N, BH, 64, kTile);
     if (rc != ATTNW_OK) return rc;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kDynamicBytes) != cudaSuccess) {
+    if (allow_smem<gr::attnw_gridrow_kernel<D>>(L::kDynamicBytes) != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
     }
@@ -441,7 +437,7 @@ int launch_attn(const void* Q, const void* K, const void* V, void* O, int BH, in
     if (rc == ATTNW_OK) rc = encode_3d(&tm_v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, V, D, N, BH, 64, kTile);
     if (rc == ATTNW_OK) rc = encode_3d(&tm_o, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, O, D, N, BH, 64, kTile);
     if (rc != ATTNW_OK) return rc;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kDynamicBytes) != cudaSuccess) {
+    if (allow_smem<av::attn_fused_kernel<D>>(L::kDynamicBytes) != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
     }
@@ -464,7 +460,7 @@ int launch_attn_onepass(const void* Q, const void* K, const void* V, void* O, in
     if (rc == ATTNW_OK) rc = encode_3d(&tm_v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, V, D, N, BH, 64, kTile);
     if (rc == ATTNW_OK) rc = encode_3d(&tm_o, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, O, D, N, BH, 64, kTile);
     if (rc != ATTNW_OK) return rc;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kDynamicBytes) != cudaSuccess) {
+    if (allow_smem<av1::attn_onepass_kernel<D>>(L::kDynamicBytes) != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
     }
@@ -527,8 +523,7 @@ int launch_project(const void* X, const void* Wq, const void* Wk, void* Q, void*
     if (rc == ATTNW_OK) rc = encode_3d(&tm_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Q, d, N, static_cast<uint64_t>(B) * H, 64, 128);
     if (rc == ATTNW_OK) rc = encode_3d(&tm_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, d, N, static_cast<uint64_t>(B) * H, 64, 128);
     if (rc != ATTNW_OK) return rc;
-    if (cudaFuncSetAttribute(proj::project_qk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, proj::kDynamicBytes) !=
-        cudaSuccess) {
+    if (allow_smem<proj::project_qk_kernel>(proj::kDynamicBytes) != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
     }
@@ -809,7 +804,7 @@ int launch_gridrow_noalloc(NoAllocState* st, const void* Q, const void* K, void*
     if (rc == ATTNW_OK) rc = encode_3d(&tm_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, D, N, BH, 64, kTile);
     if (rc == ATTNW_OK) rc = encode_3d(&tm_p, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, P, N, N, BH, 64, kTile);
     if (rc != ATTNW_OK) return rc;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kDynamicBytes) != cudaSuccess) {
+    if (allow_smem<gr::attnw_gridrow_kernel<D>>(L::kDynamicBytes) != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
     }

@@ -11,6 +11,7 @@
 // (coalesced streaming stores).
 #pragma once
 #include "attnw_fused.cuh"
+#include "launch.cuh"
 #include "softmax_rows.cuh"
 
 namespace attnw {
@@ -174,12 +175,8 @@ inline cudaError_t launch_nt(const float* S, OutT* P, long long rows, long long 
                              cudaStream_t stream) {
     const size_t smem = kControlBytes + static_cast<size_t>(slice_cols) * 4;
     auto kernel = softmax_rows_smem_kernel<OutT, NT>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    const cudaError_t e = allow_smem<softmax_rows_smem_kernel<OutT, NT>>(kControlBytes + kSliceMaxCols * 4, true);
     if (e != cudaSuccess) return e;
-    if (C > 8) {
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
-    }
     const long long per_sm = NT == 256 ? (smem * 4 <= 224 * 1024 ? 4 : 3) : 2;
     long long n_clusters = (per_sm * sm_count) / C;  // CTAs that fit at once
     if (n_clusters < 1) n_clusters = 1;
@@ -392,8 +389,7 @@ inline cudaError_t launch_regcluster(const float* S, OutT* P, long long rows, lo
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (*resident_clusters == 0) {  // once per device, output type and cluster size
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-        if (e == cudaSuccess && C > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaError_t e = allow_smem<softmax_rows_regcluster_kernel<OutT>>(kSmemMax, true);
         int n = 0;
         if (e == cudaSuccess) {
             cfg.gridDim = dim3(static_cast<unsigned>(C));

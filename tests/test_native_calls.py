@@ -1,0 +1,60 @@
+"""The native form of the tensor entry points: argument errors raise before anything touches a GPU, and what a caller passes
+for the output and the stream is honoured."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from helpers import assert_close_to_oracle, bits_to_cuda_bf16, small_fused_inputs
+
+
+@pytest.fixture(scope="module")
+def binding():
+    from paper_2407_13885_b200 import build
+    build.build_library()
+    from paper_2407_13885_b200 import binding
+    return binding
+
+
+def test_host_tensors_are_refused(binding):
+    x = torch.zeros(1, 1, 8, 64, dtype=torch.bfloat16)
+    for call in (lambda: binding.attnw_fused(x, x, 0.125), lambda: binding.attn_fused(x, x, x, 0.125),
+                 lambda: binding.project_qk(x[0], x[0], x[0]), lambda: binding.softmax_rows(x[0, 0].float()),
+                 lambda: binding.attnw_fused(None, x, 0.125)):
+        with pytest.raises(TypeError, match="must be a CUDA tensor"):
+            call()
+
+
+@pytest.mark.gpu
+def test_bad_arguments_on_the_gpu(binding):
+    q = torch.zeros(1, 2, 64, 64, dtype=torch.bfloat16, device="cuda")
+    for exc, call in ((TypeError, lambda: binding.attnw_fused(q.float(), q, 0.125)),
+                      (ValueError, lambda: binding.attnw_fused(q, q[:, :1], 0.125)),
+                      (ValueError, lambda: binding.attnw_fused(q.transpose(1, 2), q.transpose(1, 2), 0.125)),
+                      (ValueError, lambda: binding.attnw_fused(q, q, 0.125, out_dtype=torch.float16)),
+                      (ValueError, lambda: binding.attnw_fused(q, q, 0.125, P=q)),
+                      (ValueError, lambda: binding.attn_fused(q, q, q, 0.125, O=q[:, :1].contiguous())),
+                      (ValueError, lambda: binding.project_qk(q[0], q[0], q[0, :1].contiguous())),
+                      (ValueError, lambda: binding.softmax_rows(q.float())),
+                      (TypeError, lambda: binding.attnw_fused(q, q, None))):
+        with pytest.raises(exc):
+            call()
+    with pytest.raises(binding.AttnwError) as e:
+        binding.attnw_fused(q, q, -1.0)
+    assert e.value.code == 2
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_given_output_and_stream(binding, dtype):
+    q, k = small_fused_inputs(1, 2, 200, 64, stream=5)
+    Q, K = bits_to_cuda_bf16(q), bits_to_cuda_bf16(k)
+    P = torch.empty(1, 2, 200, 200, dtype=dtype, device="cuda")
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    for stream in (s, s.cuda_stream):
+        P.fill_(float("nan"))
+        torch.cuda.synchronize()
+        assert binding.attnw_fused(Q, K, np.float32(0.125), P=P, stream=stream) is P
+        s.synchronize()
+        assert_close_to_oracle(P, oracle.attnw(q, k, 0.125), f"{dtype}")
