@@ -68,11 +68,12 @@ int attnw_fused_f32(const void* Q, const void* K, void* P, int B, int H, int N, 
  * synchronisation, or in a process that has handed the rest of the GPU's memory to someone else.  attnw_fused itself
  * allocates its exchange area with cudaMalloc the first time it runs the grid-row kernel on a device; this entry
  * point never calls cudaMalloc, cudaFree or any other allocating routine.  Its exchange area is a fixed array inside
- * the library's device image (1.25 MiB, present on every GPU that loads the library until the process exits).
+ * the library's device image (3 MiB, present on every GPU that loads the library until the process exits).
  *
  * Arguments, layout and result are those of attnw_fused.  Limits, each refused with a status code and no launch:
  *   N <= 4096 (ATTNW_ERR_UNSUPPORTED beyond: one group of the grid-row kernel holds at most 4096 keys), and a device
  *   on which one group fits among at most 160 resident CTAs (the array has entries for 160; a B200 uses 144 or 148).
+ * Captured in a graph, the call clears the array (3 MB) before each replay.
  * First call on a device: looks up the array's device address (cudaGetSymbolAddress) and the device's properties.
  *   Make that first call before any stream capture begins.
  * Every call on a device shares the one array, which keeps what the previous call left in it; the messages carry
@@ -127,10 +128,11 @@ int attnw_set_attn_variant(int variant);
 
 /*
  * Which kernel attnw_fused uses (process-wide; the results are the same within the stated tolerances):
- *   0  choose by shape (default): the grid-row kernel (see 4) when P is bfloat16 and N <= 4096; the two-pass
- *      kernel otherwise (and always for attnw_fused_f32).  On a device that cannot hold a whole group of the
- *      grid-row kernel at once the older choice applies: the SRAM-resident cluster kernel, with a large call split
- *      between it and the two-pass kernel on a per-device side stream that forks from and joins `stream` with events.
+ *   0  choose by shape (default): the grid-row kernel (see 4; here it serves both types of P) for rows of up to 14336 keys
+ *      whose groups leave at most a quarter of the SMs idle (every N <= 4096 on a B200); the two-pass kernel otherwise.
+ *      On a device that cannot hold a whole group of the grid-row kernel at once the older choice applies: the SRAM-resident
+ *      cluster kernel for bfloat16 P, with a large call split between it and the two-pass kernel on a per-device side
+ *      stream that forks from and joins `stream` with events.
  *   1  two-pass kernel: statistics pass + normalise pass that recomputes the score tiles; any N
  *   2  SRAM-resident kernel: a cluster of ceil(N/512) <= 16 CTAs keeps a 128-row block of scores in tensor
  *      memory and exchanges local row maxima and sums across CTAs, as the fused kernel of Section VII
@@ -140,12 +142,12 @@ int attnw_set_attn_variant(int variant);
  *      the CTAs of the cluster, the owner of a row receives its local maxima and sums, reduces them once and
  *      sends the global values to every CTA (reduce and broadcast) instead of every CTA reducing redundantly
  *   4  grid-row kernel: the SRAM-resident design on a cooperative grid of one CTA per SM.  Consecutive ceil(N/256)
- *      CTAs form a group (the cores of one grid row in Section VII) that owns a 128-row block; every CTA keeps its
- *      128 x 256 slab of scores in half of its tensor memory, so two row blocks are in flight per CTA, and the local
- *      row maxima and sums cross the group through L2 as tagged 16-byte messages in per-device exchange areas (4.7 MB)
- *      that the library allocates on first use (cudaMalloc; never inside a stream capture).  Serves bfloat16 P and
- *      N <= 4096; any other call then returns ATTNW_ERR_UNSUPPORTED.  Launches take the exchange areas in turn, so calls on
- *      different streams of one device are safe as long as fewer than four of them are in flight at once.
+ *      CTAs form a group (the cores of one grid row in Section VII) that owns a 128-row block; every CTA keeps the
+ *      exponentials of its 128 x 256 slab in tensor memory, with three row blocks in flight, and the local row maxima and
+ *      sums cross the group through L2 as tagged 16-byte messages in an exchange area (3 MB) that belongs to the stream:
+ *      one is allocated when a stream makes its first such call (cudaMalloc), up to eight per device, which further
+ *      streams share in turn.  On a stream that is being captured the choice by shape (0) takes the other kernels
+ *      for N > 256.  On request (4) it serves bfloat16 P and N <= 4096; any other call then returns ATTNW_ERR_UNSUPPORTED.
  * Returns ATTNW_ERR_BAD_SHAPE for any other value.
  */
 int attnw_set_fused_variant(int variant);

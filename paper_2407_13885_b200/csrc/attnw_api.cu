@@ -26,9 +26,7 @@ namespace {
 
 using namespace attnw;
 
-// Consecutive launches of the grid-row kernel use different exchange areas in turn: the last CTAs of one launch may still
-// be reading the pairs of their last row block when the next launch (which starts as soon as its whole grid fits) posts.
-constexpr int kGridrowAreas = 4;
+constexpr int kMaxGridrowAreas = 8;  // exchange areas of the grid-row kernel per device
 constexpr uint32_t kSiteSelfTest = 127;  // wait site of attnw_selftest_wait_timeout (low byte of the status word)
 
 // Not part of any product path: one thread waits, with the caller's limit, on an mbarrier that nobody arrives on,
@@ -78,17 +76,29 @@ struct DeviceInfo {
     // fork/join objects for launches that split a call over two kernels (created on first use)
     cudaStream_t side_stream = nullptr;
     cudaEvent_t fork_event = nullptr, join_event = nullptr;
-    // grid-row kernel: co-resident CTAs per head dimension (0 = not asked yet), the exchange area in device memory
-    // (created on first use, zeroed once) and the next unused message tag
-    int gridrow_ctas[2] = {};
-    uint4* gridrow_xchg = nullptr;
-    int gridrow_xchg_ctas = 0;
-    uint32_t gridrow_tag = 0;
-    unsigned gridrow_launches = 0;  // selects one of kGridrowAreas exchange areas in turn
     int rc_clusters[2][17] = {};  // resident clusters of 1..16 CTAs of the register-cluster row kernel, [P is float32][CTAs]
 };
 std::mutex g_split_mutex;
 DeviceInfo g_devices[kMaxDevices];
+
+// Exchange areas of the grid-row kernel.  A launch owns its area until it ends; launches on one stream follow each other,
+// so a stream keeps the area it has, and a program with one stream uses one.  A stream that has none takes a new one, up
+// to kMaxGridrowAreas per device, or one whose last launch is known to have ended, or else waits for the area that was
+// given to its stream first.  Stream ids are never used twice, unlike stream handles.
+struct GridrowArea {
+    uint4* xchg = nullptr;
+    unsigned long long stream_id = 0;
+    uint32_t tag = 0;           // the next unused message tag
+    cudaEvent_t last = nullptr; // the end of the last launch ...
+    bool recorded = false;      // ... if it was recorded: not while the device has had one stream only
+};
+struct GridrowAreas {
+    std::mutex mutex;  // held over the launch, so that no other stream takes the area before its event is recorded
+    GridrowArea area[kMaxGridrowAreas];
+    int count = 0, next_victim = 0;
+    bool several_streams = false;
+};
+GridrowAreas g_gridrow_areas[kMaxDevices];
 
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -342,89 +352,151 @@ int launch_resident(DeviceInfo* dev, const void* Q, const void* K, void* P, int 
                  : launch_resident_impl<D, 16, false>(dev, Q, K, P, BH, N, scale, stream);
 }
 
-// Grid-row kernel: a cooperative grid of one CTA per SM; consecutive ceil(N / 256) CTAs form a group that owns a
-// 128-row block and walks a contiguous part of the list of row blocks.  Returns ATTNW_ERR_UNSUPPORTED when the
-// device cannot hold a whole group at once.
-template <int D>
-int launch_gridrow(DeviceInfo* dev, const void* Q, const void* K, void* P, int BH, int N, float scale, cudaStream_t stream) {
+// The geometry of a grid-row launch: groups of ceil(N / 256) CTAs, as many as fit one CTA per SM and have work.
+struct GridrowShape {
+    int group_ctas, n_groups, total_items;
+    uint32_t longest;  // row blocks of the longest list = message tags the launch uses
+};
+// Returns ATTNW_ERR_UNSUPPORTED when `max_ctas` cannot hold a whole group.
+int gridrow_shape(int BH, int N, int max_ctas, GridrowShape* out) {
+    const long long total = static_cast<long long>(BH) * ((N + kTile - 1) / kTile);
+    if (total > INT_MAX) return ATTNW_ERR_BAD_SHAPE;
+    out->group_ctas = (N + gr::kSlabCols - 1) / gr::kSlabCols;
+    if (out->group_ctas > max_ctas || out->group_ctas > gr::kMaxGroupCtas) return ATTNW_ERR_UNSUPPORTED;
+    out->total_items = static_cast<int>(total);
+    out->n_groups = max_ctas / out->group_ctas;
+    if (out->n_groups > total) out->n_groups = out->total_items;
+    out->longest = static_cast<uint32_t>((total + out->n_groups - 1) / out->n_groups);
+    return ATTNW_OK;
+}
+// 16-byte entries of an exchange area that serves every grid of up to `max_ctas` CTAs: the pairs of each CTA and, where the
+// rows have owners (groups of more than kMaxDirectCtas), the results of each group.
+constexpr size_t gridrow_entries(int max_ctas) {
+    return static_cast<size_t>(max_ctas + max_ctas / (gr::kMaxDirectCtas + 1)) * gr::kXchgDepth * kTile;
+}
+
+// Returns ATTNW_ERR_UNSUPPORTED when the grid does not fit at once after all (SMs taken away from this context).
+template <int D, typename OutT>
+int enqueue_gridrow(const GridrowShape& g, const void* Q, const void* K, void* P, int BH, int N, float scale, uint4* xchg,
+                    uint32_t tag_base, cudaStream_t stream) {
     using L = gr::Smem<D>;
-    auto kernel = gr::attnw_gridrow_kernel<D>;
+    auto kernel = gr::attnw_gridrow_kernel<D, OutT>;
     CUtensorMap tm_q, tm_k, tm_p;
     int rc = encode_3d(&tm_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Q, D, N, BH, 64, kTile);
     if (rc == ATTNW_OK) rc = encode_3d(&tm_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, D, N, BH, 64, kTile);
-    if (rc == ATTNW_OK) rc = encode_3d(&tm_p, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, P, N, N, BH, 64, kTile);
+    if (rc == ATTNW_OK)
+        rc = encode_3d(&tm_p, sizeof(OutT) == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sizeof(OutT), P,
+                       N, N, BH, 128 / sizeof(OutT), 32);
     if (rc != ATTNW_OK) return rc;
-    if (allow_smem<gr::attnw_gridrow_kernel<D>>(L::kDynamicBytes) != cudaSuccess) {
+    if (allow_smem<gr::attnw_gridrow_kernel<D, OutT>>(L::kDynamicBytes) != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
-    }
-    const int group_ctas = (N + gr::kSlabCols - 1) / gr::kSlabCols;
-    const int row_blocks = (N + kTile - 1) / kTile;
-    const long long total_items = static_cast<long long>(BH) * row_blocks;
-    if (total_items > INT_MAX) return ATTNW_ERR_BAD_SHAPE;
-    uint4* xchg = nullptr;
-    uint32_t tag_base = 0;
-    int n_groups = 0;
-    {
-        std::lock_guard<std::mutex> lock(g_mutex);
-        int& max_ctas = dev->gridrow_ctas[D == 128 ? 1 : 0];
-        if (max_ctas == 0) {
-            int per_sm = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, gr::kThreads, L::kDynamicBytes) != cudaSuccess ||
-                per_sm < 1) {
-                (void)cudaGetLastError();
-                max_ctas = -1;
-            } else {
-                max_ctas = dev->sm_count;  // one CTA per SM: the kernel takes all of tensor memory
-            }
-        }
-        if (max_ctas < group_ctas) return ATTNW_ERR_UNSUPPORTED;
-        n_groups = max_ctas / group_ctas;
-        if (n_groups > total_items) n_groups = static_cast<int>(total_items);
-        if (dev->gridrow_xchg == nullptr || dev->gridrow_xchg_ctas < max_ctas) {
-            // first use on this device: the exchange area, zero so that no entry carries a valid tag
-            if (dev->gridrow_xchg) cudaFree(dev->gridrow_xchg);
-            dev->gridrow_xchg = nullptr;
-            const size_t bytes = static_cast<size_t>(kGridrowAreas) * max_ctas * gr::kXchgDepth * kTile * sizeof(uint4);
-            void* p = nullptr;
-            if (cudaMalloc(&p, bytes) != cudaSuccess || cudaMemset(p, 0, bytes) != cudaSuccess ||
-                cudaDeviceSynchronize() != cudaSuccess) {
-                (void)cudaGetLastError();
-                if (p) cudaFree(p);
-                return ATTNW_ERR_CUDA;
-            }
-            dev->gridrow_xchg = static_cast<uint4*>(p);
-            dev->gridrow_xchg_ctas = max_ctas;
-            dev->gridrow_tag = 0;
-        }
-        xchg = dev->gridrow_xchg + static_cast<size_t>(dev->gridrow_launches++ % kGridrowAreas) * dev->gridrow_xchg_ctas *
-                                       gr::kXchgDepth * kTile;
-        // tags tag_base + 1 ... tag_base + (longest list) belong to this launch; 0 is never a tag
-        const uint32_t longest = static_cast<uint32_t>((total_items + n_groups - 1) / n_groups);
-        if (dev->gridrow_tag > 0xffffffffu - longest - 1u) dev->gridrow_tag = 0;
-        tag_base = dev->gridrow_tag;
-        dev->gridrow_tag += longest;
     }
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;  // every CTA of the grid is resident at once, or the launch fails
     attr[0].val.cooperative = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(gr::kThreads, 1, 1);
-    cfg.gridDim = dim3(static_cast<unsigned>(n_groups * group_ctas), 1, 1);
+    cfg.gridDim = dim3(static_cast<unsigned>(g.n_groups * g.group_ctas), 1, 1);
     cfg.dynamicSmemBytes = L::kDynamicBytes;
     cfg.stream = stream;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = g.group_ctas > 1 ? 1 : 0;  // groups of one CTA wait for nobody
     const float scale_log2e = static_cast<float>(static_cast<double>(scale) * 1.4426950408889634074);
-    const cudaError_t launched = cudaLaunchKernelEx(&cfg, kernel, tm_q, tm_k, tm_p, N, static_cast<int>(total_items), group_ctas,
-                                                    n_groups, scale_log2e, xchg, tag_base);
+    const cudaError_t launched =
+        cudaLaunchKernelEx(&cfg, kernel, tm_q, tm_k, tm_p, N, g.total_items, g.group_ctas, g.n_groups, scale_log2e, xchg, tag_base);
     if (launched != cudaSuccess) {
         (void)cudaGetLastError();
-        // the grid does not fit at once after all (SMs taken away from this context): let the caller choose another kernel
         return launched == cudaErrorCooperativeLaunchTooLarge ? ATTNW_ERR_UNSUPPORTED : ATTNW_ERR_CUDA;
     }
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return ATTNW_OK;
+}
+
+// The exchange area that a launch on `stream` uses; called with the areas' mutex held.
+int gridrow_area(GridrowAreas* areas, int sm_count, cudaStream_t stream, GridrowArea** out) {
+    unsigned long long id = 0;
+    if (cudaStreamGetId(stream, &id) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return ATTNW_ERR_CUDA;
+    }
+    for (int a = 0; a < areas->count; ++a)
+        if (areas->area[a].stream_id == id) {
+            *out = &areas->area[a];
+            return ATTNW_OK;
+        }
+    // The calls below are allowed while another thread captures a stream.
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    areas->several_streams = areas->count > 0;
+    int rc = ATTNW_OK;
+    GridrowArea* area = nullptr;
+    for (int a = 0; a < areas->count && !area; ++a)
+        if (areas->area[a].recorded && cudaEventQuery(areas->area[a].last) == cudaSuccess) area = &areas->area[a];
+    if (!area && areas->count < kMaxGridrowAreas) {
+        GridrowArea fresh;
+        const size_t bytes = gridrow_entries(sm_count) * sizeof(uint4);
+        void* p = nullptr;
+        // zero, so that no entry carries a valid tag
+        if (cudaMalloc(&p, bytes) != cudaSuccess || cudaMemset(p, 0, bytes) != cudaSuccess ||
+            cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess ||
+            cudaEventCreateWithFlags(&fresh.last, cudaEventDisableTiming) != cudaSuccess) {
+            if (p) cudaFree(p);
+            rc = ATTNW_ERR_UNSUPPORTED;  // no memory for it: the caller takes a kernel that needs none
+        } else {
+            fresh.xchg = static_cast<uint4*>(p);
+            area = &areas->area[areas->count++];
+            *area = fresh;
+        }
+    } else if (!area) {
+        for (int tries = 0; tries < kMaxGridrowAreas && !area; ++tries) {
+            GridrowArea* victim = &areas->area[areas->next_victim++ % kMaxGridrowAreas];
+            if (victim->recorded) area = victim;  // (all but the first stream's always are)
+        }
+        if (!area)
+            rc = ATTNW_ERR_UNSUPPORTED;
+        else if (cudaStreamWaitEvent(stream, area->last, 0) != cudaSuccess)
+            rc = ATTNW_ERR_CUDA;
+    }
+    (void)cudaGetLastError();  // cudaErrorNotReady of the queries
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (rc != ATTNW_OK) return rc;
+    area->stream_id = id;
+    area->recorded = false;
+    *out = area;
+    return ATTNW_OK;
+}
+
+// Grid-row kernel: a cooperative grid of one CTA per SM; consecutive ceil(N / 256) CTAs form a group that owns a
+// 128-row block and walks a contiguous part of the list of row blocks.  Returns ATTNW_ERR_UNSUPPORTED when the
+// device cannot hold a whole group at once, and for groups of several CTAs on a stream that is being captured.
+template <int D, typename OutT>
+int launch_gridrow(DeviceInfo* dev, const void* Q, const void* K, void* P, int BH, int N, float scale, cudaStream_t stream) {
+    GridrowShape g;
+    int rc = gridrow_shape(BH, N, dev->sm_count, &g);
+    if (rc != ATTNW_OK) return rc;
+    if (g.group_ctas == 1) return enqueue_gridrow<D, OutT>(g, Q, K, P, BH, N, scale, nullptr, 0, stream);
+    // A captured launch would be replayed with the tags of its capture, at any time beside any other launch.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return ATTNW_ERR_CUDA;
+    }
+    if (capture != cudaStreamCaptureStatusNone) return ATTNW_ERR_UNSUPPORTED;
+    GridrowAreas& areas = g_gridrow_areas[dev - g_devices];
+    std::lock_guard<std::mutex> lock(areas.mutex);
+    GridrowArea* area = nullptr;
+    rc = gridrow_area(&areas, dev->sm_count, stream, &area);
+    if (rc != ATTNW_OK) return rc;
+    // tags area->tag + 1 ... area->tag + (longest list) belong to this launch; 0 is never a tag
+    if (area->tag > 0xffffffffu - g.longest - 1u) area->tag = 0;
+    rc = enqueue_gridrow<D, OutT>(g, Q, K, P, BH, N, scale, area->xchg, area->tag, stream);
+    area->tag += g.longest;
+    if (rc == ATTNW_OK && areas.several_streams) {
+        area->recorded = cudaEventRecord(area->last, stream) == cudaSuccess;
+        if (!area->recorded) rc = ATTNW_ERR_CUDA;
+    }
+    return rc;
 }
 
 template <int D>
@@ -537,6 +609,17 @@ int launch_project(const void* X, const void* Wq, const void* Wk, void* Q, void*
     return ATTNW_OK;
 }
 
+// Whether the choice by shape takes the grid-row kernel for rows of N keys: it computes every score and exponential once, the
+// two-pass kernel twice, but groups of ceil(N / 256) CTAs leave SMs idle and the exchange grows with the group.
+// Measured on B200, us per call, two-pass -> grid-row: bfloat16, d = 64 or 128, B*H x N = 2 x 6000 (24 CTAs a group,
+// 144 SMs in use) 132 -> 45, 8 x 8192 (32, 128 SMs) 435 -> 360, 4 x 12288 (48, 144 SMs) 421 -> 335, 1 x 16384 (64, 128 SMs)
+// 189 -> 219; float32 2 x 512 16.4 -> 10.2, 20 x 1000 36.9 -> 22.6, 16 x 2052 111 -> 79, 32 x 4096 616 -> 506,
+// 4 x 8192 315 -> 244, 1 x 16384 314 -> 340.  So: groups of up to 56 that leave at most a quarter of the SMs idle.
+bool gridrow_pays(const DeviceInfo* dev, int N) {
+    const int group_ctas = (N + gr::kSlabCols - 1) / gr::kSlabCols;
+    return group_ctas <= 56 && dev->sm_count / group_ctas * group_ctas * 4 >= dev->sm_count * 3;
+}
+
 template <typename OutT>
 int fused_entry(const void* Q, const void* K, void* P, int B, int H, int N, int d, float scale, void* stream) {
     int rc = validate_fused(Q, K, P, B, H, N, d, scale, sizeof(OutT));
@@ -553,8 +636,8 @@ int fused_entry(const void* Q, const void* K, void* P, int B, int H, int N, int 
     if (variant == 4) {
         if constexpr (sizeof(OutT) == 2) {
             if (N > gr::kMaxN) return ATTNW_ERR_UNSUPPORTED;
-            return (d == 64) ? launch_gridrow<64>(dev, Q, K, P, B * H, N, scale, s)
-                             : launch_gridrow<128>(dev, Q, K, P, B * H, N, scale, s);
+            return (d == 64) ? launch_gridrow<64, OutT>(dev, Q, K, P, B * H, N, scale, s)
+                             : launch_gridrow<128, OutT>(dev, Q, K, P, B * H, N, scale, s);
         }
         return ATTNW_ERR_UNSUPPORTED;
     }
@@ -564,18 +647,12 @@ int fused_entry(const void* Q, const void* K, void* P, int B, int H, int N, int 
                              : launch_resident<128>(dev, Q, K, P, B * H, N, scale, s, true);
         return ATTNW_ERR_UNSUPPORTED;
     }
-    // Choice by shape, first candidate: the grid-row kernel (bfloat16 P, N <= 4096).  Measured against the cluster
-    // kernel with its split launch and against the two-pass kernel over 19 shapes (B*H = 1 ... 128, N = 256 ... 4096,
-    // d = 64 and 128) it was ahead on every one (3 to 18 %), because it runs on every SM and keeps three row blocks
-    // in flight per CTA.  A device that cannot hold a whole group at once falls through to the older choice.
-    if (variant == 0) {
-        if constexpr (sizeof(OutT) == 2) {
-            if (N <= gr::kMaxN) {
-                rc = (d == 64) ? launch_gridrow<64>(dev, Q, K, P, B * H, N, scale, s)
-                               : launch_gridrow<128>(dev, Q, K, P, B * H, N, scale, s);
-                if (rc != ATTNW_ERR_UNSUPPORTED) return rc;
-            }
-        }
+    // Choice by shape, first candidate: the grid-row kernel, where its groups fit the device well (see gridrow_pays).
+    // A device that cannot hold a whole group at once falls through to the older choice.
+    if (variant == 0 && gridrow_pays(dev, N)) {
+        rc = (d == 64) ? launch_gridrow<64, OutT>(dev, Q, K, P, B * H, N, scale, s)
+                       : launch_gridrow<128, OutT>(dev, Q, K, P, B * H, N, scale, s);
+        if (rc != ATTNW_ERR_UNSUPPORTED) return rc;
     }
     // Older choice by shape: the resident kernel whenever it can serve the call.  It spreads one 128-row block over the
     // C SMs of a cluster, so it also fills the device when B*H is small (B*H = 1, N = 4096, d = 128: 25 us
@@ -750,11 +827,11 @@ constexpr unsigned long long kHostChunkBytes = 256ull << 20;  // target size of 
 
 // ---- attnw_fused_noalloc: the grid-row kernel with its exchange area in a static device array ----------------
 // Scratch of the entry point that allocates nothing: the exchange area of the grid-row kernel for a grid of up to
-// kNoAllocMaxCtas CTAs (messages of 16 bytes: [CTA][4 row blocks in flight][128 rows]) = 1.25 MiB, held by every
+// kNoAllocMaxCtas CTAs (messages of 16 bytes: [CTA or group][8 row blocks][128 rows]) = 3 MiB, held by every
 // GPU that loads the library until the process exits.  In host code this name is only a stand-in for the symbol:
 // the device address comes from cudaGetSymbolAddress (noalloc_setup below) and is what the kernel is given.
 constexpr int kNoAllocMaxCtas = 160;
-static __device__ __align__(256) uint4 g_noalloc_xchg[kNoAllocMaxCtas * gr::kXchgDepth * kTile];
+static __device__ __align__(256) uint4 g_noalloc_xchg[gridrow_entries(kNoAllocMaxCtas)];
 
 struct NoAllocState {
     bool ready = false;
@@ -797,58 +874,32 @@ int noalloc_setup(NoAllocState** out) {
 template <int D>
 int launch_gridrow_noalloc(NoAllocState* st, const void* Q, const void* K, void* P, int BH, int N, float scale,
                            cudaStream_t stream) {
-    using L = gr::Smem<D>;
-    auto kernel = gr::attnw_gridrow_kernel<D>;
-    CUtensorMap tm_q, tm_k, tm_p;
-    int rc = encode_3d(&tm_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Q, D, N, BH, 64, kTile);
-    if (rc == ATTNW_OK) rc = encode_3d(&tm_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, D, N, BH, 64, kTile);
-    if (rc == ATTNW_OK) rc = encode_3d(&tm_p, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, P, N, N, BH, 64, kTile);
-    if (rc != ATTNW_OK) return rc;
-    if (allow_smem<gr::attnw_gridrow_kernel<D>>(L::kDynamicBytes) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return ATTNW_ERR_CUDA;
-    }
-    const int group_ctas = (N + gr::kSlabCols - 1) / gr::kSlabCols;
-    const long long total_items = static_cast<long long>(BH) * ((N + kTile - 1) / kTile);
-    if (total_items > INT_MAX) return ATTNW_ERR_BAD_SHAPE;
     // one CTA per SM, whole groups only, and never more CTAs than the static array has entries for
-    const int max_ctas = st->sm_count < kNoAllocMaxCtas ? st->sm_count : kNoAllocMaxCtas;
-    if (max_ctas < group_ctas) return ATTNW_ERR_UNSUPPORTED;
-    int n_groups = max_ctas / group_ctas;
-    if (n_groups > total_items) n_groups = static_cast<int>(total_items);
+    GridrowShape g;
+    const int rc = gridrow_shape(BH, N, st->sm_count < kNoAllocMaxCtas ? st->sm_count : kNoAllocMaxCtas, &g);
+    if (rc != ATTNW_OK) return rc;
     uint32_t tag_base = 0;
     {
         std::lock_guard<std::mutex> lock(g_mutex);
-        const uint32_t longest = static_cast<uint32_t>((total_items + n_groups - 1) / n_groups);
-        if (st->tag > 0xffffffffu - longest - 1u) {
-            // the tags are used up (after about 4e9 row blocks): start again from a cleared array, in stream order
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return ATTNW_ERR_CUDA;
+        }
+        if (capture != cudaStreamCaptureStatusNone || st->tag > 0xffffffffu - g.longest - 1u) {
+            // A captured launch is replayed with the same tags, or the tags are used up (after about 4e9 row blocks): start
+            // again from a cleared array, in stream order.
             if (cudaMemsetAsync(st->xchg, 0, sizeof(g_noalloc_xchg), stream) != cudaSuccess) {
                 (void)cudaGetLastError();
                 return ATTNW_ERR_CUDA;
             }
-            st->tag = 0;
+            if (capture == cudaStreamCaptureStatusNone) st->tag = 0;
         }
         tag_base = st->tag;
-        st->tag += longest;
+        st->tag += g.longest;
     }
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(gr::kThreads, 1, 1);
-    cfg.gridDim = dim3(static_cast<unsigned>(n_groups * group_ctas), 1, 1);
-    cfg.dynamicSmemBytes = L::kDynamicBytes;
-    cfg.stream = stream;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const float scale_log2e = static_cast<float>(static_cast<double>(scale) * 1.4426950408889634074);
-    if (cudaLaunchKernelEx(&cfg, kernel, tm_q, tm_k, tm_p, N, static_cast<int>(total_items), group_ctas, n_groups, scale_log2e,
-                           st->xchg, tag_base) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return ATTNW_ERR_CUDA;
-    }
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    return ATTNW_OK;
+    const int launched = enqueue_gridrow<D, __nv_bfloat16>(g, Q, K, P, BH, N, scale, st->xchg, tag_base, stream);
+    return launched == ATTNW_ERR_UNSUPPORTED ? ATTNW_ERR_CUDA : launched;
 }
 
 }  // namespace

@@ -3,41 +3,49 @@
 //
 // The paper lays the score matrix out over a grid of cores; the cores of one grid row hold the pieces of the
 // same rows of scores, compute LOCAL row maxima and sums and exchange them to obtain the GLOBAL ones before
-// normalising (Section VII; Eq. 1).  Here a group of C = ceil(N / 256) <= 16 CTAs owns a 128-row block of one
-// head; CTA r of the group works on the 128 x 256 slab of scores for keys [256 r, 256 r + 256).  Tensor cores
-// and exponentials run once per element, and three row blocks are in flight per CTA:
-//   tensor-memory columns [0, 256)    two landing slots of 128 columns: the MMA writes float32 scores here; a slot
-//                                     goes back to the MMA issuer as soon as its scores are in registers
-//   tensor-memory columns [256, 512)  two packed regions (one per stream = row blocks of equal parity): the
-//                                     exponentials as f16 pairs, waiting for the row's statistics
-// so the next row block's scores are computed, and its exponentials taken, while the statistics of the previous
-// ones cross the group.  (f16 keeps 11 bits of e in [0, 1]: 5e-4 relative, next to the 2e-3 of the bf16 result.)
+// normalising (Section VII; Eq. 1).  Here a group of C = ceil(N / 256) CTAs owns a 128-row block of one head; CTA r
+// of the group works on the 128 x 256 slab of scores for keys [256 r, 256 r + 256).  Tensor cores and exponentials
+// run once per element.
+//
+// Tensor memory, bfloat16 output:
+//   columns [0, 128)    the landing slot: the MMA writes float32 scores of 128 keys here; it goes back to the MMA issuer
+//                       as soon as its scores are in registers
+//   columns [128, 512)  three packed regions, used by the row blocks in turn: the exponentials as f16 pairs, waiting
+//                       for the row's statistics
+// so two further row blocks can be computed, and their exponentials taken, while the statistics of one cross the
+// group.  (f16 keeps 11 bits of e in [0, 1]: 5e-4 relative, next to the 2e-3 of the bf16 result.)
+// Tensor memory, float32 output: two regions of 256 columns; the exponentials replace the scores as float32, and a slot of
+// 128 columns goes back to the MMA issuer when its weights have been staged.
 //
 // Groups are not hardware clusters (clusters of 8 or 16 CTAs cannot occupy every SM): the grid is launched
 // cooperatively with one CTA per SM, consecutive CTAs form a group, and the 16-byte (offset, sum) pair of a row
 // travels through L2 as two 8-byte words that each carry a tag {value, tag, value, tag}; a reader accepts a
 // pair once both tags name the row block it is waiting for.  No fence, no flag, no atomics: the tag arrives
 // with the value in one 8-byte store.  Every poll is bounded.
+//   C = 1          no exchange: the pair stays in shared memory
+//   2 <= C <= 4    every CTA reads the C pairs of each row and reduces them redundantly, as the paper's kernel does
+//   C > 4          the rows of a block are dealt out to the CTAs; a row's owner reads its C pairs, reduces them once and
+//                  posts (M, 1/L) for all (the exchange of Section VIII).  One more hop through L2, but two loads per row
+//                  and CTA instead of C, and C may be larger than 16.
 //
-// Roles of a CTA (640 threads, 20 warps; warp w may touch TMEM lanes 32 (w % 4) ...):
-//   warps 0-7    exponentials, all eight on ONE row block at a time: two threads per row, thread (row, p) takes the
-//                64-column boxes p and p + 2 of the slab: scores to registers, maximum, offset mb, e = 2^(c s - mb),
-//                sum, e packed to f16 pairs into the stream's packed region; the thread's (mb, l) to shared memory;
-//                the second of a row's two warps to finish merges the halves and posts the row's pair
-//   warps 8-11   normalise, stream 0 (12-15: stream 1): a thread owns one row; waits for the C pairs of the row, forms M and 1/L - every CTA reduces redundantly, as
-//                the paper's kernel does -, then per box p = e * 2^(mb_box - M) / L (one mixed-precision FMA per
-//                element unpacks and scales), rounded to bf16, staged in 128-row boxes
-//   warp 16      TMA producer: the CTA's key slab once per head (it stays in shared memory while the group walks
-//                the head's row blocks), one 32 KB query tile per row block
-//   warp 17      tcgen05.mma issuer (one elected lane), 128 x 128 x 16 per instruction
-//   warps 18-19  store issuers, one per stream: one TMA store per filled box; P is written exactly once
-// Valid for N <= 4096 keys and bf16 output.
+// Roles of a CTA (896 threads, 28 warps; warp w may touch TMEM lanes 32 (w % 4) ...):
+//   warps 0-15   exponentials, all sixteen on ONE row block at a time: four threads per row, thread (row, g) takes columns
+//                [32 g, 32 g + 32) of both slots: scores to registers, maximum, offset mb, e = 2^(c s - mb), sum, e back
+//                to tensor memory; the thread's (mb, l) to shared memory; the last of a row's four warps to finish
+//                merges the parts and posts the row's pair
+//   warps 16-19  normalise the even row blocks (20-23: the odd ones): a thread owns one row; takes the row's M and 1/L,
+//                then per box of 128 bytes a row p = e * 2^(mb - M) / L, rounded to the output type, staged and stored by
+//                one TMA store per warp (32 rows x 128 bytes) and box; P is written exactly once
+//   warp 24      TMA producer: the CTA's key slab once per head (it stays in shared memory while the group walks
+//                the head's row blocks), one query tile per row block
+//   warp 25      tcgen05.mma issuer (one elected lane)
+//   warps 26-27  the owner's reduction of the row block, half of its rows each
 //
 // With -DATTNW_TIMELINE=<CTA> one lane per role of that CTA stamps clock64() per row block (events, by index):
-//   13 MMA of the block issued | 0 exponentials begin, 2 slot 0 ready, 17/20 load of box k, 16/19 maximum known,
-//   18/21 exponentials of box k done, 24/26 packed e stored, 4 halves posted | 10 normalise begins to wait,
-//   6 halves seen + pair posted, 11 all pairs seen, 12 box 0 read, 14/15/8/9 box 2 read / staging free / staged /
-//   handed to the store issuer, 7 block done.
+//   13 MMA of the block issued | 0 exponentials begin, 2 slot 0 ready, 17/20 load of slot k, 16/19 maximum known,
+//   18/21 exponentials of slot k done, 24/26 e stored, 4 parts posted | 22 owner begins to wait, 23 pairs seen,
+//   25 result posted | 10 normalise begins to wait, 6 own CTA done, 11 statistics seen, 12 box 0 read,
+//   14/15/8/9 box 2 read / staging free / staged / stored, 7 block done.
 #pragma once
 #include "attnw_resident.cuh"
 
@@ -45,21 +53,23 @@ namespace attnw {
 namespace gr {
 
 constexpr int kSlabCols = 256;                       // key columns per CTA and row block
-constexpr int kSub = 128;                            // columns per MMA landing slot
-constexpr int kSubsPerBlock = kSlabCols / kSub;      // 2 landing slots = tensor-memory columns [0, 256)
-constexpr int kPackedCol0 = kSlabCols;               // packed exponentials: columns [256, 512), 128 per stream
+constexpr int kSub = 128;                            // columns per MMA slot
+constexpr int kSubsPerBlock = kSlabCols / kSub;
+constexpr int kPackedCol0 = kSub;                    // packed exponentials: columns [128, 512), 128 per region
 constexpr int kPackedCols = kSlabCols / 2;           // two f16 per 32-bit column
-constexpr int kBoxCols = 64;                         // columns of one staged store box (128 bytes of bf16)
 constexpr int kChunksPerBlock = kSlabCols / kChunk;  // 32-column chunks, each with its own offset
-constexpr int kThreads = 640;                        // 8 exponential + 8 normalise warps, producer, MMA issuer, 2 store issuers
-constexpr int kNormWarp0 = 8;
-constexpr int kNormGroups = 2;                       // normalise warpgroups: one per stream
-constexpr int kProducerWarpG = kNormWarp0 + 4 * kNormGroups;
+constexpr int kExpWarps = 16;
+constexpr int kParts = kExpWarps / 4;                // threads per row
+constexpr int kNormWarp0 = kExpWarps;
+constexpr int kProducerWarpG = kNormWarp0 + 8;
 constexpr int kMmaWarpG = kProducerWarpG + 1;
-constexpr int kStoreWarpG = kProducerWarpG + 2;
-constexpr int kMaxGroupCtas = 16;
-constexpr int kMaxN = kSlabCols * kMaxGroupCtas;
-constexpr int kXchgDepth = 4;    // row blocks i and i + 4 of a group share exchange entries (see the proof at the poll)
+constexpr int kOwnerWarpG = kProducerWarpG + 2;
+constexpr int kThreads = 32 * (kOwnerWarpG + 2);
+constexpr int kStageBytes = 32 * 128;                // one staged store box: 32 rows x 128 bytes
+constexpr int kMaxDirectCtas = 4;                    // up to here every CTA reads all pairs of a row
+constexpr int kMaxGroupCtas = 128;
+constexpr int kMaxN = 4096;                          // what variant 4 and attnw_fused_noalloc serve
+constexpr int kXchgDepth = 8;    // row blocks i and i + 8 of a group share exchange entries (see the proof at the owner)
 
 enum : uint32_t {  // wait sites of this kernel (low byte of the status word)
     kSiteGrKEmpty = 32,
@@ -70,26 +80,23 @@ enum : uint32_t {  // wait sites of this kernel (low byte of the status word)
     kSiteGrSFull = 37,
     kSiteGrPosted = 38,
     kSiteGrExchange = 39,
-    kSiteGrStageFree = 40,
-    kSiteGrStageFilled = 41,
+    kSiteGrOwner = 42,
 };
 
 template <int D>
 struct Smem {
     static constexpr int kQStages = 2;  // query tiles in shared memory (with one, the load of the next tile shows: 1.28 against 1.13 ms)
-    static constexpr int kBoxes = (D == 128) ? (kQStages == 1 ? 7 : 5) : 8;  // staged store boxes of 128 rows x 128 bytes, in one ring per stream
-    static constexpr int kRing0 = (kBoxes + 1) / 2;    // (a ring has ONE filler: a parity wait is only valid one use ahead)
-    static constexpr int kRing1 = kBoxes - kRing0;
+    static constexpr int kStages = (D == 128) ? 2 : 4;  // staged boxes per normalise warp
     static constexpr int kAtoms = D / 64;
     static constexpr int kAtomBytes = kTile * 128;
     static constexpr int kTileBytes = kAtoms * kAtomBytes;
     static constexpr int kKAtomBytes = kSlabCols * 128;                 // key slab, atom-major: [d / 64][256 keys][128 bytes]
     static constexpr int kKOff = 0;
-    static constexpr int kQOff = kKOff + 2 * kTileBytes;                // one query tile per stream
-    static constexpr int kOutOff = kQOff + kQStages * kTileBytes;       // staging boxes
-    static constexpr int kMbcOff = kOutOff + kBoxes * kBoxBytes;        // float mbc[2 streams][8][128 rows]: offset per box (4 of 8 in use)
-    static constexpr int kPartOff = kMbcOff + 2 * kChunksPerBlock * kTile * 4;  // float2 part[2 streams][2 halves][128 rows]
-    static constexpr int kBarOff = kPartOff + 2 * 2 * kTile * 8;
+    static constexpr int kQOff = kKOff + 2 * kTileBytes;
+    static constexpr int kOutOff = kQOff + kQStages * kTileBytes;       // staging boxes [8 warps][kStages]
+    static constexpr int kMbcOff = kOutOff + 8 * kStages * kStageBytes; // float mbc[3 regions][8 chunks][128 rows]: offset per chunk
+    static constexpr int kPartOff = kMbcOff + 3 * kChunksPerBlock * kTile * 4;  // float2 part[3 regions][4][128 rows]
+    static constexpr int kBarOff = kPartOff + 3 * kParts * kTile * 8;
     static constexpr int kBytes = kBarOff + 512;
     static constexpr int kDynamicBytes = kBytes + 1024;
 };
@@ -98,11 +105,10 @@ static_assert(Smem<128>::kDynamicBytes <= 227 * 1024 && Smem<64>::kDynamicBytes 
 struct Barriers {
     uint64_t k_full, k_empty;
     uint64_t q_full[2], q_empty[2];
-    uint64_t s_full[kSubsPerBlock], l_free[kSubsPerBlock];  // landing slots: scores ready / scores taken to registers
-    uint64_t pk_free[2][kSlabCols / kBoxCols];              // [stream][box]: the packed exponentials have been read
-    uint64_t posted[2];
-    uint64_t out_free[8], out_filled[8];
-    uint32_t halves_done[2][4];  // [stream][TMEM lane quarter]: exponential warps that have finished a row's halves (never reset)
+    uint64_t s_full[2 * kSubsPerBlock], s_free[2 * kSubsPerBlock];  // slots: scores ready / slot may be overwritten
+    uint64_t pk_free[3][kSlabCols / 64];                    // [region][64 columns]: the packed exponentials have been read
+    uint64_t posted[3];
+    uint32_t parts_done[3][4];   // [region][TMEM lane quarter]: exponential warps that have finished a row's parts (never reset)
     uint32_t tmem_base;
     uint32_t abort_flag;
     uint32_t prior_failure;
@@ -120,15 +126,51 @@ __device__ __forceinline__ uint4 ld_message(const uint4* p) {
     return v;
 }
 
-// xchg: [grid CTAs][kXchgDepth][128 rows] messages of 16 bytes, owned by the library, zero before first use.
+// Loads `n` <= K messages until all of them carry `tag` for every lane of the warp (entries beyond n repeat the last).
+// false = the time limit ran out, or another role gave up.
+template <int K, typename Addr>
+__device__ __forceinline__ bool poll_messages(uint4 (&v)[K], int n, uint32_t tag, volatile uint32_t* abort_flag, uint32_t site, Addr addr) {
+    const long long t0 = clock64();
+    for (uint32_t spin = 1;; ++spin) {
+        // all loads first, then the tags: one round trip to L2 a round
+#pragma unroll
+        for (int c = 0; c < K; ++c) v[c] = ld_message(addr(c < n ? c : n - 1));
+        bool valid = true;
+#pragma unroll
+        for (int c = 0; c < K; ++c) valid = valid && v[c].y == tag && v[c].w == tag;
+        if (__all_sync(0xffffffffu, valid)) return true;
+        if ((spin & 15u) == 0) {
+            bool give_up = *abort_flag != 0u;
+            if (!give_up && clock64() - t0 > kWaitLimitCycles) {
+                *abort_flag = 1;
+                atomicCAS(&g_attnw_status, 0u, 0x80000000u | site);
+                give_up = true;
+            }
+            if (__any_sync(0xffffffffu, give_up)) return false;
+        }
+    }
+}
+
+// The first CTAs of a group of C > kMaxDirectCtas own the rows of a block: a power of two of them, 128 / that many rows each.
+__host__ __device__ constexpr int owner_count(int group_ctas) {
+    int n = 4;
+    while (2 * n <= group_ctas && 2 * n <= kTile) n *= 2;
+    return n;
+}
+
+// xchg: [grid CTAs][kXchgDepth][128 rows] pairs, then [groups][kXchgDepth][128 rows] results, messages of 16 bytes in
+// memory owned by the library, zero before first use.
 // tag_base: tags tag_base + 1 ... tag_base + (row blocks of the longest list) belong to this launch alone.
-template <int D>
+template <int D, typename OutT>
 __global__ void __launch_bounds__(kThreads, 1)
 attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                      const __grid_constant__ CUtensorMap tm_p, int N, int total_items, int group_ctas, int n_groups,
                      float scale_log2e, uint4* __restrict__ xchg, uint32_t tag_base) {
     using L = Smem<D>;
-    constexpr int kBoxes = L::kBoxes;
+    constexpr bool kF32 = sizeof(OutT) == 4;
+    constexpr int kBoxCols = 128 / sizeof(OutT);  // columns of one staged store box
+    constexpr int kMaxBoxes = kSlabCols / kBoxCols;
+    constexpr int kRegions = kF32 ? 2 : 3;        // row blocks whose exponentials tensor memory holds
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     Barriers* bars = reinterpret_cast<Barriers*>(smem + L::kBarOff);
@@ -142,34 +184,32 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     const int T = (N + kTile - 1) / kTile;                          // row blocks per head
     const int col0 = rank * kSlabCols;                              // first key of this CTA's slab
     const int width = (N - col0 < kSlabCols) ? N - col0 : kSlabCols;  // keys of the slab that exist (>= 1)
-    const int n_sub = (width + kSub - 1) / kSub;                    // MMA slots in use
-    const int n_boxes = (width + kBoxCols - 1) / kBoxCols;          // 64-column store boxes in use, 1..4
-    const int n_ktiles = (width + kTile - 1) / kTile;               // 128-key tiles of the slab that exist, 1..2
+    const int n_sub = (width + kSub - 1) / kSub;                    // MMA slots in use = 128-key tiles of the slab, 1..2
+    const int n_boxes = (width + kBoxCols - 1) / kBoxCols;          // store boxes in use
     // The group's list: a contiguous range of (head, row block) items, so that the key slab changes rarely.
     const long long begin_ll = static_cast<long long>(total_items) * group / n_groups;
     const long long end_ll = static_cast<long long>(total_items) * (group + 1) / n_groups;
     const int begin = static_cast<int>(begin_ll);
     const int n_items = static_cast<int>(end_ll - begin_ll);
+    uint4* const results = xchg + (static_cast<size_t>(n_groups) * group_ctas + group) * kXchgDepth * kTile;
 
     // ---- set-up ------------------------------------------------------------------------------
     if (threadIdx.x == 0) {
         ptx::mbar_init(&bars->k_full, 1);
         ptx::mbar_init(&bars->k_empty, 1);
-        for (int j = 0; j < kSubsPerBlock; ++j) {
+        for (int j = 0; j < 2 * kSubsPerBlock; ++j) {
             ptx::mbar_init(&bars->s_full[j], 1);
-            ptx::mbar_init(&bars->l_free[j], 8);  // one arrival per exponential warp
+            ptx::mbar_init(&bars->s_free[j], kF32 ? 4 : kExpWarps);  // one arrival per warp that reads the slot last
         }
         for (int s = 0; s < 2; ++s) {
             ptx::mbar_init(&bars->q_full[s], 1);
             ptx::mbar_init(&bars->q_empty[s], 1);
-            for (int b = 0; b < kSlabCols / kBoxCols; ++b) ptx::mbar_init(&bars->pk_free[s][b], 4);  // the stream's normalise warps
-            ptx::mbar_init(&bars->posted[s], 8);  // one arrival per exponential warp
         }
-        for (int b = 0; b < kBoxes; ++b) {
-            ptx::mbar_init(&bars->out_free[b], 1);
-            ptx::mbar_init(&bars->out_filled[b], 4);
+        for (int r = 0; r < 3; ++r) {
+            for (int b = 0; b < kSlabCols / 64; ++b) ptx::mbar_init(&bars->pk_free[r][b], 4);  // the row block's normalise warps
+            ptx::mbar_init(&bars->posted[r], kExpWarps);
+            for (int x = 0; x < 4; ++x) bars->parts_done[r][x] = 0;
         }
-        for (int x = 0; x < 8; ++x) (&bars->halves_done[0][0])[x] = 0;
         bars->abort_flag = 0;
         bars->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
         ptx::mbar_fence_init();
@@ -189,6 +229,10 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     const uint32_t tmem_base = bars->tmem_base;
     const bool run = bars->prior_failure == 0u && n_items > 0;  // an earlier launch step gave up: skip the work
 
+    // Slots.  bfloat16: one for all; float32: two per region.
+    auto slot_of = [](int i, int j) { return kF32 ? (i & 1) * kSubsPerBlock + j : 0; };
+    auto slot_use = [n_sub](int i, int j) { return static_cast<uint32_t>(kF32 ? i >> 1 : i * n_sub + j); };  // how often the slot has been used before
+
     if (run && warp == kProducerWarpG) {
         // ================= TMA producer =================
         if (lane == 0) {
@@ -198,12 +242,10 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             int issued = 0;
             for (int i = 0; i < n_items; ++i) {
                 const int gi = begin + i, bh = gi / T, rb = gi % T;
-                const int s = i & 1;
-                const uint32_t u = static_cast<uint32_t>(i) >> 1;
                 if (bh != cur_bh) {  // new head: the slab may be replaced once every MMA of the old head has read it
                     if (!fused_wait(&bars->k_empty, (heads & 1u) ^ 1u, abort_flag, kSiteGrKEmpty)) break;
-                    ptx::mbar_expect_tx(&bars->k_full, static_cast<uint32_t>(n_ktiles * L::kTileBytes));
-                    for (int t = 0; t < n_ktiles; ++t)
+                    ptx::mbar_expect_tx(&bars->k_full, static_cast<uint32_t>(n_sub * L::kTileBytes));
+                    for (int t = 0; t < n_sub; ++t)
                         for (int a = 0; a < L::kAtoms; ++a)
                             ptx::tma_load_3d(smem + L::kKOff + a * L::kKAtomBytes + t * L::kAtomBytes, &tm_k, &bars->k_full,
                                              a * 64, col0 + t * kTile, bh, keep);
@@ -235,9 +277,6 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         }
     } else if (run && warp == kMmaWarpG) {
         // ================= MMA issuer (warp-uniform loop, one elected lane issues) =================
-        // One slot = 128 rows x kSub keys: D / 16 instructions of shape 128 x kSub x 16.  Both operands come from shared
-        // memory, and the query tile is fetched again by every instruction: narrow slots hand tensor memory over sooner
-        // but cost shared-memory bandwidth, which this kernel is short of.
         constexpr uint32_t idesc = ptx::umma_idesc_bf16_f32(kTile, kSub);
         const uint32_t q_addr = ptx::smem_u32(smem + L::kQOff);
         const uint32_t k_addr = ptx::smem_u32(smem + L::kKOff);
@@ -246,8 +285,6 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         bool ok = true;
         for (int i = 0; ok && i < n_items; ++i) {
             const int gi = begin + i, bh = gi / T;
-            const int s = i & 1;
-            const uint32_t u = static_cast<uint32_t>(i) >> 1;
             const int qs = i % L::kQStages;
             ok = __all_sync(0xffffffffu, fused_wait(&bars->q_full[qs], static_cast<uint32_t>(i / L::kQStages) & 1u, abort_flag, kSiteGrQFull));
             if (!ok) break;
@@ -258,39 +295,13 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 cur_bh = bh;
             }
             const bool last_of_head = (i + 1 == n_items) || ((gi + 1) / T != bh);
-            if (n_sub == 2) {
-                // Both landing slots in one 128 x 256 x 16 instruction per step: the query tile is fetched from shared
-                // memory once per row block instead of once per slot (0.7 % of the launch on the headline shape).
-                ok = __all_sync(0xffffffffu, fused_wait(&bars->l_free[0], (static_cast<uint32_t>(i) & 1u) ^ 1u, abort_flag, kSiteGrSlotFree)) &&
-                     __all_sync(0xffffffffu, fused_wait(&bars->l_free[1], (static_cast<uint32_t>(i) & 1u) ^ 1u, abort_flag, kSiteGrSlotFree));
-                if (!ok) break;
-                ptx::tc_fence_after_sync();
-                if (lane == 0) ATTNW_STAMP(13, i);
-                constexpr uint32_t idesc2 = ptx::umma_idesc_bf16_f32(kTile, 2 * kSub);
-                const uint32_t a_addr = q_addr + static_cast<uint32_t>(qs * L::kTileBytes);
-                if (ptx::elect_one()) {
-#pragma unroll
-                    for (int k = 0; k < D / 16; ++k) {
-                        const uint32_t a_off = static_cast<uint32_t>((k >> 2) * L::kAtomBytes + (k & 3) * 32);
-                        const uint32_t b_off = static_cast<uint32_t>((k >> 2) * L::kKAtomBytes + (k & 3) * 32);
-                        ptx::umma_f16_ss(tmem_base, ptx::umma_desc_kmajor_sw128(a_addr + a_off),
-                                         ptx::umma_desc_kmajor_sw128(k_addr + b_off), idesc2, k > 0 ? 1u : 0u);
-                    }
-                    ptx::umma_commit(&bars->s_full[0]);
-                    ptx::umma_commit(&bars->s_full[1]);
-                    ptx::umma_commit(&bars->q_empty[qs]);                // the query tile may be replaced
-                    if (last_of_head) ptx::umma_commit(&bars->k_empty);  // ... and the key slab
-                }
-                __syncwarp();
-                continue;
-            }
-            for (int j = 0; j < n_sub; ++j) {
-                // the landing slot is free once the exponential warps have taken the scores of row block i - 1 to registers
-                ok = __all_sync(0xffffffffu, fused_wait(&bars->l_free[j], (static_cast<uint32_t>(i) & 1u) ^ 1u, abort_flag, kSiteGrSlotFree));
+            for (int j = 0; ok && j < n_sub; ++j) {
+                const int slot = slot_of(i, j);
+                ok = __all_sync(0xffffffffu, fused_wait(&bars->s_free[slot], (slot_use(i, j) & 1u) ^ 1u, abort_flag, kSiteGrSlotFree));
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 if (lane == 0 && j == 0) ATTNW_STAMP(13, i);
-                const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(j * kSub);
+                const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(slot * kSub);
                 const uint32_t a_addr = q_addr + static_cast<uint32_t>(qs * L::kTileBytes);
                 const uint32_t b_addr = k_addr + static_cast<uint32_t>(j * kSub * 128);  // keys kSub j ... of every atom
                 if (ptx::elect_one()) {
@@ -301,7 +312,7 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                         ptx::umma_f16_ss(d_tmem, ptx::umma_desc_kmajor_sw128(a_addr + a_off),
                                          ptx::umma_desc_kmajor_sw128(b_addr + b_off), idesc, k > 0 ? 1u : 0u);
                     }
-                    ptx::umma_commit(&bars->s_full[j]);
+                    ptx::umma_commit(&bars->s_full[slot]);
                     if (j == n_sub - 1) {
                         ptx::umma_commit(&bars->q_empty[qs]);                // the query tile may be replaced
                         if (last_of_head) ptx::umma_commit(&bars->k_empty);  // ... and the key slab
@@ -310,38 +321,46 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 __syncwarp();
             }
         }
-    } else if (run && (warp == kStoreWarpG || warp == kStoreWarpG + 1)) {
-        // ================= store issuer: one TMA store per filled staging box, in ring order =================
-        // Boxes are stored in the order (row block, 64 columns); the boxes of a stream use that stream's ring in turn.
-        if (lane == 0) {
-            const uint64_t stream_out = ptx::policy_evict_first();
-            const uint32_t out_base = ptx::smem_u32(smem + L::kOutOff);
-            bool ok = true;
-            for (int i = warp - kStoreWarpG; ok && i < n_items; i += 2) {  // one store issuer per stream
-                const int gi = begin + i, bh = gi / T, rb = gi % T;
-                const int s = i & 1;
-                const uint32_t ring = s ? L::kRing1 : L::kRing0, base = s ? L::kRing0 : 0;
-                const uint32_t m0 = (static_cast<uint32_t>(i) >> 1) * static_cast<uint32_t>(n_boxes);
-                for (int j = 0; j < n_boxes; ++j) {
-                    const uint32_t m = m0 + static_cast<uint32_t>(j);
-                    const uint32_t box = base + m % ring, use = m / ring;
-                    if (!fused_wait(&bars->out_filled[box], use & 1u, abort_flag, kSiteGrStageFilled)) {
-                        ok = false;
-                        break;
-                    }
-                    ptx::tma_store_3d(&tm_p, out_base + box * kBoxBytes, col0 + j * kBoxCols, rb * kTile, bh, stream_out);
-                    ptx::bulk_commit_group();
-                    ptx::bulk_wait_group_read<0>();  // the store has read the box: it may be filled again
-                    ptx::mbar_arrive(&bars->out_free[box]);
-                }
-            }
-            ptx::bulk_wait_group<0>();
+    } else if (run && warp >= kOwnerWarpG) {
+        // ================= owner's reduction =================
+        const int owners = owner_count(group_ctas);
+        const int my_rows = kTile / owners;                    // rows this CTA owns if rank < owners, at most 32
+        const int warp_rows = my_rows > 1 ? my_rows / 2 : 1;   // ... and this warp
+        const int n_lanes = 32 / warp_rows;                    // lanes that share a row
+        const int sub = lane / warp_rows;                      // this lane takes the pairs of CTAs sub, sub + n_lanes, ...
+        const int n_mine = (group_ctas - sub + n_lanes - 1) / n_lanes;  // at least 1 and, since C < 2 owners or C = owners = 128, at most 4
+        const int w = warp - kOwnerWarpG;
+        const int row = rank * my_rows + w * warp_rows + (lane & (warp_rows - 1));
+        const uint4* pairs = xchg + (static_cast<size_t>(group) * group_ctas + sub) * kXchgDepth * kTile + row;
+        const bool owner = group_ctas > kMaxDirectCtas && rank < owners && w < my_rows;
+        for (int i = 0; owner && i < n_items; ++i) {
+            // Entry reuse: row blocks i and i + 8 share entries.
+            // Pairs: a warp that posts a pair of block i + 8 has waited for the normalise warps of its CTA to read region
+            // (i + 5) mod 3, i.e. for results of block i + 5, whose owners had seen the pairs of every CTA - and this warp reads
+            // the pairs of the blocks in order, block i long before.
+            // Results: the owner posts a result of block i + 8 after every CTA has posted its pairs of that block, i.e. after
+            // the normalise warps of every CTA have read the exponentials of the blocks up to i + 5, with their statistics.
+            if (w == 0 && lane == 0) ATTNW_STAMP(22, i);
+            const uint32_t tag = tag_base + static_cast<uint32_t>(i) + 1u;
+            const uint4* src = pairs + (i & (kXchgDepth - 1)) * kTile;
+            uint4 v[4];
+            if (!poll_messages<4>(v, n_mine, tag, abort_flag, kSiteGrOwner,
+                                  [&](int c) { return src + static_cast<size_t>(c) * n_lanes * kXchgDepth * kTile; }))
+                break;
+            if (w == 0 && lane == 0) ATTNW_STAMP(23, i);
+            float m = fmaxf(fmaxf(__uint_as_float(v[0].x), __uint_as_float(v[1].x)), fmaxf(__uint_as_float(v[2].x), __uint_as_float(v[3].x)));
+            for (int off = warp_rows; off < 32; off <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+            float l = 0.0f;
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                l += (c < n_mine) ? __uint_as_float(v[c].z) * ptx::ex2_approx(__uint_as_float(v[c].x) - m) : 0.0f;
+            for (int off = warp_rows; off < 32; off <<= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+            if (sub == 0) st_message(results + (i & (kXchgDepth - 1)) * kTile + row, m, 1.0f / l, tag);
+            if (w == 0 && lane == 0) ATTNW_STAMP(25, i);
         }
     } else if (run && warp < kNormWarp0) {
-        // ================= exponential warps: TMEM lane quarter = warp % 4, box parity = warp / 4 =================
-        // All eight warps work on ONE row block at a time (both streams in turn): two threads per row, one taking the
-        // even and one the odd 64-column boxes, so that every scheduler has two warps feeding its MUFU.
-        const int par = warp >> 2;
+        // ================= exponential warps: TMEM lane quarter = warp % 4, 32 columns of each slot = warp / 4 =================
+        const int part = warp >> 2;
         const int quarter = warp & 3;
         const int row = quarter * 32 + lane;
         const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
@@ -356,86 +375,75 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         (void)stamp;
         bool ok = true;
         for (int i = 0; ok && i < n_items; ++i) {
-            const int s = i & 1;
-            const uint32_t u = static_cast<uint32_t>(i) >> 1;
-            float* mbc = mbc_all + s * kChunksPerBlock * kTile;
+            const int region = i % kRegions;
+            float* mbc = mbc_all + region * kChunksPerBlock * kTile;
             float smax = -3.0e38f, mb = -3.0e38f, l = 0.0f;
             if (stamp) ATTNW_STAMP(0, i);
-            // This thread's pieces of the row: the 64-column boxes 2k + par, k = 0, 1 (landing slot k).  A whole box is taken
-            // at once: 64 scores to registers - the landing slot goes back to the MMA issuer right there -, maximum,
-            // offset, exponentials, sum; the exponentials leave as f16 pairs for the stream's packed region, where they
-            // wait for the row's statistics without holding up the next row block's scores.
 #pragma unroll 1
-            for (int k = 0; k < kSubsPerBlock; ++k) {
-                const int bx = 2 * k + par;
-                const int valid = width - bx * kBoxCols;  // columns of this box that exist
-                uint32_t r0[kChunk], r1[kChunk];
-                if (k < n_sub) {  // (every warp waits for slot 0, so that a warp without work keeps step)
-                    ok = __all_sync(0xffffffffu, fused_wait(&bars->s_full[k], static_cast<uint32_t>(i) & 1u, abort_flag, kSiteGrSFull));
-                    if (!ok) break;
-                    ptx::tc_fence_after_sync();
-                    if (stamp && k == 0) ATTNW_STAMP(2, i);
-                }
+            for (int k = 0; k < n_sub; ++k) {
+                const int chunk = k * kParts + part;
+                const int valid = width - chunk * kChunk;  // columns of this chunk that exist
+                const int slot = slot_of(i, k);
+                ok = __all_sync(0xffffffffu, fused_wait(&bars->s_full[slot], slot_use(i, k) & 1u, abort_flag, kSiteGrSFull));
+                if (!ok) break;
+                ptx::tc_fence_after_sync();
+                if (stamp && k == 0) ATTNW_STAMP(2, i);
                 if (stamp) ATTNW_STAMP(17 + 3 * k, i);
-                if (valid <= 0) {  // nothing of the box is ever stored (the tensor map clips it); the slot's barrier counts every warp
-                    __syncwarp();
-                    if (lane == 0) ptx::mbar_arrive(&bars->l_free[k]);
+                if (valid <= 0) {  // nothing of the chunk is ever stored (the tensor map clips it); the slot's barrier counts every warp
+                    if (!kF32) {
+                        __syncwarp();
+                        if (lane == 0) ptx::mbar_arrive(&bars->s_free[slot]);
+                    }
                     continue;
                 }
-                {
-                    const uint32_t taddr = t_lane + static_cast<uint32_t>(bx * kBoxCols);
-                    ptx::tmem_ld_32x32b_x32(taddr, r0);
-                    ptx::tmem_ld_32x32b_x32(taddr + kChunk, r1);
-                    ptx::tmem_wait_ld();
+                const uint32_t taddr = t_lane + static_cast<uint32_t>(slot * kSub + part * kChunk);
+                uint32_t r[kChunk];
+                ptx::tmem_ld_32x32b_x32(taddr, r);
+                ptx::tmem_wait_ld();
+                if (!kF32) {
                     ptx::tc_fence_before_sync();
                     __syncwarp();
-                    if (lane == 0) ptx::mbar_arrive(&bars->l_free[k]);
+                    if (lane == 0) ptx::mbar_arrive(&bars->s_free[slot]);
                 }
-                if (valid < kBoxCols) {
+                if (valid < kChunk) {
 #pragma unroll
-                    for (int x = 0; x < kChunk; ++x) {
-                        if (x >= valid) r0[x] = 0xff61b1e6u;            // -3.0e38f
-                        if (x + kChunk >= valid) r1[x] = 0xff61b1e6u;
-                    }
+                    for (int x = 0; x < kChunk; ++x)
+                        if (x >= valid) r[x] = 0xff61b1e6u;  // -3.0e38f
                 }
-                float m0 = -3.0e38f, m1 = -3.0e38f, m2 = -3.0e38f, m3 = -3.0e38f;
+                float m0 = __uint_as_float(r[0]), m1 = __uint_as_float(r[1]), m2 = __uint_as_float(r[2]), m3 = __uint_as_float(r[3]);
 #pragma unroll
-                for (int x = 0; x < kChunk; x += 8) {
-                    m0 = ptx::max3(m0, __uint_as_float(r0[x + 0]), __uint_as_float(r0[x + 1]));
-                    m1 = ptx::max3(m1, __uint_as_float(r0[x + 2]), __uint_as_float(r0[x + 3]));
-                    m2 = ptx::max3(m2, __uint_as_float(r0[x + 4]), __uint_as_float(r0[x + 5]));
-                    m3 = ptx::max3(m3, __uint_as_float(r0[x + 6]), __uint_as_float(r0[x + 7]));
-                    m0 = ptx::max3(m0, __uint_as_float(r1[x + 0]), __uint_as_float(r1[x + 1]));
-                    m1 = ptx::max3(m1, __uint_as_float(r1[x + 2]), __uint_as_float(r1[x + 3]));
-                    m2 = ptx::max3(m2, __uint_as_float(r1[x + 4]), __uint_as_float(r1[x + 5]));
-                    m3 = ptx::max3(m3, __uint_as_float(r1[x + 6]), __uint_as_float(r1[x + 7]));
+                for (int x = 4; x + 7 < kChunk; x += 8) {
+                    m0 = ptx::max3(m0, __uint_as_float(r[x + 0]), __uint_as_float(r[x + 1]));
+                    m1 = ptx::max3(m1, __uint_as_float(r[x + 2]), __uint_as_float(r[x + 3]));
+                    m2 = ptx::max3(m2, __uint_as_float(r[x + 4]), __uint_as_float(r[x + 5]));
+                    m3 = ptx::max3(m3, __uint_as_float(r[x + 6]), __uint_as_float(r[x + 7]));
                 }
-                const float new_max = fmaxf(smax, ptx::max3(fmaxf(m0, m1), m2, m3));
+                m0 = ptx::max3(m0, __uint_as_float(r[kChunk - 4]), __uint_as_float(r[kChunk - 3]));
+                m1 = ptx::max3(m1, __uint_as_float(r[kChunk - 2]), __uint_as_float(r[kChunk - 1]));
+                const float new_max = ptx::max3(smax, fmaxf(m0, m1), fmaxf(m2, m3));
                 const float mb_new = fmaxf(new_max * c2, -3.0e38f);  // finite also while every column so far is masked
                 l *= ptx::ex2_approx(mb - mb_new);                   // exactly 1 while the maximum stands
                 mb = mb_new;
                 smax = new_max;
                 if (stamp) ATTNW_STAMP(16 + 3 * k, i);
-                uint32_t pk[kChunk];  // the box's 64 exponentials as f16 pairs, in column order
+                uint32_t pk[kChunk / 2];  // bfloat16 output: the exponentials as f16 pairs, in column order
                 {
                     const uint64_t off2 = ptx::pack2(-mb, -mb);
                     uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
                     // (masked columns hold -3e38 and c2 > 0, so their exponentials are exactly zero)
 #pragma unroll
                     for (int x = 0; x < kChunk; x += 2) {
-                        float a0, a1, b0, b1;
-                        const uint64_t xa = ptx::fma2(ptx::pack2(__uint_as_float(r0[x]), __uint_as_float(r0[x + 1])), c2c2, off2);
-                        const uint64_t xb = ptx::fma2(ptx::pack2(__uint_as_float(r1[x]), __uint_as_float(r1[x + 1])), c2c2, off2);
-                        ptx::unpack2(xa, a0, a1);
-                        ptx::unpack2(xb, b0, b1);
+                        float a0, a1;
+                        ptx::unpack2(ptx::fma2(ptx::pack2(__uint_as_float(r[x]), __uint_as_float(r[x + 1])), c2c2, off2), a0, a1);
                         a0 = ptx::ex2_approx(a0);
                         a1 = ptx::ex2_approx(a1);
-                        b0 = ptx::ex2_approx(b0);
-                        b1 = ptx::ex2_approx(b1);
-                        pk[x >> 1] = ptx::pack_f16x2(a0, a1);
-                        pk[(kChunk >> 1) + (x >> 1)] = ptx::pack_f16x2(b0, b1);
-                        acc[(x >> 1) & 1] = ptx::add2(acc[(x >> 1) & 1], ptx::pack2(a0, a1));
-                        acc[2 + ((x >> 1) & 1)] = ptx::add2(acc[2 + ((x >> 1) & 1)], ptx::pack2(b0, b1));
+                        if (kF32) {
+                            r[x] = __float_as_uint(a0);
+                            r[x + 1] = __float_as_uint(a1);
+                        } else {
+                            pk[x >> 1] = ptx::pack_f16x2(a0, a1);
+                        }
+                        acc[(x >> 1) & 3] = ptx::add2(acc[(x >> 1) & 3], ptx::pack2(a0, a1));
                     }
                     float s0, s1, s2, s3;
                     ptx::unpack2(ptx::add2(acc[0], acc[1]), s0, s1);
@@ -443,157 +451,170 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     l += (s0 + s1) + (s2 + s3);
                 }
                 if (stamp) ATTNW_STAMP(18 + 3 * k, i);
-                // the packed region still holds this box of row block i - 2 until its normalise warps have read it
-                ok = __all_sync(0xffffffffu, fused_wait(&bars->pk_free[s][bx], (u & 1u) ^ 1u, abort_flag, kSiteGrSlotFree));
-                if (!ok) break;
-                ptx::tc_fence_after_sync();
-                ptx::tmem_st_32x32b_x32(t_lane + static_cast<uint32_t>(kPackedCol0 + s * kPackedCols + bx * (kBoxCols / 2)), pk);
+                if (kF32) {
+                    ptx::tmem_st_32x32b_x32(taddr, r);
+                } else {
+                    // the packed region still holds these columns of row block i - 3 until its normalise warps have read them
+                    ok = __all_sync(0xffffffffu, fused_wait(&bars->pk_free[region][chunk >> 1], (static_cast<uint32_t>(i / kRegions) & 1u) ^ 1u, abort_flag, kSiteGrSlotFree));
+                    if (!ok) break;
+                    ptx::tc_fence_after_sync();
+                    ptx::tmem_st_32x32b_x16(t_lane + static_cast<uint32_t>(kPackedCol0 + region * kPackedCols + chunk * (kChunk / 2)), pk);
+                }
                 if (stamp) ATTNW_STAMP(24 + 2 * k, i);
-                mbc[bx * kTile + row] = mb;  // the offset this box's e are relative to
+                mbc[chunk * kTile + row] = mb;  // the offset this chunk's e are relative to
             }
             if (!ok) break;
-            part_all[(s * 2 + par) * kTile + row] = make_float2(mb, l);  // this thread's half of the row
-            // The second of the two warps to get here merges the halves and posts the row's pair to every CTA of the
-            // group (through L2) at once: the exchange must not wait for a normalise warp to become free.
+            part_all[(region * kParts + part) * kTile + row] = make_float2(mb, l);  // this thread's part of the row
+            // The last of the four warps to get here merges the parts and posts the row's pair for the group (through L2) at
+            // once: the exchange must not wait for a normalise warp to become free.
             __threadfence_block();
             __syncwarp();
             uint32_t before = 0;
-            if (lane == 0) before = atomicAdd(&bars->halves_done[s][quarter], 1u);
+            if (lane == 0) before = atomicAdd(&bars->parts_done[region][quarter], 1u);
             before = __shfl_sync(0xffffffffu, before, 0);
-            if (before & 1u) {
+            if ((before & (kParts - 1)) == kParts - 1) {
                 __threadfence_block();
-                const volatile float* pv = reinterpret_cast<const volatile float*>(part_all);
-                const float pax = pv[2 * ((s * 2 + 0) * kTile + row)], pay = pv[2 * ((s * 2 + 0) * kTile + row) + 1];
-                const float pbx = pv[2 * ((s * 2 + 1) * kTile + row)], pby = pv[2 * ((s * 2 + 1) * kTile + row) + 1];
-                const float mc = fmaxf(pax, pbx);
-                const float lc = pay * ptx::ex2_approx(pax - mc) + pby * ptx::ex2_approx(pbx - mc);
-                st_message(my_msg + (i & (kXchgDepth - 1)) * kTile, mc, lc, tag_base + static_cast<uint32_t>(i) + 1u);
+                const volatile float* pv = reinterpret_cast<const volatile float*>(part_all + region * kParts * kTile + row);
+                float pm[kParts], pl[kParts];
+#pragma unroll
+                for (int x = 0; x < kParts; ++x) {
+                    pm[x] = pv[2 * x * kTile];
+                    pl[x] = pv[2 * x * kTile + 1];
+                }
+                const float mc = fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3]));
+                float lc = 0.0f;
+#pragma unroll
+                for (int x = 0; x < kParts; ++x) lc += pl[x] * ptx::ex2_approx(pm[x] - mc);
+                if (group_ctas > 1)
+                    st_message(my_msg + (i & (kXchgDepth - 1)) * kTile, mc, lc, tag_base + static_cast<uint32_t>(i) + 1u);
+                else
+                    part_all[region * kParts * kTile + row] = make_float2(mc, 1.0f / lc);  // the row's statistics (this thread alone has read the parts)
             }
             ptx::tmem_wait_st();
             ptx::tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&bars->posted[s]);
+            if (lane == 0) ptx::mbar_arrive(&bars->posted[region]);
             if (stamp) ATTNW_STAMP(4, i);
         }
-    } else if (run && warp < kNormWarp0 + 4 * kNormGroups) {
-        // ================= normalise warps: stream s = (warp - 8) / 4, TMEM lane quarter = warp % 4 =================
-        const int first = (kNormGroups == 2) ? ((warp - kNormWarp0) >> 2) : 0;
+    } else if (run && warp < kNormWarp0 + 8) {
+        // ================= normalise warps: row blocks of parity (warp - 16) / 4, TMEM lane quarter = warp % 4 =================
         const int quarter = warp & 3;
         const int row = quarter * 32 + lane;
         const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
-        const uint32_t out_base = ptx::smem_u32(smem + L::kOutOff);
-        const uint32_t sw = static_cast<uint32_t>(row & 7);
+        const uint32_t stage = ptx::smem_u32(smem + L::kOutOff + (warp - kNormWarp0) * L::kStages * kStageBytes);
+        const uint32_t sw = static_cast<uint32_t>(lane & 7);
+        const uint64_t stream_out = ptx::policy_evict_first();
+        const float* mbc_all = reinterpret_cast<const float*>(smem + L::kMbcOff) + row;
+        const float2* part_all = reinterpret_cast<const float2*>(smem + L::kPartOff) + row;
         const uint4* group_msg = xchg + (static_cast<size_t>(group) * group_ctas * kXchgDepth) * kTile + row;
-        const float* mbc_all = reinterpret_cast<const float*>(smem + L::kMbcOff);
-        const int last_cta = group_ctas - 1;
+        uint32_t staged = 0;  // boxes this warp has staged
         const bool stamp = quarter == 0 && lane == 0;
         (void)stamp;
         bool ok = true;
-        for (int i = first; ok && i < n_items; i += kNormGroups) {
-            const int s = i & 1;
-            const uint32_t u = static_cast<uint32_t>(i) >> 1;
-            const float* mbc = mbc_all + s * kChunksPerBlock * kTile;
+        for (int i = (warp - kNormWarp0) >> 2; ok && i < n_items; i += 2) {
+            const int region = i % kRegions;
+            const int gi = begin + i, bh = gi / T, row0 = (gi % T) * kTile + quarter * 32;  // first row of this warp
             if (stamp) ATTNW_STAMP(10, i);
             // this CTA's exponentials of the row block are in tensor memory and its chunk offsets in shared memory
-            ok = __all_sync(0xffffffffu, fused_wait(&bars->posted[s], u & 1u, abort_flag, kSiteGrPosted));
+            ok = __all_sync(0xffffffffu, fused_wait(&bars->posted[region], static_cast<uint32_t>(i / kRegions) & 1u, abort_flag, kSiteGrPosted));
             if (!ok) break;
             ptx::tc_fence_after_sync();
             if (stamp) ATTNW_STAMP(6, i);
-            // ---- global statistics of the row: wait for the C pairs, reduce them (redundantly in every CTA) ----
-            // Entry reuse: row blocks i and i + 4 share entries.  A CTA posts block i + 4 after it has read the
-            // statistics of block i + 2, i.e. after EVERY CTA has posted block i + 2; a CTA's scores of block i + 2
-            // land in the tensor memory its normalise warps have finished reading for block i, which they did after
-            // reading these entries.  So nobody overwrites an entry that anyone still has to read.
+            // ---- global statistics of the row ----
+            const uint32_t tag = tag_base + static_cast<uint32_t>(i) + 1u;
+            const int entry = (i & (kXchgDepth - 1)) * kTile;
             float m_row, inv_l;
-            {
-                const uint32_t tag = tag_base + static_cast<uint32_t>(i) + 1u;
-                const uint4* src = group_msg + (i & (kXchgDepth - 1)) * kTile;
-                uint4 v[kMaxGroupCtas];
-                const long long t0 = clock64();
-                for (uint32_t spin = 1;; ++spin) {
-                    // all loads first (entries beyond the group repeat its last CTA), then the tags
-#pragma unroll
-                    for (int c = 0; c < kMaxGroupCtas; ++c)
-                        v[c] = ld_message(src + static_cast<size_t>(c < last_cta ? c : last_cta) * kXchgDepth * kTile);
-                    bool valid = true;
-#pragma unroll
-                    for (int c = 0; c < kMaxGroupCtas; ++c) valid = valid && v[c].y == tag && v[c].w == tag;
-                    if (__all_sync(0xffffffffu, valid)) break;
-                    if ((spin & 15u) == 0) {
-                        bool give_up = *abort_flag != 0u;
-                        if (!give_up && clock64() - t0 > kWaitLimitCycles) {
-                            *abort_flag = 1;
-                            atomicCAS(&g_attnw_status, 0u, 0x80000000u | kSiteGrExchange);
-                            give_up = true;
-                        }
-                        if (__any_sync(0xffffffffu, give_up)) {
-                            ok = false;
-                            break;
-                        }
-                    }
-                }
+            if (group_ctas == 1) {
+                const float2 st = part_all[region * kParts * kTile];
+                m_row = st.x;
+                inv_l = st.y;
+            } else if (group_ctas > kMaxDirectCtas) {
+                uint4 v[1];
+                ok = poll_messages<1>(v, 1, tag, abort_flag, kSiteGrExchange, [&](int) { return results + entry + row; });
                 if (!ok) break;
-                if (stamp) ATTNW_STAMP(11, i);
+                m_row = __uint_as_float(v[0].x);
+                inv_l = __uint_as_float(v[0].z);
+            } else {
+                // Entry reuse here: a CTA posts block i + 8 after its normalise warps have read the pairs of the blocks up to
+                // i + 5, i.e. after EVERY CTA has posted those, which a CTA does after reading the pairs up to block i + 2.
+                uint4 v[kMaxDirectCtas];
+                ok = poll_messages<kMaxDirectCtas>(v, group_ctas, tag, abort_flag, kSiteGrExchange,
+                                                   [&](int c) { return group_msg + static_cast<size_t>(c) * kXchgDepth * kTile + entry; });
+                if (!ok) break;
                 m_row = __uint_as_float(v[0].x);
 #pragma unroll
-                for (int c = 1; c < kMaxGroupCtas; ++c) m_row = fmaxf(m_row, __uint_as_float(v[c].x));
+                for (int c = 1; c < kMaxDirectCtas; ++c) m_row = fmaxf(m_row, __uint_as_float(v[c].x));
                 float l_row = 0.0f;
 #pragma unroll
-                for (int c = 0; c < kMaxGroupCtas; ++c)
+                for (int c = 0; c < kMaxDirectCtas; ++c)
                     l_row += (c < group_ctas) ? __uint_as_float(v[c].z) * ptx::ex2_approx(__uint_as_float(v[c].x) - m_row) : 0.0f;
                 inv_l = 1.0f / l_row;
             }
-            // factors of the row's boxes, read before any slot is handed back (the exponential warps write the offsets
-            // of row block i + 2 as soon as they own its scores)
-            float f[kSlabCols / kBoxCols];
+            if (stamp) ATTNW_STAMP(11, i);
+            // factors of the row's chunks, read before any of the region is handed back (the exponential warps then write the
+            // offsets of the next row block there)
+            float f[kChunksPerBlock];
 #pragma unroll
-            for (int b = 0; b < kSlabCols / kBoxCols; ++b)
-                f[b] = (b < n_boxes) ? ptx::ex2_approx(mbc[b * kTile + row] - m_row) * inv_l : 0.0f;
+            for (int c = 0; c < kChunksPerBlock; ++c)
+                f[c] = ptx::ex2_approx(mbc_all[(region * kChunksPerBlock + c) * kTile] - m_row) * inv_l;  // (chunks beyond the last key: never stored)
 #pragma unroll
-            for (int b = 0; b < kSlabCols / kBoxCols; ++b) {
-                if (b < n_boxes && ok) {
-                    uint32_t e[kChunk];  // the box's 64 exponentials as f16 pairs
-                    ptx::tmem_ld_32x32b_x32(t_lane + static_cast<uint32_t>(kPackedCol0 + s * kPackedCols + b * (kBoxCols / 2)), e);
+            for (int b = 0; b < kMaxBoxes; ++b) {
+                if (b < n_boxes) {
+                    uint32_t e[kChunk];  // 64 exponentials as f16 pairs, or 32 as float32
+                    ptx::tmem_ld_32x32b_x32(t_lane + static_cast<uint32_t>(kF32 ? region * kSlabCols + b * kChunk
+                                                                                : kPackedCol0 + region * kPackedCols + b * kChunk), e);
                     ptx::tmem_wait_ld();
-                    // the box has been read: the exponentials of row block i + 2 may take its place
+                    // the box has been read: the exponentials (float32: the scores) of the next row block may take its place
                     ptx::tc_fence_before_sync();
                     __syncwarp();
-                    if (lane == 0) ptx::mbar_arrive(&bars->pk_free[s][b]);
+                    if (kF32) {
+                        const int k = b / (kSub / kBoxCols);
+                        if (lane == 0 && (b == n_boxes - 1 || (b + 1) % (kSub / kBoxCols) == 0)) ptx::mbar_arrive(&bars->s_free[region * kSubsPerBlock + k]);
+                    } else {
+                        if (lane == 0) ptx::mbar_arrive(&bars->pk_free[region][b]);
+                    }
                     if (stamp && b == 0) ATTNW_STAMP(12, i);
-                    // staging box of this (row block, 64 columns): the stream's ring entry m % ring; the store that last
-                    // used the entry must have read it before anyone overwrites it
-                    const uint32_t m = u * static_cast<uint32_t>(n_boxes) + static_cast<uint32_t>(b);
-                    const uint32_t ring = s ? L::kRing1 : L::kRing0;
-                    const uint32_t box = (s ? L::kRing0 : 0) + m % ring, use = m / ring;
-                    const uint32_t my_row = out_base + box * kBoxBytes + static_cast<uint32_t>(row * 128);
                     if (stamp && b == 2) ATTNW_STAMP(14, i);
-                    ok = __all_sync(0xffffffffu, fused_wait(&bars->out_free[box], (use & 1u) ^ 1u, abort_flag, kSiteGrStageFree));
+                    // the staging box: the store that used it last must have read it
+                    const uint32_t box = stage + (staged % L::kStages) * kStageBytes;
+                    ++staged;
+                    if (lane == 0) ptx::bulk_wait_group_read<L::kStages - 1>();
+                    __syncwarp();
                     if (stamp && b == 2) ATTNW_STAMP(15, i);
-                    if (ok) {
-                        // p = e * f in float32 from f16 operands (one mixed-precision FMA per element unpacks and scales);
-                        // a factor below f16 range rounds to zero, where p < 6e-8 anyway
-                        const uint32_t fh = ptx::pack_f16x2(f[b], f[b]);
+                    const uint32_t my_row = box + static_cast<uint32_t>(lane * 128);
 #pragma unroll
-                        for (int gg = 0; gg < 8; ++gg) {  // 8 bf16 = one 16-byte piece of the row's 128 bytes
-                            uint32_t w[4];
+                    for (int gg = 0; gg < 8; ++gg) {  // one 16-byte piece of the row's 128 bytes
+                        uint32_t w[4];
+                        if (kF32) {
+#pragma unroll
+                            for (int x = 0; x < 4; ++x) w[x] = __float_as_uint(__uint_as_float(e[gg * 4 + x]) * f[b]);
+                        } else {
+                            // p = e * f in float32 from f16 operands (one mixed-precision FMA per element unpacks and
+                            // scales); a factor below f16 range rounds to zero, where p < 6e-8 anyway
+                            const float fc = f[2 * (b % 4) + (gg >> 2)];
+                            const uint32_t fh = ptx::pack_f16x2(fc, fc);
 #pragma unroll
                             for (int x = 0; x < 4; ++x) {
                                 float lo, hi;
                                 ptx::scale_f16x2(e[gg * 4 + x], fh, lo, hi);
                                 w[x] = ptx::pack_bf16x2(lo, hi);
                             }
-                            ptx::st_shared_v4(my_row + ((static_cast<uint32_t>(gg) ^ sw) << 4), w[0], w[1], w[2], w[3]);
                         }
-                        if (stamp && b == 2) ATTNW_STAMP(8, i);
-                        ptx::fence_proxy_async_smem();
-                        __syncwarp();
-                        if (lane == 0) ptx::mbar_arrive(&bars->out_filled[box]);
-                        if (stamp && b == 2) ATTNW_STAMP(9, i);
+                        ptx::st_shared_v4(my_row + ((static_cast<uint32_t>(gg) ^ sw) << 4), w[0], w[1], w[2], w[3]);
                     }
+                    if (stamp && b == 2) ATTNW_STAMP(8, i);
+                    ptx::fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (row0 < N) ptx::tma_store_3d(&tm_p, box, col0 + b * kBoxCols, row0, bh, stream_out);
+                        ptx::bulk_commit_group();
+                    }
+                    if (stamp && b == 2) ATTNW_STAMP(9, i);
                 }
             }
             if (stamp) ATTNW_STAMP(7, i);
         }
+        if (lane == 0) ptx::bulk_wait_group<0>();
     }
 
     // ---- teardown: every thread of the CTA arrives here, also after a wait gave up ----

@@ -1,0 +1,109 @@
+"""The grid-row kernel where the choice by shape uses it: float32 weights, groups beyond 16 CTAs, each way the row statistics
+cross a group, several streams at once, and stream capture."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from helpers import TOL, assert_close_to_oracle, assert_guards_intact, bits_to_cuda_bf16, guarded_empty, small_fused_inputs, to_f64
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def attnw():
+    from paper_2407_13885_b200 import binding
+    return binding
+
+
+def scale_of(d):
+    return float(np.float32(1.0 / math.sqrt(d)))
+
+
+# one CTA (no exchange), 2 and 4 (every CTA reads all pairs), 5, 7, 8, 15 and 16 (owners of 32, 32, 16, 16 and 8 rows);
+# a slab with one slot in use, a store box that is cut, row blocks of 4 rows, more row blocks than groups
+SHAPES = [(1, 1, 4, 64), (3, 50, 60, 64), (1, 2, 256, 128), (1, 3, 260, 64), (1, 5, 512, 64), (2, 3, 1020, 128),
+          (1, 2, 1284, 64), (1, 2, 1792, 128), (1, 9, 1924, 64), (1, 2, 3716, 64), (1, 1, 4096, 128)]
+
+
+@pytest.mark.parametrize("B,H,N,d", SHAPES)
+def test_float32_weights_match_oracle(attnw, B, H, N, d):
+    q, k = small_fused_inputs(B, H, N, d, stream=N + d + 13)
+    Q, K = bits_to_cuda_bf16(q), bits_to_cuda_bf16(k)
+    ref = oracle.attnw(q, k, scale_of(d))
+    for _ in range(2):  # the second launch finds the exchange area as the first one left it
+        raw, P, g = guarded_empty((B, H, N, N), torch.float32)
+        attnw.attnw_fused(Q, K, scale_of(d), P=P)
+        torch.cuda.synchronize()
+        assert attnw.query_status() == 0
+        assert_guards_intact(raw, g)
+        assert_close_to_oracle(P, ref, f"B{B} H{H} N{N} d{d}")
+
+
+# groups of 17, 24, 33 and 48 CTAs (owners of 8, 8, 4 and 4 rows); the last row blocks and columns ragged
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("H,N,d", [(2, 4104, 64), (1, 6000, 128), (1, 8456, 64), (1, 12288, 128)])
+def test_long_rows_match_oracle(attnw, dtype, H, N, d):
+    q, k = small_fused_inputs(1, H, N, d, sigma=1.5, stream=N + 1)
+    raw, P, g = guarded_empty((1, H, N, N), dtype)
+    attnw.attnw_fused(bits_to_cuda_bf16(q), bits_to_cuda_bf16(k), scale_of(d), P=P)
+    torch.cuda.synchronize()
+    assert attnw.query_status() == 0
+    assert_guards_intact(raw, g)
+    rows = P.view(-1, N)
+    assert float((torch.stack([r.double().sum() for r in rows.split(1)]) - 1.0).abs().max()) <= TOL[dtype]["rowsum"]
+    ids = np.unique(np.concatenate([np.arange(0, H * N, 211), [0, 127, 128, N - 1, H * N - 1]]))
+    err = np.max(np.abs(to_f64(rows[torch.from_numpy(ids).cuda()]) - oracle.attnw_rows(q, k, scale_of(d), ids)))
+    assert err <= TOL[dtype]["abs"]
+
+
+def test_more_streams_than_exchange_areas(attnw):
+    # twelve streams, two calls each in flight, on inputs of their own: no launch may read another's statistics
+    d, N = 64, 1536
+    cases = []
+    for s in range(12):
+        q, k = small_fused_inputs(1, 1, N, d, stream=700 + s)
+        cases.append((bits_to_cuda_bf16(q), bits_to_cuda_bf16(k), oracle.attnw(q, k, scale_of(d))))
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in cases]
+    for _ in range(3):
+        out = []
+        for dtype in (torch.bfloat16, torch.float32):
+            for (Q, K, _), s in zip(cases, streams):
+                with torch.cuda.stream(s):
+                    out.append(attnw.attnw_fused(Q, K, scale_of(d), out_dtype=dtype))
+        torch.cuda.synchronize()
+        assert attnw.query_status() == 0
+        for n, P in enumerate(out):
+            assert_close_to_oracle(P, cases[n % 12][2], f"stream {n % 12}")
+
+
+@pytest.mark.parametrize("entry,dtype", [("fused", torch.bfloat16), ("fused", torch.float32), ("noalloc", torch.bfloat16)])
+@pytest.mark.parametrize("N", [256, 2048])
+def test_captured_call_is_right_on_every_replay(attnw, entry, dtype, N):
+    d = 64
+    calls = [small_fused_inputs(1, 2, N, d, stream=800 + x) for x in range(3)]
+    Q, K = bits_to_cuda_bf16(calls[0][0]), bits_to_cuda_bf16(calls[0][1])
+    P = torch.empty((1, 2, N, N), dtype=dtype, device="cuda")
+
+    def call():
+        if entry == "fused":
+            attnw.attnw_fused(Q, K, scale_of(d), P=P)
+        else:
+            attnw.attnw_fused_noalloc(Q, K, scale_of(d), P=P)
+
+    call()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call()
+    for q, k in calls:  # other inputs on each replay
+        Q.copy_(bits_to_cuda_bf16(q))
+        K.copy_(bits_to_cuda_bf16(k))
+        P.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert attnw.query_status() == 0
+        assert_close_to_oracle(P, oracle.attnw(q, k, scale_of(d)), f"{entry} {dtype} N{N}")

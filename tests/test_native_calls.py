@@ -32,7 +32,7 @@ def test_bad_arguments_on_the_gpu(binding):
                       (ValueError, lambda: binding.attnw_fused(q, q[:, :1], 0.125)),
                       (ValueError, lambda: binding.attnw_fused(q.transpose(1, 2), q.transpose(1, 2), 0.125)),
                       (ValueError, lambda: binding.attnw_fused(q, q, 0.125, out_dtype=torch.float16)),
-                      (ValueError, lambda: binding.attnw_fused(q, q, 0.125, P=q)),
+                      (ValueError, lambda: binding.attnw_fused(q, q, 0.125, P=q[:, :1].contiguous())),
                       (ValueError, lambda: binding.attn_fused(q, q, q, 0.125, O=q[:, :1].contiguous())),
                       (ValueError, lambda: binding.project_qk(q[0], q[0], q[0, :1].contiguous())),
                       (ValueError, lambda: binding.softmax_rows(q.float())),
