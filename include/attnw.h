@@ -128,8 +128,9 @@ int attnw_set_attn_variant(int variant);
 
 /*
  * Which kernel attnw_fused uses (process-wide; the results are the same within the stated tolerances):
- *   0  choose by shape (default): the grid-row kernel (see 4; here it serves both types of P) for rows of up to 14336 keys
- *      whose groups leave at most a quarter of the SMs idle (every N <= 4096 on a B200); the two-pass kernel otherwise.
+ *   0  choose by shape (default): the grid-row kernel (see 4; here it serves both types of P) for rows of up to 28672 keys
+ *      whose groups leave at most a third of the SMs idle (on a B200 N <= 18944 and from 25345 on); the two-pass kernel
+ *      otherwise.
  *      On a device that cannot hold a whole group of the grid-row kernel at once the older choice applies: the SRAM-resident
  *      cluster kernel for bfloat16 P, with a large call split between it and the two-pass kernel on a per-device side
  *      stream that forks from and joins `stream` with events.

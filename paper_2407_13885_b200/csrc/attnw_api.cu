@@ -610,14 +610,15 @@ int launch_project(const void* X, const void* Wq, const void* Wk, void* Q, void*
 }
 
 // Whether the choice by shape takes the grid-row kernel for rows of N keys: it computes every score and exponential once, the
-// two-pass kernel twice, but groups of ceil(N / 256) CTAs leave SMs idle and the exchange grows with the group.
-// Measured on B200, us per call, two-pass -> grid-row: bfloat16, d = 64 or 128, B*H x N = 2 x 6000 (24 CTAs a group,
-// 144 SMs in use) 132 -> 45, 8 x 8192 (32, 128 SMs) 435 -> 360, 4 x 12288 (48, 144 SMs) 421 -> 335, 1 x 16384 (64, 128 SMs)
-// 189 -> 219; float32 2 x 512 16.4 -> 10.2, 20 x 1000 36.9 -> 22.6, 16 x 2052 111 -> 79, 32 x 4096 616 -> 506,
-// 4 x 8192 315 -> 244, 1 x 16384 314 -> 340.  So: groups of up to 56 that leave at most a quarter of the SMs idle.
+// two-pass kernel twice, but groups of ceil(N / 256) CTAs leave SMs idle, and the exchange grows with the group.
+// A 128 x 256 block costs it some 4450 cycles of an SM against 6000: it pays while two thirds of the SMs have work.
+// Measured on B200, us per call, two-pass -> grid-row, B*H x N (CTAs a group, SMs in use): bfloat16 2 x 6000 (24, 144)
+// 132 -> 39, 8 x 8192 (32, 128) 428 -> 319, 2 x 13000 (51, 102) 319 -> 233, 8 x 16384 (64, 128) 1551 -> 1212, 1 x 25600
+// (100, 100) 601 -> 425, 1 x 32768 (128, 128) 780 -> 803; float32 2 x 512 16.4 -> 10.2, 16 x 2052 112 -> 80, 32 x 4096
+// 613 -> 492, 2 x 13000 399 -> 355, 1 x 25600 776 -> 726, 1 x 32768 1193 -> 1254.
 bool gridrow_pays(const DeviceInfo* dev, int N) {
     const int group_ctas = (N + gr::kSlabCols - 1) / gr::kSlabCols;
-    return group_ctas <= 56 && dev->sm_count / group_ctas * group_ctas * 4 >= dev->sm_count * 3;
+    return group_ctas <= 112 && dev->sm_count / group_ctas * group_ctas * 3 >= dev->sm_count * 2;
 }
 
 template <typename OutT>

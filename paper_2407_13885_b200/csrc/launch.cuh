@@ -10,9 +10,10 @@ constexpr int kMaxDevices = 64;
 
 // Lets `Kernel` use `bytes` of dynamic shared memory on the current device and, with `large_clusters`, clusters of more
 // than 8 CTAs.  The setting belongs to the (kernel, device) pair and stays, so the driver is asked once per pair and not
-// on every call; every instantiation has one flag per device.  `bytes` is the most that any launch of the kernel asks for.
+// on every call; every instantiation has one flag per device (and internal linkage: two builds of the library in one
+// process have kernels of their own).  `bytes` is the most that any launch of the kernel asks for.
 template <auto Kernel>
-inline cudaError_t allow_smem(int bytes, bool large_clusters = false) {
+static inline cudaError_t allow_smem(int bytes, bool large_clusters = false) {
     static std::atomic<unsigned long long> done{0};
     static_assert(kMaxDevices <= 64, "one bit per device");
     int dev = -1;

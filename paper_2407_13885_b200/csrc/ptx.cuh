@@ -38,16 +38,26 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
+        : "r"(bar), "r"(parity)
         : "memory");
     return ok != 0;
+}
+
+__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) { return mbar_try_wait(smem_u32(bar), parity); }
+// One arrival where `pred` is not zero: predicated instead of branched around.
+__device__ __forceinline__ void mbar_arrive_if(uint32_t bar, uint32_t pred) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"(pred)
+        : "memory");
 }
 
 // ---- async-proxy fences and bulk groups --------------------------------------------------
@@ -101,6 +111,18 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* m, uint32_t smem
         "cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group.L2::cache_hint"
         " [%0, {%2, %3, %4}], [%1], %5;"
         ::"l"(reinterpret_cast<uint64_t>(m)), "r"(smem_src_addr), "r"(c0), "r"(c1), "r"(c2), "l"(policy)
+        : "memory");
+}
+
+// The same where `pred` is not zero.
+__device__ __forceinline__ void tma_store_3d_if(uint32_t pred, const CUtensorMap* m, uint32_t smem_src_addr, int c0, int c1, int c2,
+                                                uint64_t policy) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %6, 0;\n\t"
+        "@p cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group.L2::cache_hint"
+        " [%0, {%2, %3, %4}], [%1], %5;\n\t}"
+        ::"l"(reinterpret_cast<uint64_t>(m)), "r"(smem_src_addr), "r"(c0), "r"(c1), "r"(c2), "l"(policy), "r"(pred)
         : "memory");
 }
 
@@ -280,6 +302,12 @@ __device__ __forceinline__ float ex2_approx(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+// The same, kept in the order of the source among other volatile instructions.
+__device__ __forceinline__ float ex2_approx_ordered(float x) {
+    float y;
+    asm volatile("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 __device__ __forceinline__ float lg2_approx(float x) {
     float y;
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -341,6 +369,12 @@ __device__ __forceinline__ void scale_f16x2(uint32_t v, uint32_t f16_scale, floa
         "fma.rn.f32.f16 %0, l, f, 0f00000000;\n\tfma.rn.f32.f16 %1, h, f, 0f00000000;\n\t}"
         : "=f"(lo), "=f"(hi)
         : "r"(v), "r"(f16_scale));
+}
+__device__ __forceinline__ void st_shared_f32(uint32_t addr, float a) {
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(a) : "memory");
+}
+__device__ __forceinline__ void st_shared_v2(uint32_t addr, float a, float b) {
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
 }
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");

@@ -42,9 +42,9 @@ def test_float32_weights_match_oracle(attnw, B, H, N, d):
         assert_close_to_oracle(P, ref, f"B{B} H{H} N{N} d{d}")
 
 
-# groups of 17, 24, 33 and 48 CTAs (owners of 8, 8, 4 and 4 rows); the last row blocks and columns ragged
+# groups of 17, 24, 33, 48, 64 and 101 CTAs (owners of 8, 8, 4, 4, 2 and 2 rows); the last row blocks and columns ragged
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
-@pytest.mark.parametrize("H,N,d", [(2, 4104, 64), (1, 6000, 128), (1, 8456, 64), (1, 12288, 128)])
+@pytest.mark.parametrize("H,N,d", [(2, 4104, 64), (1, 6000, 128), (1, 8456, 64), (1, 12288, 128), (1, 16384, 64), (1, 25608, 64)])
 def test_long_rows_match_oracle(attnw, dtype, H, N, d):
     q, k = small_fused_inputs(1, H, N, d, sigma=1.5, stream=N + 1)
     raw, P, g = guarded_empty((1, H, N, N), dtype)
@@ -54,7 +54,7 @@ def test_long_rows_match_oracle(attnw, dtype, H, N, d):
     assert_guards_intact(raw, g)
     rows = P.view(-1, N)
     assert float((torch.stack([r.double().sum() for r in rows.split(1)]) - 1.0).abs().max()) <= TOL[dtype]["rowsum"]
-    ids = np.unique(np.concatenate([np.arange(0, H * N, 211), [0, 127, 128, N - 1, H * N - 1]]))
+    ids = np.unique(np.concatenate([np.arange(0, H * N, 211 if N < 10000 else 997), [0, 127, 128, N - 1, H * N - 1]]))
     err = np.max(np.abs(to_f64(rows[torch.from_numpy(ids).cuda()]) - oracle.attnw_rows(q, k, scale_of(d), ids)))
     assert err <= TOL[dtype]["abs"]
 
