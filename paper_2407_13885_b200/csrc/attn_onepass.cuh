@@ -1,8 +1,10 @@
 // Fused attention O = Softmax(scale * Q K^T) V for sm_100a in ONE pass over the keys: Attention(Q, K, V) of
 // Section IV (the product with V is the paper's future work, Section VIII) with the online form of Eq. 1.
 //
-// A CTA owns 256 query rows (two tiles).  Per key tile j and query tile q:
-//   MMA 1     S = Q_q K_j^T                       128 x 128 fp32 in tensor memory (one buffer per query tile)
+// A CTA holds two units that share its tensor pipe and its special function units: two query tiles of 128 rows over all
+// key tiles, or (split) ONE query tile, unit 0 over the even and unit 1 over the odd key tiles, merged at the end.
+// Per step j and unit q:
+//   MMA 1     S = Q K_j^T                         128 x 128 fp32 in tensor memory (one buffer per unit)
 //   Softmax   two threads per row, 64 columns each: a thread takes its scores to registers (the buffer is handed back
 //             at once, so the next tile's MMA 1 runs meanwhile) and also reads the other thread's 64 columns for
 //             their maximum, so both know the row maximum without an exchange; p = 2^(c s - mb) with the row's
@@ -12,19 +14,21 @@
 // The offset mb of a row follows its running maximum lazily: it moves only when the maximum has grown by more than 8
 // (in the base-2 exponent), and then O's row and l are multiplied by 2^(mb_old - mb_new) - after the first tiles
 // this is rare, and weights stay below 2^8.  The division by l happens once, in the epilogue.  One exponential and
-// two MMA passes per element.
+// two MMA passes per element.  (An offset that follows one step late, so that no exponential waits for a maximum, took 1.18 ms
+// instead of 1.01 at 128 x 4096, d = 128: 88 bytes of spills, and the maximum is not what the unit waits for.)
 // Valid for any N >= 1, d in {64, 128}; Q, K, V, O bf16 [B, H, N, d].
 #pragma once
+#include <cstddef>
+
 #include "attn_fused.cuh"
 
 namespace attnw {
 namespace av1 {
 
-constexpr int kSmWarps = 16;      // Softmax warps: query tile (2) x column half (2) x TMEM lane quarter (4)
+constexpr int kSmWarps = 16;      // Softmax warps: unit (2) x column half (2) x TMEM lane quarter (4)
 constexpr int kProducer = 16;
 constexpr int kMma = 17;
 constexpr int kThreads = 576;
-constexpr int kStages = 3;        // ring of K / V tiles (128 keys x d)
 constexpr float kLazy = 8.0f;     // the offset follows the maximum only when it has grown by more than this
 
 enum : uint32_t {  // wait sites of this kernel (low byte of the status word)
@@ -46,7 +50,8 @@ struct Smem {
     static constexpr int kAtomBytes = kTile * 128;             // 128 rows x 128 bytes
     static constexpr int kTileBytes = kAtoms * kAtomBytes;     // a Q, K or V tile
     static constexpr int kPBytes = 2 * kAtomBytes;             // a P tile: 128 rows x 128 keys, two atoms of 64 keys
-    static constexpr int kQOff = 0;
+    static constexpr int kStages = (D == 128) ? 3 : 6;         // ring of K / V tiles (128 keys x d)
+    static constexpr int kQOff = 0;                            // two query tiles; split: one, and one more stage of the ring
     static constexpr int kKOff = kQOff + 2 * kTileBytes;
     static constexpr int kPOff = kKOff + kStages * kTileBytes;
     static constexpr int kBarOff = kPOff + 2 * kPBytes;
@@ -57,11 +62,11 @@ static_assert(Smem<128>::kDynamicBytes <= 227 * 1024, "shared memory budget");
 
 struct Barriers {
     uint64_t q_full;
-    uint64_t k_full[kStages], k_empty[kStages];
-    uint64_t s_full[2], s_free[2];  // per query tile: scores written / read into registers (8 warps)
-    uint64_t p_full[2], p_free[2];  // per query tile: P tile written (8 warps) / read by its MMAs
-    uint64_t o_full;
-    uint64_t l_full[2];      // per query tile: the partial row sums of the 8 warps are in shared memory
+    uint64_t k_full[7], k_empty[7];
+    uint64_t s_full[2], s_free[2];  // per unit: scores written / read into registers (8 warps)
+    uint64_t p_full[2], p_free[2];  // per unit: P tile written (8 warps) / read by its MMAs
+    uint64_t o_full[2];             // per unit: every product complete
+    uint64_t l_full[2];             // per query tile: the row statistics of its warps are in shared memory
     uint64_t out_filled[2];
     uint32_t tmem_base;
     uint32_t abort_flag;
@@ -87,7 +92,7 @@ __device__ __forceinline__ bool wait_in_place(uint64_t* bar, uint32_t parity, vo
     }
 }
 
-template <int D>
+template <int D, bool split>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o, int N,
@@ -96,6 +101,8 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     Barriers* bars = reinterpret_cast<Barriers*>(smem + L::kBarOff);
+    const uint32_t bar = ptx::smem_u32(bars);
+    auto bar_of = [bar](size_t field, int n) { return bar + static_cast<uint32_t>(field) + 8u * static_cast<uint32_t>(n); };
     volatile uint32_t* abort_flag = &bars->abort_flag;
 
     if (threadIdx.x == 0) bars->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
@@ -105,14 +112,17 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int bh = blockIdx.x / row_blocks_per_head;
-    const int row0 = (blockIdx.x % row_blocks_per_head) * kRowsPerCta;
+    const int row0 = (blockIdx.x % row_blocks_per_head) * (split ? kTile : kRowsPerCta);
     const int T = (N + kTile - 1) / kTile;  // key tiles
-    const bool tile_active[2] = {row0 < N, row0 + kTile < N};
+    // key tiles of a unit: all of them, or every second one
+    const int steps[2] = {split ? (T + 1) >> 1 : T, split ? T >> 1 : (row0 + kTile < N ? T : 0)};
+    constexpr int kStages = L::kStages + (split ? 1 : 0);
+    auto stage_offset = [](int s) { return !split || s < L::kStages ? L::kKOff + s * L::kTileBytes : L::kQOff + L::kTileBytes; };
 
     // ---- set-up ------------------------------------------------------------------------------
     if (threadIdx.x == 0) {
         ptx::mbar_init(&bars->q_full, 1);
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < 7; ++s) {
             ptx::mbar_init(&bars->k_full[s], 1);
             ptx::mbar_init(&bars->k_empty[s], 1);
         }
@@ -121,10 +131,10 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             ptx::mbar_init(&bars->s_free[q], 8);
             ptx::mbar_init(&bars->p_full[q], 8);
             ptx::mbar_init(&bars->p_free[q], 1);
-            ptx::mbar_init(&bars->l_full[q], 8);
-            ptx::mbar_init(&bars->out_filled[q], 7);
+            ptx::mbar_init(&bars->o_full[q], 1);
+            ptx::mbar_init(&bars->l_full[q], split ? 16 : 8);
+            ptx::mbar_init(&bars->out_filled[q], split ? 15 : 7);
         }
-        ptx::mbar_init(&bars->o_full, 1);
         bars->abort_flag = 0;
         ptx::mbar_fence_init();
     }
@@ -142,35 +152,36 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bars->tmem_base;
-    // tensor memory: per query tile q, scores in columns [256 q, 256 q + 128), O in [256 q + 128, 256 q + 128 + d)
+    // tensor memory of unit q: scores in columns [256 q, 256 q + 128), O in [256 q + 128, 256 q + 128 + d)
 
     if (warp == kProducer) {
-        // ================= TMA producer: Q once, then K_0, [K_{j+1}, V_j] for j = 0 .. T-1 =================
+        // ================= TMA producer: Q once, then the K and V tiles in the order the MMA issuer reads them =========
         if (lane == 0) {
             const uint64_t keep = ptx::policy_evict_last();
-            int n_active = (tile_active[0] ? 1 : 0) + (tile_active[1] ? 1 : 0);
-            ptx::mbar_expect_tx(&bars->q_full, static_cast<uint32_t>(n_active * L::kTileBytes));
-            for (int q = 0; q < 2; ++q)
-                if (tile_active[q])
-                    for (int a = 0; a < L::kAtoms; ++a)
-                        ptx::tma_load_3d(smem + L::kQOff + q * L::kTileBytes + a * L::kAtomBytes, &tm_q, &bars->q_full,
-                                         a * 64, row0 + q * kTile, bh, keep);
+            const int q_tiles = (!split && steps[1] > 0) ? 2 : 1;
+            ptx::mbar_expect_tx(&bars->q_full, static_cast<uint32_t>(q_tiles * L::kTileBytes));
+            for (int q = 0; q < q_tiles; ++q)
+                for (int a = 0; a < L::kAtoms; ++a)
+                    ptx::tma_load_3d(smem + L::kQOff + q * L::kTileBytes + a * L::kAtomBytes, &tm_q, &bars->q_full, a * 64,
+                                     row0 + q * kTile, bh, keep);
             int n = 0;
             bool ok = true;
             auto load = [&](const CUtensorMap* map, int kt) {
+                if (!ok) return;
                 const int s = n % kStages;
                 ok = fused_wait(&bars->k_empty[s], (static_cast<uint32_t>(n / kStages) & 1u) ^ 1u, abort_flag, kSiteProducerEmpty);
                 if (!ok) return;
                 ptx::mbar_expect_tx(&bars->k_full[s], static_cast<uint32_t>(L::kTileBytes));
                 for (int a = 0; a < L::kAtoms; ++a)
-                    ptx::tma_load_3d(smem + L::kKOff + s * L::kTileBytes + a * L::kAtomBytes, map, &bars->k_full[s], a * 64,
-                                     kt * kTile, bh, keep);
+                    ptx::tma_load_3d(smem + stage_offset(n % kStages) + a * L::kAtomBytes, map, &bars->k_full[s], a * 64, kt * kTile, bh, keep);
                 ++n;
             };
-            load(&tm_k, 0);
-            for (int j = 0; ok && j < T; ++j) {
-                if (j + 1 < T) load(&tm_k, j + 1);
-                if (ok) load(&tm_v, j);
+            const int units = split ? 2 : 1;  // that have key tiles of their own
+            for (int j = -1; ok && j < steps[0]; ++j) {
+                for (int q = 0; q < units; ++q)
+                    if (j + 1 < steps[q]) load(&tm_k, units * (j + 1) + q);
+                for (int q = 0; j >= 0 && q < units; ++q)
+                    if (j < steps[q]) load(&tm_v, units * j + q);
             }
             if (*abort_flag) {
                 // Unwinding: let the copies already in flight land before shared memory is released.
@@ -186,265 +197,314 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 }
             }
         }
+        __syncwarp();
     } else if (warp == kMma) {
         // ================= MMA issuer (warp-uniform loop, one elected lane issues) =================
         constexpr uint32_t idesc_s = ptx::umma_idesc_bf16_f32(kTile, kTile);
         constexpr uint32_t idesc_o = ptx::umma_idesc_bf16_f32(kTile, D) | (1u << 16);  // B operand MN-major
-        const uint32_t q_addr = ptx::smem_u32(smem + L::kQOff);
-        const uint32_t k_addr = ptx::smem_u32(smem + L::kKOff);
-        const uint32_t p_addr = ptx::smem_u32(smem + L::kPOff);
-        bool ok = __all_sync(0xffffffffu, fused_wait(&bars->q_full, 0, abort_flag, kSiteMmaQ));
-        int n = 0;  // ring counter, in step with the producer
-        auto scores = [&](uint32_t j) {  // S_q = Q_q K_j^T for both query tiles
-            const int s = n % kStages;
-            ok = __all_sync(0xffffffffu, fused_wait(&bars->k_full[s], static_cast<uint32_t>(n / kStages) & 1u, abort_flag,
-                                                    kSiteMmaKFull));
-            if (!ok) return;
-            const uint32_t b_addr = k_addr + static_cast<uint32_t>(s * L::kTileBytes);
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                if (!tile_active[q]) continue;
-                // the row threads have the scores of tile j - 1 in registers
-                ok = __all_sync(0xffffffffu, fused_wait(&bars->s_free[q], (j & 1u) ^ 1u, abort_flag, kSiteMmaSFree));
-                if (!ok) return;
-                ptx::tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(q * 2 * kTile);
-                const uint32_t a_addr = q_addr + static_cast<uint32_t>(q * L::kTileBytes);
-                if (ptx::elect_one()) {
-#pragma unroll
-                    for (int k = 0; k < D / 16; ++k) {
-                        const uint32_t off = static_cast<uint32_t>((k >> 2) * L::kAtomBytes + (k & 3) * 32);
-                        ptx::umma_f16_ss(d_tmem, ptx::umma_desc_kmajor_sw128(a_addr + off),
-                                         ptx::umma_desc_kmajor_sw128(b_addr + off), idesc_s, k > 0 ? 1u : 0u);
-                    }
-                    ptx::umma_commit(&bars->s_full[q]);
-                }
-                __syncwarp();
-            }
-            if (ptx::elect_one()) ptx::umma_commit(&bars->k_empty[s]);
+        const uint32_t base = ptx::smem_u32(smem);
+        bool ok = warp_wait(bar_of(offsetof(Barriers, q_full), 0), 0, abort_flag, kSiteMmaQ);
+        int n = 0;            // next ring entry, in step with the producer
+        auto arrived = [&]() {
+            ok = ok && warp_wait(bar_of(offsetof(Barriers, k_full), n % kStages), static_cast<uint32_t>(n / kStages) & 1u, abort_flag, kSiteMmaKFull);
+        };
+        auto release = [&]() {  // the entry may be replaced once the MMAs issued so far are complete
+            if (ptx::elect_one()) ptx::umma_commit(&bars->k_empty[n % kStages]);
             __syncwarp();
             ++n;
         };
-        if (ok) scores(0u);
-        for (int j = 0; ok && j < T; ++j) {
-            // the scores of tile j + 1 first: the tensor pipe computes them while the row threads exponentiate tile j
-            if (j + 1 < T) scores(static_cast<uint32_t>(j) + 1u);
-            if (!ok) break;
-            const int s = n % kStages;
-            ok = __all_sync(0xffffffffu, fused_wait(&bars->k_full[s], static_cast<uint32_t>(n / kStages) & 1u, abort_flag,
-                                                    kSiteMmaKFull));
-            if (!ok) break;
-            const uint32_t v_addr = k_addr + static_cast<uint32_t>(s * L::kTileBytes);
+        auto scores = [&](int q, int j) {  // S of step j
+            // the row threads have the scores of step j - 1 in registers
+            ok = ok && warp_wait(bar_of(offsetof(Barriers, s_free), q), (static_cast<uint32_t>(j) & 1u) ^ 1u, abort_flag, kSiteMmaSFree);
+            if (!ok) return;
+            ptx::tc_fence_after_sync();
+            const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(q * 2 * kTile);
+            // (descriptors: the first of the tile plus a distance in 16-byte units)
+            const uint64_t a_desc = ptx::umma_desc_kmajor_sw128(base + L::kQOff + (split ? 0u : static_cast<uint32_t>(q * L::kTileBytes)));
+            const uint64_t b_desc = ptx::umma_desc_kmajor_sw128(base + static_cast<uint32_t>(stage_offset(n % kStages)));
+            if (ptx::elect_one()) {
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                if (!tile_active[q]) continue;
-                ok = __all_sync(0xffffffffu, fused_wait(&bars->p_full[q], static_cast<uint32_t>(j) & 1u, abort_flag, kSiteMmaPFull));
-                if (!ok) break;
-                ptx::tc_fence_after_sync();
-                const uint32_t o_tmem = tmem_base + static_cast<uint32_t>((q * 2 + 1) * kTile);
-                const uint32_t a_base = p_addr + static_cast<uint32_t>(q * L::kPBytes);
-                if (ptx::elect_one()) {
-#pragma unroll
-                    for (int kk = 0; kk < kTile / 16; ++kk) {  // 16 keys per instruction
-                        const uint32_t a_off = static_cast<uint32_t>((kk >> 2) * L::kAtomBytes + (kk & 3) * 32);
-                        ptx::umma_f16_ss(o_tmem, ptx::umma_desc_kmajor_sw128(a_base + a_off),
-                                         av::umma_desc_mnmajor_sw128(v_addr + static_cast<uint32_t>(kk * 16 * 128), L::kAtomBytes),
-                                         idesc_o, (j > 0 || kk > 0) ? 1u : 0u);
-                    }
-                    ptx::umma_commit(&bars->p_free[q]);
+                for (int k = 0; k < D / 16; ++k) {
+                    const uint64_t off = static_cast<uint64_t>(((k >> 2) * L::kAtomBytes + (k & 3) * 32) >> 4);
+                    ptx::umma_f16_ss(d_tmem, a_desc + off, b_desc + off, idesc_s, k > 0 ? 1u : 0u);
                 }
-                __syncwarp();
+                ptx::umma_commit(&bars->s_full[q]);
             }
-            if (!ok) break;
-            if (ptx::elect_one()) ptx::umma_commit(&bars->k_empty[s]);
             __syncwarp();
-            ++n;
+        };
+        auto product = [&](int q, int j) {  // O += P V of step j
+            ok = ok && warp_wait(bar_of(offsetof(Barriers, p_full), q), static_cast<uint32_t>(j) & 1u, abort_flag, kSiteMmaPFull);
+            if (!ok) return;
+            ptx::tc_fence_after_sync();
+            const uint32_t o_tmem = tmem_base + static_cast<uint32_t>((q * 2 + 1) * kTile);
+            const uint64_t a_desc = ptx::umma_desc_kmajor_sw128(base + L::kPOff + static_cast<uint32_t>(q * L::kPBytes));
+            const uint64_t b_desc = av::umma_desc_mnmajor_sw128(base + static_cast<uint32_t>(stage_offset(n % kStages)), L::kAtomBytes);
+            if (ptx::elect_one()) {
+#pragma unroll
+                for (int kk = 0; kk < kTile / 16; ++kk)  // 16 keys per instruction
+                    ptx::umma_f16_ss(o_tmem, a_desc + static_cast<uint64_t>(((kk >> 2) * L::kAtomBytes + (kk & 3) * 32) >> 4),
+                                     b_desc + static_cast<uint64_t>(kk * 16 * 128 >> 4), idesc_o, (j > 0 || kk > 0) ? 1u : 0u);
+                ptx::umma_commit(&bars->p_free[q]);
+                if (j + 1 == steps[q]) ptx::umma_commit(&bars->o_full[q]);
+            }
+            __syncwarp();
+        };
+        // The scores of step j + 1 first: the tensor pipe computes them while the row threads exponentiate step j.  Two query
+        // tiles alternate - scores of one, product of one, scores of the other, product of the other - which keeps their
+        // row threads half a step apart (d = 64, 128 x 4096: 888 -> 841 us against both scores first).
+        for (int j = -1; ok && j < steps[0]; ++j) {
+            if (split) {
+                for (int q = 0; q < 2; ++q)
+                    if (ok && j + 1 < steps[q]) {
+                        arrived();
+                        scores(q, j + 1);
+                        release();
+                    }
+                for (int q = 0; q < 2; ++q)
+                    if (ok && j >= 0 && j < steps[q]) {
+                        arrived();
+                        product(q, j);
+                        release();
+                    }
+            } else {
+                const bool next = j + 1 < T;
+                const int k_entry = n, v_entry = next ? n + 1 : n;  // K of step j + 1, V of step j
+                if (next) {
+                    arrived();
+                    scores(0, j + 1);
+                }
+                n = v_entry;
+                if (ok && j >= 0) {
+                    arrived();
+                    product(0, j);
+                }
+                if (ok && next) {
+                    n = k_entry;
+                    if (steps[1] > 0) scores(1, j + 1);
+                    release();
+                }
+                if (ok && j >= 0) {
+                    n = v_entry;
+                    if (steps[1] > 0) product(1, j);
+                    release();
+                }
+            }
         }
-        if (ok && ptx::elect_one()) ptx::umma_commit(&bars->o_full);
-        __syncwarp();
     } else if (warp < kSmWarps) {
         // ================= Softmax warps: two threads per query row, 64 key columns of a tile each =================
         const int q = warp >> 3;
         const int half = (warp >> 2) & 1;
         const int quarter = warp & 3;
-        if (tile_active[q]) {
-            const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(q * 2 * kTile);
-            const uint32_t t_own = t_lane + static_cast<uint32_t>(half * kHalf);
-            const uint32_t t_other = t_lane + static_cast<uint32_t>((half ^ 1) * kHalf);
-            const uint32_t o_own = t_lane + static_cast<uint32_t>(kTile + half * (D / 2));  // this thread's D/2 columns of O
-            const float c2 = scale_log2e;
-            const uint64_t c2c2 = ptx::pack2(c2, c2);
-            // this row in the P tile's atom of this column half (64 keys = 128 bytes, 16-byte pieces XOR-swizzled)
-            const int row = quarter * 32 + lane;
-            const uint32_t p_tile = ptx::smem_u32(smem + L::kPOff + q * L::kPBytes);
-            const uint32_t p_row = p_tile + static_cast<uint32_t>(half * L::kAtomBytes + row * 128);
-            const uint32_t sw = static_cast<uint32_t>(lane & 7);
-            float smax = -3.0e38f;  // running maximum of the raw scores of this row (all columns: both threads of a row
-                                    // compute it, each from the whole tile, so they agree without an exchange)
-            float mb = -3.0e38f;    // the offset the weights, l and O's row are relative to (follows smax * c2 lazily)
-            float l = 0.0f;         // sum of this thread's weights
-            bool ok = true;
+        const uint32_t t_quarter = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+        const uint32_t t_own = t_quarter + static_cast<uint32_t>(q * 2 * kTile + half * kHalf);
+        const uint32_t o_own = t_quarter + static_cast<uint32_t>((q * 2 + 1) * kTile + half * (D / 2));  // this thread's D/2 columns of O
+        const float c2 = scale_log2e;
+        const uint64_t c2c2 = ptx::pack2(c2, c2);
+        // this row in the P tile's atom of this column half (64 keys = 128 bytes, 16-byte pieces XOR-swizzled)
+        const int row = quarter * 32 + lane;
+        const uint32_t t_other = t_quarter + static_cast<uint32_t>(q * 2 * kTile + (half ^ 1) * kHalf);
+        const uint32_t lane0 = lane == 0;
+        const uint32_t p_row = ptx::smem_u32(smem + L::kPOff + q * L::kPBytes) + static_cast<uint32_t>(half * L::kAtomBytes + row * 128);
+        const uint32_t sw = static_cast<uint32_t>(lane & 7);
+        float smax = -3.0e38f;  // running maximum of the raw scores of this row (all columns: both threads of a row
+                                // compute it, each from the whole tile, so they agree without an exchange)
+        float mb = -3.0e38f;    // the offset the weights, l and O's row are relative to (follows smax * c2 lazily)
+        float l = 0.0f;         // sum of this thread's weights
+        bool ok = true;
 
-            for (int j = 0; ok && j < T; ++j) {
-                ok = __all_sync(0xffffffffu, fused_wait(&bars->s_full[q], static_cast<uint32_t>(j) & 1u, abort_flag, kSiteSFull));
-                if (!ok) break;
-                ptx::tc_fence_after_sync();
-                const int valid = N - j * kTile;  // key columns of this tile that exist
-                // ---- maximum of the other thread's 64 columns (read and dropped) ----
-                float mo = -3.0e38f;
+        for (int j = 0; ok && j < steps[q]; ++j) {
+            ok = __all_sync(0xffffffffu, fused_wait(&bars->s_full[q], static_cast<uint32_t>(j) & 1u, abort_flag, kSiteSFull));
+            if (!ok) break;
+            ptx::tc_fence_after_sync();
+            const int valid = N - (split ? 2 * j + q : j) * kTile;  // key columns of this tile that exist
+            // ---- maximum of the other thread's 64 columns (read and dropped) ----
+            float mo = -3.0e38f;
 #pragma unroll
-                for (int c = 0; c < kHalf / kChunk; ++c) {
-                    uint32_t r[kChunk];
-                    ptx::tmem_ld_32x32b_x32(t_other + static_cast<uint32_t>(c * kChunk), r);
-                    ptx::tmem_wait_ld();
-                    if (valid < kTile) {
-#pragma unroll
-                        for (int i = 0; i < kChunk; ++i)
-                            if ((half ^ 1) * kHalf + c * kChunk + i >= valid) r[i] = __float_as_uint(-3.0e38f);
-                    }
-                    float m0 = __uint_as_float(r[0]), m1 = __uint_as_float(r[1]), m2 = __uint_as_float(r[2]), m3 = __uint_as_float(r[3]);
-#pragma unroll
-                    for (int i = 4; i < kChunk; i += 8) {
-                        m0 = ptx::max3(m0, __uint_as_float(r[i + 0]), __uint_as_float(r[i + 1]));
-                        m1 = ptx::max3(m1, __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
-                        if (i + 4 < kChunk) {
-                            m2 = ptx::max3(m2, __uint_as_float(r[i + 4]), __uint_as_float(r[i + 5]));
-                            m3 = ptx::max3(m3, __uint_as_float(r[i + 6]), __uint_as_float(r[i + 7]));
-                        }
-                    }
-                    mo = fmaxf(mo, ptx::max3(fmaxf(m0, m1), m2, m3));
-                }
-                // ---- this thread's 64 scores into registers; the buffer goes back to the MMA issuer at once ----
-                float s[kHalf];
-                {
-                    uint32_t r0[kChunk], r1[kChunk];
-                    ptx::tmem_ld_32x32b_x32(t_own, r0);
-                    ptx::tmem_ld_32x32b_x32(t_own + kChunk, r1);
-                    ptx::tmem_wait_ld();
-#pragma unroll
-                    for (int i = 0; i < kChunk; ++i) {
-                        s[i] = __uint_as_float(r0[i]);
-                        s[kChunk + i] = __uint_as_float(r1[i]);
-                    }
-                }
-                ptx::tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(&bars->s_free[q]);
+            for (int c = 0; c < kHalf / kChunk; ++c) {
+                uint32_t r[kChunk];
+                ptx::tmem_ld_32x32b_x32(t_other + static_cast<uint32_t>(c * kChunk), r);
+                ptx::tmem_wait_ld();
                 if (valid < kTile) {
 #pragma unroll
-                    for (int i = 0; i < kHalf; ++i)
-                        if (half * kHalf + i >= valid) s[i] = -3.0e38f;
+                    for (int i = 0; i < kChunk; ++i)
+                        if ((half ^ 1) * kHalf + c * kChunk + i >= valid) r[i] = __float_as_uint(-3.0e38f);
                 }
-                // ---- row maximum, lazy offset ----
-                float m0 = s[0], m1 = s[1], m2 = s[2], m3 = s[3];
+                float m0 = __uint_as_float(r[0]), m1 = __uint_as_float(r[1]), m2 = __uint_as_float(r[2]), m3 = __uint_as_float(r[3]);
 #pragma unroll
-                for (int i = 4; i < kHalf; i += 8) {
-                    m0 = ptx::max3(m0, s[i + 0], s[i + 1]);
-                    m1 = ptx::max3(m1, s[i + 2], s[i + 3]);
-                    if (i + 4 < kHalf) {
-                        m2 = ptx::max3(m2, s[i + 4], s[i + 5]);
-                        m3 = ptx::max3(m3, s[i + 6], s[i + 7]);
+                for (int i = 4; i < kChunk; i += 8) {
+                    m0 = ptx::max3(m0, __uint_as_float(r[i + 0]), __uint_as_float(r[i + 1]));
+                    m1 = ptx::max3(m1, __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
+                    if (i + 4 < kChunk) {
+                        m2 = ptx::max3(m2, __uint_as_float(r[i + 4]), __uint_as_float(r[i + 5]));
+                        m3 = ptx::max3(m3, __uint_as_float(r[i + 6]), __uint_as_float(r[i + 7]));
                     }
                 }
-                smax = ptx::max3(smax, mo, ptx::max3(fmaxf(m0, m1), m2, m3));
-                const float mb_cand = fmaxf(smax * c2, -3.0e38f);
-                const bool move = j == 0 || mb_cand - mb > kLazy;
-                // the P tile and O are free once the MMAs of the previous key tile are complete
-                ok = __all_sync(0xffffffffu, wait_in_place(&bars->p_free[q], (static_cast<uint32_t>(j) & 1u) ^ 1u, abort_flag, kSitePFree));
-                if (!ok) break;
-                if (j == 0) {
-                    mb = mb_cand;
-                } else if (__any_sync(0xffffffffu, move)) {
-                    // rescale this thread's part of O's row and l to the new offset (factor 1 for the rows of the warp
-                    // that do not move; the other thread of the row takes the same decision)
-                    const float alpha = move ? ptx::ex2_approx(mb - mb_cand) : 1.0f;
-                    if (move) mb = mb_cand;
-                    l *= alpha;
-                    ptx::tc_fence_after_sync();
-#pragma unroll 1
-                    for (int c = 0; c < D / 2; c += 8) {  // 8 columns at a time: the row of scores stays in registers
-                        uint32_t r[8];
-                        ptx::tmem_ld_32x32b_x8(o_own + static_cast<uint32_t>(c), r);
-                        ptx::tmem_wait_ld();
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
-                        ptx::tmem_st_32x32b_x8(o_own + static_cast<uint32_t>(c), r);
-                    }
-                    ptx::tmem_wait_st();
-                }
-                // ---- weights: p = 2^(c2 s - mb) (below 2^8), row sum, bf16, into the P tile ----
-                const uint64_t nmb2 = ptx::pack2(-mb, -mb);
-                uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
-#pragma unroll
-                for (int g = 0; g < kHalf / 8; ++g) {  // 8 keys = one 16-byte piece of the row
-                    float p[8];
-#pragma unroll
-                    for (int i = 0; i < 8; i += 2) {
-                        float x0, x1;
-                        ptx::unpack2(ptx::fma2(ptx::pack2(s[g * 8 + i], s[g * 8 + i + 1]), c2c2, nmb2), x0, x1);
-                        p[i] = ptx::ex2_approx(x0);
-                        p[i + 1] = ptx::ex2_approx(x1);
-                        if (valid < kTile) {  // columns beyond N: weight zero
-                            p[i] = (half * kHalf + g * 8 + i < valid) ? p[i] : 0.0f;
-                            p[i + 1] = (half * kHalf + g * 8 + i + 1 < valid) ? p[i + 1] : 0.0f;
-                        }
-                        acc[(i >> 1) & 3] = ptx::add2(acc[(i >> 1) & 3], ptx::pack2(p[i], p[i + 1]));
-                    }
-                    ptx::st_shared_v4(p_row + ((static_cast<uint32_t>(g) ^ sw) << 4), ptx::pack_bf16x2(p[0], p[1]),
-                                      ptx::pack_bf16x2(p[2], p[3]), ptx::pack_bf16x2(p[4], p[5]), ptx::pack_bf16x2(p[6], p[7]));
-                }
-                float a0, a1, a2, a3;
-                ptx::unpack2(ptx::add2(acc[0], acc[1]), a0, a1);
-                ptx::unpack2(ptx::add2(acc[2], acc[3]), a2, a3);
-                l += (a0 + a1) + (a2 + a3);
-                ptx::tc_fence_before_sync();  // orders the rescale of O before the MMAs that accumulate into it
-                ptx::fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(&bars->p_full[q]);
+                mo = fmaxf(mo, ptx::max3(fmaxf(m0, m1), m2, m3));
             }
-
-            // ---- epilogue: O / l -> bf16 -> the P tile's shared memory -> TMA stores ----
-            if (ok) ok = __all_sync(0xffffffffu, fused_wait(&bars->o_full, 0, abort_flag, kSiteOFull));
-            if (ok) {
-                // every MMA is complete: the K / V ring is free and carries the two partial row sums to each other
-                float* lx = reinterpret_cast<float*>(smem + L::kKOff);
-                lx[(q * 2 + half) * kTile + row] = l;
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(&bars->l_full[q]);
-                ok = __all_sync(0xffffffffu, fused_wait(&bars->l_full[q], 0, abort_flag, kSiteLFull));
+            // ---- this thread's 64 scores into registers; the buffer goes back to the MMA issuer at once ----
+            float s[kHalf];
+            {
+                uint32_t r0[kChunk], r1[kChunk];
+                ptx::tmem_ld_32x32b_x32(t_own, r0);
+                ptx::tmem_ld_32x32b_x32(t_own + kChunk, r1);
+                ptx::tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < kChunk; ++i) {
+                    s[i] = __uint_as_float(r0[i]);
+                    s[kChunk + i] = __uint_as_float(r1[i]);
+                }
             }
-            if (ok) {
-                const float* lx = reinterpret_cast<const float*>(smem + L::kKOff);
-                const float inv_l = 1.0f / (l + lx[(q * 2 + (half ^ 1)) * kTile + row]);
+            ptx::tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&bars->s_free[q]);
+            if (valid < kTile) {
+#pragma unroll
+                for (int i = 0; i < kHalf; ++i)
+                    if (half * kHalf + i >= valid) s[i] = -3.0e38f;
+            }
+            // ---- row maximum, lazy offset ----
+            float m0 = s[0], m1 = s[1], m2 = s[2], m3 = s[3];
+#pragma unroll
+            for (int i = 4; i < kHalf; i += 8) {
+                m0 = ptx::max3(m0, s[i + 0], s[i + 1]);
+                m1 = ptx::max3(m1, s[i + 2], s[i + 3]);
+                if (i + 4 < kHalf) {
+                    m2 = ptx::max3(m2, s[i + 4], s[i + 5]);
+                    m3 = ptx::max3(m3, s[i + 6], s[i + 7]);
+                }
+            }
+            smax = ptx::max3(smax, mo, ptx::max3(fmaxf(m0, m1), m2, m3));
+            const float mb_cand = fmaxf(smax * c2, -3.0e38f);
+            const bool move = j == 0 || mb_cand - mb > kLazy;
+            // the P tile and O are free once the MMAs of the previous key tile are complete
+            ok = __all_sync(0xffffffffu, wait_in_place(&bars->p_free[q], (static_cast<uint32_t>(j) & 1u) ^ 1u, abort_flag, kSitePFree));
+            if (!ok) break;
+            if (j == 0) {
+                mb = mb_cand;
+            } else if (__any_sync(0xffffffffu, move)) {
+                // rescale this thread's part of O's row and l to the new offset (factor 1 for the rows of the warp
+                // that do not move; the other thread of the row takes the same decision)
+                const float alpha = move ? ptx::ex2_approx(mb - mb_cand) : 1.0f;
+                if (move) mb = mb_cand;
+                l *= alpha;
                 ptx::tc_fence_after_sync();
 #pragma unroll 1
-                for (int c = 0; c < D / 2 / kChunk; ++c) {
-                    float o[kChunk];
-                    load_chunk(o_own + static_cast<uint32_t>(c * kChunk), o);
-                    const int col = half * (D / 2) + c * kChunk;  // first of these 32 columns of O
-                    const uint32_t dst = p_tile + static_cast<uint32_t>((col >> 6) * L::kAtomBytes + row * 128);
-                    const uint32_t piece0 = static_cast<uint32_t>((col & 63) >> 3);
+                for (int c = 0; c < D / 2; c += 8) {  // 8 columns at a time: the row of scores stays in registers
+                    uint32_t r[8];
+                    ptx::tmem_ld_32x32b_x8(o_own + static_cast<uint32_t>(c), r);
+                    ptx::tmem_wait_ld();
 #pragma unroll
-                    for (int g = 0; g < 4; ++g)
-                        ptx::st_shared_v4(dst + (((piece0 + static_cast<uint32_t>(g)) ^ sw) << 4),
-                                          ptx::pack_bf16x2(o[g * 8 + 0] * inv_l, o[g * 8 + 1] * inv_l),
-                                          ptx::pack_bf16x2(o[g * 8 + 2] * inv_l, o[g * 8 + 3] * inv_l),
-                                          ptx::pack_bf16x2(o[g * 8 + 4] * inv_l, o[g * 8 + 5] * inv_l),
-                                          ptx::pack_bf16x2(o[g * 8 + 6] * inv_l, o[g * 8 + 7] * inv_l));
+                    for (int i = 0; i < 8; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
+                    ptx::tmem_st_32x32b_x8(o_own + static_cast<uint32_t>(c), r);
+                }
+                ptx::tmem_wait_st();
+            }
+            // ---- weights: p = 2^(c2 s - mb) (below 2^8), row sum, bf16, into the P tile ----
+            const uint64_t nmb2 = ptx::pack2(-mb, -mb);
+            uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+            for (int g = 0; g < kHalf / 8; ++g) {  // 8 keys = one 16-byte piece of the row
+                float p[8];
+#pragma unroll
+                for (int i = 0; i < 8; i += 2) {
+                    float x0, x1;
+                    ptx::unpack2(ptx::fma2(ptx::pack2(s[g * 8 + i], s[g * 8 + i + 1]), c2c2, nmb2), x0, x1);
+                    p[i] = ptx::ex2_approx(x0);
+                    p[i + 1] = ptx::ex2_approx(x1);
+                    if (valid < kTile) {  // columns beyond N: weight zero
+                        p[i] = (half * kHalf + g * 8 + i < valid) ? p[i] : 0.0f;
+                        p[i + 1] = (half * kHalf + g * 8 + i + 1 < valid) ? p[i + 1] : 0.0f;
+                    }
+                    acc[(i >> 1) & 3] = ptx::add2(acc[(i >> 1) & 3], ptx::pack2(p[i], p[i + 1]));
+                }
+                ptx::st_shared_v4(p_row + ((static_cast<uint32_t>(g) ^ sw) << 4), ptx::pack_bf16x2(p[0], p[1]),
+                                  ptx::pack_bf16x2(p[2], p[3]), ptx::pack_bf16x2(p[4], p[5]), ptx::pack_bf16x2(p[6], p[7]));
+            }
+            float a0, a1, a2, a3;
+            ptx::unpack2(ptx::add2(acc[0], acc[1]), a0, a1);
+            ptx::unpack2(ptx::add2(acc[2], acc[3]), a2, a3);
+            l += (a0 + a1) + (a2 + a3);
+            ptx::tc_fence_before_sync();  // orders the rescale of O before the MMAs that accumulate into it
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&bars->p_full[q]);
+        }
+
+        // ---- epilogue: O / l -> bf16 -> the P tile's shared memory -> TMA stores ----
+        if (steps[q] > 0) {
+            // Two units of one query tile each finish alone.  Two units of the same query tile meet here: the four threads of a
+            // row take D / 4 columns each of 2^(mb_0 - mb) O_0 + 2^(mb_1 - mb) O_1.
+            const int u = split ? 0 : q;  // the barriers and the P tile this epilogue uses
+            float* lx = reinterpret_cast<float*>(smem + L::kKOff);  // (every MMA is complete: the K / V ring is free)
+            float* ox = lx + 4 * kTile;
+            if (ok) ok = warp_wait(bar_of(offsetof(Barriers, o_full), q), 0, abort_flag, kSiteOFull);
+            if (ok && steps[q ^ 1] > 0) ok = warp_wait(bar_of(offsetof(Barriers, o_full), q ^ 1), 0, abort_flag, kSiteOFull);
+            if (ok) {
+                lx[(q * 2 + half) * kTile + row] = l;
+                if (half == 0) ox[q * kTile + row] = mb;
+                __syncwarp();
+                ptx::mbar_arrive_if(bar_of(offsetof(Barriers, l_full), u), lane0);
+                ok = warp_wait(bar_of(offsetof(Barriers, l_full), u), 0, abort_flag, kSiteLFull);
+            }
+            if (ok) {
+                float f_own, f_other = 0.0f;
+                const float l_own = l + lx[(q * 2 + (half ^ 1)) * kTile + row];
+                if (split) {
+                    const float mb_other = ox[(q ^ 1) * kTile + row];
+                    const float top = fmaxf(mb, mb_other);
+                    f_own = ptx::ex2_approx(mb - top);
+                    f_other = ptx::ex2_approx(mb_other - top);
+                    const float* lo = lx + (q ^ 1) * 2 * kTile + row;
+                    const float inv = 1.0f / (l_own * f_own + (lo[0] + lo[kTile]) * f_other);
+                    f_own *= inv;
+                    f_other *= inv;
+                } else {
+                    f_own = 1.0f / l_own;
+                }
+                ptx::tc_fence_after_sync();
+                const int cols = split ? D / 4 : D / 2;
+                const int col0 = split ? (q * 2 + half) * (D / 4) : half * (D / 2);
+                const uint32_t o_unit = t_quarter + static_cast<uint32_t>((q * 2 + 1) * kTile);
+                const uint32_t o_peer = t_quarter + static_cast<uint32_t>(((q ^ 1) * 2 + 1) * kTile);
+                const uint32_t dst_row = ptx::smem_u32(smem + L::kPOff + u * L::kPBytes) + static_cast<uint32_t>(row * 128);
+#pragma unroll 1
+                for (int c = col0; c < col0 + cols; c += 16) {
+                    uint32_t o[16];
+                    ptx::tmem_ld_32x32b_x16(o_unit + static_cast<uint32_t>(c), o);
+                    ptx::tmem_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f_own);
+                    if (split) {
+                        uint32_t r[16];
+                        ptx::tmem_ld_32x32b_x16(o_peer + static_cast<uint32_t>(c), r);
+                        ptx::tmem_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(fmaf(__uint_as_float(r[i]), f_other, __uint_as_float(o[i])));
+                    }
+                    const uint32_t dst = dst_row + static_cast<uint32_t>((c >> 6) * L::kAtomBytes);
+                    const uint32_t piece = static_cast<uint32_t>((c & 63) >> 3);
+#pragma unroll
+                    for (int g = 0; g < 2; ++g) {
+                        uint32_t w[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            w[i] = ptx::pack_bf16x2(__uint_as_float(o[g * 8 + 2 * i]), __uint_as_float(o[g * 8 + 2 * i + 1]));
+                        ptx::st_shared_v4(dst + (((piece + static_cast<uint32_t>(g)) ^ sw) << 4), w[0], w[1], w[2], w[3]);
+                    }
                 }
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
-                if (quarter == 0 && half == 0) {
-                    ok = __all_sync(0xffffffffu, fused_wait(&bars->out_filled[q], 0, abort_flag, kSiteOutFilled));
+                if (quarter == 0 && half == 0 && q == u) {
+                    ok = warp_wait(bar_of(offsetof(Barriers, out_filled), u), 0, abort_flag, kSiteOutFilled);
                     if (ok && lane == 0) {
                         for (int a = 0; a < L::kAtoms; ++a)
-                            ptx::tma_store_3d(&tm_o, p_tile + static_cast<uint32_t>(a * L::kAtomBytes), a * 64, row0 + q * kTile, bh,
-                                              ptx::policy_evict_first());
+                            ptx::tma_store_3d(&tm_o, ptx::smem_u32(smem + L::kPOff + u * L::kPBytes + a * L::kAtomBytes), a * 64,
+                                              row0 + u * kTile, bh, ptx::policy_evict_first());
                         ptx::bulk_commit_group();
                         ptx::bulk_wait_group<0>();
                     }
-                } else if (lane == 0) {
-                    ptx::mbar_arrive(&bars->out_filled[q]);
+                } else {
+                    ptx::mbar_arrive_if(bar_of(offsetof(Barriers, out_filled), u), lane0);
                 }
             }
         }

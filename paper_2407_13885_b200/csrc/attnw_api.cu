@@ -523,21 +523,29 @@ int launch_attn(const void* Q, const void* K, const void* V, void* O, int BH, in
 }
 
 template <int D>
-int launch_attn_onepass(const void* Q, const void* K, const void* V, void* O, int BH, int N, float scale, cudaStream_t stream) {
+int launch_attn_onepass(const DeviceInfo* dev, const void* Q, const void* K, const void* V, void* O, int BH, int N, float scale, cudaStream_t stream) {
     using L = av1::Smem<D>;
-    auto kernel = av1::attn_onepass_kernel<D>;
     CUtensorMap tm_q, tm_k, tm_v, tm_o;
     int rc = encode_3d(&tm_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Q, D, N, BH, 64, kTile);
     if (rc == ATTNW_OK) rc = encode_3d(&tm_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, D, N, BH, 64, kTile);
     if (rc == ATTNW_OK) rc = encode_3d(&tm_v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, V, D, N, BH, 64, kTile);
     if (rc == ATTNW_OK) rc = encode_3d(&tm_o, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, O, D, N, BH, 64, kTile);
     if (rc != ATTNW_OK) return rc;
-    if (allow_smem<av1::attn_onepass_kernel<D>>(L::kDynamicBytes) != cudaSuccess) {
+    // Two query tiles per CTA, or one whose even and odd key tiles are worked on side by side: twice the CTAs of half the
+    // length, chosen when that takes 5 % fewer rounds of key tiles on the device.
+    const long long tiles = (N + kTile - 1) / kTile, pairs = (tiles + 1) / 2;
+    const long long rounds = (BH * pairs + dev->sm_count - 1) / dev->sm_count * tiles;
+    const long long rounds_split = (BH * tiles + dev->sm_count - 1) / dev->sm_count * pairs;
+    const bool split = tiles > 1 && BH * tiles <= INT_MAX && rounds_split * 105 < rounds * 100;
+    const int row_blocks = static_cast<int>(split ? tiles : pairs);
+    const float scale_log2e = static_cast<float>(static_cast<double>(scale) * 1.4426950408889634074);
+    const cudaError_t allowed = split ? allow_smem<av1::attn_onepass_kernel<D, true>>(L::kDynamicBytes)
+                                      : allow_smem<av1::attn_onepass_kernel<D, false>>(L::kDynamicBytes);
+    if (allowed != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
     }
-    const int row_blocks = (N + kRowsPerCta - 1) / kRowsPerCta;
-    const float scale_log2e = static_cast<float>(static_cast<double>(scale) * 1.4426950408889634074);
+    auto kernel = split ? av1::attn_onepass_kernel<D, true> : av1::attn_onepass_kernel<D, false>;
     kernel<<<static_cast<unsigned>(BH * row_blocks), av1::kThreads, L::kDynamicBytes, stream>>>(tm_q, tm_k, tm_v, tm_o, N,
                                                                                                  row_blocks, scale_log2e);
     if (cudaGetLastError() != cudaSuccess) return ATTNW_ERR_CUDA;
@@ -919,8 +927,8 @@ int attn_fused(const void* Q, const void* K, const void* V, void* O, int B, int 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (g_attn_variant.load(std::memory_order_relaxed) == 1)
         return d == 64 ? launch_attn<64>(Q, K, V, O, B * H, N, scale, s) : launch_attn<128>(Q, K, V, O, B * H, N, scale, s);
-    return d == 64 ? launch_attn_onepass<64>(Q, K, V, O, B * H, N, scale, s)
-                   : launch_attn_onepass<128>(Q, K, V, O, B * H, N, scale, s);
+    return d == 64 ? launch_attn_onepass<64>(dev, Q, K, V, O, B * H, N, scale, s)
+                   : launch_attn_onepass<128>(dev, Q, K, V, O, B * H, N, scale, s);
 }
 
 int attnw_project_qk(const void* X, const void* Wq, const void* Wk, void* Q, void* K, int B, int N, int d_model, int H, int d,

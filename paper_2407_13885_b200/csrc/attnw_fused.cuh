@@ -138,6 +138,28 @@ __device__ __forceinline__ bool fused_wait(uint64_t* bar, uint32_t parity, volat
     return fused_wait_slow(bar, parity, abort_flag, site);
 }
 
+// Bounded wait of a whole warp on an mbarrier phase; the same answer in every lane.  false = gave up.  For kernels whose waits
+// are many and short: one vote and one branch where the phase is over, and 32-bit shared-memory addresses.
+__device__ __noinline__ bool warp_wait_slow(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t site) {
+    const long long t0 = clock64();
+    for (uint32_t spin = 1;; ++spin) {
+        if (__all_sync(0xffffffffu, ptx::mbar_try_wait(bar, parity))) return true;
+        if ((spin & 63u) == 0) {
+            bool give_up = *abort_flag != 0u;
+            if (!give_up && clock64() - t0 > kWaitLimitCycles) {
+                *abort_flag = 1;
+                atomicCAS(&g_attnw_status, 0u, 0x80000000u | site);
+                give_up = true;
+            }
+            if (__any_sync(0xffffffffu, give_up)) return false;
+        }
+    }
+}
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t site) {
+    if (__all_sync(0xffffffffu, ptx::mbar_try_wait(bar, parity))) return true;
+    return warp_wait_slow(bar, parity, abort_flag, site);
+}
+
 // One thread's 32 consecutive columns of a score tile (TMEM lane = row).
 __device__ __forceinline__ void load_chunk(uint32_t taddr, float (&s)[kChunk]) {
     uint32_t r[32];

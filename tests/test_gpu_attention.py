@@ -167,3 +167,15 @@ def test_attention_full_size_sampled(attnw):
     err = np.abs(got - ref)
     tol = tolerance_map(q, k, v, w.scale, ref, row_ids=ids)
     assert np.all(err <= tol), (float(err.max()), float((err / tol).max()))
+
+
+# One query tile per CTA over two halves of the keys (few CTAs) against two query tiles per CTA (many): 2, 3, 8 and 16 key tiles,
+# an odd number of them, ragged last tiles, a second query tile that does not exist
+@pytest.mark.parametrize("B,H,N,d", [(1, 1, 129, 64), (1, 2, 300, 128), (1, 3, 1021, 64), (2, 2, 2048, 128), (4, 37, 200, 64), (4, 37, 257, 128)])
+def test_attention_split_and_whole(attnw, B, H, N, d):
+    q, k = small_fused_inputs(B, H, N, d, sigma=2.0, stream=N + d + 23)
+    v = rand_v(B, H, N, d, stream=N + d + 25)
+    scale = float(np.float32(1.0 / math.sqrt(d)))
+    ref = oracle.attn(q, k, v, scale)
+    got = run_attn(attnw, q, k, v, scale).double().cpu().numpy().reshape(ref.shape)
+    assert np.all(np.abs(got - ref) <= tolerance_map(q, k, v, scale, ref))
