@@ -577,9 +577,9 @@ int validate_project(const void* X, const void* Wq, const void* Wk, const void* 
     if (N > (1 << 24) || d_model > (1 << 20)) return ATTNW_ERR_BAD_SHAPE;  // keeps every tensor-map stride below 2^40 bytes
     const long long bh = static_cast<long long>(B) * H;
     if (bh > INT_MAX || static_cast<long long>(H) * d > INT_MAX) return ATTNW_ERR_BAD_SHAPE;
-    const long long col_tiles = (static_cast<long long>(H) * d + proj::kCols - 1) / proj::kCols;
-    const long long row_tiles = (static_cast<long long>(N) + proj::kRows - 1) / proj::kRows;
-    if (2 * col_tiles * row_tiles * B > INT_MAX) return ATTNW_ERR_BAD_SHAPE;
+    const long long col_tiles = (static_cast<long long>(H) * d + 127) / 128;  // the smallest tiles the call may be cut into
+    const long long row_tiles = (static_cast<long long>(N) + 127) / 128;
+    if (2 * col_tiles * row_tiles > INT_MAX / B) return ATTNW_ERR_BAD_SHAPE;
     if (d != 64 && d != 128) return ATTNW_ERR_UNSUPPORTED;
     if (d_model % 8 != 0) return ATTNW_ERR_MISALIGNED;  // rows of X and of the weights must start on 16-byte boundaries
     if (!aligned16(X) || !aligned16(Wq) || !aligned16(Wk) || !aligned16(Q) || !aligned16(K)) return ATTNW_ERR_MISALIGNED;
@@ -593,28 +593,50 @@ int validate_project(const void* X, const void* Wq, const void* Wk, const void* 
     return ATTNW_OK;
 }
 
-int launch_project(const void* X, const void* Wq, const void* Wk, void* Q, void* K, int B, int N, int d_model, int H, int d,
-                   cudaStream_t stream) {
-    CUtensorMap tm_x, tm_wq, tm_wk, tm_q, tm_k;
-    const uint64_t hd = static_cast<uint64_t>(H) * d;
-    int rc = encode_3d(&tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, d_model, N, B, proj::kKSlice, 128);
-    if (rc == ATTNW_OK) rc = encode_3d(&tm_wq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Wq, d_model, hd, 1, proj::kKSlice, 128);
-    if (rc == ATTNW_OK) rc = encode_3d(&tm_wk, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Wk, d_model, hd, 1, proj::kKSlice, 128);
-    if (rc == ATTNW_OK) rc = encode_3d(&tm_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Q, d, N, static_cast<uint64_t>(B) * H, 64, 128);
-    if (rc == ATTNW_OK) rc = encode_3d(&tm_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, d, N, static_cast<uint64_t>(B) * H, 64, 128);
-    if (rc != ATTNW_OK) return rc;
-    if (allow_smem<proj::project_qk_kernel>(proj::kDynamicBytes) != cudaSuccess) {
+struct ProjectMaps {
+    CUtensorMap x, wq, wk, q, k;
+};
+
+template <int RB, int CB>
+int launch_project_tile(const ProjectMaps& m, int B, int N, int d_model, int H, int d, cudaStream_t stream) {
+    using L = proj::Tile<RB, CB>;
+    if (allow_smem<proj::project_qk_kernel<RB, CB>>(L::kDynamicBytes) != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
     }
-    const int col_tiles = static_cast<int>((hd + proj::kCols - 1) / proj::kCols);
-    const int row_tiles = (N + proj::kRows - 1) / proj::kRows;
+    const int col_tiles = static_cast<int>((static_cast<long long>(H) * d + L::kCols - 1) / L::kCols);
+    const int row_tiles = (N + L::kRows - 1) / L::kRows;
     const unsigned ctas = static_cast<unsigned>(2 * col_tiles) * static_cast<unsigned>(row_tiles) * static_cast<unsigned>(B);
-    proj::project_qk_kernel<<<ctas, proj::kThreads, proj::kDynamicBytes, stream>>>(tm_x, tm_wq, tm_wk, tm_q, tm_k, N, d_model, H,
-                                                                                     d, col_tiles, row_tiles);
+    proj::project_qk_kernel<RB, CB><<<ctas, proj::kThreads, L::kDynamicBytes, stream>>>(m.x, m.wq, m.wk, m.q, m.k, N, d_model, H, d,
+                                                                                         col_tiles, row_tiles);
     if (cudaGetLastError() != cudaSuccess) return ATTNW_ERR_CUDA;
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return ATTNW_OK;
+}
+
+int launch_project(const DeviceInfo* dev, const void* X, const void* Wq, const void* Wk, void* Q, void* K, int B, int N, int d_model,
+                   int H, int d, cudaStream_t stream) {
+    ProjectMaps m;
+    const uint64_t hd = static_cast<uint64_t>(H) * d;
+    int rc = encode_3d(&m.x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, d_model, N, B, proj::kKSlice, 128);
+    if (rc == ATTNW_OK) rc = encode_3d(&m.wq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Wq, d_model, hd, 1, proj::kKSlice, 128);
+    if (rc == ATTNW_OK) rc = encode_3d(&m.wk, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Wk, d_model, hd, 1, proj::kKSlice, 128);
+    if (rc == ATTNW_OK) rc = encode_3d(&m.q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Q, d, N, static_cast<uint64_t>(B) * H, 64, 128);
+    if (rc == ATTNW_OK) rc = encode_3d(&m.k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, d, N, static_cast<uint64_t>(B) * H, 64, 128);
+    if (rc != ATTNW_OK) return rc;
+    // Rounds of tiles on the device times the cost of a tile: a tile of a half or a quarter of the work takes 0.55 or 0.32 of
+    // the time, since it fetches more bytes a flop.  Measured, us per call, 256 x 256 / 128 x 256 / 128 x 128 tiles, for
+    // B x N x d_model to H x d: 1 x 1024 x 1024 to 16 x 64 (32 / 64 / 128 tiles) 17.6 / 12.5 / 10.4, 1 x 146 x 1080 to 29 x 128
+    // 18.6 / 16.6 / 13.5, 1 x 512 x 4096 to 32 x 128 (64 / 128 / 256) 47.7 / 38.5 / 45.2, 2 x 469 x 3840 to 60 x 64
+    // (120 / 240 / 480) 54.9 / 61.4 / 77.8, 4 x 4096 x 4096 to 32 x 128 837 / 923 / 1199.
+    auto cost = [&](int rb, int cb, double per_tile) {
+        const long long tiles = 2 * ((static_cast<long long>(hd) + 128 * cb - 1) / (128 * cb)) * ((N + 128 * rb - 1) / (128 * rb)) * B;
+        return static_cast<double>((tiles + dev->sm_count - 1) / dev->sm_count) * per_tile;
+    };
+    const double c22 = cost(2, 2, 1.0), c12 = cost(1, 2, 0.55), c11 = cost(1, 1, 0.32);
+    if (c22 <= c12 && c22 <= c11) return launch_project_tile<2, 2>(m, B, N, d_model, H, d, stream);
+    if (c12 <= c11) return launch_project_tile<1, 2>(m, B, N, d_model, H, d, stream);
+    return launch_project_tile<1, 1>(m, B, N, d_model, H, d, stream);
 }
 
 // Whether the choice by shape takes the grid-row kernel for rows of N keys: it computes every score and exponential once, the
@@ -940,7 +962,7 @@ int attnw_project_qk(const void* X, const void* Wq, const void* Wk, void* Q, voi
     if (rc != ATTNW_OK) return rc;
     rc = load_encoder();
     if (rc != ATTNW_OK) return rc;
-    return launch_project(X, Wq, Wk, Q, K, B, N, d_model, H, d, static_cast<cudaStream_t>(stream));
+    return launch_project(dev, X, Wq, Wk, Q, K, B, N, d_model, H, d, static_cast<cudaStream_t>(stream));
 }
 
 int attnw_set_rows_variant(int variant) {

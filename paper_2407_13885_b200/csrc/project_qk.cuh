@@ -6,7 +6,7 @@
 // A plain dense contraction, so it runs on the tensor cores: a CTA owns a 256 x 256 tile of one of the two
 // outputs (256 rows of one batch entry x 256 output features = 2 or 4 heads), four 128 x 128 fp32 accumulators in
 // tensor memory (all 512 columns), a 3-stage TMA ring of [256 x 64] slices of X and of the weights (64 KB a stage),
-// tcgen05 MMAs of shape 128 x 256 x 16.  Weights are stored [H, d, d_model] (feature c of head h contiguous along
+// tcgen05 MMAs of shape 128 x 256 x 16.  Smaller calls take tiles of 128 x 256 or 128 x 128, which fill more SMs.  Weights are stored [H, d, d_model] (feature c of head h contiguous along
 // d_model), which is the K-major B operand TMA can deliver as it is.
 #pragma once
 #include "attnw_fused.cuh"
@@ -14,20 +14,27 @@
 namespace attnw {
 namespace proj {
 
-constexpr int kRows = 256;        // rows of X per CTA (two MMA row blocks)
-constexpr int kCols = 256;        // output features per CTA
 constexpr int kKSlice = 64;       // d_model elements per stage: one 128-byte swizzle atom
-constexpr int kStages = 3;
 constexpr int kGroupCols = 16;    // column tiles walked together (32 MB of weights at d_model = 4096)
 constexpr int kEpiWarps = 8;      // TMEM lane quarter (4) x column half (2)
 constexpr int kProducer = 8;
 constexpr int kMma = 9;
 constexpr int kThreads = 320;
 constexpr int kAtomBytes = 128 * 128;             // 128 rows x 128 bytes
-constexpr int kStageBytes = 4 * kAtomBytes;       // X rows 0-127, X rows 128-255, features 0-127, features 128-255
-constexpr int kBarOff = kStages * kStageBytes;
-constexpr int kDynamicBytes = kBarOff + 256 + 1024;
-static_assert(kDynamicBytes <= 227 * 1024, "shared memory budget");
+
+// A CTA's tile: RB blocks of 128 rows of X times CB blocks of 128 output features.
+template <int RB, int CB>
+struct Tile {
+    static constexpr int kRows = 128 * RB;
+    static constexpr int kCols = 128 * CB;
+    static constexpr int kStageBytes = (RB + CB) * kAtomBytes;  // the blocks of X, then the blocks of features
+    static constexpr int kStages = 12 / (RB + CB);              // 192 KB of stages
+    static constexpr int kBarOff = kStages * kStageBytes;
+    static constexpr int kDynamicBytes = kBarOff + 256 + 1024;
+    static constexpr int kTmemCols = kCols * RB;
+};
+static_assert(Tile<2, 2>::kDynamicBytes <= 227 * 1024 && Tile<1, 2>::kDynamicBytes <= 227 * 1024 &&
+              Tile<1, 1>::kDynamicBytes <= 227 * 1024, "shared memory budget");
 
 enum : uint32_t {  // wait sites of this kernel (low byte of the status word)
     kSiteProducerEmpty = 112,
@@ -37,7 +44,7 @@ enum : uint32_t {  // wait sites of this kernel (low byte of the status word)
 };
 
 struct Barriers {
-    uint64_t full[kStages], empty[kStages];
+    uint64_t full[6], empty[6];
     uint64_t acc_full;     // every MMA of the tile is complete
     uint64_t out_filled;   // the 7 warps that do not issue the stores have staged their part of the tile
     uint32_t tmem_base;
@@ -49,13 +56,16 @@ static_assert(sizeof(Barriers) <= 256, "barrier block must fit its slot");
 // grid: 2 * col_tiles * B * row_tiles CTAs.  The column tiles (Q's, then K's) are walked in groups of kGroupCols: within
 // a group the tiles of one block of rows are neighbours (that block of X is fetched once per group) and the group's
 // slice of the weights (kGroupCols x 256 x d_model) is small enough to stay in L2 while all row blocks pass.
+template <int RB, int CB>
 __global__ void __launch_bounds__(kThreads, 1)
 project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_wq,
                   const __grid_constant__ CUtensorMap tm_wk, const __grid_constant__ CUtensorMap tm_q,
                   const __grid_constant__ CUtensorMap tm_k, int N, int d_model, int H, int d, int col_tiles, int row_tiles) {
+    using L = Tile<RB, CB>;
+    constexpr int kStages = L::kStages, kStageBytes = L::kStageBytes, kCols = L::kCols, kRows = L::kRows;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    Barriers* bars = reinterpret_cast<Barriers*>(smem + kBarOff);
+    Barriers* bars = reinterpret_cast<Barriers*>(smem + L::kBarOff);
     volatile uint32_t* abort_flag = &bars->abort_flag;
 
     if (threadIdx.x == 0) bars->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
@@ -95,7 +105,7 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         ptx::prefetch_tensormap(tm_out);
     }
     if (warp == kMma) {
-        ptx::tmem_alloc(&bars->tmem_base, kTmemCols);
+        ptx::tmem_alloc(&bars->tmem_base, L::kTmemCols);
         ptx::tmem_relinquish();
     }
     ptx::tc_fence_before_sync();
@@ -104,7 +114,7 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     const uint32_t tmem_base = bars->tmem_base;
 
     if (warp == kProducer) {
-        // ================= TMA producer: one [256 x 64] slice of X and one of the weights per stage =================
+        // ================= TMA producer: one 64-wide slice of X and one of the weights per stage =================
         if (lane == 0) {
             const uint64_t keep = ptx::policy_evict_last();
             int kt = 0;
@@ -114,10 +124,10 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 uint8_t* st = smem + s * kStageBytes;
                 ptx::mbar_expect_tx(&bars->full[s], static_cast<uint32_t>(kStageBytes));
                 // rows or features beyond the tensor's extent, and d_model's ragged tail, arrive as zeros
-                ptx::tma_load_3d(st + 0 * kAtomBytes, &tm_x, &bars->full[s], kt * kKSlice, r0, b, keep);
-                ptx::tma_load_3d(st + 1 * kAtomBytes, &tm_x, &bars->full[s], kt * kKSlice, r0 + 128, b, keep);
-                ptx::tma_load_3d(st + 2 * kAtomBytes, tm_w, &bars->full[s], kt * kKSlice, c0, 0, keep);
-                ptx::tma_load_3d(st + 3 * kAtomBytes, tm_w, &bars->full[s], kt * kKSlice, c0 + 128, 0, keep);
+                for (int m = 0; m < RB; ++m)
+                    ptx::tma_load_3d(st + m * kAtomBytes, &tm_x, &bars->full[s], kt * kKSlice, r0 + m * 128, b, keep);
+                for (int c = 0; c < CB; ++c)
+                    ptx::tma_load_3d(st + (RB + c) * kAtomBytes, tm_w, &bars->full[s], kt * kKSlice, c0 + c * 128, 0, keep);
             }
             if (*abort_flag) {
                 // Unwinding: let the copies already in flight land before shared memory is released.
@@ -140,17 +150,15 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             ok = __all_sync(0xffffffffu, fused_wait(&bars->full[s], static_cast<uint32_t>(kt / kStages) & 1u, abort_flag, kSiteMmaFull));
             if (!ok) break;
             ptx::tc_fence_after_sync();
-            const uint32_t st = base + static_cast<uint32_t>(s * kStageBytes);
+            const uint64_t st = ptx::umma_desc_kmajor_sw128(base + static_cast<uint32_t>(s * kStageBytes));
             if (ptx::elect_one()) {
 #pragma unroll
-                for (int mi = 0; mi < 2; ++mi) {
+                for (int mi = 0; mi < RB; ++mi) {
 #pragma unroll
                     for (int k = 0; k < kKSlice / 16; ++k)
-                        // A: 128 rows of X; B: 256 features = the two weight atoms, contiguous (8-row groups 1024 bytes apart)
-                        ptx::umma_f16_ss(tmem_base + static_cast<uint32_t>(mi * kCols),
-                                         ptx::umma_desc_kmajor_sw128(st + static_cast<uint32_t>(mi * kAtomBytes + k * 32)),
-                                         ptx::umma_desc_kmajor_sw128(st + static_cast<uint32_t>(2 * kAtomBytes + k * 32)), idesc,
-                                         (kt > 0 || k > 0) ? 1u : 0u);
+                        // A: 128 rows of X; B: the weight atoms, contiguous (8-row groups 1024 bytes apart)
+                        ptx::umma_f16_ss(tmem_base + static_cast<uint32_t>(mi * kCols), st + static_cast<uint64_t>((mi * kAtomBytes + k * 32) >> 4),
+                                         st + static_cast<uint64_t>((RB * kAtomBytes + k * 32) >> 4), idesc, (kt > 0 || k > 0) ? 1u : 0u);
                 }
                 ptx::umma_commit(&bars->empty[s]);
             }
@@ -161,23 +169,23 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     } else {
         // ================= Epilogue warps: accumulators -> bf16 -> shared memory -> TMA stores, head-major =================
         const int quarter = warp & 3;
-        const int ch = warp >> 2;  // column half of the tile (features ch*128 .. +127)
+        const int ch = warp >> 2;  // column half of the tile
         const int row = quarter * 32 + lane;
         const uint32_t sw = static_cast<uint32_t>(lane & 7);
         bool ok = __all_sync(0xffffffffu, fused_wait(&bars->acc_full, 0, abort_flag, kSiteEpiAcc));
         if (ok) {
             ptx::tc_fence_after_sync();
-            // every load was consumed and every MMA is complete: the ring is free and stages the tile as 2 x 4 boxes of
+            // every load was consumed and every MMA is complete: the ring is free and stages the tile as RB x 2 CB boxes of
             // [128 rows x 64 features]
             const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
 #pragma unroll 1
-            for (int mi = 0; mi < 2; ++mi) {
+            for (int mi = 0; mi < RB; ++mi) {
 #pragma unroll 1
-                for (int c = 0; c < 4; ++c) {
+                for (int c = 0; c < 2 * CB; ++c) {
                     float v[kChunk];
-                    load_chunk(t_lane + static_cast<uint32_t>(mi * kCols + ch * 128 + c * kChunk), v);
-                    const int atom = ch * 2 + (c >> 1);
-                    const uint32_t dst = ptx::smem_u32(smem + (mi * 4 + atom) * kAtomBytes + row * 128);
+                    load_chunk(t_lane + static_cast<uint32_t>(mi * kCols + ch * (kCols / 2) + c * kChunk), v);
+                    const int atom = ch * CB + (c >> 1);
+                    const uint32_t dst = ptx::smem_u32(smem + (mi * 2 * CB + atom) * kAtomBytes + row * 128);
 #pragma unroll
                     for (int g = 0; g < 4; ++g)
                         ptx::st_shared_v4(dst + ((static_cast<uint32_t>((c & 1) * 4 + g) ^ sw) << 4),
@@ -191,12 +199,12 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 ok = __all_sync(0xffffffffu, fused_wait(&bars->out_filled, 0, abort_flag, kSiteEpiFilled));
                 if (ok && lane == 0) {
                     const uint64_t stream_out = ptx::policy_evict_last();  // the attention kernels read Q and K next
-                    for (int mi = 0; mi < 2; ++mi) {
+                    for (int mi = 0; mi < RB; ++mi) {
                         if (r0 + mi * 128 >= N) continue;
-                        for (int atom = 0; atom < 4; ++atom) {
+                        for (int atom = 0; atom < 2 * CB; ++atom) {
                             const int col = c0 + atom * 64;  // output feature of H * d: head col / d, offset col % d
                             if (col >= H * d) continue;
-                            ptx::tma_store_3d(tm_out, ptx::smem_u32(smem + (mi * 4 + atom) * kAtomBytes), col % d, r0 + mi * 128,
+                            ptx::tma_store_3d(tm_out, ptx::smem_u32(smem + (mi * 2 * CB + atom) * kAtomBytes), col % d, r0 + mi * 128,
                                               b * H + col / d, stream_out);
                         }
                     }
@@ -214,7 +222,7 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     __syncthreads();
     if (warp == kMma) {
         ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem_base, kTmemCols);
+        ptx::tmem_dealloc(tmem_base, L::kTmemCols);
     }
 }
 

@@ -60,7 +60,9 @@ def check(got: torch.Tensor, ref: np.ndarray, x, w):
 # several row tiles and column tiles, ragged rows, ragged d_model (not a multiple of 64), H*d not a multiple of 256,
 # a single row, more than one batch entry
 SHAPES = [(1, 256, 64, 2, 128), (1, 128, 128, 1, 64), (2, 300, 192, 3, 64), (1, 1, 64, 1, 128), (1, 520, 328, 5, 64),
-          (2, 77, 72, 1, 128), (1, 1024, 512, 4, 128), (3, 130, 256, 6, 64), (1, 257, 8, 2, 64)]
+          (2, 77, 72, 1, 128), (1, 1024, 512, 4, 128), (3, 130, 256, 6, 64), (1, 257, 8, 2, 64),
+          # tiles of 256 x 256 and of 128 x 256 on a device of 148 SMs, with a last tile that is partly empty (the others: 128 x 128)
+          (2, 469, 136, 60, 64), (1, 3872, 72, 7, 64)]
 
 
 @pytest.mark.parametrize("B,N,d_model,H,d", SHAPES)
