@@ -105,10 +105,6 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     auto bar_of = [bar](size_t field, int n) { return bar + static_cast<uint32_t>(field) + 8u * static_cast<uint32_t>(n); };
     volatile uint32_t* abort_flag = &bars->abort_flag;
 
-    if (threadIdx.x == 0) bars->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
-    __syncthreads();
-    if (bars->prior_failure != 0u) return;  // an earlier CTA gave up: do not queue more waits behind it
-
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int bh = blockIdx.x / row_blocks_per_head;
@@ -148,13 +144,17 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         ptx::tmem_alloc(&bars->tmem_base, kTmemCols);
         ptx::tmem_relinquish();
     }
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();
+    if (threadIdx.x == 0) bars->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bars->tmem_base;
+    const bool run = bars->prior_failure == 0u;  // an earlier CTA gave up: do not queue more waits behind it
     // tensor memory of unit q: scores in columns [256 q, 256 q + 128), O in [256 q + 128, 256 q + 128 + d)
 
-    if (warp == kProducer) {
+    if (run && warp == kProducer) {
         // ================= TMA producer: Q once, then the K and V tiles in the order the MMA issuer reads them =========
         if (lane == 0) {
             const uint64_t keep = ptx::policy_evict_last();
@@ -198,7 +198,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             }
         }
         __syncwarp();
-    } else if (warp == kMma) {
+    } else if (run && warp == kMma) {
         // ================= MMA issuer (warp-uniform loop, one elected lane issues) =================
         constexpr uint32_t idesc_s = ptx::umma_idesc_bf16_f32(kTile, kTile);
         constexpr uint32_t idesc_o = ptx::umma_idesc_bf16_f32(kTile, D) | (1u << 16);  // B operand MN-major
@@ -290,7 +290,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 }
             }
         }
-    } else if (warp < kSmWarps) {
+    } else if (run && warp < kSmWarps) {
         // ================= Softmax warps: two threads per query row, 64 key columns of a tile each =================
         const int q = warp >> 3;
         const int half = (warp >> 2) & 1;

@@ -76,6 +76,7 @@ struct DeviceInfo {
     // fork/join objects for launches that split a call over two kernels (created on first use)
     cudaStream_t side_stream = nullptr;
     cudaEvent_t fork_event = nullptr, join_event = nullptr;
+    std::atomic<int> gridrow_clusters[2][2][17] = {};  // resident clusters of 2..16 CTAs of the grid-row kernel, [d == 128][P is float32][CTAs], 0 = not asked yet
     int rc_clusters[2][17] = {};  // resident clusters of 1..16 CTAs of the register-cluster row kernel, [P is float32][CTAs]
 };
 std::mutex g_split_mutex;
@@ -355,18 +356,63 @@ int launch_resident(DeviceInfo* dev, const void* Q, const void* K, void* P, int 
 // The geometry of a grid-row launch: groups of ceil(N / 256) CTAs, as many as fit one CTA per SM and have work.
 struct GridrowShape {
     int group_ctas, n_groups, total_items;
+    bool clusters;     // each group is a cluster (else: the grid is cooperative)
     uint32_t longest;  // row blocks of the longest list = message tags the launch uses
 };
+// How many clusters of `ctas` CTAs of the grid-row kernel the device holds at once; -1 = none.
+template <int D, typename OutT>
+int gridrow_max_clusters(DeviceInfo* dev, int ctas) {
+    std::atomic<int>& memo = dev->gridrow_clusters[D == 128][sizeof(OutT) == 4][ctas];
+    int n = memo.load(std::memory_order_relaxed);
+    if (n != 0) return n;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(ctas);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(gr::kThreads, 1, 1);
+    cfg.gridDim = dim3(static_cast<unsigned>(ctas * dev->sm_count), 1, 1);
+    cfg.dynamicSmemBytes = gr::Smem<D>::kDynamicBytes;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, gr::attnw_gridrow_kernel<D, OutT>, &cfg) != cudaSuccess || n < 1) {
+        (void)cudaGetLastError();
+        n = -1;
+    }
+    memo.store(n, std::memory_order_relaxed);
+    return n;
+}
+
 // Returns ATTNW_ERR_UNSUPPORTED when `max_ctas` cannot hold a whole group.
-int gridrow_shape(int BH, int N, int max_ctas, GridrowShape* out) {
+template <int D, typename OutT>
+int gridrow_shape(DeviceInfo* dev, int BH, int N, int max_ctas, GridrowShape* out) {
     const long long total = static_cast<long long>(BH) * ((N + kTile - 1) / kTile);
     if (total > INT_MAX) return ATTNW_ERR_BAD_SHAPE;
-    out->group_ctas = (N + gr::kSlabCols - 1) / gr::kSlabCols;
-    if (out->group_ctas > max_ctas || out->group_ctas > gr::kMaxGroupCtas) return ATTNW_ERR_UNSUPPORTED;
+    const int C = (N + gr::kSlabCols - 1) / gr::kSlabCols;
+    if (C > max_ctas || C > gr::kMaxGroupCtas) return ATTNW_ERR_UNSUPPORTED;
+    if (allow_smem<gr::attnw_gridrow_kernel<D, OutT>>(gr::Smem<D>::kDynamicBytes, true) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return ATTNW_ERR_CUDA;
+    }
+    out->group_ctas = C;
     out->total_items = static_cast<int>(total);
-    out->n_groups = max_ctas / out->group_ctas;
+    out->n_groups = max_ctas / C;
+    auto rounds = [&](int groups) { return (total + groups - 1) / groups; };
+    // The CTAs of a group wait for one another, so they must be resident together: as a cluster, or with the whole grid
+    // (cooperative).  Large clusters do not reach every SM (16 CTAs: 7 clusters, where 9 groups fit), but a cluster launch may
+    // overlap the end of the kernel in front: taken where it needs no more rounds of row blocks.  us per call, cooperative ->
+    // clusters: 2 x 512 10.3 -> 7.2, 24 x 1000 20.5 -> 18.0, 3 x 1504 12.3 -> 10.3; with one round more (1 x 2048) 10.2 -> 10.5.
+    out->clusters = false;
+    if (C > 1 && C <= 16) {
+        const int clusters = gridrow_max_clusters<D, OutT>(dev, C);
+        if (clusters > 0 && rounds(clusters < out->n_groups ? clusters : out->n_groups) <= rounds(out->n_groups)) {
+            out->clusters = true;
+            if (clusters < out->n_groups) out->n_groups = clusters;
+        }
+    }
     if (out->n_groups > total) out->n_groups = out->total_items;
-    out->longest = static_cast<uint32_t>((total + out->n_groups - 1) / out->n_groups);
+    out->longest = static_cast<uint32_t>(rounds(out->n_groups));
     return ATTNW_OK;
 }
 // 16-byte entries of an exchange area that serves every grid of up to `max_ctas` CTAs: the pairs of each CTA and, where the
@@ -388,23 +434,27 @@ int enqueue_gridrow(const GridrowShape& g, const void* Q, const void* K, void* P
         rc = encode_3d(&tm_p, sizeof(OutT) == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sizeof(OutT), P,
                        N, N, BH, 128 / sizeof(OutT), 32);
     if (rc != ATTNW_OK) return rc;
-    if (allow_smem<gr::attnw_gridrow_kernel<D, OutT>>(L::kDynamicBytes) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return ATTNW_ERR_CUDA;
-    }
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;  // every CTA of the grid is resident at once, or the launch fails
-    attr[0].val.cooperative = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(gr::kThreads, 1, 1);
-    cfg.gridDim = dim3(static_cast<unsigned>(g.n_groups * g.group_ctas), 1, 1);
-    cfg.dynamicSmemBytes = L::kDynamicBytes;
-    cfg.stream = stream;
-    cfg.attrs = attr;
-    cfg.numAttrs = g.group_ctas > 1 ? 1 : 0;  // groups of one CTA wait for nobody
     const float scale_log2e = static_cast<float>(static_cast<double>(scale) * 1.4426950408889634074);
-    const cudaError_t launched =
-        cudaLaunchKernelEx(&cfg, kernel, tm_q, tm_k, tm_p, N, g.total_items, g.group_ctas, g.n_groups, scale_log2e, xchg, tag_base);
+    cudaError_t launched;
+    if (g.group_ctas == 1 || g.clusters) {
+        launched = launch_overlapped(kernel, static_cast<unsigned>(g.n_groups * g.group_ctas), gr::kThreads, L::kDynamicBytes, stream,
+                                     g.group_ctas, false, tm_q, tm_k, tm_p, N, g.total_items, g.group_ctas, g.n_groups, scale_log2e, xchg,
+                                     tag_base);
+    } else {
+        // Not overlapped: CTAs that wait for the kernel in front while another stream's cooperative grid holds the other SMs
+        // could leave both grids incomplete.
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;  // every CTA of the grid is resident at once, or the launch fails
+        attr[0].val.cooperative = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.blockDim = dim3(gr::kThreads, 1, 1);
+        cfg.gridDim = dim3(static_cast<unsigned>(g.n_groups * g.group_ctas), 1, 1);
+        cfg.dynamicSmemBytes = L::kDynamicBytes;
+        cfg.stream = stream;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        launched = cudaLaunchKernelEx(&cfg, kernel, tm_q, tm_k, tm_p, N, g.total_items, g.group_ctas, g.n_groups, scale_log2e, xchg, tag_base);
+    }
     if (launched != cudaSuccess) {
         (void)cudaGetLastError();
         return launched == cudaErrorCooperativeLaunchTooLarge ? ATTNW_ERR_UNSUPPORTED : ATTNW_ERR_CUDA;
@@ -473,7 +523,7 @@ int gridrow_area(GridrowAreas* areas, int sm_count, cudaStream_t stream, Gridrow
 template <int D, typename OutT>
 int launch_gridrow(DeviceInfo* dev, const void* Q, const void* K, void* P, int BH, int N, float scale, cudaStream_t stream) {
     GridrowShape g;
-    int rc = gridrow_shape(BH, N, dev->sm_count, &g);
+    int rc = gridrow_shape<D, OutT>(dev, BH, N, dev->sm_count, &g);
     if (rc != ATTNW_OK) return rc;
     if (g.group_ctas == 1) return enqueue_gridrow<D, OutT>(g, Q, K, P, BH, N, scale, nullptr, 0, stream);
     // A captured launch would be replayed with the tags of its capture, at any time beside any other launch.
@@ -546,9 +596,11 @@ int launch_attn_onepass(const DeviceInfo* dev, const void* Q, const void* K, con
         return ATTNW_ERR_CUDA;
     }
     auto kernel = split ? av1::attn_onepass_kernel<D, true> : av1::attn_onepass_kernel<D, false>;
-    kernel<<<static_cast<unsigned>(BH * row_blocks), av1::kThreads, L::kDynamicBytes, stream>>>(tm_q, tm_k, tm_v, tm_o, N,
-                                                                                                 row_blocks, scale_log2e);
-    if (cudaGetLastError() != cudaSuccess) return ATTNW_ERR_CUDA;
+    if (launch_overlapped(kernel, static_cast<unsigned>(BH * row_blocks), av1::kThreads, L::kDynamicBytes, stream, 1, false, tm_q, tm_k, tm_v,
+                          tm_o, N, row_blocks, scale_log2e) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return ATTNW_ERR_CUDA;
+    }
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return ATTNW_OK;
 }
@@ -607,9 +659,11 @@ int launch_project_tile(const ProjectMaps& m, int B, int N, int d_model, int H, 
     const int col_tiles = static_cast<int>((static_cast<long long>(H) * d + L::kCols - 1) / L::kCols);
     const int row_tiles = (N + L::kRows - 1) / L::kRows;
     const unsigned ctas = static_cast<unsigned>(2 * col_tiles) * static_cast<unsigned>(row_tiles) * static_cast<unsigned>(B);
-    proj::project_qk_kernel<RB, CB><<<ctas, proj::kThreads, L::kDynamicBytes, stream>>>(m.x, m.wq, m.wk, m.q, m.k, N, d_model, H, d,
-                                                                                         col_tiles, row_tiles);
-    if (cudaGetLastError() != cudaSuccess) return ATTNW_ERR_CUDA;
+    if (launch_overlapped(proj::project_qk_kernel<RB, CB>, ctas, proj::kThreads, L::kDynamicBytes, stream, 1, false, m.x, m.wq, m.wk, m.q, m.k,
+                          N, d_model, H, d, col_tiles, row_tiles) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return ATTNW_ERR_CUDA;
+    }
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return ATTNW_OK;
 }
@@ -867,7 +921,6 @@ static __device__ __align__(256) uint4 g_noalloc_xchg[gridrow_entries(kNoAllocMa
 struct NoAllocState {
     bool ready = false;
     uint4* xchg = nullptr;   // device address of g_noalloc_xchg on this device
-    int sm_count = 0;
     uint32_t tag = 0;        // next unused message tag of this device's array
 };
 NoAllocState g_noalloc[kMaxDevices];
@@ -882,14 +935,7 @@ int noalloc_setup(NoAllocState** out) {
     std::lock_guard<std::mutex> lock(g_mutex);
     NoAllocState& st = g_noalloc[dev];
     if (!st.ready) {
-        int major = 0;
         void* ptr = nullptr;
-        if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&st.sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-            (void)cudaGetLastError();
-            return ATTNW_ERR_CUDA;
-        }
-        if (major != 10) return ATTNW_ERR_UNSUPPORTED;
         if (cudaGetSymbolAddress(&ptr, g_noalloc_xchg) != cudaSuccess || ptr == nullptr) {
             (void)cudaGetLastError();
             return ATTNW_ERR_CUDA;
@@ -903,11 +949,11 @@ int noalloc_setup(NoAllocState** out) {
 }
 
 template <int D>
-int launch_gridrow_noalloc(NoAllocState* st, const void* Q, const void* K, void* P, int BH, int N, float scale,
+int launch_gridrow_noalloc(DeviceInfo* dev, NoAllocState* st, const void* Q, const void* K, void* P, int BH, int N, float scale,
                            cudaStream_t stream) {
     // one CTA per SM, whole groups only, and never more CTAs than the static array has entries for
     GridrowShape g;
-    const int rc = gridrow_shape(BH, N, st->sm_count < kNoAllocMaxCtas ? st->sm_count : kNoAllocMaxCtas, &g);
+    int rc = gridrow_shape<D, __nv_bfloat16>(dev, BH, N, dev->sm_count < kNoAllocMaxCtas ? dev->sm_count : kNoAllocMaxCtas, &g);
     if (rc != ATTNW_OK) return rc;
     uint32_t tag_base = 0;
     {
@@ -988,11 +1034,14 @@ int attnw_fused_noalloc(const void* Q, const void* K, void* P, int B, int H, int
     NoAllocState* st = nullptr;
     rc = noalloc_setup(&st);
     if (rc != ATTNW_OK) return rc;
+    DeviceInfo* dev = nullptr;
+    rc = current_device(&dev);
+    if (rc != ATTNW_OK) return rc;
     rc = load_encoder();
     if (rc != ATTNW_OK) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    return d == 64 ? launch_gridrow_noalloc<64>(st, Q, K, P, B * H, N, scale, s)
-                   : launch_gridrow_noalloc<128>(st, Q, K, P, B * H, N, scale, s);
+    return d == 64 ? launch_gridrow_noalloc<64>(dev, st, Q, K, P, B * H, N, scale, s)
+                   : launch_gridrow_noalloc<128>(dev, st, Q, K, P, B * H, N, scale, s);
 }
 
 int attnw_fused_f32(const void* Q, const void* K, void* P, int B, int H, int N, int d, float scale, void* stream) {

@@ -17,8 +17,10 @@
 // Tensor memory, float32 output: two regions of 256 columns; the exponentials replace the scores as float32, and a slot of
 // 64 columns goes back to the MMA issuer when its weights have been read.
 //
-// Groups are not hardware clusters (clusters of 8 or 16 CTAs cannot occupy every SM): the grid is launched
-// cooperatively with one CTA per SM, consecutive CTAs form a group, and the 16-byte (offset, sum) pair of a row
+// The CTAs of a group wait for one another, so they must be resident together.  Large hardware clusters do not occupy
+// every SM (8 CTAs: 15 clusters of the device's 148 SMs, 16: 7), so large calls are launched cooperatively with one CTA per SM
+// and consecutive CTAs form a group; small ones, and groups of 2 to 4, are clusters, whose launch may overlap the kernel in
+// front (2 x 512 10.3 -> 8.2 us).  Either way the 16-byte (offset, sum) pair of a row
 // travels through L2 as two 8-byte words that each carry a tag {value, tag, value, tag}; a reader accepts a
 // pair once both tags name the row block it is waiting for.  No fence, no flag, no atomics: the tag arrives
 // with the value in one 8-byte store.  Every poll is bounded.
@@ -237,7 +239,6 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             ptx::mbar_init(&bars->merged[r], 2);
         }
         bars->abort_flag = 0;
-        bars->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
         ptx::mbar_fence_init();
     }
     if (warp == kOwnerWarpG && lane == 0) {
@@ -252,6 +253,9 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         ptx::tmem_alloc(&bars->tmem_base, kTmemCols);
         ptx::tmem_relinquish();
     }
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();
+    if (threadIdx.x == 0) bars->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();

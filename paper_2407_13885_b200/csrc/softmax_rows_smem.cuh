@@ -73,11 +73,13 @@ softmax_rows_smem_kernel(const float* S, OutT* P, long long rows, long long cols
     const int nvec = n >> 2;
 
     if (threadIdx.x == 0) {
-        ctl->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
         ptx::mbar_init(&ctl->full, 1);
         ctl->abort_flag = 0;
         ptx::mbar_fence_init();
     }
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();
+    if (threadIdx.x == 0) ctl->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
     __syncthreads();
     // A CTA that sees an earlier failure still takes part in every cluster barrier below, without touching memory.
     bool ok = ctl->prior_failure == 0u;
@@ -174,26 +176,14 @@ template <typename OutT, int NT>
 inline cudaError_t launch_nt(const float* S, OutT* P, long long rows, long long cols, int sm_count, int C, int slice_cols,
                              cudaStream_t stream) {
     const size_t smem = kControlBytes + static_cast<size_t>(slice_cols) * 4;
-    auto kernel = softmax_rows_smem_kernel<OutT, NT>;
     const cudaError_t e = allow_smem<softmax_rows_smem_kernel<OutT, NT>>(kControlBytes + kSliceMaxCols * 4, true);
     if (e != cudaSuccess) return e;
     const long long per_sm = NT == 256 ? (smem * 4 <= 224 * 1024 ? 4 : 3) : 2;
     long long n_clusters = (per_sm * sm_count) / C;  // CTAs that fit at once
     if (n_clusters < 1) n_clusters = 1;
     if (n_clusters > rows) n_clusters = rows;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(n_clusters * C));
-    cfg.blockDim = dim3(NT);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = static_cast<unsigned>(C);
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, S, P, rows, cols, slice_cols, C);
+    return launch_overlapped(softmax_rows_smem_kernel<OutT, NT>, static_cast<unsigned>(n_clusters * C), NT, smem, stream, C, false, S, P,
+                             rows, cols, slice_cols, C);
 }
 
 template <typename OutT>
@@ -257,13 +247,15 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
     const bool full = v1 - v0 == kRcVecPerThread * 32;  // this warp's piece has all its 256 vectors
 
     if (threadIdx.x == 0) {
-        ctl->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
         for (int w = 0; w < kWarpsRc; ++w) ptx::mbar_init(&ctl->full[w], 1);
         ptx::mbar_init(&ctl->pairs_in[0], 1);
         ptx::mbar_init(&ctl->pairs_in[1], 1);
         ctl->abort_flag = 0;
         ptx::mbar_fence_init();
     }
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();
+    if (threadIdx.x == 0) ctl->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
     __syncthreads();
     bool ok = ctl->prior_failure == 0u;
     if (C > 1) {  // every CTA of the cluster runs before anyone writes into a peer
@@ -379,8 +371,7 @@ inline cudaError_t launch_regcluster(const float* S, OutT* P, long long rows, lo
     auto kernel = softmax_rows_regcluster_kernel<OutT>;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(kRcThreads);
-    cfg.dynamicSmemBytes = kRcControlBytes + static_cast<size_t>(slice_cols) * 4;
-    cfg.stream = stream;
+    cfg.dynamicSmemBytes = kSmemMax;  // the memo serves every row length of this cluster size
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = static_cast<unsigned>(C);
@@ -393,10 +384,7 @@ inline cudaError_t launch_regcluster(const float* S, OutT* P, long long rows, lo
         int n = 0;
         if (e == cudaSuccess) {
             cfg.gridDim = dim3(static_cast<unsigned>(C));
-            const size_t asked = cfg.dynamicSmemBytes;
-            cfg.dynamicSmemBytes = kSmemMax;  // the memo serves every row length of this cluster size
             e = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
-            cfg.dynamicSmemBytes = asked;
         }
         *resident_clusters = (e == cudaSuccess && n > 0) ? n : -1;
         if (e != cudaSuccess) (void)cudaGetLastError();
@@ -404,8 +392,8 @@ inline cudaError_t launch_regcluster(const float* S, OutT* P, long long rows, lo
     if (*resident_clusters < 0) return cudaErrorInvalidConfiguration;
     long long n_clusters = *resident_clusters;
     if (n_clusters > rows) n_clusters = rows;
-    cfg.gridDim = dim3(static_cast<unsigned>(n_clusters * C));
-    return cudaLaunchKernelEx(&cfg, kernel, S, P, rows, cols, slice_cols, C);
+    return launch_overlapped(kernel, static_cast<unsigned>(n_clusters * C), kRcThreads, kRcControlBytes + static_cast<size_t>(slice_cols) * 4,
+                             stream, C, false, S, P, rows, cols, slice_cols, C);
 }
 
 }  // namespace srs

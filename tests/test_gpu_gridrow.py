@@ -107,3 +107,35 @@ def test_captured_call_is_right_on_every_replay(attnw, entry, dtype, N):
         torch.cuda.synchronize()
         assert attnw.query_status() == 0
         assert_close_to_oracle(P, oracle.attnw(q, k, scale_of(d)), f"{entry} {dtype} N{N}")
+
+
+def test_chain_of_calls_sees_the_results_in_front(attnw):
+    # each launch may begin before the kernel in front of it has ended: every call here reads what the call before has just
+    # written, among ordinary kernels of torch, and the last result is that of the same chain with a wait after each call
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    X = torch.randn(1, 200, 256, generator=gen, device="cuda", dtype=torch.bfloat16)
+    W = [torch.randn(4, 64, 256, generator=gen, device="cuda", dtype=torch.bfloat16) / 16 for _ in range(2)]
+
+    def chain(wait):
+        x = X
+        for _ in range(6):
+            Q, K = attnw.project_qk(x, *W)
+            wait()
+            O = attnw.attn_fused(Q, K, Q, 0.125)
+            wait()
+            P = attnw.attnw_fused(O, K, 0.125, out_dtype=torch.float32)
+            wait()
+            R = attnw.softmax_rows(P.view(-1, 200), out_dtype=torch.float32)
+            wait()
+            P2 = attnw.attnw_fused(O, Q, 0.125)
+            wait()
+            x = (O + torch.matmul(R.view(1, 4, 200, 200).bfloat16() + P2, Q)).transpose(1, 2).reshape(1, 200, 256).contiguous()
+            wait()
+        return x
+
+    want = chain(torch.cuda.synchronize)
+    for _ in range(3):
+        got = chain(lambda: None)
+        torch.cuda.synchronize()
+        assert attnw.query_status() == 0
+        assert torch.equal(got, want)
