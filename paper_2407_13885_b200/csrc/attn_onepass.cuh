@@ -116,7 +116,10 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     auto stage_offset = [](int s) { return !split || s < L::kStages ? L::kKOff + s * L::kTileBytes : L::kQOff + L::kTileBytes; };
 
     // ---- set-up ------------------------------------------------------------------------------
+    ptx::grid_launch_dependents();
     if (threadIdx.x == 0) {
+        ptx::grid_dependency_wait();
+        const uint32_t prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);  // (arrives meanwhile)
         ptx::mbar_init(&bars->q_full, 1);
         for (int s = 0; s < 7; ++s) {
             ptx::mbar_init(&bars->k_full[s], 1);
@@ -132,6 +135,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             ptx::mbar_init(&bars->out_filled[q], split ? 15 : 7);
         }
         bars->abort_flag = 0;
+        bars->prior_failure = prior_failure;
         ptx::mbar_fence_init();
     }
     if (warp == kProducer && lane == 0) {
@@ -144,9 +148,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         ptx::tmem_alloc(&bars->tmem_base, kTmemCols);
         ptx::tmem_relinquish();
     }
-    ptx::grid_launch_dependents();
     ptx::grid_dependency_wait();
-    if (threadIdx.x == 0) bars->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();

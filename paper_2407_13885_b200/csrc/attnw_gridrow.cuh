@@ -222,7 +222,10 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     uint4* const results = xchg + (static_cast<size_t>(n_groups) * group_ctas + group) * kXchgDepth * kTile;
 
     // ---- set-up ------------------------------------------------------------------------------
+    ptx::grid_launch_dependents();
     if (threadIdx.x == 0) {
+        ptx::grid_dependency_wait();
+        const uint32_t prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);  // (arrives meanwhile)
         ptx::mbar_init(&bars->k_full, 1);
         ptx::mbar_init(&bars->k_empty, 1);
         for (int j = 0; j < 8; ++j) {
@@ -239,6 +242,7 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             ptx::mbar_init(&bars->merged[r], 2);
         }
         bars->abort_flag = 0;
+        bars->prior_failure = prior_failure;
         ptx::mbar_fence_init();
     }
     if (warp == kOwnerWarpG && lane == 0) {
@@ -253,9 +257,7 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         ptx::tmem_alloc(&bars->tmem_base, kTmemCols);
         ptx::tmem_relinquish();
     }
-    ptx::grid_launch_dependents();
     ptx::grid_dependency_wait();
-    if (threadIdx.x == 0) bars->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();

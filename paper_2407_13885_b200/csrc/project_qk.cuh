@@ -85,7 +85,10 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     const CUtensorMap* tm_w = keys ? &tm_wk : &tm_wq;
     const CUtensorMap* tm_out = keys ? &tm_k : &tm_q;
 
+    ptx::grid_launch_dependents();
     if (threadIdx.x == 0) {
+        ptx::grid_dependency_wait();
+        const uint32_t prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);  // (arrives meanwhile)
         for (int s = 0; s < kStages; ++s) {
             ptx::mbar_init(&bars->full[s], 1);
             ptx::mbar_init(&bars->empty[s], 1);
@@ -93,6 +96,7 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         ptx::mbar_init(&bars->acc_full, 1);
         ptx::mbar_init(&bars->out_filled, kEpiWarps - 1);
         bars->abort_flag = 0;
+        bars->prior_failure = prior_failure;
         ptx::mbar_fence_init();
     }
     if (warp == kProducer && lane == 0) {
@@ -104,9 +108,7 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         ptx::tmem_alloc(&bars->tmem_base, L::kTmemCols);
         ptx::tmem_relinquish();
     }
-    ptx::grid_launch_dependents();
     ptx::grid_dependency_wait();
-    if (threadIdx.x == 0) bars->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();

@@ -72,14 +72,16 @@ softmax_rows_smem_kernel(const float* S, OutT* P, long long rows, long long cols
     const int n = static_cast<int>(c0 >= cols ? 0 : (cols - c0 < slice_cols ? cols - c0 : slice_cols));  // its length
     const int nvec = n >> 2;
 
+    ptx::grid_launch_dependents();
     if (threadIdx.x == 0) {
+        ptx::grid_dependency_wait();
+        const uint32_t prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);  // (arrives meanwhile)
         ptx::mbar_init(&ctl->full, 1);
         ctl->abort_flag = 0;
+        ctl->prior_failure = prior_failure;
         ptx::mbar_fence_init();
     }
-    ptx::grid_launch_dependents();
     ptx::grid_dependency_wait();
-    if (threadIdx.x == 0) ctl->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
     __syncthreads();
     // A CTA that sees an earlier failure still takes part in every cluster barrier below, without touching memory.
     bool ok = ctl->prior_failure == 0u;
@@ -246,16 +248,18 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
     const uint32_t bytes = static_cast<uint32_t>(v1 - v0) * 16u;
     const bool full = v1 - v0 == kRcVecPerThread * 32;  // this warp's piece has all its 256 vectors
 
+    ptx::grid_launch_dependents();
     if (threadIdx.x == 0) {
+        ptx::grid_dependency_wait();
+        const uint32_t prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);  // (arrives meanwhile)
         for (int w = 0; w < kWarpsRc; ++w) ptx::mbar_init(&ctl->full[w], 1);
         ptx::mbar_init(&ctl->pairs_in[0], 1);
         ptx::mbar_init(&ctl->pairs_in[1], 1);
         ctl->abort_flag = 0;
+        ctl->prior_failure = prior_failure;
         ptx::mbar_fence_init();
     }
-    ptx::grid_launch_dependents();
     ptx::grid_dependency_wait();
-    if (threadIdx.x == 0) ctl->prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
     __syncthreads();
     bool ok = ctl->prior_failure == 0u;
     if (C > 1) {  // every CTA of the cluster runs before anyone writes into a peer
