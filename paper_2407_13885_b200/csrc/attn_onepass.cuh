@@ -8,7 +8,9 @@
 //   Softmax   two threads per row, 64 columns each: a thread takes its scores to registers (the buffer is handed back
 //             at once, so the next tile's MMA 1 runs meanwhile) and also reads the other thread's 64 columns for
 //             their maximum, so both know the row maximum without an exchange; p = 2^(c s - mb) with the row's
-//             offset mb; l += sum p; P (bf16) is written to shared memory as a K-major MMA operand
+//             offset mb; l += sum p; P (bf16) becomes the A operand of MMA 2: through shared memory (d = 128), or, since d = 64
+//             leaves room, in tensor memory (128 x 4096 839 -> 801 us: the MMAs of d = 64 fetch 256 KB a step of two tiles
+//             from shared memory otherwise, as long as the exponentials take)
 //   MMA 2     O_q += P V_j                        128 x d fp32 in tensor memory; V_j as TMA delivers it
 //             ([128 keys x d], an MN-major B operand)
 // The offset mb of a row follows its running maximum lazily: it moves only when the maximum has grown by more than 8
@@ -51,6 +53,9 @@ struct Smem {
     static constexpr int kTileBytes = kAtoms * kAtomBytes;     // a Q, K or V tile
     static constexpr int kPBytes = 2 * kAtomBytes;             // a P tile: 128 rows x 128 keys, two atoms of 64 keys
     static constexpr int kStages = (D == 128) ? 3 : 6;         // ring of K / V tiles (128 keys x d)
+    // d = 64 leaves 64 columns of tensor memory per unit beside the scores and O: P goes there as the product's A operand
+    // instead of through shared memory.
+    static constexpr bool kPInTmem = D == 64;
     static constexpr int kQOff = 0;                            // two query tiles; split: one, and one more stage of the ring
     static constexpr int kKOff = kQOff + 2 * kTileBytes;
     static constexpr int kPOff = kKOff + kStages * kTileBytes;
@@ -154,7 +159,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bars->tmem_base;
     const bool run = bars->prior_failure == 0u;  // an earlier CTA gave up: do not queue more waits behind it
-    // tensor memory of unit q: scores in columns [256 q, 256 q + 128), O in [256 q + 128, 256 q + 128 + d)
+    // tensor memory of unit q: scores in columns [256 q, 256 q + 128), O in [256 q + 128, 256 q + 128 + d), then P (d = 64)
 
     if (run && warp == kProducer) {
         // ================= TMA producer: Q once, then the K and V tiles in the order the MMA issuer reads them =========
@@ -243,9 +248,15 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             const uint64_t b_desc = av::umma_desc_mnmajor_sw128(base + static_cast<uint32_t>(stage_offset(n % kStages)), L::kAtomBytes);
             if (ptx::elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < kTile / 16; ++kk)  // 16 keys per instruction
+                for (int kk = 0; kk < kTile / 16; ++kk) {  // 16 keys per instruction
+                    if constexpr (L::kPInTmem) {
+                        ptx::umma_f16_ts(o_tmem, o_tmem + static_cast<uint32_t>(D + kk * 8), b_desc + static_cast<uint64_t>(kk * 16 * 128 >> 4),
+                                         idesc_o, (j > 0 || kk > 0) ? 1u : 0u);
+                        continue;
+                    }
                     ptx::umma_f16_ss(o_tmem, a_desc + static_cast<uint64_t>(((kk >> 2) * L::kAtomBytes + (kk & 3) * 32) >> 4),
                                      b_desc + static_cast<uint64_t>(kk * 16 * 128 >> 4), idesc_o, (j > 0 || kk > 0) ? 1u : 0u);
+                }
                 ptx::umma_commit(&bars->p_free[q]);
                 if (j + 1 == steps[q]) ptx::umma_commit(&bars->o_full[q]);
             }
@@ -308,6 +319,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         const uint32_t lane0 = lane == 0;
         const uint32_t p_row = ptx::smem_u32(smem + L::kPOff + q * L::kPBytes) + static_cast<uint32_t>(half * L::kAtomBytes + row * 128);
         const uint32_t sw = static_cast<uint32_t>(lane & 7);
+        const uint32_t p_own = t_quarter + static_cast<uint32_t>((q * 2 + 1) * kTile + D + half * 32);  // kPInTmem: its 64 keys of P
         float smax = -3.0e38f;  // running maximum of the raw scores of this row (all columns: both threads of a row
                                 // compute it, each from the whole tile, so they agree without an exchange)
         float mb = -3.0e38f;    // the offset the weights, l and O's row are relative to (follows smax * c2 lazily)
@@ -381,6 +393,9 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             // the P tile and O are free once the MMAs of the previous key tile are complete
             ok = __all_sync(0xffffffffu, wait_in_place(&bars->p_free[q], (static_cast<uint32_t>(j) & 1u) ^ 1u, abort_flag, kSitePFree));
             if (!ok) break;
+            if constexpr (L::kPInTmem) ptx::tc_fence_after_sync();
+            uint32_t w[16];  // 32 keys of P on their way to tensor memory
+            (void)w;
             if (j == 0) {
                 mb = mb_cand;
             } else if (__any_sync(0xffffffffu, move)) {
@@ -419,15 +434,22 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                     }
                     acc[(i >> 1) & 3] = ptx::add2(acc[(i >> 1) & 3], ptx::pack2(p[i], p[i + 1]));
                 }
-                ptx::st_shared_v4(p_row + ((static_cast<uint32_t>(g) ^ sw) << 4), ptx::pack_bf16x2(p[0], p[1]),
-                                  ptx::pack_bf16x2(p[2], p[3]), ptx::pack_bf16x2(p[4], p[5]), ptx::pack_bf16x2(p[6], p[7]));
+                if constexpr (L::kPInTmem) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) w[(g & 3) * 4 + i] = ptx::pack_bf16x2(p[2 * i], p[2 * i + 1]);
+                    if ((g & 3) == 3) ptx::tmem_st_32x32b_x16(p_own + static_cast<uint32_t>((g >> 2) * 16), w);
+                } else {
+                    ptx::st_shared_v4(p_row + ((static_cast<uint32_t>(g) ^ sw) << 4), ptx::pack_bf16x2(p[0], p[1]),
+                                      ptx::pack_bf16x2(p[2], p[3]), ptx::pack_bf16x2(p[4], p[5]), ptx::pack_bf16x2(p[6], p[7]));
+                }
             }
             float a0, a1, a2, a3;
             ptx::unpack2(ptx::add2(acc[0], acc[1]), a0, a1);
             ptx::unpack2(ptx::add2(acc[2], acc[3]), a2, a3);
             l += (a0 + a1) + (a2 + a3);
-            ptx::tc_fence_before_sync();  // orders the rescale of O before the MMAs that accumulate into it
-            ptx::fence_proxy_async_smem();
+            if constexpr (L::kPInTmem) ptx::tmem_wait_st();
+            ptx::tc_fence_before_sync();  // orders P in tensor memory and the rescale of O before the MMAs that use them
+            if constexpr (!L::kPInTmem) ptx::fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&bars->p_full[q]);
         }

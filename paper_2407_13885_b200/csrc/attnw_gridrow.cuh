@@ -329,16 +329,14 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 ptx::tc_fence_after_sync();
                 if (lane == 0 && j == 0) ATTNW_STAMP(13, i);
                 const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(slot * kSub);
-                const uint32_t a_addr = q_addr + static_cast<uint32_t>((i & 1) * L::kTileBytes);
-                const uint32_t b_addr = k_addr + static_cast<uint32_t>(j * kSub * 128);  // keys kSub j ... of every atom
+                // (descriptors: the first of the tile plus a distance in 16-byte units)
+                const uint64_t a_desc = ptx::umma_desc_kmajor_sw128(q_addr + static_cast<uint32_t>((i & 1) * L::kTileBytes));
+                const uint64_t b_desc = ptx::umma_desc_kmajor_sw128(k_addr + static_cast<uint32_t>(j * kSub * 128));  // keys kSub j ... of every atom
                 if (ptx::elect_one()) {
 #pragma unroll
-                    for (int k = 0; k < D / 16; ++k) {
-                        const uint32_t a_off = static_cast<uint32_t>((k >> 2) * L::kAtomBytes + (k & 3) * 32);
-                        const uint32_t b_off = static_cast<uint32_t>((k >> 2) * L::kKAtomBytes + (k & 3) * 32);
-                        ptx::umma_f16_ss(d_tmem, ptx::umma_desc_kmajor_sw128(a_addr + a_off),
-                                         ptx::umma_desc_kmajor_sw128(b_addr + b_off), idesc, k > 0 ? 1u : 0u);
-                    }
+                    for (int k = 0; k < D / 16; ++k)
+                        ptx::umma_f16_ss(d_tmem, a_desc + static_cast<uint64_t>(((k >> 2) * L::kAtomBytes + (k & 3) * 32) >> 4),
+                                         b_desc + static_cast<uint64_t>(((k >> 2) * L::kKAtomBytes + (k & 3) * 32) >> 4), idesc, k > 0 ? 1u : 0u);
                     ptx::umma_commit(&bars->s_full[slot]);
                     if (j == n_sub - 1) {
                         ptx::umma_commit(&bars->q_empty[i & 1]);                               // the query tile may be replaced
