@@ -171,7 +171,7 @@ int softmax_rows_f32(const void* S, void* P, long long rows, long long cols, voi
  * Which form of the row Softmax softmax_rows uses (process-wide; Section VI-A compares the two on its hardware):
  *   0  by row length (default): rows of up to 262144 columns are read once and kept on chip ("caching": one
  *      exponential per element) - in registers up to 8192 columns, in the shared memory of one CTA up to 24576 and
- *      of a cluster of two CTAs up to 32768, in the registers of a cluster of 3 to 16 CTAs from 45057 to 262144;
+ *      of a cluster of two CTAs up to 32768, in the registers of a cluster of 3 to 16 CTAs from 43009 (few rows: 32769) to 262144;
  *      rows in between and longer rows are read twice (the second time out of L2), their exponentials recomputed
  *   1  caching only: rows of up to 393216 columns are kept in the shared memory of a thread-block cluster of up to
  *      16 CTAs that exchange local maxima and sums through distributed shared memory; a call with cols > 393216
@@ -204,8 +204,8 @@ int attnw_host_release(void);
  * up records a code in a per-device status word, makes the kernel unwind and return normally, and the output of
  * that launch is then undefined.
  * The word is STICKY: while it is non-zero, every later launch of the tensor-core kernels (attnw_fused*, attn_fused,
- * attnw_project_qk) and of the shared-memory and cluster tiers of softmax_rows* (rows of 8193 to 32768 and of 45057
- * to 262144 columns) returns at once WITHOUT WRITING ITS OUTPUT - the
+ * attnw_project_qk) and of the shared-memory and cluster tiers of softmax_rows* (rows of 8193 to 262144 columns, but
+ * for those that are read twice) returns at once WITHOUT WRITING ITS OUTPUT - the
  * call itself still returns ATTNW_OK, since it only enqueues - so that no work piles up behind a device that has
  * stopped making progress.  The register and streaming tiers of softmax_rows* have no waits and ignore the word.
  * attnw_query_status() synchronises `stream`, stores the word in *device_status (0 = no failure; otherwise

@@ -17,7 +17,7 @@
 namespace attnw {
 
 constexpr long long kSoftmaxRowsSmemTierMinCols = 8192;  // rows longer than this may leave the register tier
-constexpr long long kSoftmaxRowsRegClusterMinCols = 45056;  // rows longer than this live in the registers of a cluster
+constexpr long long kSoftmaxRowsRegClusterMinCols = 43008;  // rows longer than this live in the registers of a cluster
 
 namespace srs {
 
@@ -205,6 +205,9 @@ inline cudaError_t launch(const float* S, OutT* P, long long rows, long long col
 // the bulk copy of the same piece of the next row, so no barrier sits in the load pipeline and the HBM read stream
 // does not pause for the reductions, the cluster exchange and the stores.  One read and one write per element, where
 // the two-read kernel moves every element through L2 twice.
+// The statistics cross the CTA and the cluster by mbarriers that only the readers wait on: with two block reductions and a
+// serial loop over the CTAs' pairs 628 x 198496 took 181 us (now 169), 1024 x 262144 318 (308), 12 x 60000 6.4 (5.6);
+// sending every warp's pair to every CTA instead of one per CTA was slower for many rows (2048 x 131072 280 -> 305).
 // CTAs of 512 threads, two per SM, whose phases overlap (CTAs of 1024 threads with slices of 32768 columns were slower
 // at every length: fewer clusters of them are resident at once, 15 of 8 CTAs against 14 of 16).
 constexpr int kRcThreads = 512;
@@ -216,10 +219,10 @@ constexpr uint32_t kSiteRcExchange = 122;
 
 struct RcControl {
     uint64_t full[kRcThreads / 32];  // one per warp: its piece of the current row has landed
-    float red_max[kRcThreads / 32];
-    float red_sum[kRcThreads / 32];
-    uint64_t pairs_in[2];            // by row parity: the (maximum, sum) pairs of every CTA of the cluster have arrived
-    float2 xch[2][kMaxCluster];      // [row parity][CTA]: (local maximum, local sum)
+    uint64_t pieces_in[2];           // by row parity: the (maximum, sum) pairs of the CTA's warps are in place
+    uint64_t pairs_in[2];            // by row parity: the pairs of every CTA of the cluster have arrived
+    float2 piece[2][kRcThreads / 32];  // [row parity][warp]
+    float2 xch[2][kMaxCluster];      // [row parity][CTA]
     uint32_t abort_flag;
     uint32_t prior_failure;
 };
@@ -253,8 +256,10 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
         ptx::grid_dependency_wait();
         const uint32_t prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);  // (arrives meanwhile)
         for (int w = 0; w < kWarpsRc; ++w) ptx::mbar_init(&ctl->full[w], 1);
-        ptx::mbar_init(&ctl->pairs_in[0], 1);
-        ptx::mbar_init(&ctl->pairs_in[1], 1);
+        for (int i = 0; i < 2; ++i) {
+            ptx::mbar_init(&ctl->pieces_in[i], kWarpsRc);
+            ptx::mbar_init(&ctl->pairs_in[i], 1);
+        }
         ctl->abort_flag = 0;
         ctl->prior_failure = prior_failure;
         ptx::mbar_fence_init();
@@ -275,10 +280,11 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
 
     uint32_t it = 0;
     for (long long row = cluster; row < rows; row += n_clusters, ++it) {
-        if (ok && bytes > 0) ok = fused_wait(&ctl->full[warp], it & 1u, abort_flag, kSiteRcRowLoad);
+        if (ok && bytes > 0) ok = warp_wait(ptx::smem_u32(&ctl->full[warp]), it & 1u, abort_flag, kSiteRcRowLoad);
+        if (!ok) break;  // (the warps that wait for this one's pair give up as well)
         float4 v[kRcVecPerThread];
         float m = -INFINITY;
-        if (ok && full) {  // the common case, free of per-vector bounds checks
+        if (full) {  // the common case, free of per-vector bounds checks
 #pragma unroll
             for (int k = 0; k < kRcVecPerThread; ++k) {
                 v[k] = x[v0 + k * 32 + lane];
@@ -288,7 +294,7 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
 #pragma unroll
             for (int k = 0; k < kRcVecPerThread; ++k) {
                 const int idx = v0 + k * 32 + lane;
-                if (ok && idx < v1) {
+                if (idx < v1) {
                     v[k] = x[idx];
                     m = fmaxf(m, fmaxf(fmaxf(v[k].x, v[k].y), fmaxf(v[k].z, v[k].w)));
                 } else {
@@ -298,12 +304,11 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
         }
         ptx::fence_proxy_async_smem();  // orders these reads before the next bulk copy into the same bytes
         __syncwarp();
-        if (ok && lane == 0 && bytes > 0 && row + n_clusters < rows) issue(row + n_clusters);
+        if (lane == 0 && bytes > 0 && row + n_clusters < rows) issue(row + n_clusters);
 
-        m = sr_row_reduce<kRcThreads, true>(m, ctl->red_max);
-        // a warp that gave up has set the flag before the barrier inside the reduction: all or none of the CTA goes on
-        ok = *abort_flag == 0u && ctl->prior_failure == 0u;
-        const float mc = (m > -INFINITY) ? m : 0.0f;  // an empty slice (or a failure upstream): keeps inf - inf out
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        const float mc = (m > -INFINITY) ? m : 0.0f;  // an empty piece: keeps inf - inf out
         float l = 0.0f;
 #pragma unroll
         for (int k = 0; k < kRcVecPerThread; ++k) {
@@ -314,31 +319,48 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
             v[k].w = sr_ex2((v[k].w - mc) * kLog2e);
             l += (v[k].x + v[k].y) + (v[k].z + v[k].w);
         }
-        l = sr_row_reduce<kRcThreads, false>(l, ctl->red_sum);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
 
-        float factor;
-        if (C > 1) {
-            // One exchange of (maximum, sum) across the cluster without a cluster barrier: every CTA sends its pair into
-            // every CTA's slots (two sets by row parity) with a store that completes bytes on the receiver's mbarrier,
-            // and waits only for its own slots to fill.  A CTA can send the pair of row r + 2 (the same parity) only
-            // after receiving every pair of row r + 1, which its peers sent after reading their slots of row r.
-            const uint32_t par = it & 1u;
-            if (threadIdx.x < static_cast<unsigned>(C))
-                ptx::st_async_b64(ptx::map_to_cta(ptx::smem_u32(&ctl->xch[par][rank]), threadIdx.x), ptx::pack2(m, l),
-                                  ptx::map_to_cta(ptx::smem_u32(&ctl->pairs_in[par]), threadIdx.x));
-            if (threadIdx.x == 0) ptx::mbar_expect_tx(&ctl->pairs_in[par], static_cast<uint32_t>(C) * 8u);
-            if (ok) ok = fused_wait(&ctl->pairs_in[par], (it >> 1) & 1u, abort_flag, kSiteRcExchange);
-            float M = ctl->xch[par][0].x;
-            for (int c = 1; c < C; ++c) M = fmaxf(M, ctl->xch[par][c].x);
-            if (!(M > -INFINITY)) M = 0.0f;
-            float L = 0.0f;
-            for (int c = 0; c < C; ++c)  // the same order in every CTA; an empty slice has sum 0 and maximum -inf
-                L += ctl->xch[par][c].y * sr_ex2((ctl->xch[par][c].x - M) * kLog2e);
-            factor = sr_ex2((mc - M) * kLog2e) / L;
-        } else {
-            factor = 1.0f / l;
+        // One exchange of (maximum, sum) per row, without a barrier of the CTA or of the cluster: a warp leaves the pair of its
+        // piece in shared memory, warp 0 merges them and sends the CTA's pair into every CTA's slots with stores that
+        // complete bytes on the receiver's mbarrier, and every warp waits only for its own CTA's slots to fill.  All slots
+        // are double, by row parity: a pair of row r + 2 can be written only after every pair of row r + 1 has been received,
+        // which the others sent after reading those of row r.
+        const uint32_t par = it & 1u, phase = (it >> 1) & 1u;
+        if (lane == 0) {
+            ctl->piece[par][warp] = make_float2(m, l);
+            ptx::mbar_arrive(&ctl->pieces_in[par]);
         }
-        if (ok) {
+        __syncwarp();
+        if (warp == 0) {
+            ok = warp_wait(ptx::smem_u32(&ctl->pieces_in[par]), phase, abort_flag, kSiteRcExchange);
+            if (!ok) break;
+            const float2 p = ctl->piece[par][lane & (kWarpsRc - 1)];
+            float pm = p.x;
+#pragma unroll
+            for (int off = kWarpsRc / 2; off > 0; off >>= 1) pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, off));
+            float pl = p.y * sr_ex2((p.x - (pm > -INFINITY ? pm : 0.0f)) * kLog2e);
+#pragma unroll
+            for (int off = kWarpsRc / 2; off > 0; off >>= 1) pl += __shfl_xor_sync(0xffffffffu, pl, off);
+            if (lane < C)
+                ptx::st_async_b64(ptx::map_to_cta(ptx::smem_u32(&ctl->xch[par][rank]), lane), ptx::pack2(pm, pl),
+                                  ptx::map_to_cta(ptx::smem_u32(&ctl->pairs_in[par]), lane));
+            if (lane == 0) ptx::mbar_expect_tx(&ctl->pairs_in[par], static_cast<uint32_t>(C) * 8u);
+        }
+        ok = warp_wait(ptx::smem_u32(&ctl->pairs_in[par]), phase, abort_flag, kSiteRcExchange);
+        if (!ok) break;
+        // every warp reduces the CTAs' pairs, in the same order
+        const float2 pair = (lane & 15) < C ? ctl->xch[par][lane & 15] : make_float2(-INFINITY, 0.0f);
+        float M = pair.x;
+#pragma unroll
+        for (int off = kMaxCluster / 2; off > 0; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
+        if (!(M > -INFINITY)) M = 0.0f;
+        float L = pair.y * sr_ex2((pair.x - M) * kLog2e);
+#pragma unroll
+        for (int off = kMaxCluster / 2; off > 0; off >>= 1) L += __shfl_xor_sync(0xffffffffu, L, off);
+        const float factor = sr_ex2((mc - M) * kLog2e) / L;
+        {
             OutT* dst = P + row * cols + c0 + 4ll * (v0 + lane);
             if (full) {
 #pragma unroll
@@ -369,7 +391,7 @@ template <typename OutT>
 inline cudaError_t launch_regcluster(const float* S, OutT* P, long long rows, long long cols, int* resident_clusters,
                                      cudaStream_t stream) {
     const int C = rc_cluster_ctas_for(cols);
-    if (C == 0) return cudaErrorInvalidValue;
+    if (C < 2) return cudaErrorInvalidValue;  // the exchange needs a cluster launch, also to reach the CTA itself
     constexpr int kSmemMax = kRcControlBytes + kRcSliceMaxCols * 4;
     const int slice_cols = static_cast<int>(((cols / 4 + C - 1) / C) * 4);
     auto kernel = softmax_rows_regcluster_kernel<OutT>;
