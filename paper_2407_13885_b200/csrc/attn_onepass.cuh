@@ -2,7 +2,8 @@
 // Section IV (the product with V is the paper's future work, Section VIII) with the online form of Eq. 1.
 //
 // A CTA holds two units that share its tensor pipe and its special function units: two query tiles of 128 rows over all
-// key tiles, or (split) ONE query tile, unit 0 over the even and unit 1 over the odd key tiles, merged at the end.
+// key tiles, or (split) ONE query tile, unit 0 over the even and unit 1 over the odd key tiles, merged at the end; or the
+// 2 G units of a cluster of G CTAs share one query tile, unit u over the key tiles u, u + 2 G, ...
 // Per step j and unit q:
 //   MMA 1     S = Q K_j^T                         128 x 128 fp32 in tensor memory (one buffer per unit)
 //   Softmax   two threads per row, 64 columns each: a thread takes its scores to registers (the buffer is handed back
@@ -31,6 +32,7 @@ constexpr int kSmWarps = 16;      // Softmax warps: unit (2) x column half (2) x
 constexpr int kProducer = 16;
 constexpr int kMma = 17;
 constexpr int kThreads = 576;
+constexpr int kMaxCluster = 4;    // CTAs that share a query tile (of 8, 15 clusters fit, and a call that needs them has 16 tiles)
 constexpr float kLazy = 8.0f;     // the offset follows the maximum only when it has grown by more than this
 
 enum : uint32_t {  // wait sites of this kernel (low byte of the status word)
@@ -97,12 +99,16 @@ __device__ __forceinline__ bool wait_in_place(uint64_t* bar, uint32_t parity, vo
     }
 }
 
-template <int D, bool split>
+// How the keys of a query tile are worked on.
+enum Mode { kWhole, kSplit, kCluster };
+
+template <int D, Mode M>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o, int N,
-                    int row_blocks_per_head, float scale_log2e) {
+                    int row_blocks_per_head, float scale_log2e, __nv_bfloat16* O, int cluster_ctas) {
     using L = Smem<D>;
+    constexpr bool split = M != kWhole;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     Barriers* bars = reinterpret_cast<Barriers*>(smem + L::kBarOff);
@@ -112,11 +118,17 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const int bh = blockIdx.x / row_blocks_per_head;
-    const int row0 = (blockIdx.x % row_blocks_per_head) * (split ? kTile : kRowsPerCta);
+    const int G = M == kCluster ? cluster_ctas : 1;  // CTAs that share a query tile
+    const int rank = M == kCluster ? static_cast<int>(ptx::cluster_ctarank()) : 0;
+    const int block = static_cast<int>(blockIdx.x) / G;
+    const int bh = block / row_blocks_per_head;
+    const int row0 = (block % row_blocks_per_head) * (split ? kTile : kRowsPerCta);
     const int T = (N + kTile - 1) / kTile;  // key tiles
-    // key tiles of a unit: all of them, or every second one
-    const int steps[2] = {split ? (T + 1) >> 1 : T, split ? T >> 1 : (row0 + kTile < N ? T : 0)};
+    // The key tiles of a unit: all of them, or one in 2 G.
+    const int units = split ? 2 * G : 1;
+    auto key_tile = [&](int j, int q) { return split ? units * j + 2 * rank + q : j; };
+    const int steps[2] = {split ? (T - 2 * rank + units - 1) / units : T,
+                          split ? (T - 2 * rank + units - 2) / units : (row0 + kTile < N ? T : 0)};
     constexpr int kStages = L::kStages + (split ? 1 : 0);
     auto stage_offset = [](int s) { return !split || s < L::kStages ? L::kKOff + s * L::kTileBytes : L::kQOff + L::kTileBytes; };
 
@@ -183,12 +195,12 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                     ptx::tma_load_3d(smem + stage_offset(n % kStages) + a * L::kAtomBytes, map, &bars->k_full[s], a * 64, kt * kTile, bh, keep);
                 ++n;
             };
-            const int units = split ? 2 : 1;  // that have key tiles of their own
+            const int lists = split ? 2 : 1;  // units that have key tiles of their own
             for (int j = -1; ok && j < steps[0]; ++j) {
-                for (int q = 0; q < units; ++q)
-                    if (j + 1 < steps[q]) load(&tm_k, units * (j + 1) + q);
-                for (int q = 0; j >= 0 && q < units; ++q)
-                    if (j < steps[q]) load(&tm_v, units * j + q);
+                for (int q = 0; q < lists; ++q)
+                    if (j + 1 < steps[q]) load(&tm_k, key_tile(j + 1, q));
+                for (int q = 0; j >= 0 && q < lists; ++q)
+                    if (j < steps[q]) load(&tm_v, key_tile(j, q));
             }
             if (*abort_flag) {
                 // Unwinding: let the copies already in flight land before shared memory is released.
@@ -330,7 +342,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             ok = __all_sync(0xffffffffu, fused_wait(&bars->s_full[q], static_cast<uint32_t>(j) & 1u, abort_flag, kSiteSFull));
             if (!ok) break;
             ptx::tc_fence_after_sync();
-            const int valid = N - (split ? 2 * j + q : j) * kTile;  // key columns of this tile that exist
+            const int valid = N - key_tile(j, q) * kTile;  // key columns of this tile that exist
             // ---- maximum of the other thread's 64 columns (read and dropped) ----
             float mo = -3.0e38f;
 #pragma unroll
@@ -455,7 +467,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         }
 
         // ---- epilogue: O / l -> bf16 -> the P tile's shared memory -> TMA stores ----
-        if (steps[q] > 0) {
+        if (split || steps[q] > 0) {  // (split: each unit has a step)
             // Two units of one query tile each finish alone.  Two units of the same query tile meet here: the four threads of a
             // row take D / 4 columns each of 2^(mb_0 - mb) O_0 + 2^(mb_1 - mb) O_1.
             const int u = split ? 0 : q;  // the barriers and the P tile this epilogue uses
@@ -470,7 +482,83 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 ptx::mbar_arrive_if(bar_of(offsetof(Barriers, l_full), u), lane0);
                 ok = warp_wait(bar_of(offsetof(Barriers, l_full), u), 0, abort_flag, kSiteLFull);
             }
-            if (ok) {
+            if constexpr (M == kCluster) {
+                // The CTAs of a cluster have worked on other key tiles of the same query tile.  Each leaves its rows' (offset, sum) in
+                // its shared memory; after the cluster's barrier every thread knows its row's global ones, scales its
+                // part of O and sends it to the CTA that owns the row (128 / G rows each); after another barrier the
+                // owners add the G parts, in the order of the CTAs, and write O.
+                float2* pairs = reinterpret_cast<float2*>(smem + L::kKOff + 4096);
+                const uint32_t parts = ptx::smem_u32(smem + L::kKOff + 8192);  // float [G CTAs][128 / G rows][D], 16-byte pieces XOR-swizzled by row
+                const int my_rows = kTile / G;
+                const float l_own = ok ? l + lx[(q * 2 + (half ^ 1)) * kTile + row] : 1.0f;
+                const float mb_other = ok ? ox[(q ^ 1) * kTile + row] : 0.0f;
+                if (ok && q == 0 && half == 0) {
+                    const float* lo = lx + (q ^ 1) * 2 * kTile + row;
+                    const float top = fmaxf(mb, mb_other);
+                    pairs[row] = make_float2(top, l_own * ptx::ex2_approx(mb - top) + (lo[0] + lo[kTile]) * ptx::ex2_approx(mb_other - top));
+                }
+                __syncwarp();
+                ptx::cluster_arrive_release();
+                ptx::cluster_wait_acquire();
+                if (ok) {
+                    float2 pair[kMaxCluster];
+                    float top = -3.0e38f, sum = 0.0f;
+#pragma unroll
+                    for (int g = 0; g < kMaxCluster; ++g) {
+                        pair[g] = ptx::ld_cluster_v2(ptx::map_to_cta(ptx::smem_u32(pairs + row), static_cast<uint32_t>(g < G ? g : 0)));
+                        top = fmaxf(top, pair[g].x);
+                    }
+#pragma unroll
+                    for (int g = 0; g < kMaxCluster; ++g) sum += g < G ? pair[g].y * ptx::ex2_approx(pair[g].x - top) : 0.0f;
+                    const float inv = 1.0f / sum;
+                    const float f_own = ptx::ex2_approx(mb - top) * inv, f_other = ptx::ex2_approx(mb_other - top) * inv;
+                    ptx::tc_fence_after_sync();
+                    const uint32_t o_unit = t_quarter + static_cast<uint32_t>((q * 2 + 1) * kTile);
+                    const uint32_t o_peer = t_quarter + static_cast<uint32_t>(((q ^ 1) * 2 + 1) * kTile);
+                    const uint32_t dst = ptx::map_to_cta(parts + static_cast<uint32_t>((rank * my_rows + row % my_rows) * D * 4),
+                                                         static_cast<uint32_t>(row / my_rows));
+                    const int col0 = (q * 2 + half) * (D / 4);
+#pragma unroll 1
+                    for (int c = col0; c < col0 + D / 4; c += 16) {
+                        uint32_t o[16], r[16];
+                        ptx::tmem_ld_32x32b_x16(o_unit + static_cast<uint32_t>(c), o);
+                        ptx::tmem_ld_32x32b_x16(o_peer + static_cast<uint32_t>(c), r);
+                        ptx::tmem_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            float v[4];
+#pragma unroll
+                            for (int x = 0; x < 4; ++x)
+                                v[x] = fmaf(__uint_as_float(r[4 * i + x]), f_other, __uint_as_float(o[4 * i + x]) * f_own);
+                            ptx::st_cluster_v4(dst + (((static_cast<uint32_t>(c) >> 2) + static_cast<uint32_t>(i)) ^ static_cast<uint32_t>(lane & 7)) * 16u,
+                                               v[0], v[1], v[2], v[3]);
+                        }
+                    }
+                }
+                __syncwarp();
+                ptx::cluster_arrive_release();
+                ptx::cluster_wait_acquire();
+                if (ok) {
+                    for (int idx = static_cast<int>(threadIdx.x); idx < my_rows * (D / 8); idx += kSmWarps * 32) {
+                        const int r = idx / (D / 8), piece = idx % (D / 8);  // 8 columns of row r of this CTA's
+                        const int at = row0 + rank * my_rows + r;
+                        if (at >= N) continue;
+                        float v[8] = {};
+                        for (int g = 0; g < G; ++g) {
+                            const float4* src = reinterpret_cast<const float4*>(smem + L::kKOff + 8192) + (g * my_rows + r) * (D / 4);
+                            const float4 a = src[(2 * piece) ^ (r & 7)], b = src[(2 * piece + 1) ^ (r & 7)];
+                            v[0] += a.x, v[1] += a.y, v[2] += a.z, v[3] += a.w;
+                            v[4] += b.x, v[5] += b.y, v[6] += b.z, v[7] += b.w;
+                        }
+                        uint4 out;
+                        out.x = ptx::pack_bf16x2(v[0], v[1]);
+                        out.y = ptx::pack_bf16x2(v[2], v[3]);
+                        out.z = ptx::pack_bf16x2(v[4], v[5]);
+                        out.w = ptx::pack_bf16x2(v[6], v[7]);
+                        reinterpret_cast<uint4*>(O + (static_cast<size_t>(bh) * N + at) * D)[piece] = out;
+                    }
+                }
+            } else if (ok) {
                 float f_own, f_other = 0.0f;
                 const float l_own = l + lx[(q * 2 + (half ^ 1)) * kTile + row];
                 if (split) {
@@ -534,6 +622,15 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         }
     }
 
+    if constexpr (M == kCluster) {
+        if (!run || warp >= kSmWarps) {  // the Softmax warps' two barriers
+            __syncwarp();
+            ptx::cluster_arrive_release();
+            ptx::cluster_wait_acquire();
+            ptx::cluster_arrive_release();
+            ptx::cluster_wait_acquire();
+        }
+    }
     // ---- teardown: every role falls through to here, also after a wait gave up ----
     ptx::tc_fence_before_sync();
     __syncthreads();

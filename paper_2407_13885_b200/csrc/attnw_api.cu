@@ -77,6 +77,7 @@ struct DeviceInfo {
     cudaStream_t side_stream = nullptr;
     cudaEvent_t fork_event = nullptr, join_event = nullptr;
     std::atomic<int> gridrow_clusters[2][2][17] = {};  // resident clusters of 2..16 CTAs of the grid-row kernel, [d == 128][P is float32][CTAs], 0 = not asked yet
+    std::atomic<int> attn_clusters[2][5] = {};  // resident clusters of 2 and 4 CTAs of the one-pass attention kernel, [d == 128][CTAs]
     int rc_clusters[2][17] = {};  // resident clusters of 1..16 CTAs of the register-cluster row kernel, [P is float32][CTAs]
 };
 std::mutex g_split_mutex;
@@ -572,8 +573,35 @@ int launch_attn(const void* Q, const void* K, const void* V, void* O, int BH, in
     return ATTNW_OK;
 }
 
+// How many clusters of `ctas` CTAs of the one-pass attention kernel the device holds at once; -1 = none.
 template <int D>
-int launch_attn_onepass(const DeviceInfo* dev, const void* Q, const void* K, const void* V, void* O, int BH, int N, float scale, cudaStream_t stream) {
+int attn_max_clusters(DeviceInfo* dev, int ctas) {
+    std::atomic<int>& memo = dev->attn_clusters[D == 128][ctas];
+    int n = memo.load(std::memory_order_relaxed);
+    if (n != 0) return n;
+    auto kernel = av1::attn_onepass_kernel<D, av1::kCluster>;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(ctas);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(av1::kThreads, 1, 1);
+    cfg.gridDim = dim3(static_cast<unsigned>(ctas * dev->sm_count), 1, 1);
+    cfg.dynamicSmemBytes = av1::Smem<D>::kDynamicBytes;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (allow_smem<av1::attn_onepass_kernel<D, av1::kCluster>>(av1::Smem<D>::kDynamicBytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
+        (void)cudaGetLastError();
+        n = -1;
+    }
+    memo.store(n, std::memory_order_relaxed);
+    return n;
+}
+
+template <int D>
+int launch_attn_onepass(DeviceInfo* dev, const void* Q, const void* K, const void* V, void* O, int BH, int N, float scale, cudaStream_t stream) {
     using L = av1::Smem<D>;
     CUtensorMap tm_q, tm_k, tm_v, tm_o;
     int rc = encode_3d(&tm_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Q, D, N, BH, 64, kTile);
@@ -581,23 +609,43 @@ int launch_attn_onepass(const DeviceInfo* dev, const void* Q, const void* K, con
     if (rc == ATTNW_OK) rc = encode_3d(&tm_v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, V, D, N, BH, 64, kTile);
     if (rc == ATTNW_OK) rc = encode_3d(&tm_o, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, O, D, N, BH, 64, kTile);
     if (rc != ATTNW_OK) return rc;
-    // Two query tiles per CTA, or one whose even and odd key tiles are worked on side by side: twice the CTAs of half the
-    // length, chosen when that takes 5 % fewer rounds of key tiles on the device.
+    // Two query tiles per CTA; or one whose even and odd key tiles are worked on side by side; or one for a cluster of 2 or 4
+    // CTAs.  Chosen by the rounds of key tiles on the device (about 2 us each) plus what a round of CTAs costs besides: 1.5 of
+    // them for set-up and epilogue, 2 more for a cluster's merge.  us per call, one CTA -> cluster: 1 x 4744 (d = 64)
+    // 43.5 -> 28.5, 1 x 9260 (d = 128) 85.6 -> 53.6, 4 x 2155 24.2 -> 19.8, 3 x 824 11.9 -> 10.8, 1 x 1000 13.3 -> 13.2.
     const long long tiles = (N + kTile - 1) / kTile, pairs = (tiles + 1) / 2;
-    const long long rounds = (BH * pairs + dev->sm_count - 1) / dev->sm_count * tiles;
-    const long long rounds_split = (BH * tiles + dev->sm_count - 1) / dev->sm_count * pairs;
-    const bool split = tiles > 1 && BH * tiles <= INT_MAX && rounds_split * 105 < rounds * 100;
-    const int row_blocks = static_cast<int>(split ? tiles : pairs);
-    const float scale_log2e = static_cast<float>(static_cast<double>(scale) * 1.4426950408889634074);
-    const cudaError_t allowed = split ? allow_smem<av1::attn_onepass_kernel<D, true>>(L::kDynamicBytes)
-                                      : allow_smem<av1::attn_onepass_kernel<D, false>>(L::kDynamicBytes);
-    if (allowed != cudaSuccess) {
-        (void)cudaGetLastError();
-        return ATTNW_ERR_CUDA;
+    auto waves = [](long long work, long long at_once) { return static_cast<double>((work + at_once - 1) / at_once); };
+    av1::Mode mode = av1::kWhole;
+    int ctas = 1;  // per row block
+    double best = waves(BH * pairs, dev->sm_count) * (static_cast<double>(tiles) + 1.5);
+    if (tiles > 1 && BH * tiles <= INT_MAX) {
+        const double cost = waves(BH * tiles, dev->sm_count) * (static_cast<double>(pairs) + 1.5);
+        if (cost * 1.05 < best) {
+            best = cost;
+            mode = av1::kSplit;
+        }
+        for (int g = 2; g <= av1::kMaxCluster && 2 * g <= tiles && BH * tiles * g <= INT_MAX; g *= 2) {
+            const int clusters = attn_max_clusters<D>(dev, g);
+            if (clusters < 1) break;
+            const double c = waves(BH * tiles, clusters) * (static_cast<double>((tiles + 2 * g - 1) / (2 * g)) + 3.5);
+            if (c * 1.05 < best) {
+                best = c;
+                mode = av1::kCluster;
+                ctas = g;
+            }
+        }
     }
-    auto kernel = split ? av1::attn_onepass_kernel<D, true> : av1::attn_onepass_kernel<D, false>;
-    if (launch_overlapped(kernel, static_cast<unsigned>(BH * row_blocks), av1::kThreads, L::kDynamicBytes, stream, 1, false, tm_q, tm_k, tm_v,
-                          tm_o, N, row_blocks, scale_log2e) != cudaSuccess) {
+    const int row_blocks = static_cast<int>(mode == av1::kWhole ? pairs : tiles);
+    const float scale_log2e = static_cast<float>(static_cast<double>(scale) * 1.4426950408889634074);
+    const cudaError_t allowed = mode == av1::kWhole   ? allow_smem<av1::attn_onepass_kernel<D, av1::kWhole>>(L::kDynamicBytes)
+                                : mode == av1::kSplit ? allow_smem<av1::attn_onepass_kernel<D, av1::kSplit>>(L::kDynamicBytes)
+                                                      : allow_smem<av1::attn_onepass_kernel<D, av1::kCluster>>(L::kDynamicBytes);
+    auto kernel = mode == av1::kWhole   ? av1::attn_onepass_kernel<D, av1::kWhole>
+                  : mode == av1::kSplit ? av1::attn_onepass_kernel<D, av1::kSplit>
+                                        : av1::attn_onepass_kernel<D, av1::kCluster>;
+    if (allowed != cudaSuccess ||
+        launch_overlapped(kernel, static_cast<unsigned>(BH * row_blocks * ctas), av1::kThreads, L::kDynamicBytes, stream, ctas, false, tm_q,
+                          tm_k, tm_v, tm_o, N, row_blocks, scale_log2e, static_cast<__nv_bfloat16*>(O), ctas) != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
     }

@@ -170,8 +170,10 @@ def test_attention_full_size_sampled(attnw):
 
 
 # One query tile per CTA over two halves of the keys (few CTAs) against two query tiles per CTA (many): 2, 3, 8 and 16 key tiles,
-# an odd number of them, ragged last tiles, a second query tile that does not exist
-@pytest.mark.parametrize("B,H,N,d", [(1, 1, 129, 64), (1, 2, 300, 128), (1, 3, 1021, 64), (2, 2, 2048, 128), (4, 37, 200, 64), (4, 37, 257, 128)])
+# an odd number of them, ragged last tiles, a second query tile that does not exist; then clusters of 4 and 2 CTAs per query tile
+# (12, 17 and 41 key tiles, 1 to 5 steps a unit, rows of the last tile beyond N)
+@pytest.mark.parametrize("B,H,N,d", [(1, 1, 129, 64), (1, 2, 300, 128), (1, 3, 1021, 64), (2, 2, 2048, 128), (4, 37, 200, 64), (4, 37, 257, 128), (1, 1, 1536, 64),
+                                     (1, 2, 2049, 128), (1, 1, 5131, 64), (1, 1, 5131, 128)])
 def test_attention_split_and_whole(attnw, B, H, N, d):
     q, k = small_fused_inputs(B, H, N, d, sigma=2.0, stream=N + d + 23)
     v = rand_v(B, H, N, d, stream=N + d + 25)
