@@ -13,7 +13,11 @@
 //   columns [128, 512)  three packed regions, used by the row blocks in turn: the exponentials as f16 pairs, waiting
 //                       for the row's statistics
 // so two further row blocks can be computed, and their exponentials taken, while the statistics of one cross the
-// group.  (f16 keeps 11 bits of e in [0, 1]: 5e-4 relative, next to the 2e-3 of the bf16 result.)
+// group.  f16 keeps 11 bits of an exponential, 2.4e-4 relative next to the 2e-3 of the bf16 result, and no more than its
+// range: the offset therefore leaves 2^15 of headroom above 1, which keeps those bits down to 2^-29 of the largest of a
+// chunk, and the row's factor is applied in float32.  (With the largest at 1 and an f16 factor, weights of 1e-9 .. 1e-6 were
+// 0.75 off in relative rms at N = 16384, logits of sigma 16; now 1.7e-3, the rounding of bf16.  It costs 0.5 %: 128 x 4096
+// 1090 and 1095 us, 12 x 2048 28.7 and 29.1.)
 // Tensor memory, float32 output: two regions of 256 columns; the exponentials replace the scores as float32, and a slot of
 // 64 columns goes back to the MMA issuer when its weights have been read.
 //
@@ -77,6 +81,7 @@ constexpr int kMergeWarpG = kMmaWarpG + 1;
 constexpr int kOwnerWarpG = kMmaWarpG + 3;
 constexpr int kThreads = 32 * (kOwnerWarpG + 1);
 constexpr int kStageBytes = 32 * 128;                // one staged store box: 32 rows x 128 bytes
+constexpr float kHeadroom = 15.0f;                   // bfloat16: exponentials are parked as f16 up to 2^15
 constexpr int kMaxDirectCtas = 4;                    // up to here every CTA reads all pairs of a row
 constexpr int kMaxGroupCtas = 128;
 constexpr int kMaxN = 4096;                          // what variant 4 and attnw_fused_noalloc serve
@@ -512,7 +517,8 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 m0 = ptx::max3(m0, __uint_as_float(r[kChunk - 4]), __uint_as_float(r[kChunk - 3]));
                 m1 = ptx::max3(m1, __uint_as_float(r[kChunk - 2]), __uint_as_float(r[kChunk - 1]));
                 smax = ptx::max3(smax, ptx::max3(m0, m1, m2), m3);
-                const float mb_new = fmaxf(smax * c2, -3.0e38f);  // finite also while every column so far is masked
+                // finite also while every column so far is masked; rounded up, so that no exponential passes 2^kHeadroom
+                const float mb_new = fmaxf(kF32 ? smax * c2 : __fmaf_ru(smax, c2, -kHeadroom), -3.0e38f);
                 if (k > 0) l *= ptx::ex2_approx(mb - mb_new);     // exactly 1 while the maximum stands
                 mb = mb_new;
                 if (stamp) ATTNW_STAMP(16 + 3 * k, i);
@@ -658,14 +664,13 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
 #pragma unroll
                             for (int x = 0; x < 4; ++x) w[x] = __float_as_uint(__uint_as_float(e[gg * 4 + x]) * f[b]);
                         } else {
-                            // p = e * f in float32 from f16 operands (one mixed-precision FMA per element unpacks and
-                            // scales); a factor below f16 range rounds to zero, where p < 6e-8 anyway
                             const float fc = f[(2 * b + (gg >> 2)) % kParts];
-                            const uint32_t fh = ptx::pack_f16x2(fc, fc);
+                            const uint64_t ff = ptx::pack2(fc, fc);
 #pragma unroll
                             for (int x = 0; x < 4; ++x) {
                                 float lo, hi;
-                                ptx::scale_f16x2(e[gg * 4 + x], fh, lo, hi);
+                                ptx::unpack_f16x2(e[gg * 4 + x], lo, hi);
+                                ptx::unpack2(ptx::mul2(ptx::pack2(lo, hi), ff), lo, hi);
                                 w[x] = ptx::pack_bf16x2(lo, hi);
                             }
                         }

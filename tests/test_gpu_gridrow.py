@@ -59,6 +59,27 @@ def test_long_rows_match_oracle(attnw, dtype, H, N, d):
     assert err <= TOL[dtype]["abs"]
 
 
+# one CTA, an exchange where all read all, owners, and a group beyond 16 CTAs; a row whose largest logit is large itself
+@pytest.mark.parametrize("N,d,sigma", [(256, 64, 4.0), (1000, 128, 4.0), (2048, 128, 4.0), (8192, 128, 4.0), (2048, 64, 60.0)])
+def test_small_weights_keep_their_digits(attnw, N, d, sigma):
+    # A weight's relative error: its logit and its row's sum in float32 (d products, each step within 2^-23 of the sum of the
+    # products' sizes, twice), the exponential in f16 (2^-11) and the result in bf16 (2^-9), with a factor 2 on these.
+    g = torch.Generator(device="cuda").manual_seed(N + d)
+    Q, K = (torch.randn(1, 1, N, d, generator=g, device="cuda", dtype=torch.bfloat16).mul_(sigma) for _ in range(2))
+    P = attnw.attnw_fused(Q, K, scale_of(d))
+    torch.cuda.synchronize()
+    assert attnw.query_status() == 0
+    S = (Q[0, 0, :512].double() @ K[0, 0].double().T) * scale_of(d)
+    ref = torch.softmax(S, -1)
+    # within 2^-28 of its row's largest weight a weight is still a normal f16 number, whichever chunk it lies in
+    m = ref >= ref.amax(-1, keepdim=True) * 2.0 ** -28
+    size = (Q[0, 0, :512].double().abs() @ K[0, 0].double().abs().T) * scale_of(d)
+    bound = 2.0 ** -8 + 2.0 ** -10 + 2 * size * d * 2.0 ** -23
+    rel = (P[0, 0, :512].double() - ref).abs() / ref
+    assert int(m.sum()) > 512
+    assert bool((rel <= bound)[m].all()), float((rel / bound)[m].max())
+
+
 def test_more_streams_than_exchange_areas(attnw):
     # twelve streams, two calls each in flight, on inputs of their own: no launch may read another's statistics
     d, N = 64, 1536
