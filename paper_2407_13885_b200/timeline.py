@@ -70,17 +70,20 @@ def run(cta: int = 1, heads: int = 64, n: int = 4096, d: int = 128, launches: in
     period = float(np.mean(np.diff(buf[13, lo:hi])))
     table = {
         "period_per_row_block": period,
-        "exponential_role": {
-            "slot0_ready_to_halves_posted": span(2, 4),
-            "box0_load_and_maximum": span(17, 16), "box0_exponentials": span(16, 18), "box0_wait_region_and_store": span(18, 24),
-            "box1_load_and_maximum": span(20, 19), "box1_exponentials": span(19, 21), "box1_wait_region_and_store": span(21, 26),
-            "mma_issue_to_exponentials_begin": span(13, 0),
+        "exponential_role": {  # the first of the sixteen warps
+            "slot0_ready_to_posted": span(2, 4),
+            "slot0_load_and_maximum": span(17, 16), "slot0_exponentials": span(16, 18), "slot0_wait_region_and_store": span(18, 24),
+            "slot1_wait": span(24, 20),
+            "slot1_load_and_maximum": span(20, 19), "slot1_exponentials": span(19, 21), "slot1_store": span(21, 26),
+            "mma_issue_to_slot0_ready": span(13, 2),
+        },
+        "statistics": {
+            "first_warp_done_to_merge_begins": span(4, 1), "merge_and_post": span(1, 3), "post_to_owner_has_all_pairs": span(3, 23),
+            "owner_reduces_and_posts": span(23, 25), "result_to_normalise_warps": span(25, 11),
         },
         "normalise_role": {
-            "first_warp_done_to_block_visible_to_normalise": float(np.mean(buf[6, it] - buf[4, it])),
-            "wait_for_group": span(6, 11), "reduce_and_read_box0": span(11, 12),
-            "box2_wait_staging": span(14, 15), "box2_scale_round_stage": span(15, 8), "box2_fence_and_hand_over": span(8, 9),
-            "all_pairs_seen_to_block_done": span(11, 7),
+            "factors_and_read_box0": span(11, 12), "box1_wait_staging": span(14, 15), "box1_scale_round_stage": span(15, 8),
+            "box1_fence_and_store": span(8, 9), "statistics_seen_to_block_done": span(11, 7),
         },
     }
     return {"timeline_run": True, "case": f"attnw_fused (grid-row kernel) B=1 H={heads} N={n} d={d}, CTA {cta}, "
