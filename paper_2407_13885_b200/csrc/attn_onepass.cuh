@@ -5,13 +5,15 @@
 // key tiles, or (split) ONE query tile, unit 0 over the even and unit 1 over the odd key tiles, merged at the end; or the
 // 2 G units of a cluster of G CTAs share one query tile, unit u over the key tiles u, u + 2 G, ...
 // Per step j and unit q:
-//   MMA 1     S = Q K_j^T                         128 x 128 fp32 in tensor memory (one buffer per unit)
+//   MMA 1     S = Q K_j^T                         128 x 128 fp32 in tensor memory
 //   Softmax   two threads per row, 64 columns each: a thread takes its scores to registers (the buffer is handed back
-//             at once, so the next tile's MMA 1 runs meanwhile) and also reads the other thread's 64 columns for
+//             at once, so the next MMA 1 runs meanwhile) and also reads the other thread's 64 columns for
 //             their maximum, so both know the row maximum without an exchange; p = 2^(c s - mb) with the row's
-//             offset mb; l += sum p; P (bf16) becomes the A operand of MMA 2: through shared memory (d = 128), or, since d = 64
-//             leaves room, in tensor memory (128 x 4096 839 -> 801 us: the MMAs of d = 64 fetch 256 KB a step of two tiles
-//             from shared memory otherwise, as long as the exponentials take)
+//             offset mb; l += sum p; P (bf16) becomes the A operand of MMA 2 in tensor memory.  (Through shared memory its
+//             port was busy 3072 of 4200 cycles a step, and the clock lower under the power cap.  128 x 4096, d = 64: 839 -> 801 us;
+//             d = 128: 985 -> 941 at a burst, 1106 -> 1056 in a loop.)
+//             d = 64 has room for scores of both units beside P and O.  d = 128 has one buffer of scores: the units are half
+//             a step apart and hold it only from MMA 1 until their scores are in registers, less than half a step.
 //   MMA 2     O_q += P V_j                        128 x d fp32 in tensor memory; V_j as TMA delivers it
 //             ([128 keys x d], an MN-major B operand)
 // The offset mb of a row follows its running maximum lazily: it moves only when the maximum has grown by more than 8
@@ -53,15 +55,17 @@ struct Smem {
     static constexpr int kAtoms = D / 64;
     static constexpr int kAtomBytes = kTile * 128;             // 128 rows x 128 bytes
     static constexpr int kTileBytes = kAtoms * kAtomBytes;     // a Q, K or V tile
-    static constexpr int kPBytes = 2 * kAtomBytes;             // a P tile: 128 rows x 128 keys, two atoms of 64 keys
     static constexpr int kStages = (D == 128) ? 3 : 6;         // ring of K / V tiles (128 keys x d)
-    // d = 64 leaves 64 columns of tensor memory per unit beside the scores and O: P goes there as the product's A operand
-    // instead of through shared memory.
-    static constexpr bool kPInTmem = D == 64;
+    // Tensor memory: d = 64 has room for scores, O and P (the product's A operand) of both units; d = 128 for P and O of
+    // both and ONE buffer of scores, which the units use in turn.
+    static constexpr bool kSharedS = D == 128;
+    static __host__ __device__ constexpr uint32_t s_col(int q) { return kSharedS ? 0u : static_cast<uint32_t>(q * 256); }
+    static __host__ __device__ constexpr uint32_t p_col(int q) { return kSharedS ? 128u + static_cast<uint32_t>(q * 64) : static_cast<uint32_t>(q * 256 + 192); }
+    static __host__ __device__ constexpr uint32_t o_col(int q) { return kSharedS ? 256u + static_cast<uint32_t>(q * 128) : static_cast<uint32_t>(q * 256 + 128); }
     static constexpr int kQOff = 0;                            // two query tiles; split: one, and one more stage of the ring
     static constexpr int kKOff = kQOff + 2 * kTileBytes;
-    static constexpr int kPOff = kKOff + kStages * kTileBytes;
-    static constexpr int kBarOff = kPOff + 2 * kPBytes;
+    static constexpr int kOutOff = kKOff + kStages * kTileBytes;  // a unit's part of O on its way out
+    static constexpr int kBarOff = kOutOff + 2 * kTileBytes;
     static constexpr int kBytes = kBarOff + 256;
     static constexpr int kDynamicBytes = kBytes + 1024;
 };
@@ -71,7 +75,7 @@ struct Barriers {
     uint64_t q_full;
     uint64_t k_full[7], k_empty[7];
     uint64_t s_full[2], s_free[2];  // per unit: scores written / read into registers (8 warps)
-    uint64_t p_full[2], p_free[2];  // per unit: P tile written (8 warps) / read by its MMAs
+    uint64_t p_full[2], p_free[2];  // per unit: P written (8 warps) / read by its MMAs
     uint64_t o_full[2];             // per unit: every product complete
     uint64_t l_full[2];             // per query tile: the row statistics of its warps are in shared memory
     uint64_t out_filled[2];
@@ -171,7 +175,6 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bars->tmem_base;
     const bool run = bars->prior_failure == 0u;  // an earlier CTA gave up: do not queue more waits behind it
-    // tensor memory of unit q: scores in columns [256 q, 256 q + 128), O in [256 q + 128, 256 q + 128 + d), then P (d = 64)
 
     if (run && warp == kProducer) {
         // ================= TMA producer: Q once, then the K and V tiles in the order the MMA issuer reads them =========
@@ -197,10 +200,10 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             };
             const int lists = split ? 2 : 1;  // units that have key tiles of their own
             for (int j = -1; ok && j < steps[0]; ++j) {
-                for (int q = 0; q < lists; ++q)
+                for (int q = 0; q < lists; ++q) {
                     if (j + 1 < steps[q]) load(&tm_k, key_tile(j + 1, q));
-                for (int q = 0; j >= 0 && q < lists; ++q)
-                    if (j < steps[q]) load(&tm_v, key_tile(j, q));
+                    if (j >= 0 && j < steps[q]) load(&tm_v, key_tile(j, q));
+                }
             }
             if (*abort_flag) {
                 // Unwinding: let the copies already in flight land before shared memory is released.
@@ -232,12 +235,16 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             __syncwarp();
             ++n;
         };
+        int last_q = 0, last_j = -1;  // kSharedS: whose scores the buffer holds
         auto scores = [&](int q, int j) {  // S of step j
-            // the row threads have the scores of step j - 1 in registers
-            ok = ok && warp_wait(bar_of(offsetof(Barriers, s_free), q), (static_cast<uint32_t>(j) & 1u) ^ 1u, abort_flag, kSiteMmaSFree);
+            // the row threads have the scores that are in the buffer in registers
+            const int before_q = L::kSharedS ? last_q : q, before_j = L::kSharedS ? last_j : j - 1;
+            ok = ok && warp_wait(bar_of(offsetof(Barriers, s_free), before_q), static_cast<uint32_t>(before_j) & 1u, abort_flag, kSiteMmaSFree);
             if (!ok) return;
+            last_q = q;
+            last_j = j;
             ptx::tc_fence_after_sync();
-            const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(q * 2 * kTile);
+            const uint32_t d_tmem = tmem_base + L::s_col(q);
             // (descriptors: the first of the tile plus a distance in 16-byte units)
             const uint64_t a_desc = ptx::umma_desc_kmajor_sw128(base + L::kQOff + (split ? 0u : static_cast<uint32_t>(q * L::kTileBytes)));
             const uint64_t b_desc = ptx::umma_desc_kmajor_sw128(base + static_cast<uint32_t>(stage_offset(n % kStages)));
@@ -255,42 +262,35 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             ok = ok && warp_wait(bar_of(offsetof(Barriers, p_full), q), static_cast<uint32_t>(j) & 1u, abort_flag, kSiteMmaPFull);
             if (!ok) return;
             ptx::tc_fence_after_sync();
-            const uint32_t o_tmem = tmem_base + static_cast<uint32_t>((q * 2 + 1) * kTile);
-            const uint64_t a_desc = ptx::umma_desc_kmajor_sw128(base + L::kPOff + static_cast<uint32_t>(q * L::kPBytes));
+            const uint32_t o_tmem = tmem_base + L::o_col(q), p_tmem = tmem_base + L::p_col(q);
             const uint64_t b_desc = av::umma_desc_mnmajor_sw128(base + static_cast<uint32_t>(stage_offset(n % kStages)), L::kAtomBytes);
             if (ptx::elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < kTile / 16; ++kk) {  // 16 keys per instruction
-                    if constexpr (L::kPInTmem) {
-                        ptx::umma_f16_ts(o_tmem, o_tmem + static_cast<uint32_t>(D + kk * 8), b_desc + static_cast<uint64_t>(kk * 16 * 128 >> 4),
-                                         idesc_o, (j > 0 || kk > 0) ? 1u : 0u);
-                        continue;
-                    }
-                    ptx::umma_f16_ss(o_tmem, a_desc + static_cast<uint64_t>(((kk >> 2) * L::kAtomBytes + (kk & 3) * 32) >> 4),
-                                     b_desc + static_cast<uint64_t>(kk * 16 * 128 >> 4), idesc_o, (j > 0 || kk > 0) ? 1u : 0u);
-                }
+                for (int kk = 0; kk < kTile / 16; ++kk)  // 16 keys per instruction
+                    ptx::umma_f16_ts(o_tmem, p_tmem + static_cast<uint32_t>(kk * 8), b_desc + static_cast<uint64_t>(kk * 16 * 128 >> 4), idesc_o,
+                                     (j > 0 || kk > 0) ? 1u : 0u);
                 ptx::umma_commit(&bars->p_free[q]);
                 if (j + 1 == steps[q]) ptx::umma_commit(&bars->o_full[q]);
             }
             __syncwarp();
         };
-        // The scores of step j + 1 first: the tensor pipe computes them while the row threads exponentiate step j.  Two query
-        // tiles alternate - scores of one, product of one, scores of the other, product of the other - which keeps their
+        // The scores of step j + 1 first: the tensor pipe computes them while the row threads exponentiate step j.  The two
+        // units alternate - scores of one, product of one, scores of the other, product of the other - which keeps their
         // row threads half a step apart (d = 64, 128 x 4096: 888 -> 841 us against both scores first).
         for (int j = -1; ok && j < steps[0]; ++j) {
             if (split) {
-                for (int q = 0; q < 2; ++q)
+                for (int q = 0; q < 2; ++q) {
                     if (ok && j + 1 < steps[q]) {
                         arrived();
                         scores(q, j + 1);
                         release();
                     }
-                for (int q = 0; q < 2; ++q)
                     if (ok && j >= 0 && j < steps[q]) {
                         arrived();
                         product(q, j);
                         release();
                     }
+                }
             } else {
                 const bool next = j + 1 < T;
                 const int k_entry = n, v_entry = next ? n + 1 : n;  // K of step j + 1, V of step j
@@ -321,17 +321,15 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         const int half = (warp >> 2) & 1;
         const int quarter = warp & 3;
         const uint32_t t_quarter = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
-        const uint32_t t_own = t_quarter + static_cast<uint32_t>(q * 2 * kTile + half * kHalf);
-        const uint32_t o_own = t_quarter + static_cast<uint32_t>((q * 2 + 1) * kTile + half * (D / 2));  // this thread's D/2 columns of O
+        const uint32_t t_own = t_quarter + L::s_col(q) + static_cast<uint32_t>(half * kHalf);
+        const uint32_t o_own = t_quarter + L::o_col(q) + static_cast<uint32_t>(half * (D / 2));  // this thread's D/2 columns of O
         const float c2 = scale_log2e;
         const uint64_t c2c2 = ptx::pack2(c2, c2);
-        // this row in the P tile's atom of this column half (64 keys = 128 bytes, 16-byte pieces XOR-swizzled)
         const int row = quarter * 32 + lane;
-        const uint32_t t_other = t_quarter + static_cast<uint32_t>(q * 2 * kTile + (half ^ 1) * kHalf);
+        const uint32_t t_other = t_quarter + L::s_col(q) + static_cast<uint32_t>((half ^ 1) * kHalf);
         const uint32_t lane0 = lane == 0;
-        const uint32_t p_row = ptx::smem_u32(smem + L::kPOff + q * L::kPBytes) + static_cast<uint32_t>(half * L::kAtomBytes + row * 128);
         const uint32_t sw = static_cast<uint32_t>(lane & 7);
-        const uint32_t p_own = t_quarter + static_cast<uint32_t>((q * 2 + 1) * kTile + D + half * 32);  // kPInTmem: its 64 keys of P
+        const uint32_t p_own = t_quarter + L::p_col(q) + static_cast<uint32_t>(half * 32);  // its 64 keys of P
         float smax = -3.0e38f;  // running maximum of the raw scores of this row (all columns: both threads of a row
                                 // compute it, each from the whole tile, so they agree without an exchange)
         float mb = -3.0e38f;    // the offset the weights, l and O's row are relative to (follows smax * c2 lazily)
@@ -402,12 +400,11 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             smax = ptx::max3(smax, mo, ptx::max3(fmaxf(m0, m1), m2, m3));
             const float mb_cand = fmaxf(smax * c2, -3.0e38f);
             const bool move = j == 0 || mb_cand - mb > kLazy;
-            // the P tile and O are free once the MMAs of the previous key tile are complete
+            // P and O are free once the MMAs of the previous key tile are complete
             ok = __all_sync(0xffffffffu, wait_in_place(&bars->p_free[q], (static_cast<uint32_t>(j) & 1u) ^ 1u, abort_flag, kSitePFree));
             if (!ok) break;
-            if constexpr (L::kPInTmem) ptx::tc_fence_after_sync();
+            ptx::tc_fence_after_sync();
             uint32_t w[16];  // 32 keys of P on their way to tensor memory
-            (void)w;
             if (j == 0) {
                 mb = mb_cand;
             } else if (__any_sync(0xffffffffu, move)) {
@@ -428,7 +425,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 }
                 ptx::tmem_wait_st();
             }
-            // ---- weights: p = 2^(c2 s - mb) (below 2^8), row sum, bf16, into the P tile ----
+            // ---- weights: p = 2^(c2 s - mb) (below 2^8), row sum, bf16, into tensor memory ----
             const uint64_t nmb2 = ptx::pack2(-mb, -mb);
             uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
@@ -446,31 +443,25 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                     }
                     acc[(i >> 1) & 3] = ptx::add2(acc[(i >> 1) & 3], ptx::pack2(p[i], p[i + 1]));
                 }
-                if constexpr (L::kPInTmem) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) w[(g & 3) * 4 + i] = ptx::pack_bf16x2(p[2 * i], p[2 * i + 1]);
-                    if ((g & 3) == 3) ptx::tmem_st_32x32b_x16(p_own + static_cast<uint32_t>((g >> 2) * 16), w);
-                } else {
-                    ptx::st_shared_v4(p_row + ((static_cast<uint32_t>(g) ^ sw) << 4), ptx::pack_bf16x2(p[0], p[1]),
-                                      ptx::pack_bf16x2(p[2], p[3]), ptx::pack_bf16x2(p[4], p[5]), ptx::pack_bf16x2(p[6], p[7]));
-                }
+                for (int i = 0; i < 4; ++i) w[(g & 3) * 4 + i] = ptx::pack_bf16x2(p[2 * i], p[2 * i + 1]);
+                if ((g & 3) == 3) ptx::tmem_st_32x32b_x16(p_own + static_cast<uint32_t>((g >> 2) * 16), w);
             }
             float a0, a1, a2, a3;
             ptx::unpack2(ptx::add2(acc[0], acc[1]), a0, a1);
             ptx::unpack2(ptx::add2(acc[2], acc[3]), a2, a3);
             l += (a0 + a1) + (a2 + a3);
-            if constexpr (L::kPInTmem) ptx::tmem_wait_st();
+            ptx::tmem_wait_st();
             ptx::tc_fence_before_sync();  // orders P in tensor memory and the rescale of O before the MMAs that use them
-            if constexpr (!L::kPInTmem) ptx::fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&bars->p_full[q]);
         }
 
-        // ---- epilogue: O / l -> bf16 -> the P tile's shared memory -> TMA stores ----
+        // ---- epilogue: O / l -> bf16 -> shared memory -> TMA stores ----
         if (split || steps[q] > 0) {  // (split: each unit has a step)
             // Two units of one query tile each finish alone.  Two units of the same query tile meet here: the four threads of a
             // row take D / 4 columns each of 2^(mb_0 - mb) O_0 + 2^(mb_1 - mb) O_1.
-            const int u = split ? 0 : q;  // the barriers and the P tile this epilogue uses
+            const int u = split ? 0 : q;  // the barriers and the output tile this epilogue uses
             float* lx = reinterpret_cast<float*>(smem + L::kKOff);  // (every MMA is complete: the K / V ring is free)
             float* ox = lx + 4 * kTile;
             if (ok) ok = warp_wait(bar_of(offsetof(Barriers, o_full), q), 0, abort_flag, kSiteOFull);
@@ -513,8 +504,8 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                     const float inv = 1.0f / sum;
                     const float f_own = ptx::ex2_approx(mb - top) * inv, f_other = ptx::ex2_approx(mb_other - top) * inv;
                     ptx::tc_fence_after_sync();
-                    const uint32_t o_unit = t_quarter + static_cast<uint32_t>((q * 2 + 1) * kTile);
-                    const uint32_t o_peer = t_quarter + static_cast<uint32_t>(((q ^ 1) * 2 + 1) * kTile);
+                    const uint32_t o_unit = t_quarter + L::o_col(q);
+                    const uint32_t o_peer = t_quarter + L::o_col(q ^ 1);
                     const uint32_t dst = ptx::map_to_cta(parts + static_cast<uint32_t>((rank * my_rows + row % my_rows) * D * 4),
                                                          static_cast<uint32_t>(row / my_rows));
                     const int col0 = (q * 2 + half) * (D / 4);
@@ -576,9 +567,9 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 ptx::tc_fence_after_sync();
                 const int cols = split ? D / 4 : D / 2;
                 const int col0 = split ? (q * 2 + half) * (D / 4) : half * (D / 2);
-                const uint32_t o_unit = t_quarter + static_cast<uint32_t>((q * 2 + 1) * kTile);
-                const uint32_t o_peer = t_quarter + static_cast<uint32_t>(((q ^ 1) * 2 + 1) * kTile);
-                const uint32_t dst_row = ptx::smem_u32(smem + L::kPOff + u * L::kPBytes) + static_cast<uint32_t>(row * 128);
+                const uint32_t o_unit = t_quarter + L::o_col(q);
+                const uint32_t o_peer = t_quarter + L::o_col(q ^ 1);
+                const uint32_t dst_row = ptx::smem_u32(smem + L::kOutOff + u * L::kTileBytes) + static_cast<uint32_t>(row * 128);
 #pragma unroll 1
                 for (int c = col0; c < col0 + cols; c += 16) {
                     uint32_t o[16];
@@ -610,7 +601,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                     ok = warp_wait(bar_of(offsetof(Barriers, out_filled), u), 0, abort_flag, kSiteOutFilled);
                     if (ok && lane == 0) {
                         for (int a = 0; a < L::kAtoms; ++a)
-                            ptx::tma_store_3d(&tm_o, ptx::smem_u32(smem + L::kPOff + u * L::kPBytes + a * L::kAtomBytes), a * 64,
+                            ptx::tma_store_3d(&tm_o, ptx::smem_u32(smem + L::kOutOff + u * L::kTileBytes + a * L::kAtomBytes), a * 64,
                                               row0 + u * kTile, bh, ptx::policy_evict_first());
                         ptx::bulk_commit_group();
                         ptx::bulk_wait_group<0>();
