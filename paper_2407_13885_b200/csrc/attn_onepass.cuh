@@ -7,13 +7,8 @@
 // Per step j and unit q:
 //   MMA 1     S = Q K_j^T                         128 x 128 fp32 in tensor memory
 //   Softmax   two threads per row, 64 columns each: a thread takes its scores to registers (the buffer is handed back
-//             at once, so the next MMA 1 runs meanwhile) and also reads the other thread's 64 columns for
-//             their maximum, so both know the row maximum without an exchange; p = 2^(c s - mb) with the row's
-//             offset mb; l += sum p; P (bf16) becomes the A operand of MMA 2 in tensor memory.  (Through shared memory its
-//             port was busy 3072 of 4200 cycles a step, and the clock lower under the power cap.  128 x 4096, d = 64: 839 -> 801 us;
-//             d = 128: 985 -> 941 at a burst, 1106 -> 1056 in a loop.)
-//             d = 64 has room for scores of both units beside P and O.  d = 128 has one buffer of scores: the units are half
-//             a step apart and hold it only from MMA 1 until their scores are in registers, less than half a step.
+//             at once, so the next MMA 1 runs meanwhile); the two tell each other their maximum through shared memory;
+//             p = 2^(c s - mb) with the row's offset mb; l += sum p; P (bf16) becomes the A operand of MMA 2 in tensor memory
 //   MMA 2     O_q += P V_j                        128 x d fp32 in tensor memory; V_j as TMA delivers it
 //             ([128 keys x d], an MN-major B operand)
 // The offset mb of a row follows its running maximum lazily: it moves only when the maximum has grown by more than 8
@@ -21,6 +16,18 @@
 // this is rare, and weights stay below 2^8.  The division by l happens once, in the epilogue.  One exponential and
 // two MMA passes per element.  (An offset that follows one step late, so that no exponential waits for a maximum, took 1.18 ms
 // instead of 1.01 at 128 x 4096, d = 128: 88 bytes of spills, and the maximum is not what the unit waits for.)
+// What bounds it: in a loop of large calls, the power cap; at a burst, the chain of a unit's step and the tensor pipe, whose
+// instructions the operand fetch from shared memory holds up.  So what leaves shared memory counts twice:
+//   * P goes through tensor memory (through shared memory its port was busy 3072 of 4200 cycles a step): 128 x 4096, d = 64
+//     839 -> 801 us; d = 128 985 -> 941 at a burst, 1106 -> 1056 in a loop.  d = 64 has room for the scores of both units beside P
+//     and O.  d = 128 has one buffer of scores: the units are half a step apart and hold it only from MMA 1 until their
+//     scores are in registers, less than half a step.
+//   * The two threads of a row exchange maxima (each read the other's scores too, which held the buffer longer), and the
+//     room of P's tiles makes the ring of K and V a stage longer: d = 128 941 -> 910 and 1057 -> 1027; d = 64 793 -> 768;
+//     12 x 1021, d = 64 13.0 -> 12.1.
+// Slower: the wait for the previous product put off until half of the weights are there (d = 64 780 -> 821 us, d = 128 no change);
+// one thread per row, 8 Softmax warps of 168 registers (d = 64 795 -> 1000: a lone warp of a scheduler gets half of
+// its special function unit).
 // Valid for any N >= 1, d in {64, 128}; Q, K, V, O bf16 [B, H, N, d].
 #pragma once
 #include <cstddef>
@@ -48,14 +55,17 @@ enum : uint32_t {  // wait sites of this kernel (low byte of the status word)
     kSiteOFull = 103,
     kSiteOutFilled = 104,
     kSiteLFull = 105,
+    kSiteMaxFull = 106,
 };
+
+constexpr int kUnitStats = 4 * kTile;
 
 template <int D>
 struct Smem {
     static constexpr int kAtoms = D / 64;
     static constexpr int kAtomBytes = kTile * 128;             // 128 rows x 128 bytes
     static constexpr int kTileBytes = kAtoms * kAtomBytes;     // a Q, K or V tile
-    static constexpr int kStages = (D == 128) ? 3 : 6;         // ring of K / V tiles (128 keys x d)
+    static constexpr int kStages = (D == 128) ? 4 : 6;         // ring of K / V tiles (128 keys x d)
     // Tensor memory: d = 64 has room for scores, O and P (the product's A operand) of both units; d = 128 for P and O of
     // both and ONE buffer of scores, which the units use in turn.
     static constexpr bool kSharedS = D == 128;
@@ -64,9 +74,9 @@ struct Smem {
     static __host__ __device__ constexpr uint32_t o_col(int q) { return kSharedS ? 256u + static_cast<uint32_t>(q * 128) : static_cast<uint32_t>(q * 256 + 128); }
     static constexpr int kQOff = 0;                            // two query tiles; split: one, and one more stage of the ring
     static constexpr int kKOff = kQOff + 2 * kTileBytes;
-    static constexpr int kOutOff = kKOff + kStages * kTileBytes;  // a unit's part of O on its way out
-    static constexpr int kBarOff = kOutOff + 2 * kTileBytes;
-    static constexpr int kBytes = kBarOff + 256;
+    static constexpr int kStatOff = kKOff + kStages * kTileBytes;  // per unit: maxima, float [2 steps][2 halves][128 rows]; at the end sums and offset
+    static constexpr int kBarOff = kStatOff + 2 * kUnitStats * 4;
+    static constexpr int kBytes = kBarOff + 512;
     static constexpr int kDynamicBytes = kBytes + 1024;
 };
 static_assert(Smem<128>::kDynamicBytes <= 227 * 1024, "shared memory budget");
@@ -77,13 +87,14 @@ struct Barriers {
     uint64_t s_full[2], s_free[2];  // per unit: scores written / read into registers (8 warps)
     uint64_t p_full[2], p_free[2];  // per unit: P written (8 warps) / read by its MMAs
     uint64_t o_full[2];             // per unit: every product complete
+    uint64_t max_full[2][4];        // per unit and lane quarter: the maxima of both halves are in shared memory (2 warps)
     uint64_t l_full[2];             // per query tile: the row statistics of its warps are in shared memory
     uint64_t out_filled[2];
     uint32_t tmem_base;
     uint32_t abort_flag;
     uint32_t prior_failure;
 };
-static_assert(sizeof(Barriers) <= 256, "barrier block must fit its slot");
+static_assert(sizeof(Barriers) <= 512, "barrier block must fit its slot");
 
 // The bounded wait of the other kernels, but expanded in place: where a thread holds a row of scores in registers,
 // a call would spill them around it.
@@ -152,6 +163,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             ptx::mbar_init(&bars->p_full[q], 8);
             ptx::mbar_init(&bars->p_free[q], 1);
             ptx::mbar_init(&bars->o_full[q], 1);
+            for (int w = 0; w < 4; ++w) ptx::mbar_init(&bars->max_full[q][w], 2);
             ptx::mbar_init(&bars->l_full[q], split ? 16 : 8);
             ptx::mbar_init(&bars->out_filled[q], split ? 15 : 7);
         }
@@ -326,12 +338,14 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         const float c2 = scale_log2e;
         const uint64_t c2c2 = ptx::pack2(c2, c2);
         const int row = quarter * 32 + lane;
-        const uint32_t t_other = t_quarter + L::s_col(q) + static_cast<uint32_t>((half ^ 1) * kHalf);
+        // The two threads of a row tell each other their maximum through shared memory, even and odd steps in places of their own
+        // (a thread is at most one step ahead of the other).
+        float* const stats = reinterpret_cast<float*>(smem + L::kStatOff) + q * kUnitStats;
+        const uint32_t max_own = ptx::smem_u32(stats + half * kTile + row), max_other = ptx::smem_u32(stats + (half ^ 1) * kTile + row);
         const uint32_t lane0 = lane == 0;
         const uint32_t sw = static_cast<uint32_t>(lane & 7);
         const uint32_t p_own = t_quarter + L::p_col(q) + static_cast<uint32_t>(half * 32);  // its 64 keys of P
-        float smax = -3.0e38f;  // running maximum of the raw scores of this row (all columns: both threads of a row
-                                // compute it, each from the whole tile, so they agree without an exchange)
+        float smax = -3.0e38f;  // running maximum of the raw scores of this row (all columns)
         float mb = -3.0e38f;    // the offset the weights, l and O's row are relative to (follows smax * c2 lazily)
         float l = 0.0f;         // sum of this thread's weights
         bool ok = true;
@@ -341,30 +355,6 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             if (!ok) break;
             ptx::tc_fence_after_sync();
             const int valid = N - key_tile(j, q) * kTile;  // key columns of this tile that exist
-            // ---- maximum of the other thread's 64 columns (read and dropped) ----
-            float mo = -3.0e38f;
-#pragma unroll
-            for (int c = 0; c < kHalf / kChunk; ++c) {
-                uint32_t r[kChunk];
-                ptx::tmem_ld_32x32b_x32(t_other + static_cast<uint32_t>(c * kChunk), r);
-                ptx::tmem_wait_ld();
-                if (valid < kTile) {
-#pragma unroll
-                    for (int i = 0; i < kChunk; ++i)
-                        if ((half ^ 1) * kHalf + c * kChunk + i >= valid) r[i] = __float_as_uint(-3.0e38f);
-                }
-                float m0 = __uint_as_float(r[0]), m1 = __uint_as_float(r[1]), m2 = __uint_as_float(r[2]), m3 = __uint_as_float(r[3]);
-#pragma unroll
-                for (int i = 4; i < kChunk; i += 8) {
-                    m0 = ptx::max3(m0, __uint_as_float(r[i + 0]), __uint_as_float(r[i + 1]));
-                    m1 = ptx::max3(m1, __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
-                    if (i + 4 < kChunk) {
-                        m2 = ptx::max3(m2, __uint_as_float(r[i + 4]), __uint_as_float(r[i + 5]));
-                        m3 = ptx::max3(m3, __uint_as_float(r[i + 6]), __uint_as_float(r[i + 7]));
-                    }
-                }
-                mo = fmaxf(mo, ptx::max3(fmaxf(m0, m1), m2, m3));
-            }
             // ---- this thread's 64 scores into registers; the buffer goes back to the MMA issuer at once ----
             float s[kHalf];
             {
@@ -397,7 +387,14 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                     m3 = ptx::max3(m3, s[i + 6], s[i + 7]);
                 }
             }
-            smax = ptx::max3(smax, mo, ptx::max3(fmaxf(m0, m1), m2, m3));
+            m0 = ptx::max3(fmaxf(m0, m1), m2, m3);
+            const uint32_t place = static_cast<uint32_t>(j & 1) * (2 * kTile * 4);
+            ptx::st_shared_f32(max_own + place, m0);
+            __syncwarp();
+            ptx::mbar_arrive_if(bar_of(offsetof(Barriers, max_full), q * 4 + quarter), lane0);
+            ok = __all_sync(0xffffffffu, wait_in_place(&bars->max_full[q][quarter], static_cast<uint32_t>(j) & 1u, abort_flag, kSiteMaxFull));
+            if (!ok) break;
+            smax = ptx::max3(smax, m0, ptx::ld_shared_f32(max_other + place));
             const float mb_cand = fmaxf(smax * c2, -3.0e38f);
             const bool move = j == 0 || mb_cand - mb > kLazy;
             // P and O are free once the MMAs of the previous key tile are complete
@@ -457,18 +454,18 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             if (lane == 0) ptx::mbar_arrive(&bars->p_full[q]);
         }
 
-        // ---- epilogue: O / l -> bf16 -> shared memory -> TMA stores ----
+        // ---- epilogue: O / l -> bf16 -> the query tile's shared memory -> TMA stores ----
         if (split || steps[q] > 0) {  // (split: each unit has a step)
             // Two units of one query tile each finish alone.  Two units of the same query tile meet here: the four threads of a
             // row take D / 4 columns each of 2^(mb_0 - mb) O_0 + 2^(mb_1 - mb) O_1.
-            const int u = split ? 0 : q;  // the barriers and the output tile this epilogue uses
-            float* lx = reinterpret_cast<float*>(smem + L::kKOff);  // (every MMA is complete: the K / V ring is free)
-            float* ox = lx + 4 * kTile;
+            const int u = split ? 0 : q;  // the barriers and the query tile this epilogue uses
+            const float* peer = reinterpret_cast<const float*>(smem + L::kStatOff) + (q ^ 1) * kUnitStats;
+            const float *l_peer = peer + row, *mb_peer = peer + 2 * kTile + row;  // split: the other unit's sums (of both halves) and offset
             if (ok) ok = warp_wait(bar_of(offsetof(Barriers, o_full), q), 0, abort_flag, kSiteOFull);
-            if (ok && steps[q ^ 1] > 0) ok = warp_wait(bar_of(offsetof(Barriers, o_full), q ^ 1), 0, abort_flag, kSiteOFull);
+            if (ok && split) ok = warp_wait(bar_of(offsetof(Barriers, o_full), q ^ 1), 0, abort_flag, kSiteOFull);
             if (ok) {
-                lx[(q * 2 + half) * kTile + row] = l;
-                if (half == 0) ox[q * kTile + row] = mb;
+                stats[half * kTile + row] = l;  // (the maxima have all been read: the last product has them behind it)
+                if (half == 0) stats[2 * kTile + row] = mb;
                 __syncwarp();
                 ptx::mbar_arrive_if(bar_of(offsetof(Barriers, l_full), u), lane0);
                 ok = warp_wait(bar_of(offsetof(Barriers, l_full), u), 0, abort_flag, kSiteLFull);
@@ -481,12 +478,11 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 float2* pairs = reinterpret_cast<float2*>(smem + L::kKOff + 4096);
                 const uint32_t parts = ptx::smem_u32(smem + L::kKOff + 8192);  // float [G CTAs][128 / G rows][D], 16-byte pieces XOR-swizzled by row
                 const int my_rows = kTile / G;
-                const float l_own = ok ? l + lx[(q * 2 + (half ^ 1)) * kTile + row] : 1.0f;
-                const float mb_other = ok ? ox[(q ^ 1) * kTile + row] : 0.0f;
+                const float l_own = ok ? l + stats[(half ^ 1) * kTile + row] : 1.0f;
+                const float mb_other = ok ? *mb_peer : 0.0f;
                 if (ok && q == 0 && half == 0) {
-                    const float* lo = lx + (q ^ 1) * 2 * kTile + row;
                     const float top = fmaxf(mb, mb_other);
-                    pairs[row] = make_float2(top, l_own * ptx::ex2_approx(mb - top) + (lo[0] + lo[kTile]) * ptx::ex2_approx(mb_other - top));
+                    pairs[row] = make_float2(top, l_own * ptx::ex2_approx(mb - top) + (l_peer[0] + l_peer[kTile]) * ptx::ex2_approx(mb_other - top));
                 }
                 __syncwarp();
                 ptx::cluster_arrive_release();
@@ -551,14 +547,13 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 }
             } else if (ok) {
                 float f_own, f_other = 0.0f;
-                const float l_own = l + lx[(q * 2 + (half ^ 1)) * kTile + row];
+                const float l_own = l + stats[(half ^ 1) * kTile + row];
                 if (split) {
-                    const float mb_other = ox[(q ^ 1) * kTile + row];
+                    const float mb_other = *mb_peer;
                     const float top = fmaxf(mb, mb_other);
                     f_own = ptx::ex2_approx(mb - top);
                     f_other = ptx::ex2_approx(mb_other - top);
-                    const float* lo = lx + (q ^ 1) * 2 * kTile + row;
-                    const float inv = 1.0f / (l_own * f_own + (lo[0] + lo[kTile]) * f_other);
+                    const float inv = 1.0f / (l_own * f_own + (l_peer[0] + l_peer[kTile]) * f_other);
                     f_own *= inv;
                     f_other *= inv;
                 } else {
@@ -569,7 +564,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 const int col0 = split ? (q * 2 + half) * (D / 4) : half * (D / 2);
                 const uint32_t o_unit = t_quarter + L::o_col(q);
                 const uint32_t o_peer = t_quarter + L::o_col(q ^ 1);
-                const uint32_t dst_row = ptx::smem_u32(smem + L::kOutOff + u * L::kTileBytes) + static_cast<uint32_t>(row * 128);
+                const uint32_t dst_row = ptx::smem_u32(smem + L::kQOff + u * L::kTileBytes) + static_cast<uint32_t>(row * 128);
 #pragma unroll 1
                 for (int c = col0; c < col0 + cols; c += 16) {
                     uint32_t o[16];
@@ -601,7 +596,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                     ok = warp_wait(bar_of(offsetof(Barriers, out_filled), u), 0, abort_flag, kSiteOutFilled);
                     if (ok && lane == 0) {
                         for (int a = 0; a < L::kAtoms; ++a)
-                            ptx::tma_store_3d(&tm_o, ptx::smem_u32(smem + L::kOutOff + u * L::kTileBytes + a * L::kAtomBytes), a * 64,
+                            ptx::tma_store_3d(&tm_o, ptx::smem_u32(smem + L::kQOff + u * L::kTileBytes + a * L::kAtomBytes), a * 64,
                                               row0 + u * kTile, bh, ptx::policy_evict_first());
                         ptx::bulk_commit_group();
                         ptx::bulk_wait_group<0>();

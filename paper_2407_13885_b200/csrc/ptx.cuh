@@ -389,6 +389,11 @@ __device__ __forceinline__ void unpack_f16x2(uint32_t v, float& lo, float& hi) {
 __device__ __forceinline__ void st_shared_f32(uint32_t addr, float a) {
     asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(a) : "memory");
 }
+__device__ __forceinline__ float ld_shared_f32(uint32_t addr) {
+    float a;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(a) : "r"(addr) : "memory");
+    return a;
+}
 __device__ __forceinline__ void st_shared_v2(uint32_t addr, float a, float b) {
     asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
 }

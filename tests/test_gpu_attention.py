@@ -181,3 +181,16 @@ def test_attention_split_and_whole(attnw, B, H, N, d):
     ref = oracle.attn(q, k, v, scale)
     got = run_attn(attnw, q, k, v, scale).double().cpu().numpy().reshape(ref.shape)
     assert np.all(np.abs(got - ref) <= tolerance_map(q, k, v, scale, ref))
+
+
+# Two query tiles per CTA (calls with many of them) over 9 and 8 key tiles: the units take turns at one buffer of scores (d = 128) or
+# have one each (d = 64); an odd number of query tiles, so that the last CTA of a head has one unit, and ragged last tiles
+@pytest.mark.parametrize("B,H,N,d", [(1, 40, 1100, 128), (1, 64, 900, 64), (1, 40, 1152, 128)])
+def test_attention_of_many_query_tiles(attnw, B, H, N, d):
+    q, k = small_fused_inputs(B, H, N, d, sigma=2.0, stream=N + d + 31)
+    v = rand_v(B, H, N, d, stream=N + d + 33)
+    scale = float(np.float32(1.0 / math.sqrt(d)))
+    ref = oracle.attn(q, k, v, scale)
+    for _ in range(2):
+        got = run_attn(attnw, q, k, v, scale).double().cpu().numpy().reshape(ref.shape)
+        assert np.all(np.abs(got - ref) <= tolerance_map(q, k, v, scale, ref))
