@@ -40,7 +40,7 @@ namespace av1 {
 constexpr int kSmWarps = 16;      // Softmax warps: unit (2) x column half (2) x TMEM lane quarter (4)
 constexpr int kProducer = 16;
 constexpr int kMma = 17;
-constexpr int kThreads = 576;
+constexpr int kMmaProduct = 18;   // kTwoIssuers: the products' issuer
 constexpr int kMaxCluster = 4;    // CTAs that share a query tile (of 8, 15 clusters fit, and a call that needs them has 16 tiles)
 constexpr float kLazy = 8.0f;     // the offset follows the maximum only when it has grown by more than this
 
@@ -69,6 +69,12 @@ struct Smem {
     // Tensor memory: d = 64 has room for scores, O and P (the product's A operand) of both units; d = 128 for P and O of
     // both and ONE buffer of scores, which the units use in turn.
     static constexpr bool kSharedS = D == 128;
+    // A second warp issues the products: an issuer spends 200 to 550 cycles on the waits in front of each set of MMAs, 1360 of a
+    // step's 3450 at d = 128, and nothing of the other kind was queued meanwhile.  128 x 4096 902 -> 856 us at a burst, 1012 -> 950
+    // in a loop; 12 x 2048 34.8 -> 32.4.  At d = 64 the MMAs take half as long and the exponentials set the pace: 780 us with
+    // one issuer, 811 with two (796 where the scores still keep the order).
+    static constexpr bool kTwoIssuers = D == 128;
+    static constexpr int kThreads = kTwoIssuers ? 608 : 576;
     static __host__ __device__ constexpr uint32_t s_col(int q) { return kSharedS ? 0u : static_cast<uint32_t>(q * 256); }
     static __host__ __device__ constexpr uint32_t p_col(int q) { return kSharedS ? 128u + static_cast<uint32_t>(q * 64) : static_cast<uint32_t>(q * 256 + 192); }
     static __host__ __device__ constexpr uint32_t o_col(int q) { return kSharedS ? 256u + static_cast<uint32_t>(q * 128) : static_cast<uint32_t>(q * 256 + 128); }
@@ -118,7 +124,7 @@ __device__ __forceinline__ bool wait_in_place(uint64_t* bar, uint32_t parity, vo
 enum Mode { kWhole, kSplit, kCluster };
 
 template <int D, Mode M>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(Smem<D>::kThreads, 1)
 attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o, int N,
                     int row_blocks_per_head, float scale_log2e, __nv_bfloat16* O, int cluster_ctas) {
@@ -232,8 +238,8 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             }
         }
         __syncwarp();
-    } else if (run && warp == kMma) {
-        // ================= MMA issuer (warp-uniform loop, one elected lane issues) =================
+    } else if (run && (warp == kMma || (L::kTwoIssuers && warp == kMmaProduct))) {
+        // ================= MMA issuers (warp-uniform loops, one elected lane issues): of scores, of products, or of both =================
         constexpr uint32_t idesc_s = ptx::umma_idesc_bf16_f32(kTile, kTile);
         constexpr uint32_t idesc_o = ptx::umma_idesc_bf16_f32(kTile, D) | (1u << 16);  // B operand MN-major
         const uint32_t base = ptx::smem_u32(smem);
@@ -287,43 +293,71 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             __syncwarp();
         };
         // The scores of step j + 1 first: the tensor pipe computes them while the row threads exponentiate step j.  The two
-        // units alternate - scores of one, product of one, scores of the other, product of the other - which keeps their
+        // units alternate (with two issuers, because the scores take turns at their buffer) - scores of one, product of one, scores of the other, product of the other - which keeps their
         // row threads half a step apart (d = 64, 128 x 4096: 888 -> 841 us against both scores first).
-        for (int j = -1; ok && j < steps[0]; ++j) {
-            if (split) {
-                for (int q = 0; q < 2; ++q) {
-                    if (ok && j + 1 < steps[q]) {
-                        arrived();
-                        scores(q, j + 1);
-                        release();
+        if constexpr (L::kTwoIssuers) {
+            const bool for_scores = warp == kMma;
+            for (int j = -1; ok && j < steps[0]; ++j) {
+                for (int q = 0; ok && q < (split ? 2 : 1); ++q) {
+                    if (j + 1 < steps[q]) {  // K of step j + 1
+                        if (for_scores) {
+                            arrived();
+                            scores(q, j + 1);
+                            if (!split && steps[1] > 0) scores(1, j + 1);
+                            release();
+                        } else {
+                            ++n;
+                        }
                     }
-                    if (ok && j >= 0 && j < steps[q]) {
-                        arrived();
-                        product(q, j);
-                        release();
+                    if (j >= 0 && j < steps[q]) {  // V of step j
+                        if (!for_scores) {
+                            arrived();
+                            product(q, j);
+                            if (!split && steps[1] > 0) product(1, j);
+                            release();
+                        } else {
+                            ++n;
+                        }
                     }
                 }
-            } else {
-                const bool next = j + 1 < T;
-                const int k_entry = n, v_entry = next ? n + 1 : n;  // K of step j + 1, V of step j
-                if (next) {
-                    arrived();
-                    scores(0, j + 1);
-                }
-                n = v_entry;
-                if (ok && j >= 0) {
-                    arrived();
-                    product(0, j);
-                }
-                if (ok && next) {
-                    n = k_entry;
-                    if (steps[1] > 0) scores(1, j + 1);
-                    release();
-                }
-                if (ok && j >= 0) {
+            }
+        } else {
+            for (int j = -1; ok && j < steps[0]; ++j) {
+                if (split) {
+                    for (int q = 0; q < 2; ++q) {
+                        if (ok && j + 1 < steps[q]) {
+                            arrived();
+                            scores(q, j + 1);
+                            release();
+                        }
+                        if (ok && j >= 0 && j < steps[q]) {
+                            arrived();
+                            product(q, j);
+                            release();
+                        }
+                    }
+                } else {
+                    const bool next = j + 1 < T;
+                    const int k_entry = n, v_entry = next ? n + 1 : n;  // K of step j + 1, V of step j
+                    if (next) {
+                        arrived();
+                        scores(0, j + 1);
+                    }
                     n = v_entry;
-                    if (steps[1] > 0) product(1, j);
-                    release();
+                    if (ok && j >= 0) {
+                        arrived();
+                        product(0, j);
+                    }
+                    if (ok && next) {
+                        n = k_entry;
+                        if (steps[1] > 0) scores(1, j + 1);
+                        release();
+                    }
+                    if (ok && j >= 0) {
+                        n = v_entry;
+                        if (steps[1] > 0) product(1, j);
+                        release();
+                    }
                 }
             }
         }
