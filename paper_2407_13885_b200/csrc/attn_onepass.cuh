@@ -16,8 +16,9 @@
 // this is rare, and weights stay below 2^8.  The division by l happens once, in the epilogue.  One exponential and
 // two MMA passes per element.  (An offset that follows one step late, so that no exponential waits for a maximum, took 1.18 ms
 // instead of 1.01 at 128 x 4096, d = 128: 88 bytes of spills, and the maximum is not what the unit waits for.)
-// What bounds it: in a loop of large calls, the power cap; at a burst, the chain of a unit's step and the tensor pipe, whose
-// instructions the operand fetch from shared memory holds up.  So what leaves shared memory counts twice:
+// What bounds it: in a loop of large calls, the power cap; at a burst, the chain of the Softmax warps' step (d = 128: 3100 cycles
+// of which the special function units and the tensor pipe need 2048 each).  Operand fetch from shared memory holds up
+// the tensor pipe, and the issuers' waits keep it idle (kTwoIssuers), so:
 //   * P goes through tensor memory (through shared memory its port was busy 3072 of 4200 cycles a step): 128 x 4096, d = 64
 //     839 -> 801 us; d = 128 985 -> 941 at a burst, 1106 -> 1056 in a loop.  d = 64 has room for the scores of both units beside P
 //     and O.  d = 128 has one buffer of scores: the units are half a step apart and hold it only from MMA 1 until their
@@ -27,7 +28,9 @@
 //     12 x 1021, d = 64 13.0 -> 12.1.
 // Slower: the wait for the previous product put off until half of the weights are there (d = 64 780 -> 821 us, d = 128 no change);
 // one thread per row, 8 Softmax warps of 168 registers (d = 64 795 -> 1000: a lone warp of a scheduler gets half of
-// its special function unit).
+// its special function unit); products before scores (780 -> 978); 1/8 or 1/4 of the exponentials by a polynomial of degree 5 on
+// the FMA pipes (d = 64 778 -> 776, 790; d = 128 965 -> 984, 1002 in a loop); CTAs that stay for several row blocks and store
+// O from registers (d = 128 905 -> 896 at a burst, d = 64 800 -> 843).
 // Valid for any N >= 1, d in {64, 128}; Q, K, V, O bf16 [B, H, N, d].
 #pragma once
 #include <cstddef>
