@@ -429,14 +429,21 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             ptx::st_shared_f32(max_own + place, m0);
             __syncwarp();
             ptx::mbar_arrive_if(bar_of(offsetof(Barriers, max_full), q * 4 + quarter), lane0);
+            // P and O are free once the MMAs of the previous key tile are complete.  At d = 64 they are by now, as a rule, and the wait runs
+            // beside the other half's (128 x 4096 780 -> 763 us); at d = 128 they take longer than the maxima (976 -> 1022).
+            if constexpr (D == 64) {
+                ok = __all_sync(0xffffffffu, wait_in_place(&bars->p_free[q], (static_cast<uint32_t>(j) & 1u) ^ 1u, abort_flag, kSitePFree));
+                if (!ok) break;
+            }
             ok = __all_sync(0xffffffffu, wait_in_place(&bars->max_full[q][quarter], static_cast<uint32_t>(j) & 1u, abort_flag, kSiteMaxFull));
             if (!ok) break;
             smax = ptx::max3(smax, m0, ptx::ld_shared_f32(max_other + place));
             const float mb_cand = fmaxf(smax * c2, -3.0e38f);
             const bool move = j == 0 || mb_cand - mb > kLazy;
-            // P and O are free once the MMAs of the previous key tile are complete
-            ok = __all_sync(0xffffffffu, wait_in_place(&bars->p_free[q], (static_cast<uint32_t>(j) & 1u) ^ 1u, abort_flag, kSitePFree));
-            if (!ok) break;
+            if constexpr (D != 64) {
+                ok = __all_sync(0xffffffffu, wait_in_place(&bars->p_free[q], (static_cast<uint32_t>(j) & 1u) ^ 1u, abort_flag, kSitePFree));
+                if (!ok) break;
+            }
             ptx::tc_fence_after_sync();
             uint32_t w[16];  // 32 keys of P on their way to tensor memory
             if (j == 0) {
