@@ -20,6 +20,9 @@ namespace {
 
 PyObject* g_error = nullptr;  // binding.AttnwError, handed over once by binding.py
 
+// A tensor without storage (torch.func's wrappers) throws when it is asked for its address, so every entry point asks while it
+// holds the interpreter's lock: HANDLE_TH_ERRORS needs the lock to turn the exception into a Python one.
+
 // A CUDA tensor of the wanted type, contiguous; nullptr with a Python exception set otherwise.
 const at::Tensor* tensor_arg(PyObject* obj, const char* name, at::ScalarType type, const char* type_name) {
     if (!THPVariable_Check(obj) || !THPVariable_Unpack(obj).is_cuda()) {
@@ -121,6 +124,7 @@ PyObject* py_attnw_fused(PyObject*, PyObject* const* a, Py_ssize_t n) {
     bool f32 = false;
     float scale;
     if ((a[3] == Py_None && !is_float32(a[4], &f32)) || !float_arg(a[2], &scale)) return nullptr;
+    const void *q_ptr = q->data_ptr(), *k_ptr = k->data_ptr();
     const c10::cuda::CUDAGuard guard(q->device());
     at::Tensor p;
     if (!output_arg(a[3], "P", {B, H, N, N}, f32 ? at::kFloat : at::kBFloat16, true, false,
@@ -128,11 +132,11 @@ PyObject* py_attnw_fused(PyObject*, PyObject* const* a, Py_ssize_t n) {
         return nullptr;
     void* stream;
     if (!stream_arg(a[5], &stream)) return nullptr;
+    const auto entry = p.scalar_type() == at::kBFloat16 ? attnw_fused : attnw_fused_f32;
+    void* p_ptr = p.data_ptr();
     int rc;
     Py_BEGIN_ALLOW_THREADS
-    rc = (p.scalar_type() == at::kBFloat16 ? attnw_fused : attnw_fused_f32)(q->data_ptr(), k->data_ptr(), p.data_ptr(),
-                                                                            static_cast<int>(B), static_cast<int>(H),
-                                                                            static_cast<int>(N), static_cast<int>(d), scale, stream);
+    rc = entry(q_ptr, k_ptr, p_ptr, static_cast<int>(B), static_cast<int>(H), static_cast<int>(N), static_cast<int>(d), scale, stream);
     Py_END_ALLOW_THREADS
     if (rc != ATTNW_OK) return failed(rc, "attnw_fused");
     if (a[3] != Py_None) return Py_NewRef(a[3]);
@@ -152,15 +156,17 @@ PyObject* py_attn_fused(PyObject*, PyObject* const* a, Py_ssize_t n) {
     }
     float scale;
     if (!float_arg(a[3], &scale)) return nullptr;
+    const void *q_ptr = q->data_ptr(), *k_ptr = k->data_ptr(), *v_ptr = v->data_ptr();
+    const int B = static_cast<int>(q->size(0)), H = static_cast<int>(q->size(1)), N = static_cast<int>(q->size(2)), d = static_cast<int>(q->size(3));
     const c10::cuda::CUDAGuard guard(q->device());
     at::Tensor o;
     if (!output_arg(a[4], "O", q->sizes(), at::kBFloat16, false, true, "[B, H, N, d]", *q, &o)) return nullptr;
     void* stream;
     if (!stream_arg(a[5], &stream)) return nullptr;
+    void* o_ptr = o.data_ptr();
     int rc;
     Py_BEGIN_ALLOW_THREADS
-    rc = attn_fused(q->data_ptr(), k->data_ptr(), v->data_ptr(), o.data_ptr(), static_cast<int>(q->size(0)),
-                    static_cast<int>(q->size(1)), static_cast<int>(q->size(2)), static_cast<int>(q->size(3)), scale, stream);
+    rc = attn_fused(q_ptr, k_ptr, v_ptr, o_ptr, B, H, N, d, scale, stream);
     Py_END_ALLOW_THREADS
     if (rc != ATTNW_OK) return failed(rc, "attn_fused");
     if (a[4] != Py_None) return Py_NewRef(a[4]);
@@ -179,6 +185,7 @@ PyObject* py_project_qk(PyObject*, PyObject* const* a, Py_ssize_t n) {
         return nullptr;
     }
     const int64_t B = x->size(0), N = x->size(1), d_model = x->size(2), H = wq->size(0), d = wq->size(1);
+    const void *x_ptr = x->data_ptr(), *wq_ptr = wq->data_ptr(), *wk_ptr = wk->data_ptr();
     const c10::cuda::CUDAGuard guard(x->device());
     at::Tensor q, k;
     if (!output_arg(a[3], "Q", {B, H, N, d}, at::kBFloat16, false, true, "[B, H, N, d]", *x, &q) ||
@@ -186,10 +193,11 @@ PyObject* py_project_qk(PyObject*, PyObject* const* a, Py_ssize_t n) {
         return nullptr;
     void* stream;
     if (!stream_arg(a[5], &stream)) return nullptr;
+    void *q_ptr = q.data_ptr(), *k_ptr = k.data_ptr();
     int rc;
     Py_BEGIN_ALLOW_THREADS
-    rc = attnw_project_qk(x->data_ptr(), wq->data_ptr(), wk->data_ptr(), q.data_ptr(), k.data_ptr(), static_cast<int>(B),
-                          static_cast<int>(N), static_cast<int>(d_model), static_cast<int>(H), static_cast<int>(d), stream);
+    rc = attnw_project_qk(x_ptr, wq_ptr, wk_ptr, q_ptr, k_ptr, static_cast<int>(B), static_cast<int>(N), static_cast<int>(d_model),
+                          static_cast<int>(H), static_cast<int>(d), stream);
     Py_END_ALLOW_THREADS
     if (rc != ATTNW_OK) return failed(rc, "attnw_project_qk");
     PyObject* pq = a[3] != Py_None ? Py_NewRef(a[3]) : THPVariable_Wrap(std::move(q));
@@ -213,6 +221,8 @@ PyObject* py_softmax_rows(PyObject*, PyObject* const* a, Py_ssize_t n) {
     }
     bool f32 = false;
     if (a[1] == Py_None && !is_float32(a[2], &f32)) return nullptr;
+    const long long rows = s->size(0), cols = s->size(1);
+    const void* s_ptr = s->data_ptr();
     const c10::cuda::CUDAGuard guard(s->device());
     at::Tensor p;
     if (!output_arg(a[1], "P", s->sizes(), f32 ? at::kFloat : at::kBFloat16, true, false,
@@ -220,10 +230,11 @@ PyObject* py_softmax_rows(PyObject*, PyObject* const* a, Py_ssize_t n) {
         return nullptr;
     void* stream;
     if (!stream_arg(a[3], &stream)) return nullptr;
+    const auto entry = p.scalar_type() == at::kBFloat16 ? softmax_rows : softmax_rows_f32;
+    void* p_ptr = p.data_ptr();
     int rc;
     Py_BEGIN_ALLOW_THREADS
-    rc = (p.scalar_type() == at::kBFloat16 ? softmax_rows : softmax_rows_f32)(s->data_ptr(), p.data_ptr(), s->size(0), s->size(1),
-                                                                              stream);
+    rc = entry(s_ptr, p_ptr, rows, cols, stream);
     Py_END_ALLOW_THREADS
     if (rc != ATTNW_OK) return failed(rc, "softmax_rows");
     if (a[1] != Py_None) return Py_NewRef(a[1]);

@@ -58,3 +58,25 @@ def test_given_output_and_stream(binding, dtype):
         assert binding.attnw_fused(Q, K, np.float32(0.125), P=P, stream=stream) is P
         s.synchronize()
         assert_close_to_oracle(P, oracle.attnw(q, k, 0.125), f"{dtype}")
+
+
+def test_tensors_without_storage_are_refused(binding):
+    # torch.func.vmap hands over wrappers that have no address: the calls raise, also where there is no GPU (fake tensors)
+    from torch._subclasses.fake_tensor import FakeTensorMode
+    with FakeTensorMode():
+        q = torch.empty(2, 1, 1, 64, 64, dtype=torch.bfloat16, device="cuda")
+        for call, x in ((lambda x: binding.attnw_fused(x, x, 0.125), q), (lambda x: binding.attn_fused(x, x, x, 0.125), q),
+                        (lambda x: binding.project_qk(x, x, x), q[0]), (binding.softmax_rows, q[0, 0].float())):
+            with pytest.raises(RuntimeError, match="storage"):
+                torch.func.vmap(call)(x)
+
+
+@pytest.mark.gpu
+def test_vmap_is_refused(binding):
+    q = torch.zeros(2, 1, 1, 64, 64, dtype=torch.bfloat16, device="cuda")
+    p = torch.zeros(1, 1, 64, 64, dtype=torch.bfloat16, device="cuda")
+    for call, x in ((lambda x: binding.attnw_fused(x, x, 0.125), q), (lambda x: binding.attnw_fused(p, p, 0.125, P=x), q),
+                    (lambda x: binding.attn_fused(x, x, x, 0.125), q), (lambda x: binding.attn_fused(p, p, p, 0.125, O=x), q),
+                    (lambda x: binding.project_qk(x, x, x), q[0]), (binding.softmax_rows, q[0, 0].float())):
+        with pytest.raises(RuntimeError, match="storage"):
+            torch.func.vmap(call)(x)
