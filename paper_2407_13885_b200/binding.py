@@ -129,13 +129,15 @@ def _check(code: int, where: str) -> None:
         raise AttnwError(code, where)
 
 
-def _require_cuda(t: torch.Tensor, name: str, dtype) -> None:
+def _require_cuda(t: torch.Tensor, name: str, dtype, like: torch.Tensor | None = None) -> None:
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
         raise TypeError(f"{name} must have dtype {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
+    if like is not None and t.device != like.device:
+        raise ValueError(f"{name} must be on {like.device} like the other tensors, got {t.device}")
 
 
 def attnw_fused(Q: torch.Tensor, K: torch.Tensor, scale: float, P: torch.Tensor | None = None,
@@ -223,14 +225,14 @@ def attnw_fused_noalloc(Q: torch.Tensor, K: torch.Tensor, scale: float, P: torch
     that may not call cudaMalloc (a memory pool owns the device, or the call sits in a latency-critical loop).  The
     output tensor is still the caller's (or allocated here by torch, outside the library)."""
     _require_cuda(Q, "Q", torch.bfloat16)
-    _require_cuda(K, "K", torch.bfloat16)
+    _require_cuda(K, "K", torch.bfloat16, Q)
     if Q.dim() != 4 or Q.shape != K.shape:
         raise ValueError("Q and K must both be [B, H, N, d]")
     B, H, N, d = Q.shape
     if P is None:
         P = torch.empty((B, H, N, N), dtype=torch.bfloat16, device=Q.device)
     else:
-        _require_cuda(P, "P", torch.bfloat16)
+        _require_cuda(P, "P", torch.bfloat16, Q)
         if tuple(P.shape) != (B, H, N, N):
             raise ValueError("P must be [B, H, N, N] in bfloat16")
     with torch.cuda.device(Q.device):

@@ -23,8 +23,9 @@ PyObject* g_error = nullptr;  // binding.AttnwError, handed over once by binding
 // A tensor without storage (torch.func's wrappers) throws when it is asked for its address, so every entry point asks while it
 // holds the interpreter's lock: HANDLE_TH_ERRORS needs the lock to turn the exception into a Python one.
 
-// A CUDA tensor of the wanted type, contiguous; nullptr with a Python exception set otherwise.
-const at::Tensor* tensor_arg(PyObject* obj, const char* name, at::ScalarType type, const char* type_name) {
+// A CUDA tensor of the wanted type, contiguous and on the device of the call's first tensor (`like`; nullptr for that one itself, and
+// its kernel would read another GPU's memory); nullptr with a Python exception set otherwise.
+const at::Tensor* tensor_arg(PyObject* obj, const char* name, at::ScalarType type, const char* type_name, const at::Tensor* like) {
     if (!THPVariable_Check(obj) || !THPVariable_Unpack(obj).is_cuda()) {
         PyErr_Format(PyExc_TypeError, "%s must be a CUDA tensor", name);
         return nullptr;
@@ -38,11 +39,16 @@ const at::Tensor* tensor_arg(PyObject* obj, const char* name, at::ScalarType typ
         PyErr_Format(PyExc_ValueError, "%s must be contiguous", name);
         return nullptr;
     }
+    if (like && t.device() != like->device()) {
+        PyErr_Format(PyExc_ValueError, "%s must be on %s like the other tensors, got %s", name, like->device().str().c_str(),
+                     t.device().str().c_str());
+        return nullptr;
+    }
     return &t;
 }
 
-const at::Tensor* bf16_arg(PyObject* obj, const char* name) {
-    return tensor_arg(obj, name, at::kBFloat16, "torch.bfloat16");
+const at::Tensor* bf16_arg(PyObject* obj, const char* name, const at::Tensor* like) {
+    return tensor_arg(obj, name, at::kBFloat16, "torch.bfloat16", like);
 }
 
 // The result: the caller's tensor `obj` (bfloat16, or also float32 where `f32_allowed`), or a new one where it is None.
@@ -54,7 +60,7 @@ bool output_arg(PyObject* obj, const char* name, at::IntArrayRef shape, at::Scal
     }
     const bool f32 = f32_allowed && THPVariable_Check(obj) && THPVariable_Unpack(obj).scalar_type() == at::kFloat;
     if (exact_type || f32 || (THPVariable_Check(obj) && THPVariable_Unpack(obj).scalar_type() == at::kBFloat16)) {
-        const at::Tensor* t = tensor_arg(obj, name, f32 ? at::kFloat : at::kBFloat16, f32 ? "torch.float32" : "torch.bfloat16");
+        const at::Tensor* t = tensor_arg(obj, name, f32 ? at::kFloat : at::kBFloat16, f32 ? "torch.float32" : "torch.bfloat16", &like);
         if (!t) return false;
         if (t->sizes() == shape) {
             *out = *t;
@@ -115,7 +121,7 @@ PyObject* py_attnw_fused(PyObject*, PyObject* const* a, Py_ssize_t n) {
     HANDLE_TH_ERRORS
     if (!count_is(n, 6)) return nullptr;
     const at::Tensor *q, *k;
-    if (!(q = bf16_arg(a[0], "Q")) || !(k = bf16_arg(a[1], "K"))) return nullptr;
+    if (!(q = bf16_arg(a[0], "Q", nullptr)) || !(k = bf16_arg(a[1], "K", q))) return nullptr;
     if (q->dim() != 4 || q->sizes() != k->sizes()) {
         PyErr_SetString(PyExc_ValueError, "Q and K must both be [B, H, N, d]");
         return nullptr;
@@ -125,11 +131,11 @@ PyObject* py_attnw_fused(PyObject*, PyObject* const* a, Py_ssize_t n) {
     float scale;
     if ((a[3] == Py_None && !is_float32(a[4], &f32)) || !float_arg(a[2], &scale)) return nullptr;
     const void *q_ptr = q->data_ptr(), *k_ptr = k->data_ptr();
-    const c10::cuda::CUDAGuard guard(q->device());
     at::Tensor p;
     if (!output_arg(a[3], "P", {B, H, N, N}, f32 ? at::kFloat : at::kBFloat16, true, false,
                     "[B, H, N, N] in bfloat16 or float32", *q, &p))
         return nullptr;
+    const c10::cuda::CUDAGuard guard(q->device());
     void* stream;
     if (!stream_arg(a[5], &stream)) return nullptr;
     const auto entry = p.scalar_type() == at::kBFloat16 ? attnw_fused : attnw_fused_f32;
@@ -149,7 +155,7 @@ PyObject* py_attn_fused(PyObject*, PyObject* const* a, Py_ssize_t n) {
     HANDLE_TH_ERRORS
     if (!count_is(n, 6)) return nullptr;
     const at::Tensor *q, *k, *v;
-    if (!(q = bf16_arg(a[0], "Q")) || !(k = bf16_arg(a[1], "K")) || !(v = bf16_arg(a[2], "V"))) return nullptr;
+    if (!(q = bf16_arg(a[0], "Q", nullptr)) || !(k = bf16_arg(a[1], "K", q)) || !(v = bf16_arg(a[2], "V", q))) return nullptr;
     if (q->dim() != 4 || q->sizes() != k->sizes() || q->sizes() != v->sizes()) {
         PyErr_SetString(PyExc_ValueError, "Q, K and V must all be [B, H, N, d]");
         return nullptr;
@@ -158,9 +164,9 @@ PyObject* py_attn_fused(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!float_arg(a[3], &scale)) return nullptr;
     const void *q_ptr = q->data_ptr(), *k_ptr = k->data_ptr(), *v_ptr = v->data_ptr();
     const int B = static_cast<int>(q->size(0)), H = static_cast<int>(q->size(1)), N = static_cast<int>(q->size(2)), d = static_cast<int>(q->size(3));
-    const c10::cuda::CUDAGuard guard(q->device());
     at::Tensor o;
     if (!output_arg(a[4], "O", q->sizes(), at::kBFloat16, false, true, "[B, H, N, d]", *q, &o)) return nullptr;
+    const c10::cuda::CUDAGuard guard(q->device());
     void* stream;
     if (!stream_arg(a[5], &stream)) return nullptr;
     void* o_ptr = o.data_ptr();
@@ -179,18 +185,18 @@ PyObject* py_project_qk(PyObject*, PyObject* const* a, Py_ssize_t n) {
     HANDLE_TH_ERRORS
     if (!count_is(n, 6)) return nullptr;
     const at::Tensor *x, *wq, *wk;
-    if (!(x = bf16_arg(a[0], "X")) || !(wq = bf16_arg(a[1], "Wq")) || !(wk = bf16_arg(a[2], "Wk"))) return nullptr;
+    if (!(x = bf16_arg(a[0], "X", nullptr)) || !(wq = bf16_arg(a[1], "Wq", x)) || !(wk = bf16_arg(a[2], "Wk", x))) return nullptr;
     if (x->dim() != 3 || wq->dim() != 3 || wq->sizes() != wk->sizes() || wq->size(2) != x->size(2)) {
         PyErr_SetString(PyExc_ValueError, "X must be [B, N, d_model] and Wq, Wk [H, d, d_model]");
         return nullptr;
     }
     const int64_t B = x->size(0), N = x->size(1), d_model = x->size(2), H = wq->size(0), d = wq->size(1);
     const void *x_ptr = x->data_ptr(), *wq_ptr = wq->data_ptr(), *wk_ptr = wk->data_ptr();
-    const c10::cuda::CUDAGuard guard(x->device());
     at::Tensor q, k;
     if (!output_arg(a[3], "Q", {B, H, N, d}, at::kBFloat16, false, true, "[B, H, N, d]", *x, &q) ||
         !output_arg(a[4], "K", {B, H, N, d}, at::kBFloat16, false, true, "[B, H, N, d]", *x, &k))
         return nullptr;
+    const c10::cuda::CUDAGuard guard(x->device());
     void* stream;
     if (!stream_arg(a[5], &stream)) return nullptr;
     void *q_ptr = q.data_ptr(), *k_ptr = k.data_ptr();
@@ -213,7 +219,7 @@ PyObject* py_project_qk(PyObject*, PyObject* const* a, Py_ssize_t n) {
 PyObject* py_softmax_rows(PyObject*, PyObject* const* a, Py_ssize_t n) {
     HANDLE_TH_ERRORS
     if (!count_is(n, 4)) return nullptr;
-    const at::Tensor* s = tensor_arg(a[0], "S", at::kFloat, "torch.float32");
+    const at::Tensor* s = tensor_arg(a[0], "S", at::kFloat, "torch.float32", nullptr);
     if (!s) return nullptr;
     if (s->dim() != 2) {
         PyErr_SetString(PyExc_ValueError, "S must be [rows, cols]");
@@ -223,11 +229,11 @@ PyObject* py_softmax_rows(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (a[1] == Py_None && !is_float32(a[2], &f32)) return nullptr;
     const long long rows = s->size(0), cols = s->size(1);
     const void* s_ptr = s->data_ptr();
-    const c10::cuda::CUDAGuard guard(s->device());
     at::Tensor p;
     if (!output_arg(a[1], "P", s->sizes(), f32 ? at::kFloat : at::kBFloat16, true, false,
                     "[rows, cols] in bfloat16 or float32", *s, &p))
         return nullptr;
+    const c10::cuda::CUDAGuard guard(s->device());
     void* stream;
     if (!stream_arg(a[3], &stream)) return nullptr;
     const auto entry = p.scalar_type() == at::kBFloat16 ? softmax_rows : softmax_rows_f32;

@@ -80,3 +80,20 @@ def test_vmap_is_refused(binding):
                     (lambda x: binding.project_qk(x, x, x), q[0]), (binding.softmax_rows, q[0, 0].float())):
         with pytest.raises(RuntimeError, match="storage"):
             torch.func.vmap(call)(x)
+
+
+def test_tensors_of_several_devices_are_refused(binding):
+    # (fake tensors: the check comes before anything asks for an address, and needs neither one GPU nor two)
+    from torch._subclasses.fake_tensor import FakeTensorMode
+    with FakeTensorMode():
+        q, far = (torch.empty(1, 1, 64, 64, dtype=torch.bfloat16, device=f"cuda:{n}") for n in range(2))
+        s, far_s = q[0, 0].float(), far[0, 0].float()
+        for call in (lambda: binding.attnw_fused(q, far, 0.125), lambda: binding.attnw_fused(q, q, 0.125, P=far),
+                     lambda: binding.attn_fused(q, far, q, 0.125), lambda: binding.attn_fused(q, q, far, 0.125),
+                     lambda: binding.attn_fused(q, q, q, 0.125, O=far), lambda: binding.project_qk(q[0], far[0], q[0]),
+                     lambda: binding.project_qk(q[0], q[0], far[0]), lambda: binding.project_qk(q[0], q[0], q[0], Q=far),
+                     lambda: binding.project_qk(q[0], q[0], q[0], Q=q, K=far), lambda: binding.softmax_rows(s, P=far_s),
+                     lambda: binding.softmax_rows(s, P=far[0, 0]), lambda: binding.attnw_fused_noalloc(q, far, 0.125),
+                     lambda: binding.attnw_fused_noalloc(q, q, 0.125, P=far)):
+            with pytest.raises(ValueError, match="must be on cuda:0"):
+                call()
