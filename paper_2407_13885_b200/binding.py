@@ -69,7 +69,11 @@ class AttnwError(RuntimeError):
 def _load_native():
     if not os.path.exists(_build.EXT_PATH):
         raise ImportError(f"{_build.EXT_PATH} is missing: build it with `python -m paper_2407_13885_b200.build`.")
-    from . import _attnw_torch
+    try:
+        from . import _attnw_torch
+    except ImportError as e:
+        raise ImportError(f"{_build.EXT_PATH} does not load (it was built for another torch or Python, or against another "
+                          "libattnw.so): build it again with `python -m paper_2407_13885_b200.build`.") from e
     _attnw_torch.set_error(AttnwError)
     return _attnw_torch
 

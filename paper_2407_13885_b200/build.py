@@ -35,6 +35,12 @@ def nvcc_command(out: str, verbose_ptxas: bool = False, defines: tuple[str, ...]
     return cmd
 
 
+def built_for() -> str:
+    """What ``_attnw_torch`` is bound to: the C++ interface of one torch and the C interface of one Python.  The module carries it."""
+    import torch
+    return f"attnw for torch {torch.__version__}, {sysconfig.get_config_var('SOABI')}"
+
+
 def ext_command(out: str) -> list[str]:
     import torch
     from torch.utils import cpp_extension
@@ -42,7 +48,8 @@ def ext_command(out: str) -> list[str]:
     cuda_home = os.path.dirname(os.path.dirname(nvcc_path()))
     includes = [sysconfig.get_paths()["include"], *cpp_extension.include_paths(), os.path.join(cuda_home, "include")]
     return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
-            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *["-isystem" + i for i in includes],
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DATTNW_BUILT_FOR="{built_for()}"',
+            *["-isystem" + i for i in includes],
             "-o", out, EXT_SOURCE, "-L" + _PKG, "-l:" + os.path.basename(LIB_PATH), "-L" + torch_lib, "-ltorch_python",
             "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN"]
 
@@ -55,6 +62,13 @@ def is_stale() -> bool:
     return _older(LIB_PATH, _DEPS)
 
 
+def ext_is_stale() -> bool:
+    if _older(EXT_PATH, [EXT_SOURCE, os.path.join(os.path.dirname(_PKG), "include", "attnw.h")]):
+        return True
+    with open(EXT_PATH, "rb") as f:
+        return built_for().encode() + b"\0" not in f.read()
+
+
 def _compile(cmd: list[str], tmp: str, target: str) -> str:
     proc = subprocess.run(cmd, capture_output=True, text=True)
     if proc.returncode != 0:
@@ -64,8 +78,9 @@ def _compile(cmd: list[str], tmp: str, target: str) -> str:
 
 
 def build_extension(force: bool = False) -> str:
-    """Compile ``_attnw_torch`` if it is missing or older than its source or the C header; returns its path."""
-    if force or _older(EXT_PATH, [EXT_SOURCE, os.path.join(os.path.dirname(_PKG), "include", "attnw.h")]):
+    """Compile ``_attnw_torch`` if it is missing, older than its source or the C header, or built for another torch or Python;
+    returns its path."""
+    if force or ext_is_stale():
         tmp = EXT_PATH + f".tmp{os.getpid()}"
         _compile(ext_command(tmp), tmp, EXT_PATH)
     return EXT_PATH

@@ -266,7 +266,10 @@ PyMethodDef g_methods[] = {
     {"set_error", py_set_error, METH_O, "the exception type for attnw status codes"},
     {nullptr, nullptr, 0, nullptr},
 };
-PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_attnw_torch", nullptr, -1, g_methods, nullptr, nullptr, nullptr, nullptr};
+#ifndef ATTNW_BUILT_FOR
+#error "build.py passes the torch and the Python that the module is built for and looks for them in it later"
+#endif
+PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_attnw_torch", ATTNW_BUILT_FOR, -1, g_methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace
 

@@ -97,3 +97,18 @@ def test_tensors_of_several_devices_are_refused(binding):
                      lambda: binding.attnw_fused_noalloc(q, q, 0.125, P=far)):
             with pytest.raises(ValueError, match="must be on cuda:0"):
                 call()
+
+
+def test_extension_is_built_again_for_another_torch_or_python(binding, monkeypatch):
+    import sysconfig
+
+    from paper_2407_13885_b200 import build
+    assert not build.ext_is_stale() and binding._native.__doc__ == build.built_for()
+    with monkeypatch.context() as m:
+        m.setattr(torch, "__version__", torch.__version__ + ".1")
+        assert build.ext_is_stale()
+    soabi = sysconfig.get_config_var("SOABI")
+    with monkeypatch.context() as m:
+        m.setattr(sysconfig, "get_config_var", lambda name: soabi + "x" if name == "SOABI" else None)
+        assert build.ext_is_stale()
+    assert not build.ext_is_stale()
