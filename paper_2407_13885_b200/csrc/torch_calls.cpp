@@ -106,9 +106,10 @@ bool count_is(Py_ssize_t n, Py_ssize_t want) {
     return n == want;
 }
 
+// None = torch's default type, as everywhere in torch.
 bool is_float32(PyObject* dtype, bool* f32) {
-    if (THPDtype_Check(dtype)) {
-        const at::ScalarType t = reinterpret_cast<THPDtype*>(dtype)->scalar_type;
+    if (dtype == Py_None || THPDtype_Check(dtype)) {
+        const at::ScalarType t = dtype == Py_None ? c10::get_default_dtype_as_scalartype() : reinterpret_cast<THPDtype*>(dtype)->scalar_type;
         *f32 = t == at::kFloat;
         if (*f32 || t == at::kBFloat16) return true;
     }

@@ -45,6 +45,15 @@ def test_bad_arguments_on_the_gpu(binding):
 
 
 @pytest.mark.gpu
+def test_no_type_is_the_default_type(binding):
+    q, k = small_fused_inputs(1, 1, 64, 64, stream=7)
+    P = binding.attnw_fused(bits_to_cuda_bf16(q), bits_to_cuda_bf16(k), 0.125, out_dtype=None)
+    assert P.dtype == torch.float32
+    assert_close_to_oracle(P, oracle.attnw(q, k, 0.125))
+    assert binding.softmax_rows(P[0, 0].contiguous(), out_dtype=None).dtype == torch.float32
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 def test_given_output_and_stream(binding, dtype):
     q, k = small_fused_inputs(1, 2, 200, 64, stream=5)
