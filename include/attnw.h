@@ -223,6 +223,14 @@ int attnw_query_status(void* stream, unsigned int* device_status);
  */
 int attnw_selftest_wait_timeout(long long limit_cycles, void* stream);
 
+/*
+ * Self-test of the message tags of the grid-row kernel (see attnw_set_fused_variant): the next launch that exchanges messages on
+ * `stream`, and the next one of attnw_fused_noalloc on the device, number them from `next` + 1 on, as they would after that many
+ * row blocks; near 2^32 the tags run out and start over.  Forward only (ATTNW_ERR_BAD_SHAPE otherwise), so no tag comes twice;
+ * ATTNW_ERR_UNSUPPORTED on a stream that has no exchange area yet.
+ */
+int attnw_selftest_exchange_tags(unsigned int next, void* stream);
+
 /* Number of kernels this library has launched in the calling process since load / last reset
  * (reset = 1 returns the count and then sets it to zero). */
 long long attnw_launch_count(int reset);

@@ -30,6 +30,7 @@ SIGNATURES = {
     "attnw_fused_noalloc": (_int, [_vp, _vp, _vp, _int, _int, _int, _int, ctypes.c_float, _vp]),
     "attnw_query_status": (_int, [_vp, ctypes.POINTER(ctypes.c_uint)]),
     "attnw_selftest_wait_timeout": (_int, [_ll, _vp]),
+    "attnw_selftest_exchange_tags": (_int, [ctypes.c_uint, _vp]),
     "attnw_set_fused_variant": (_int, [_int]),
     "attnw_set_attn_variant": (_int, [_int]),
     "attnw_set_rows_variant": (_int, [_int]),
@@ -221,6 +222,12 @@ def selftest_wait_timeout(limit_cycles: int = 1_000_000, stream=None) -> None:
     """Launches the failure-path self-test: one warp waits ``limit_cycles`` SM clocks on a barrier nobody arrives on,
     gives up and records site 127 in the device status word (see ``attnw_selftest_wait_timeout``)."""
     _check(lib.attnw_selftest_wait_timeout(int(limit_cycles), _stream_ptr(stream)), "attnw_selftest_wait_timeout")
+
+
+def selftest_exchange_tags(next_tag: int, stream=None) -> None:
+    """Moves the message tags of ``stream``'s exchange area, and of ``attnw_fused_noalloc``, forward to ``next_tag``
+    (see ``attnw_selftest_exchange_tags``)."""
+    _check(lib.attnw_selftest_exchange_tags(int(next_tag), _stream_ptr(stream)), "attnw_selftest_exchange_tags")
 
 
 def attnw_fused_noalloc(Q: torch.Tensor, K: torch.Tensor, scale: float, P: torch.Tensor | None = None,

@@ -102,6 +102,18 @@ struct GridrowAreas {
 };
 GridrowAreas g_gridrow_areas[kMaxDevices];
 
+// The tags *base + 1 ... *base + n of an exchange area's messages for one launch, from the counter `next`; 0 is never a tag.
+// true: the tags had run out (after about 4e9 row blocks) and start over, so the area must be cleared in front of the launch.  Where
+// a message lies depends on the launch's groups: messages of other shapes may have stood there since the low tags were last in use.
+constexpr uint32_t kLastTag = 0xffffffffu;
+bool take_tags(uint32_t* next, uint32_t n, uint32_t* base) {
+    const bool start_over = n > kLastTag - *next;
+    if (start_over) *next = 0;
+    *base = *next;
+    *next += n;
+    return start_over;
+}
+
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -539,10 +551,14 @@ int launch_gridrow(DeviceInfo* dev, const void* Q, const void* K, void* P, int B
     GridrowArea* area = nullptr;
     rc = gridrow_area(&areas, dev->sm_count, stream, &area);
     if (rc != ATTNW_OK) return rc;
-    // tags area->tag + 1 ... area->tag + (longest list) belong to this launch; 0 is never a tag
-    if (area->tag > 0xffffffffu - g.longest - 1u) area->tag = 0;
-    rc = enqueue_gridrow<D, OutT>(g, Q, K, P, BH, N, scale, area->xchg, area->tag, stream);
-    area->tag += g.longest;
+    uint32_t tag_base = 0;
+    if (take_tags(&area->tag, g.longest, &tag_base) &&
+        cudaMemsetAsync(area->xchg, 0, gridrow_entries(dev->sm_count) * sizeof(uint4), stream) != cudaSuccess) {
+        (void)cudaGetLastError();
+        area->tag = kLastTag;
+        return ATTNW_ERR_CUDA;
+    }
+    rc = enqueue_gridrow<D, OutT>(g, Q, K, P, BH, N, scale, area->xchg, tag_base, stream);
     if (rc == ATTNW_OK && areas.several_streams) {
         area->recorded = cudaEventRecord(area->last, stream) == cudaSuccess;
         if (!area->recorded) rc = ATTNW_ERR_CUDA;
@@ -1234,6 +1250,28 @@ int attnw_selftest_wait_timeout(long long limit_cycles, void* stream) {
     wait_timeout_selftest_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(limit_cycles);
     if (cudaGetLastError() != cudaSuccess) return ATTNW_ERR_CUDA;
     g_launches.fetch_add(1, std::memory_order_relaxed);
+    return ATTNW_OK;
+}
+
+int attnw_selftest_exchange_tags(unsigned int next, void* stream) {
+    DeviceInfo* dev = nullptr;
+    int rc = current_device(&dev);
+    if (rc != ATTNW_OK) return rc;
+    unsigned long long id = 0;
+    if (cudaStreamGetId(static_cast<cudaStream_t>(stream), &id) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return ATTNW_ERR_CUDA;
+    }
+    GridrowAreas& areas = g_gridrow_areas[dev - g_devices];
+    std::lock_guard<std::mutex> areas_lock(areas.mutex);
+    uint32_t* tag = nullptr;
+    for (int a = 0; a < areas.count && !tag; ++a)
+        if (areas.area[a].stream_id == id) tag = &areas.area[a].tag;
+    if (!tag) return ATTNW_ERR_UNSUPPORTED;
+    std::lock_guard<std::mutex> noalloc_lock(g_mutex);
+    uint32_t* noalloc_tag = &g_noalloc[dev - g_devices].tag;
+    if (*tag > next || *noalloc_tag > next) return ATTNW_ERR_BAD_SHAPE;
+    *tag = *noalloc_tag = next;
     return ATTNW_OK;
 }
 

@@ -101,6 +101,29 @@ def test_more_streams_than_exchange_areas(attnw):
             assert_close_to_oracle(P, cases[n % 12][2], f"stream {n % 12}")
 
 
+LAST_TAG = 0xffffffff
+
+
+@pytest.mark.parametrize("entry", ["fused", "noalloc"])
+def test_message_tags_start_over(attnw, entry):
+    # before each call the tags run out, so that it starts over with those which the calls before have left in the exchange area:
+    # the same groups on other inputs (4 CTAs, where all read all pairs, and 6, with owners), and groups of 16 in between
+    d = 64
+    call = attnw.attnw_fused if entry == "fused" else attnw.attnw_fused_noalloc
+    for x, N in enumerate((1000, 1000, 1288, 1288, 4096, 1288, 1000)):
+        q, k = small_fused_inputs(1, 2, N, d, sigma=2.0, stream=900 + x)
+        Q, K = bits_to_cuda_bf16(q), bits_to_cuda_bf16(k)
+        if x == 0:
+            attnw.attnw_fused(Q, K, scale_of(d))  # the stream's exchange area
+            with pytest.raises(attnw.AttnwError):
+                attnw.selftest_exchange_tags(0)   # forward only
+        attnw.selftest_exchange_tags(LAST_TAG)
+        P = call(Q, K, scale_of(d))
+        torch.cuda.synchronize()
+        assert attnw.query_status() == 0
+        assert_close_to_oracle(P, oracle.attnw(q, k, scale_of(d)), f"{entry} N{N}")
+
+
 @pytest.mark.parametrize("entry,dtype", [("fused", torch.bfloat16), ("fused", torch.float32), ("noalloc", torch.bfloat16)])
 @pytest.mark.parametrize("N", [256, 2048])
 def test_captured_call_is_right_on_every_replay(attnw, entry, dtype, N):
