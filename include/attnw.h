@@ -77,7 +77,7 @@ int attnw_fused_f32(const void* Q, const void* K, void* P, int B, int H, int N, 
  * First call on a device: looks up the array's device address (cudaGetSymbolAddress) and the device's properties.
  *   Make that first call before any stream capture begins.
  * Every call on a device shares the one array, which keeps what the previous call left in it; the messages carry
- *   tags that no later call repeats, so nothing has to be cleared between calls (after about 4e9 row blocks the tags
+ *   tags that no later call repeats, so nothing has to be cleared between calls (after about 2e9 row blocks the tags
  *   start over and the call first clears the array, in stream order).  Two calls that overlap in time on one device
  *   - different streams with nothing ordering them - race on the array: order them, or use attnw_fused for one.
  */
@@ -226,7 +226,7 @@ int attnw_selftest_wait_timeout(long long limit_cycles, void* stream);
 /*
  * Self-test of the message tags of the grid-row kernel (see attnw_set_fused_variant): the next launch that exchanges messages on
  * `stream`, and the next one of attnw_fused_noalloc on the device, number them from `next` + 1 on, as they would after that many
- * row blocks; near 2^32 the tags run out and start over.  Forward only (ATTNW_ERR_BAD_SHAPE otherwise), so no tag comes twice;
+ * row blocks; at 2^31 - 1 the tags run out and start over.  Forward only (ATTNW_ERR_BAD_SHAPE otherwise), so no tag comes twice;
  * ATTNW_ERR_UNSUPPORTED on a stream that has no exchange area yet.
  */
 int attnw_selftest_exchange_tags(unsigned int next, void* stream);

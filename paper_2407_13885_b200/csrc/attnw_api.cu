@@ -103,9 +103,10 @@ struct GridrowAreas {
 GridrowAreas g_gridrow_areas[kMaxDevices];
 
 // The tags *base + 1 ... *base + n of an exchange area's messages for one launch, from the counter `next`; 0 is never a tag.
-// true: the tags had run out (after about 4e9 row blocks) and start over, so the area must be cleared in front of the launch.  Where
+// true: the tags had run out (after about 2e9 row blocks) and start over, so the area must be cleared in front of the launch.  Where
 // a message lies depends on the launch's groups: messages of other shapes may have stood there since the low tags were last in use.
-constexpr uint32_t kLastTag = 0xffffffffu;
+// The upper half of the tags belongs to launches of attnw_fused_noalloc in graphs, which repeat them on every replay.
+constexpr uint32_t kLastTag = 0x7fffffffu, kCapturedTagBase = kLastTag;
 bool take_tags(uint32_t* next, uint32_t n, uint32_t* base) {
     const bool start_over = n > kLastTag - *next;
     if (start_over) *next = 0;
@@ -1030,17 +1031,16 @@ int launch_gridrow_noalloc(DeviceInfo* dev, NoAllocState* st, const void* Q, con
             (void)cudaGetLastError();
             return ATTNW_ERR_CUDA;
         }
-        if (capture != cudaStreamCaptureStatusNone || st->tag > 0xffffffffu - g.longest - 1u) {
-            // A captured launch is replayed with the same tags, or the tags are used up (after about 4e9 row blocks): start
-            // again from a cleared array, in stream order.
-            if (cudaMemsetAsync(st->xchg, 0, sizeof(g_noalloc_xchg), stream) != cudaSuccess) {
-                (void)cudaGetLastError();
-                return ATTNW_ERR_CUDA;
-            }
-            if (capture == cudaStreamCaptureStatusNone) st->tag = 0;
+        // A captured launch has tags that no uncaptured one uses, and repeats them, like the graph's other launches, from an array
+        // that it clears first.
+        const bool captured = capture != cudaStreamCaptureStatusNone;
+        const bool start_over = !captured && take_tags(&st->tag, g.longest, &tag_base);
+        if (captured) tag_base = kCapturedTagBase;
+        if ((captured || start_over) && cudaMemsetAsync(st->xchg, 0, sizeof(g_noalloc_xchg), stream) != cudaSuccess) {
+            (void)cudaGetLastError();
+            if (start_over) st->tag = kLastTag;
+            return ATTNW_ERR_CUDA;
         }
-        tag_base = st->tag;
-        st->tag += g.longest;
     }
     const int launched = enqueue_gridrow<D, __nv_bfloat16>(g, Q, K, P, BH, N, scale, st->xchg, tag_base, stream);
     return launched == ATTNW_ERR_UNSUPPORTED ? ATTNW_ERR_CUDA : launched;
@@ -1270,7 +1270,7 @@ int attnw_selftest_exchange_tags(unsigned int next, void* stream) {
     if (!tag) return ATTNW_ERR_UNSUPPORTED;
     std::lock_guard<std::mutex> noalloc_lock(g_mutex);
     uint32_t* noalloc_tag = &g_noalloc[dev - g_devices].tag;
-    if (*tag > next || *noalloc_tag > next) return ATTNW_ERR_BAD_SHAPE;
+    if (next > kLastTag || *tag > next || *noalloc_tag > next) return ATTNW_ERR_BAD_SHAPE;
     *tag = *noalloc_tag = next;
     return ATTNW_OK;
 }

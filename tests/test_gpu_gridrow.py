@@ -101,7 +101,7 @@ def test_more_streams_than_exchange_areas(attnw):
             assert_close_to_oracle(P, cases[n % 12][2], f"stream {n % 12}")
 
 
-LAST_TAG = 0xffffffff
+LAST_TAG = 0x7fffffff
 
 
 @pytest.mark.parametrize("entry", ["fused", "noalloc"])
@@ -122,6 +122,28 @@ def test_message_tags_start_over(attnw, entry):
         torch.cuda.synchronize()
         assert attnw.query_status() == 0
         assert_close_to_oracle(P, oracle.attnw(q, k, scale_of(d)), f"{entry} N{N}")
+
+
+def test_captured_noalloc_calls_have_tags_of_their_own(attnw):
+    # captured when the tags had run out; then replays and uncaptured calls, on other inputs each time, in turn
+    d, N = 64, 1288
+    calls = [small_fused_inputs(1, 2, N, d, sigma=2.0, stream=950 + x) for x in range(6)]
+    Q, K = bits_to_cuda_bf16(calls[0][0]), bits_to_cuda_bf16(calls[0][1])
+    P = torch.empty((1, 2, N, N), dtype=torch.bfloat16, device="cuda")
+    attnw.attnw_fused(Q, K, scale_of(d))
+    attnw.attnw_fused_noalloc(Q, K, scale_of(d), P=P)
+    attnw.selftest_exchange_tags(LAST_TAG)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        attnw.attnw_fused_noalloc(Q, K, scale_of(d), P=P)
+    for x, (q, k) in enumerate(calls):
+        Q.copy_(bits_to_cuda_bf16(q))
+        K.copy_(bits_to_cuda_bf16(k))
+        P.fill_(float("nan"))
+        graph.replay() if x % 2 == 0 else attnw.attnw_fused_noalloc(Q, K, scale_of(d), P=P)
+        torch.cuda.synchronize()
+        assert attnw.query_status() == 0
+        assert_close_to_oracle(P, oracle.attnw(q, k, scale_of(d)), f"call {x}")
 
 
 @pytest.mark.parametrize("entry,dtype", [("fused", torch.bfloat16), ("fused", torch.float32), ("noalloc", torch.bfloat16)])
