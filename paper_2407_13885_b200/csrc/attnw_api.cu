@@ -770,6 +770,40 @@ bool gridrow_pays(const DeviceInfo* dev, int N) {
     return group_ctas <= 112 && dev->sm_count / group_ctas * group_ctas * 3 >= dev->sm_count * 2;
 }
 
+// Enqueues `first` and `second` on a stream that is being captured as two branches of its graph, which may run side by side.  By
+// the capture's own dependencies and not by a second stream: a stream belongs to one capture until that ends, so two captures
+// open at once could not share it.
+template <typename First, typename Second>
+int capture_side_by_side(cudaStream_t s, First first, Second second) {
+    constexpr size_t kMost = 16;
+    cudaGraphNode_t before[kMost], behind_first[kMost];
+    auto dependencies = [s](cudaGraphNode_t* out, size_t* n) {
+        cudaStreamCaptureStatus status;
+        const cudaGraphNode_t* nodes = nullptr;
+        if (cudaStreamGetCaptureInfo(s, &status, nullptr, nullptr, &nodes, n) != cudaSuccess || *n > kMost) {
+            (void)cudaGetLastError();
+            return false;
+        }
+        for (size_t i = 0; i < *n; ++i) out[i] = nodes[i];
+        return true;
+    };
+    size_t n_before = 0, n_first = 0;
+    const bool known = dependencies(before, &n_before);
+    int rc = first(s);
+    if (rc != ATTNW_OK) return rc;
+    if (!known || !dependencies(behind_first, &n_first)) return second(s);  // one behind the other
+    if (cudaStreamUpdateCaptureDependencies(s, before, n_before, cudaStreamSetCaptureDependencies) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return ATTNW_ERR_CUDA;
+    }
+    rc = second(s);
+    if (cudaStreamUpdateCaptureDependencies(s, behind_first, n_first, cudaStreamAddCaptureDependencies) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return ATTNW_ERR_CUDA;
+    }
+    return rc;
+}
+
 template <typename OutT>
 int fused_entry(const void* Q, const void* K, void* P, int B, int H, int N, int d, float scale, void* stream) {
     int rc = validate_fused(Q, K, P, B, H, N, d, scale, sizeof(OutT));
@@ -842,6 +876,26 @@ int fused_entry(const void* Q, const void* K, void* P, int B, int H, int N, int 
                 }
             }
             if (bh_two_pass > 0) {
+                const int bh_res = bh - bh_two_pass;
+                const size_t qk_off = static_cast<size_t>(bh_res) * N * d * 2;
+                const size_t p_off = static_cast<size_t>(bh_res) * N * N * 2;
+                const char* q2 = static_cast<const char*>(Q) + qk_off;
+                const char* k2 = static_cast<const char*>(K) + qk_off;
+                char* p2 = static_cast<char*>(P) + p_off;
+                auto resident = [&](cudaStream_t on) {
+                    return (d == 64) ? launch_resident<64>(dev, Q, K, P, bh_res, N, scale, on)
+                                     : launch_resident<128>(dev, Q, K, P, bh_res, N, scale, on);
+                };
+                auto two_pass = [&](cudaStream_t on) {
+                    return (d == 64) ? launch_fused<64, OutT>(dev, q2, k2, p2, bh_two_pass, N, scale, on, false)
+                                     : launch_fused<128, OutT>(dev, q2, k2, p2, bh_two_pass, N, scale, on, false);
+                };
+                cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+                if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
+                    (void)cudaGetLastError();
+                    return ATTNW_ERR_CUDA;
+                }
+                if (capture != cudaStreamCaptureStatusNone) return capture_side_by_side(s, resident, two_pass);
                 std::lock_guard<std::mutex> lock(g_split_mutex);
                 if (!dev->side_stream) {
                     if (cudaStreamCreateWithFlags(&dev->side_stream, cudaStreamNonBlocking) != cudaSuccess ||
@@ -851,19 +905,11 @@ int fused_entry(const void* Q, const void* K, void* P, int B, int H, int N, int 
                         return ATTNW_ERR_CUDA;
                     }
                 }
-                const int bh_res = bh - bh_two_pass;
-                const size_t qk_off = static_cast<size_t>(bh_res) * N * d * 2;
-                const size_t p_off = static_cast<size_t>(bh_res) * N * N * 2;
-                const char* q2 = static_cast<const char*>(Q) + qk_off;
-                const char* k2 = static_cast<const char*>(K) + qk_off;
-                char* p2 = static_cast<char*>(P) + p_off;
                 if (cudaEventRecord(dev->fork_event, s) != cudaSuccess) return ATTNW_ERR_CUDA;
-                rc = (d == 64) ? launch_resident<64>(dev, Q, K, P, bh_res, N, scale, s)
-                               : launch_resident<128>(dev, Q, K, P, bh_res, N, scale, s);
+                rc = resident(s);
                 if (rc != ATTNW_OK) return rc;
                 if (cudaStreamWaitEvent(dev->side_stream, dev->fork_event, 0) != cudaSuccess) return ATTNW_ERR_CUDA;
-                rc = (d == 64) ? launch_fused<64, OutT>(dev, q2, k2, p2, bh_two_pass, N, scale, dev->side_stream, false)
-                               : launch_fused<128, OutT>(dev, q2, k2, p2, bh_two_pass, N, scale, dev->side_stream, false);
+                rc = two_pass(dev->side_stream);
                 if (cudaEventRecord(dev->join_event, dev->side_stream) != cudaSuccess ||
                     cudaStreamWaitEvent(s, dev->join_event, 0) != cudaSuccess)
                     return ATTNW_ERR_CUDA;

@@ -175,6 +175,65 @@ def test_captured_call_is_right_on_every_replay(attnw, entry, dtype, N):
         assert_close_to_oracle(P, oracle.attnw(q, k, scale_of(d)), f"{entry} {dtype} N{N}")
 
 
+# captured calls of many heads: one part on the resident kernel, the others beside it on the two-pass kernel
+@pytest.mark.parametrize("H,N,d", [(12, 4096, 64), (8, 4040, 128)])
+def test_captured_call_in_two_parts(attnw, H, N, d):
+    X = torch.zeros(1, 64, 64, dtype=torch.bfloat16, device="cuda")
+    W = torch.zeros(1, 64, 64, dtype=torch.bfloat16, device="cuda")
+    calls = [small_fused_inputs(1, H, N, d, stream=820 + x) for x in range(2)]
+    ids = np.unique(np.concatenate([np.arange(0, H * N, 617), [0, H * N - 1]]))
+    Q, K = (bits_to_cuda_bf16(x) for x in calls[0])
+    for behind_another in (False, True):  # the first node of its graph, and behind a launch that may overlap its own
+        P = torch.empty((1, H, N, N), dtype=torch.bfloat16, device="cuda")
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            if behind_another:
+                attnw.project_qk(X, W, W)
+            launches = attnw.launch_count()
+            attnw.attnw_fused(Q, K, scale_of(d), P=P)
+            assert attnw.launch_count() == launches + 2
+        for q, k in calls:
+            Q.copy_(bits_to_cuda_bf16(q))
+            K.copy_(bits_to_cuda_bf16(k))
+            P.fill_(float("nan"))
+            graph.replay()
+            torch.cuda.synchronize()
+            assert attnw.query_status() == 0
+            assert not bool(torch.isnan(P).any())
+            rows = P.view(-1, N)[torch.from_numpy(ids).cuda()]
+            err = np.max(np.abs(to_f64(rows) - oracle.attnw_rows(q, k, scale_of(d), ids)))
+            assert err <= TOL[torch.bfloat16]["abs"], err
+
+
+def test_two_captures_open_at_once(attnw):
+    from cuda.bindings import runtime as rt
+    H, N, d = 8, 4040, 64
+    relaxed = rt.cudaStreamCaptureMode.cudaStreamCaptureModeRelaxed
+
+    def ok(result):
+        assert result[0] == rt.cudaError_t.cudaSuccess, result[0]
+        return result[1] if len(result) > 1 else None
+
+    calls = [tuple(bits_to_cuda_bf16(x) for x in small_fused_inputs(1, H, N, d, stream=840 + 2 * n)) for n in range(2)]
+    want = [attnw.attnw_fused(Q, K, scale_of(d)) for Q, K in calls]
+    P = [torch.full_like(w, float("nan")) for w in want]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in calls]
+    for n, s in enumerate(streams):
+        ok(rt.cudaStreamBeginCapture(s.cuda_stream, relaxed))
+        attnw.attnw_fused(*calls[n], scale_of(d), P=P[n], stream=s)
+    graphs = [ok(rt.cudaStreamEndCapture(s.cuda_stream)) for s in streams]
+    for s, graph in zip(streams, graphs):
+        run = ok(rt.cudaGraphInstantiate(graph, 0))
+        ok(rt.cudaGraphLaunch(run, s.cuda_stream))
+        torch.cuda.synchronize()
+        ok(rt.cudaGraphExecDestroy(run))
+        ok(rt.cudaGraphDestroy(graph))
+    assert attnw.query_status() == 0
+    for p, w in zip(P, want):
+        assert float((p.float() - w.float()).abs().max()) <= TOL[torch.bfloat16]["abs"]
+
+
 def test_chain_of_calls_sees_the_results_in_front(attnw):
     # each launch may begin before the kernel in front of it has ended: every call here reads what the call before has just
     # written, among ordinary kernels of torch, and the last result is that of the same chain with a wait after each call
