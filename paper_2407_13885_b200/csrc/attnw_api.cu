@@ -501,10 +501,11 @@ int gridrow_area(GridrowAreas* areas, int sm_count, cudaStream_t stream, Gridrow
         GridrowArea fresh;
         const size_t bytes = gridrow_entries(sm_count) * sizeof(uint4);
         void* p = nullptr;
-        // zero, so that no entry carries a valid tag
-        if (cudaMalloc(&p, bytes) != cudaSuccess || cudaMemset(p, 0, bytes) != cudaSuccess ||
-            cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess ||
-            cudaEventCreateWithFlags(&fresh.last, cudaEventDisableTiming) != cudaSuccess) {
+        // Zero, so that no entry carries a valid tag: by the stream itself, which runs the area's first launch (the legacy stream may
+        // not be used while another thread captures a stream that synchronises with it, and doing so spoils that capture).
+        if (cudaMalloc(&p, bytes) != cudaSuccess || cudaEventCreateWithFlags(&fresh.last, cudaEventDisableTiming) != cudaSuccess ||
+            cudaMemsetAsync(p, 0, bytes, stream) != cudaSuccess) {
+            if (fresh.last) cudaEventDestroy(fresh.last);
             if (p) cudaFree(p);
             rc = ATTNW_ERR_UNSUPPORTED;  // no memory for it: the caller takes a kernel that needs none
         } else {

@@ -205,6 +205,35 @@ def test_captured_call_in_two_parts(attnw, H, N, d):
             assert err <= TOL[torch.bfloat16]["abs"], err
 
 
+def test_exchange_area_for_a_new_stream_while_another_is_captured():
+    # in a process of its own, where no exchange area is free: a second stream needs one while a blocking stream is captured
+    import os
+    import subprocess
+    import sys
+    code = """if True:
+        import torch
+        from cuda.bindings import runtime as rt
+        from paper_2407_13885_b200 import binding
+        Q, K = (torch.randn(1, 2, 1000, 64, device="cuda").bfloat16() for _ in range(2))
+        P = [torch.zeros(1, 2, 1000, 1000, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+        first, second = torch.cuda.Stream(), torch.cuda.Stream()
+        torch.cuda.synchronize()
+        binding.attnw_fused(Q, K, 0.125, P=P[0], stream=first)
+        torch.cuda.synchronize()
+        _, blocking = rt.cudaStreamCreate()
+        (err,) = rt.cudaStreamBeginCapture(blocking, rt.cudaStreamCaptureMode.cudaStreamCaptureModeRelaxed)
+        assert err == rt.cudaError_t.cudaSuccess
+        binding.attnw_fused(Q, K, 0.125, P=P[1], stream=second)
+        err, graph = rt.cudaStreamEndCapture(blocking)
+        assert err == rt.cudaError_t.cudaSuccess, err
+        torch.cuda.synchronize()
+        assert binding.query_status() == 0 and torch.equal(P[0], P[1])
+        binding.selftest_exchange_tags(100, stream=second)  # refused for a stream without an area
+        """
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", code], cwd=root, check=True, timeout=300)
+
+
 def test_two_captures_open_at_once(attnw):
     from cuda.bindings import runtime as rt
     H, N, d = 8, 4040, 64
