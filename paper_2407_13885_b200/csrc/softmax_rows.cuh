@@ -73,8 +73,9 @@ __device__ __forceinline__ float sr_row_reduce(float v, float* red) {
     return v;
 }
 
-// S and P carry no __restrict__ and every load is a coherent one: the float32 variant may run
-// in place (P == S), where each thread overwrites exactly the elements it has loaded.
+// S and P carry no __restrict__ and every load is a coherent one (no __ldg): the float32 variant may run in place (P == S), where
+// each thread overwrites exactly the elements it has loaded, and a kernel may begin while the one in front still writes S
+// (launch_overlapped), where a read-only load need not see what was written after the begin.
 //
 // Register tier: TPR threads per row, VPT float4 vectors per thread, row kept in registers.
 // A CTA has max(TPR, 256) threads and handles CTA_THREADS / TPR rows per sweep.
@@ -177,7 +178,7 @@ softmax_rows_stream_kernel(const float* S, OutT* P, long long rows, long long co
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const long long idx = base + j * THREADS;
-                x[j] = idx < nvec ? __ldg(src + idx) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+                x[j] = idx < nvec ? src[idx] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
             }
             float vm = m;
 #pragma unroll

@@ -134,3 +134,12 @@ def test_attention_variant_knob(lib):
 
 def test_query_status_rejects_null(lib):
     assert lib.attnw_query_status(None, None) == 1
+
+
+def test_kernels_have_no_read_only_loads():
+    # A kernel may begin while the kernel in front still writes what it will read; a read-only load (ld.global.nc) promises that
+    # nobody writes as long as the kernel runs.
+    csrc = os.path.join(ROOT, "paper_2407_13885_b200", "csrc")
+    for name in sorted(os.listdir(csrc)):
+        code = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+        assert not re.search(r"__ldg\s*\(|ld\.global\.nc|const\s+\w+\s*\*\s*__restrict__", code), name

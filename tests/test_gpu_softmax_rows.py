@@ -160,3 +160,24 @@ def test_cluster_tier_edges(attnw, rows, cols):
         assert attnw.query_status() == 0
         assert_guards_intact(raw, g)
         assert_close_to_oracle(P, oracle.softmax_rows(S), f"{rows} x {cols} {dtype}")
+
+
+# each launch may begin while the kernel in front still writes what it reads: register, shared-memory, two-read and cluster kernels
+@pytest.mark.parametrize("rows,cols", [(900, 1000), (200, 12000), (300, 36864), (100, 65536)])
+def test_chain_reads_what_the_kernel_in_front_wrote(attnw, rows, cols):
+    S = torch.from_numpy(inputs.normal_f32(12, rows + cols, rows * cols, 3.0).reshape(rows, cols)).cuda()
+
+    def chain(wait):
+        a, b = S.clone(), torch.empty_like(S)
+        wait()
+        for src, dst in ((a, b), (b, a), (a, b), (b, b)):
+            attnw.softmax_rows(src, P=dst)
+            wait()
+        return a, b
+
+    want = chain(torch.cuda.synchronize)
+    for _ in range(3):
+        got = chain(lambda: None)
+        torch.cuda.synchronize()
+        assert attnw.query_status() == 0
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
