@@ -157,7 +157,6 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     auto stage_offset = [](int s) { return !split || s < L::kStages ? L::kKOff + s * L::kTileBytes : L::kQOff + L::kTileBytes; };
 
     // ---- set-up ------------------------------------------------------------------------------
-    ptx::grid_launch_dependents();
     if (threadIdx.x == 0) {
         ptx::grid_dependency_wait();
         const uint32_t prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);  // (arrives meanwhile)
@@ -189,6 +188,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     if (warp == kMma) {
         ptx::tmem_alloc(&bars->tmem_base, kTmemCols);
         ptx::tmem_relinquish();
+        ptx::grid_launch_dependents();  // not before this CTA has its tensor memory (launch_overlapped)
     }
     ptx::grid_dependency_wait();
     ptx::tc_fence_before_sync();

@@ -227,7 +227,6 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     uint4* const results = xchg + (static_cast<size_t>(n_groups) * group_ctas + group) * kXchgDepth * kTile;
 
     // ---- set-up ------------------------------------------------------------------------------
-    ptx::grid_launch_dependents();
     if (threadIdx.x == 0) {
         ptx::grid_dependency_wait();
         const uint32_t prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);  // (arrives meanwhile)
@@ -261,6 +260,7 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     if (warp == kMmaWarpG) {
         ptx::tmem_alloc(&bars->tmem_base, kTmemCols);
         ptx::tmem_relinquish();
+        ptx::grid_launch_dependents();  // not before this CTA has its tensor memory (launch_overlapped)
     }
     ptx::grid_dependency_wait();
     ptx::tc_fence_before_sync();

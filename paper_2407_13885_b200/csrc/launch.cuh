@@ -30,6 +30,8 @@ static inline cudaError_t allow_smem(int bytes, bool large_clusters = false) {
 // Launches `kernel` so that it may begin before the kernel in front of it on the stream has ended: its CTAs take the SMs as that
 // kernel's CTAs leave them, set up their barriers and tensor memory, and wait (ptx::grid_dependency_wait) until the kernel
 // has ended and its results are visible.  Every kernel launched this way waits before it touches global memory.
+// A kernel that takes tensor memory lets the one behind it begin (ptx::grid_launch_dependents) only once its CTA has it: a CTA of
+// that kernel on the same SM might otherwise take it first, then wait for this kernel, and keep it for good.
 // Back to back, small calls took 2 us more each: 4096 x 1000 float32 row Softmax 6.2 -> 4.6 us, attention of 2 x 128 8.2 -> 5.4,
 // projection of 64 rows 8.2 -> 5.3, weights of one head of 256 8.4 -> 6.5.
 // `cluster` CTAs form a cluster; `cooperative`: the whole grid is resident at once, or the launch fails.

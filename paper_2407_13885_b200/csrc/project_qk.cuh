@@ -85,7 +85,6 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     const CUtensorMap* tm_w = keys ? &tm_wk : &tm_wq;
     const CUtensorMap* tm_out = keys ? &tm_k : &tm_q;
 
-    ptx::grid_launch_dependents();
     if (threadIdx.x == 0) {
         ptx::grid_dependency_wait();
         const uint32_t prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);  // (arrives meanwhile)
@@ -107,6 +106,7 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     if (warp == kMma) {
         ptx::tmem_alloc(&bars->tmem_base, L::kTmemCols);
         ptx::tmem_relinquish();
+        ptx::grid_launch_dependents();  // not before this CTA has its tensor memory (launch_overlapped)
     }
     ptx::grid_dependency_wait();
     ptx::tc_fence_before_sync();
