@@ -39,6 +39,13 @@ struct Control {
 constexpr int kControlBytes = 512;
 static_assert(sizeof(Control) <= kControlBytes, "control block must fit its slot");
 
+// Unwinding after a wait gave up: the bulk copy that completes phase `parity` of `bar` lands before shared memory is released.
+__device__ __noinline__ void drain_copy(uint32_t bar, uint32_t parity) {
+    const long long t0 = clock64();
+    while (!ptx::mbar_try_wait(bar, parity) && clock64() - t0 < kWaitLimitCycles / 8) {
+    }
+}
+
 template <bool IS_MAX, int NT>
 __device__ __forceinline__ float block_reduce(float v, float* red) {
 #pragma unroll
@@ -100,7 +107,10 @@ softmax_rows_smem_kernel(const float* S, OutT* P, long long rows, long long cols
                 ptx::bulk_load_1d(ptx::smem_u32(x) + off, reinterpret_cast<const uint8_t*>(src) + off,
                                   bytes - off < kPieceBytes ? bytes - off : kPieceBytes, &ctl->full);
         }
-        if (ok && n > 0) ok = fused_wait(&ctl->full, it & 1u, abort_flag, kSiteRowLoad);
+        if (ok && n > 0 && !fused_wait(&ctl->full, it & 1u, abort_flag, kSiteRowLoad)) {
+            drain_copy(ptx::smem_u32(&ctl->full), it & 1u);
+            ok = false;
+        }
         ok = __syncthreads_and(ok);  // all or none of the CTA goes on
 
         // ---- pass 1: maximum of the slice ----
@@ -216,6 +226,7 @@ constexpr int kRcSliceMaxCols = kRcThreads * kRcVecPerThread * 4;               
 constexpr long long kRcMaxCols = static_cast<long long>(kRcSliceMaxCols) * kMaxCluster;  // 262144
 constexpr uint32_t kSiteRcRowLoad = 121;
 constexpr uint32_t kSiteRcExchange = 122;
+constexpr long long kLatePairCycles = 1ll << 17;  // some 70 us
 
 struct RcControl {
     uint64_t full[kRcThreads / 32];  // one per warp: its piece of the current row has landed
@@ -278,10 +289,15 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
     };
     if (ok && lane == 0 && bytes > 0 && cluster < rows) issue(cluster);
 
+    // Where a wait gives up, the copy of this warp's next piece that is in flight has to land first (the warps that wait for this
+    // one's pair give up as well).
     uint32_t it = 0;
-    for (long long row = cluster; row < rows; row += n_clusters, ++it) {
-        if (ok && bytes > 0) ok = warp_wait(ptx::smem_u32(&ctl->full[warp]), it & 1u, abort_flag, kSiteRcRowLoad);
-        if (!ok) break;  // (the warps that wait for this one's pair give up as well)
+    for (long long row = cluster; ok && row < rows; row += n_clusters, ++it) {
+        if (bytes > 0) ok = warp_wait(ptx::smem_u32(&ctl->full[warp]), it & 1u, abort_flag, kSiteRcRowLoad);
+        if (!ok) {
+            drain_copy(ptx::smem_u32(&ctl->full[warp]), it & 1u);
+            break;
+        }
         float4 v[kRcVecPerThread];
         float m = -INFINITY;
         if (full) {  // the common case, free of per-vector bounds checks
@@ -335,7 +351,10 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
         __syncwarp();
         if (warp == 0) {
             ok = warp_wait(ptx::smem_u32(&ctl->pieces_in[par]), phase, abort_flag, kSiteRcExchange);
-            if (!ok) break;
+            if (!ok) {
+                if (bytes > 0 && row + n_clusters < rows) drain_copy(ptx::smem_u32(&ctl->full[warp]), (it + 1) & 1u);
+                break;
+            }
             const float2 p = ctl->piece[par][lane & (kWarpsRc - 1)];
             float pm = p.x;
 #pragma unroll
@@ -349,7 +368,10 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
             if (lane == 0) ptx::mbar_expect_tx(&ctl->pairs_in[par], static_cast<uint32_t>(C) * 8u);
         }
         ok = warp_wait(ptx::smem_u32(&ctl->pairs_in[par]), phase, abort_flag, kSiteRcExchange);
-        if (!ok) break;
+        if (!ok) {
+            if (bytes > 0 && row + n_clusters < rows) drain_copy(ptx::smem_u32(&ctl->full[warp]), (it + 1) & 1u);
+            break;
+        }
         // every warp reduces the CTAs' pairs, in the same order
         const float2 pair = (lane & 15) < C ? ctl->xch[par][lane & 15] : make_float2(-INFINITY, 0.0f);
         float M = pair.x;
@@ -377,6 +399,13 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
     if (C > 1) {  // no CTA leaves while a peer may still write into its control block
         ptx::cluster_arrive_release();
         ptx::cluster_wait_acquire();
+    }
+    if (!ok) {
+        // Pairs that peers sent to a CTA that did not wait for them: the barrier does not order them, but no more are sent behind
+        // it, and the last ones arrive within microseconds.
+        const long long t0 = clock64();
+        while (clock64() - t0 < kLatePairCycles) {
+        }
     }
 }
 
