@@ -32,6 +32,11 @@ static inline cudaError_t allow_smem(int bytes, bool large_clusters = false) {
 // has ended and its results are visible.  Every kernel launched this way waits before it touches global memory.
 // A kernel that takes tensor memory lets the one behind it begin (ptx::grid_launch_dependents) only once its CTA has it: a CTA of
 // that kernel on the same SM might otherwise take it first, then wait for this kernel, and keep it for good.
+// A kernel that does not call ptx::grid_launch_dependents lets the kernel behind begin as its own CTAs end, and still saves most of
+// the gap.  So do the row kernels of more than 8192 columns: several of their CTAs fit an SM, so those of the kernel behind would
+// begin beside the ones that work and lie unevenly when their turn comes, and each has a fixed share of the rows.  us per call, calling it at
+// the begin -> not at all (without overlap): two-read bfloat16 3937 x 43008 217 -> 186 (189), float32 5081 x 40632 317 -> 296 (298), bfloat16
+// 60 x 36864 12.4 -> 6.2 (8.2); cluster bfloat16 300 x 44000 21.1 -> 17.3 (19.3); shared memory bfloat16 500 x 30000 24.5 -> 22.1 (24.7).
 // Back to back, small calls took 2 us more each: 4096 x 1000 float32 row Softmax 6.2 -> 4.6 us, attention of 2 x 128 8.2 -> 5.4,
 // projection of 64 rows 8.2 -> 5.3, weights of one head of 256 8.4 -> 6.5.
 // `cluster` CTAs form a cluster; `cooperative`: the whole grid is resident at once, or the launch fails.

@@ -163,8 +163,7 @@ softmax_rows_stream_kernel(const float* S, OutT* P, long long rows, long long co
     constexpr int kWarps = THREADS / 32;
     __shared__ float red_m[kWarps];
     __shared__ float red_l[kWarps];
-    ptx::grid_launch_dependents();
-    ptx::grid_dependency_wait();
+    ptx::grid_dependency_wait();  // (no grid_launch_dependents: see launch_overlapped)
     const long long nvec = cols >> 2;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 

@@ -79,7 +79,6 @@ softmax_rows_smem_kernel(const float* S, OutT* P, long long rows, long long cols
     const int n = static_cast<int>(c0 >= cols ? 0 : (cols - c0 < slice_cols ? cols - c0 : slice_cols));  // its length
     const int nvec = n >> 2;
 
-    ptx::grid_launch_dependents();
     if (threadIdx.x == 0) {
         ptx::grid_dependency_wait();
         const uint32_t prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);  // (arrives meanwhile)
@@ -262,7 +261,6 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
     const uint32_t bytes = static_cast<uint32_t>(v1 - v0) * 16u;
     const bool full = v1 - v0 == kRcVecPerThread * 32;  // this warp's piece has all its 256 vectors
 
-    ptx::grid_launch_dependents();
     if (threadIdx.x == 0) {
         ptx::grid_dependency_wait();
         const uint32_t prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);  // (arrives meanwhile)
