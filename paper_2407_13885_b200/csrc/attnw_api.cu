@@ -744,16 +744,18 @@ int launch_project(const DeviceInfo* dev, const void* X, const void* Wq, const v
     if (rc == ATTNW_OK) rc = encode_3d(&m.q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Q, d, N, static_cast<uint64_t>(B) * H, 64, 128);
     if (rc == ATTNW_OK) rc = encode_3d(&m.k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, d, N, static_cast<uint64_t>(B) * H, 64, 128);
     if (rc != ATTNW_OK) return rc;
-    // Rounds of tiles on the device times the cost of a tile: a tile of a half or a quarter of the work takes 0.55 or 0.32 of
-    // the time, since it fetches more bytes a flop.  Measured, us per call, 256 x 256 / 128 x 256 / 128 x 128 tiles, for
-    // B x N x d_model to H x d: 1 x 1024 x 1024 to 16 x 64 (32 / 64 / 128 tiles) 17.6 / 12.5 / 10.4, 1 x 146 x 1080 to 29 x 128
-    // 18.6 / 16.6 / 13.5, 1 x 512 x 4096 to 32 x 128 (64 / 128 / 256) 47.7 / 38.5 / 45.2, 2 x 469 x 3840 to 60 x 64
-    // (120 / 240 / 480) 54.9 / 61.4 / 77.8, 4 x 4096 x 4096 to 32 x 128 837 / 923 / 1199.
+    // Rounds of tiles on the device times the cost of a round: one of tiles of a half or a quarter of the work takes 0.6 or 0.44 of
+    // the time, since they fetch more bytes a flop.  Measured, us per call, 256 x 256 / 128 x 256 / 128 x 128 tiles, for
+    // B x N x d_model to H x d: 1 x 1000 x 1024 to 16 x 64 (32 / 64 / 128 tiles) 19.0 / 11.8 / 9.9, 1 x 763 x 2816 to 22 x 128
+    // (66 / 132 / 264) 33.7 / 22.0 / 29.1, 2 x 1377 x 1024 to 8 x 128 (96 / 176 / 352) 16.4 / 18.1 / 21.8, 1 x 2109 x 2432 to 19 x 128
+    // (180 / 340 / 646) 61.1 / 53.6 / 67.0, 4 x 2825 x 1664 to 13 x 128 (672 / 1288 / 2392) 118 / 130 / 190, 4 x 4096 x 4096 to 32 x 128 804 /
+    // 861 / 1317.  Over 70 drawn sizes the choice is the fastest but for one (3 %); with 0.55 and 0.32 it was up to 33 % slower
+    // than 256 x 256 tiles.
     auto cost = [&](int rb, int cb, double per_tile) {
         const long long tiles = 2 * ((static_cast<long long>(hd) + 128 * cb - 1) / (128 * cb)) * ((N + 128 * rb - 1) / (128 * rb)) * B;
         return static_cast<double>((tiles + dev->sm_count - 1) / dev->sm_count) * per_tile;
     };
-    const double c22 = cost(2, 2, 1.0), c12 = cost(1, 2, 0.55), c11 = cost(1, 1, 0.32);
+    const double c22 = cost(2, 2, 1.0), c12 = cost(1, 2, 0.6), c11 = cost(1, 1, 0.44);
     if (c22 <= c12 && c22 <= c11) return launch_project_tile<2, 2>(m, B, N, d_model, H, d, stream);
     if (c12 <= c11) return launch_project_tile<1, 2>(m, B, N, d_model, H, d, stream);
     return launch_project_tile<1, 1>(m, B, N, d_model, H, d, stream);
