@@ -188,7 +188,6 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     if (warp == kMma) {
         ptx::tmem_alloc(&bars->tmem_base, kTmemCols);
         ptx::tmem_relinquish();
-        ptx::grid_launch_dependents();  // not before this CTA has its tensor memory (launch_overlapped)
     }
     ptx::grid_dependency_wait();
     ptx::tc_fence_before_sync();

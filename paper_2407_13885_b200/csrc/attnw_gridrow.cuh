@@ -260,11 +260,6 @@ attnw_gridrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     if (warp == kMmaWarpG) {
         ptx::tmem_alloc(&bars->tmem_base, kTmemCols);
         ptx::tmem_relinquish();
-        // Not before this CTA has its tensor memory (launch_overlapped).  Clusters of 3 and 5 say it by ending: those of the kernel
-        // behind, placed one by one as others leave, would not all find their SMs (bfloat16 82 x 752 46.3 us per call, now 30.3, and
-        // 32.7 without overlap; 43 x 752 29.8, 18.1, 20.5; 15 x 1280 23.2, 18.5, 20.5).  The other sizes gain by saying it early:
-        // 24 x 1000 18.5 -> 18.0, 1 x 256 7.2 -> 6.8.
-        if (group_ctas != 3 && group_ctas != 5) ptx::grid_launch_dependents();
     }
     ptx::grid_dependency_wait();
     ptx::tc_fence_before_sync();

@@ -27,18 +27,17 @@ static inline cudaError_t allow_smem(int bytes, bool large_clusters = false) {
     return e;
 }
 
-// Launches `kernel` so that it may begin before the kernel in front of it on the stream has ended: its CTAs take the SMs as that
-// kernel's CTAs leave them, set up their barriers and tensor memory, and wait (ptx::grid_dependency_wait) until the kernel
-// has ended and its results are visible.  Every kernel launched this way waits before it touches global memory.
-// A kernel that takes tensor memory lets the one behind it begin (ptx::grid_launch_dependents) only once its CTA has it: a CTA of
-// that kernel on the same SM might otherwise take it first, then wait for this kernel, and keep it for good.
-// A kernel that does not call ptx::grid_launch_dependents lets the kernel behind begin as its own CTAs end, and still saves most of
-// the gap.  So do the row kernels of more than 8192 columns: several of their CTAs fit an SM, so those of the kernel behind would
-// begin beside the ones that work and lie unevenly when their turn comes, and each has a fixed share of the rows.  us per call, calling it at
-// the begin -> not at all (without overlap): two-read bfloat16 3937 x 43008 217 -> 186 (189), float32 5081 x 40632 317 -> 296 (298), bfloat16
-// 60 x 36864 12.4 -> 6.2 (8.2); cluster bfloat16 300 x 44000 21.1 -> 17.3 (19.3); shared memory bfloat16 500 x 30000 24.5 -> 22.1 (24.7).
-// Back to back, small calls took 2 us more each: 4096 x 1000 float32 row Softmax 6.2 -> 4.6 us, attention of 2 x 128 8.2 -> 5.4,
-// projection of 64 rows 8.2 -> 5.3, weights of one head of 256 8.4 -> 6.5.
+// Launches `kernel` so that it may begin as soon as every CTA of the kernel in front on the stream has ended: what lies between the
+// end of one kernel and the begin of the next runs beside its set-up, and it waits (ptx::grid_dependency_wait) until the results in
+// front are visible.  Every kernel launched this way waits before it touches global memory.  Back to back, small calls took about 2 us
+// more each: 4096 x 1000 float32 row Softmax 6.2 -> 4.6 us, attention of 2 x 128 8.2 -> 5.9, projection of 64 rows 6.2 -> 4.3, weights
+// of one head of 256 8.6 -> 7.2.
+// No kernel lets the one behind begin earlier (griddepcontrol.launch_dependents).  Its CTAs would take room as CTAs of the kernel in front
+// leave it, not evenly, where each has a fixed share of the work, and clusters would not all find their SMs.  us, two calls one behind the
+// other, early / as now / without overlap: rows 1000 x 131072 behind weights of 24 x 1000 236 / 160 / 162, rows 600 x 44000 behind 9 x 256
+// 55.9 / 39.1 / 43.3, weights of 82 x 752 behind themselves 46.3 / 30.3 / 32.7.  It saved another 0.3 to 0.5 us between the smallest
+// calls of the tensor-core kernels (one head of 256 7.2 -> 6.8), and it has to come after a CTA has its tensor memory: a CTA of the
+// kernel behind on the same SM might otherwise take that first, then wait for this kernel, and keep it for good.
 // `cluster` CTAs form a cluster; `cooperative`: the whole grid is resident at once, or the launch fails.
 template <typename... Params, typename... Args>
 inline cudaError_t launch_overlapped(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream,

@@ -106,7 +106,6 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     if (warp == kMma) {
         ptx::tmem_alloc(&bars->tmem_base, L::kTmemCols);
         ptx::tmem_relinquish();
-        ptx::grid_launch_dependents();  // not before this CTA has its tensor memory (launch_overlapped)
     }
     ptx::grid_dependency_wait();
     ptx::tc_fence_before_sync();

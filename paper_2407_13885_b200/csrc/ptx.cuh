@@ -27,8 +27,6 @@ __device__ __forceinline__ bool elect_one() {
 // ---- programmatic dependent launch (launch_overlapped) ----------------------------------------
 // Until the kernel in front on the stream has ended and its writes are visible (no-op after an ordinary launch).
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// The kernel behind on the stream may be given the SMs that this kernel's CTAs leave, once every CTA has said so.
-__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---- mbarrier ------------------------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {

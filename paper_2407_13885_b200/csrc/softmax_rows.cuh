@@ -91,7 +91,6 @@ softmax_rows_reg_kernel(const float* S, OutT* P, long long rows, int cols) {
     __shared__ float red_max[TPR > 32 ? TPR / 32 : 1];
     __shared__ float red_sum[TPR > 32 ? TPR / 32 : 1];
 
-    ptx::grid_launch_dependents();
     ptx::grid_dependency_wait();
     const int nvec = cols >> 2;
     const int sub = threadIdx.x % TPR;          // position inside the row group
@@ -163,7 +162,7 @@ softmax_rows_stream_kernel(const float* S, OutT* P, long long rows, long long co
     constexpr int kWarps = THREADS / 32;
     __shared__ float red_m[kWarps];
     __shared__ float red_l[kWarps];
-    ptx::grid_dependency_wait();  // (no grid_launch_dependents: see launch_overlapped)
+    ptx::grid_dependency_wait();
     const long long nvec = cols >> 2;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
