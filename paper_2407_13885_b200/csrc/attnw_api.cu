@@ -963,11 +963,12 @@ int rows_entry(const void* S, void* P, long long rows, long long cols, void* str
         (void)cudaGetLastError();  // no cluster of that size on this device: fall through to the two-read kernel
         if (variant == 1) return ATTNW_ERR_UNSUPPORTED;
     }
-    // Rows of 43009 to 262144 columns, and from 32769 where there are fewer rows than SMs: kept in the registers of a
-    // cluster, one read and one write per element.  With many rows of up to 43008 columns the slices of a cluster of three are
-    // short and the two-read kernel is ahead (6000 x 36864: 256 against 269 us, x 40960: 277 against 292, x 45000: 357 against
-    // 315); with few, it has one CTA a row (10 x 40000: 7.0 against 5.3).
-    const bool few_rows = cols > kSoftmaxRowsRegTierMaxCols && rows <= dev->sm_count;
+    // Rows of 43009 to 262144 columns, and from 32769 where rows are few: kept in the registers of a cluster, one read and
+    // one write per element.  With many rows of up to 43008 columns the slices of a cluster of three are short and the two-read
+    // kernel is ahead (6000 x 36864: 256 against 269 us, x 40960: 277 against 292, x 45000: 357 against 315); with few it has one CTA a
+    // row where the clusters have three SMs.  us, two-read / cluster: bfloat16 10, 37, 49, 74, 148 x 36864 6.1 / 5.0, 6.2 / 5.1, 6.3 / 6.2,
+    // 6.3 / 6.5, 7.1 / 9.4, x 43008 6.9 / 5.1, 7.0 / 5.2, 7.0 / 6.4, 7.1 / 6.7, 8.3 / 9.8; float32 37, 49 x 32772 6.4 / 5.7, 6.4 / 7.3.
+    const bool few_rows = cols > kSoftmaxRowsRegTierMaxCols && rows <= dev->sm_count / 4;
     if (variant == 0 && (cols > kSoftmaxRowsRegClusterMinCols || few_rows) && cols <= srs::kRcMaxCols) {
         const int C = srs::rc_cluster_ctas_for(cols);
         const cudaError_t ce = srs::launch_regcluster<OutT>(static_cast<const float*>(S), static_cast<OutT*>(P), rows, cols,

@@ -147,9 +147,9 @@ def test_bad_arguments_on_device(attnw):
     assert e.value.code == 7
 
 
-# the cluster tier at its edges: few rows from 32769 columns on (more than one per SM: the two-read kernel), 43009 columns, each
+# the cluster tier at its edges: few rows from 32769 columns on (more than one per four SMs: the two-read kernel), 43009 columns, each
 # cluster size with a slice that is cut, warps and a whole CTA without columns, more rows than clusters
-@pytest.mark.parametrize("rows,cols", [(3, 32772), (149, 32772), (2, 43008), (200, 43012), (97, 49156), (5, 65540), (75, 81924), (3, 98308),
+@pytest.mark.parametrize("rows,cols", [(3, 32772), (37, 36864), (38, 36864), (149, 32772), (2, 43008), (200, 43012), (97, 49156), (5, 65540), (75, 81924), (3, 98308),
                                        (2, 114692), (40, 131076), (2, 163844), (23, 212996), (2, 262144)])
 def test_cluster_tier_edges(attnw, rows, cols):
     S = inputs.normal_f32(11, rows * 149 + cols, rows * cols, 3.0).reshape(rows, cols)
