@@ -38,11 +38,11 @@ static inline cudaError_t allow_smem(int bytes, bool large_clusters = false) {
 // 55.9 / 39.1 / 43.3, weights of 82 x 752 behind themselves 46.3 / 30.3 / 32.7.  It saved another 0.3 to 0.5 us between the smallest
 // calls of the tensor-core kernels (one head of 256 7.2 -> 6.8), and it has to come after a CTA has its tensor memory: a CTA of the
 // kernel behind on the same SM might otherwise take that first, then wait for this kernel, and keep it for good.
-// `cluster` CTAs form a cluster; `cooperative`: the whole grid is resident at once, or the launch fails.
+// `cluster` CTAs form a cluster.
 template <typename... Params, typename... Args>
 inline cudaError_t launch_overlapped(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream,
-                                     int cluster, bool cooperative, Args... args) {
-    cudaLaunchAttribute attr[3];
+                                     int cluster, Args... args) {
+    cudaLaunchAttribute attr[2];
     unsigned n = 0;
     attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[n++].val.programmaticStreamSerializationAllowed = 1;
@@ -51,10 +51,6 @@ inline cudaError_t launch_overlapped(void (*kernel)(Params...), unsigned grid, u
         attr[n].val.clusterDim.x = static_cast<unsigned>(cluster);
         attr[n].val.clusterDim.y = 1;
         attr[n++].val.clusterDim.z = 1;
-    }
-    if (cooperative) {
-        attr[n].id = cudaLaunchAttributeCooperative;
-        attr[n++].val.cooperative = 1;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid, 1, 1);
