@@ -452,7 +452,7 @@ int enqueue_gridrow(const GridrowShape& g, const void* Q, const void* K, void* P
     cudaError_t launched;
     if (g.group_ctas == 1 || g.clusters) {
         launched = launch_overlapped(kernel, static_cast<unsigned>(g.n_groups * g.group_ctas), gr::kThreads, L::kDynamicBytes, stream,
-                                     g.group_ctas, false, tm_q, tm_k, tm_p, N, g.total_items, g.group_ctas, g.n_groups, scale_log2e, xchg,
+                                     g.group_ctas, tm_q, tm_k, tm_p, N, g.total_items, g.group_ctas, g.n_groups, scale_log2e, xchg,
                                      tag_base);
     } else {
         // Not overlapped: CTAs that wait for the kernel in front while another stream's cooperative grid holds the other SMs
@@ -662,7 +662,7 @@ int launch_attn_onepass(DeviceInfo* dev, const void* Q, const void* K, const voi
                   : mode == av1::kSplit ? av1::attn_onepass_kernel<D, av1::kSplit>
                                         : av1::attn_onepass_kernel<D, av1::kCluster>;
     if (allowed != cudaSuccess ||
-        launch_overlapped(kernel, static_cast<unsigned>(BH * row_blocks * ctas), L::kThreads, L::kDynamicBytes, stream, ctas, false, tm_q,
+        launch_overlapped(kernel, static_cast<unsigned>(BH * row_blocks * ctas), L::kThreads, L::kDynamicBytes, stream, ctas, tm_q,
                           tm_k, tm_v, tm_o, N, row_blocks, scale_log2e, static_cast<__nv_bfloat16*>(O), ctas) != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
@@ -725,7 +725,7 @@ int launch_project_tile(const ProjectMaps& m, int B, int N, int d_model, int H, 
     const int col_tiles = static_cast<int>((static_cast<long long>(H) * d + L::kCols - 1) / L::kCols);
     const int row_tiles = (N + L::kRows - 1) / L::kRows;
     const unsigned ctas = static_cast<unsigned>(2 * col_tiles) * static_cast<unsigned>(row_tiles) * static_cast<unsigned>(B);
-    if (launch_overlapped(proj::project_qk_kernel<RB, CB>, ctas, proj::kThreads, L::kDynamicBytes, stream, 1, false, m.x, m.wq, m.wk, m.q, m.k,
+    if (launch_overlapped(proj::project_qk_kernel<RB, CB>, ctas, proj::kThreads, L::kDynamicBytes, stream, 1, m.x, m.wq, m.wk, m.q, m.k,
                           N, d_model, H, d, col_tiles, row_tiles) != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;

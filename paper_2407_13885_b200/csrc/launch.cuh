@@ -34,8 +34,8 @@ static inline cudaError_t allow_smem(int bytes, bool large_clusters = false) {
 // of one head of 256 8.6 -> 7.2.
 // No kernel lets the one behind begin earlier (griddepcontrol.launch_dependents).  Its CTAs would take room as CTAs of the kernel in front
 // leave it, not evenly, where each has a fixed share of the work, and clusters would not all find their SMs.  us, two calls one behind the
-// other, early / as now / without overlap: rows 1000 x 131072 behind weights of 24 x 1000 236 / 160 / 162, rows 600 x 44000 behind 9 x 256
-// 55.9 / 39.1 / 43.3, weights of 82 x 752 behind themselves 46.3 / 30.3 / 32.7.  It saved another 0.3 to 0.5 us between the smallest
+// other, early / as now / without overlap: rows 1000 x 131072 behind weights of 24 x 1000 236 / 157 / 162, rows 600 x 44000 behind 9 x 256
+// 55.9 / 39.7 / 43.9, weights of 82 x 752 behind themselves 46.3 / 30.3 / 32.7.  It saved another 0.3 to 0.5 us between the smallest
 // calls of the tensor-core kernels (one head of 256 7.2 -> 6.8), and it has to come after a CTA has its tensor memory: a CTA of the
 // kernel behind on the same SM might otherwise take that first, then wait for this kernel, and keep it for good.
 // `cluster` CTAs form a cluster.

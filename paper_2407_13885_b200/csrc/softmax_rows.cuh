@@ -243,7 +243,7 @@ inline cudaError_t sr_launch_reg(const float* S, OutT* P, long long rows, int co
     auto kernel = mode == 1   ? softmax_rows_reg_kernel<TPR, VPT, OutT, 1>
                   : mode == 2 ? softmax_rows_reg_kernel<TPR, VPT, OutT, 2>
                               : softmax_rows_reg_kernel<TPR, VPT, OutT>;
-    return launch_overlapped(kernel, grid, kThreads, 0, stream, 1, false, S, P, rows, cols);
+    return launch_overlapped(kernel, grid, kThreads, 0, stream, 1, S, P, rows, cols);
 }
 
 constexpr long long kSoftmaxRowsRegTierMaxCols = 32768;
@@ -262,11 +262,11 @@ inline cudaError_t softmax_rows_launch(const float* S, OutT* P, long long rows, 
         if (row_bytes * sm_count * 2 <= (80ll << 20)) {
             const long long cap = static_cast<long long>(sm_count) * 2;
             const unsigned grid = static_cast<unsigned>(rows < cap ? rows : cap);
-            return launch_overlapped(softmax_rows_stream_kernel<OutT, 512>, grid, 512, 0, stream, 1, false, S, P, rows, cols);
+            return launch_overlapped(softmax_rows_stream_kernel<OutT, 512>, grid, 512, 0, stream, 1, S, P, rows, cols);
         } else {
             const long long cap = static_cast<long long>(sm_count);
             const unsigned grid = static_cast<unsigned>(rows < cap ? rows : cap);
-            return launch_overlapped(softmax_rows_stream_kernel<OutT, 1024>, grid, 1024, 0, stream, 1, false, S, P, rows, cols);
+            return launch_overlapped(softmax_rows_stream_kernel<OutT, 1024>, grid, 1024, 0, stream, 1, S, P, rows, cols);
         }
     }
     const int c = static_cast<int>(cols);

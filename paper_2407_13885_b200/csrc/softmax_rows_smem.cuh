@@ -193,7 +193,7 @@ inline cudaError_t launch_nt(const float* S, OutT* P, long long rows, long long 
     long long n_clusters = (per_sm * sm_count) / C;  // CTAs that fit at once
     if (n_clusters < 1) n_clusters = 1;
     if (n_clusters > rows) n_clusters = rows;
-    return launch_overlapped(softmax_rows_smem_kernel<OutT, NT>, static_cast<unsigned>(n_clusters * C), NT, smem, stream, C, false, S, P,
+    return launch_overlapped(softmax_rows_smem_kernel<OutT, NT>, static_cast<unsigned>(n_clusters * C), NT, smem, stream, C, S, P,
                              rows, cols, slice_cols, C);
 }
 
@@ -446,7 +446,7 @@ inline cudaError_t launch_regcluster(const float* S, OutT* P, long long rows, lo
     long long n_clusters = *resident_clusters;
     if (n_clusters > rows) n_clusters = rows;
     return launch_overlapped(kernel, static_cast<unsigned>(n_clusters * C), kRcThreads, kRcControlBytes + static_cast<size_t>(slice_cols) * 4,
-                             stream, C, false, S, P, rows, cols, slice_cols, C);
+                             stream, C, S, P, rows, cols, slice_cols, C);
 }
 
 }  // namespace srs
