@@ -54,7 +54,12 @@ typedef enum attnw_status {
  *          N % 4 == 0 for float32);  d in {64, 128}
  *   scale  finite, >= 0 (1/sqrt(d) in the paper); applied to the scores before the max
  * Scores are accumulated in float32 on the tensor cores; max, exponentials and sums are
- * float32; only P is rounded (to nearest even for bfloat16).
+ * float32; only P is rounded (to nearest even for bfloat16) - but for the exponentials of attnw_fused where the choice by
+ * shape takes the grid-row kernel (see attnw_set_fused_variant): they wait for the row's statistics as 16-bit floats,
+ * relative to the largest of some 64 scores of their row.  A bfloat16 weight down to 2^-29 of the largest weight of its row keeps
+ * bfloat16's digits; smaller ones may lose digits (the error stays below 2^-39 of the largest) and may be exactly zero below
+ * 2^-40.  Callers that take logarithms of such weights: attnw_fused_f32, or attnw_set_fused_variant(1), which keep float32's
+ * range to the end.
  */
 int attnw_fused(const void* Q, const void* K, void* P, int B, int H, int N, int d, float scale, void* stream);
 int attnw_fused_f32(const void* Q, const void* K, void* P, int B, int H, int N, int d, float scale, void* stream);

@@ -293,3 +293,33 @@ def test_chain_of_calls_sees_the_results_in_front(attnw):
         torch.cuda.synchronize()
         assert attnw.query_status() == 0
         assert torch.equal(got, want)
+
+
+# logits of sigma 16: weights far below the largest of their row
+@pytest.mark.parametrize("N,d", [(256, 64), (1000, 128), (2048, 64), (8192, 128)])
+def test_range_of_small_weights(attnw, N, d):
+    g = torch.Generator(device="cuda").manual_seed(N + 3 * d)
+    Q, K = (torch.randn(1, 1, N, d, generator=g, device="cuda", dtype=torch.bfloat16).mul_(4.0) for _ in range(2))
+    S = (Q[0, 0, :256].double() @ K[0, 0].double().T) * scale_of(d)
+    ref = torch.softmax(S, -1)
+    top = ref.amax(-1, keepdim=True)
+    size = (Q[0, 0, :256].double().abs() @ K[0, 0].double().abs().T) * scale_of(d)
+    bound = 2.0 ** -8 + 2.0 ** -10 + 2 * size * d * 2.0 ** -23  # relative, as in test_small_weights_keep_their_digits
+    assert bool((ref < top * 2.0 ** -60).any())
+
+    def error(P):
+        torch.cuda.synchronize()
+        assert attnw.query_status() == 0
+        return (P[0, 0, :256].double() - ref).abs()
+
+    # half of the smallest 16-bit float, 2^-25, next to the largest, 2^15: absolute, with a factor 2
+    assert bool((error(attnw.attnw_fused(Q, K, scale_of(d))) <= bound * ref + 2.0 ** -39 * top).all())
+    # float32 to the end: float32 weights, and the two-pass kernel
+    whole = ref >= top * 2.0 ** -100
+    assert bool((error(attnw.attnw_fused(Q, K, scale_of(d), out_dtype=torch.float32)) <= bound * ref)[whole].all())
+    attnw.set_fused_variant("two_pass")
+    try:
+        P = attnw.attnw_fused(Q, K, scale_of(d))
+    finally:
+        attnw.set_fused_variant("auto")
+    assert bool((error(P) <= bound * ref)[whole].all())
