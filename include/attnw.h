@@ -71,7 +71,7 @@ int attnw_fused_f32(const void* Q, const void* K, void* P, int B, int H, int N, 
  * Who needs it: code that runs where cudaMalloc is not allowed or not wanted - inside a framework whose memory pool
  * owns all device memory, in a real-time loop that must not take the allocator's lock or its implicit
  * synchronisation, or in a process that has handed the rest of the GPU's memory to someone else.  attnw_fused itself
- * allocates its exchange area with cudaMalloc the first time it runs the grid-row kernel on a device; this entry
+ * allocates an exchange area with cudaMalloc the first time it runs the grid-row kernel on a stream; this entry
  * point never calls cudaMalloc, cudaFree or any other allocating routine.  Its exchange area is a fixed array inside
  * the library's device image (3 MiB, present on every GPU that loads the library until the process exits).
  *
@@ -147,13 +147,17 @@ int attnw_set_attn_variant(int variant);
  *   3  the same kernel with the exchange the paper leaves as future work (Section VIII): the rows are dealt out to
  *      the CTAs of the cluster, the owner of a row receives its local maxima and sums, reduces them once and
  *      sends the global values to every CTA (reduce and broadcast) instead of every CTA reducing redundantly
- *   4  grid-row kernel: the SRAM-resident design on a cooperative grid of one CTA per SM.  Consecutive ceil(N/256)
- *      CTAs form a group (the cores of one grid row in Section VII) that owns a 128-row block; every CTA keeps the
+ *   4  grid-row kernel: the SRAM-resident design with one CTA per SM.  Consecutive ceil(N/256) CTAs form a group (the
+ *      cores of one grid row in Section VII; launched as clusters, or all together as a cooperative grid where clusters would
+ *      not reach enough SMs) that owns a 128-row block; every CTA keeps the
  *      exponentials of its 128 x 256 slab in tensor memory, with three row blocks in flight, and the local row maxima and
  *      sums cross the group through L2 as tagged 16-byte messages in an exchange area (3 MB) that belongs to the stream:
  *      one is allocated when a stream makes its first such call (cudaMalloc), up to eight per device, which further
- *      streams share in turn.  On a stream that is being captured the choice by shape (0) takes the other kernels
- *      for N > 256.  On request (4) it serves bfloat16 P and N <= 4096; any other call then returns ATTNW_ERR_UNSUPPORTED.
+ *      streams share in turn.  On a stream that is being captured the choice by shape (0) takes the older choice
+ *      for N > 256, since a replay would repeat its capture's tags; that is slower (bfloat16, us per call, uncaptured and
+ *      captured: 2 x 512 7.7 and 10.8, 12 x 2048 31 and 35, 12 x 4096 92 and 126, 128 x 4096 1215 and 1445, 8 x 8192 293 and 438).
+ *      attnw_fused_noalloc keeps the grid-row kernel in a capture.  On request (4) it serves bfloat16 P and N <= 4096, in a capture
+ *      N <= 256; any other call then returns ATTNW_ERR_UNSUPPORTED.
  * Returns ATTNW_ERR_BAD_SHAPE for any other value.
  */
 int attnw_set_fused_variant(int variant);

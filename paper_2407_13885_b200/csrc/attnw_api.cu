@@ -416,7 +416,8 @@ int gridrow_shape(DeviceInfo* dev, int BH, int N, int max_ctas, GridrowShape* ou
     // The CTAs of a group wait for one another, so they must be resident together: as a cluster, or with the whole grid
     // (cooperative).  Large clusters do not reach every SM (16 CTAs: 7 clusters, where 9 groups fit), but a cluster launch may
     // overlap the end of the kernel in front: taken where it needs no more rounds of row blocks.  us per call, cooperative ->
-    // clusters: 2 x 512 10.3 -> 7.2, 24 x 1000 20.5 -> 18.0, 3 x 1504 12.3 -> 10.3; with one round more (1 x 2048) 10.2 -> 10.5.
+    // clusters: 1 x 512 10.3 -> 7.6, 7 x 752 10.3 -> 8.1, 24 x 1000 20.5 -> 18.5, 7 x 1536 16.4 -> 14.8; with one round more (1 x 2048)
+    // 10.2 -> 10.5.
     out->clusters = false;
     if (C > 1 && C <= 16) {
         const int clusters = gridrow_max_clusters<D, OutT>(dev, C);
@@ -532,8 +533,8 @@ int gridrow_area(GridrowAreas* areas, int sm_count, cudaStream_t stream, Gridrow
     return ATTNW_OK;
 }
 
-// Grid-row kernel: a cooperative grid of one CTA per SM; consecutive ceil(N / 256) CTAs form a group that owns a
-// 128-row block and walks a contiguous part of the list of row blocks.  Returns ATTNW_ERR_UNSUPPORTED when the
+// Grid-row kernel: one CTA per SM; consecutive ceil(N / 256) CTAs, a cluster or a part of a cooperative grid, form a group that owns
+// a 128-row block and walks a contiguous part of the list of row blocks.  Returns ATTNW_ERR_UNSUPPORTED when the
 // device cannot hold a whole group at once, and for groups of several CTAs on a stream that is being captured.
 template <int D, typename OutT>
 int launch_gridrow(DeviceInfo* dev, const void* Q, const void* K, void* P, int BH, int N, float scale, cudaStream_t stream) {

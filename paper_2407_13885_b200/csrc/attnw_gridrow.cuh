@@ -17,15 +17,14 @@
 // range: the offset therefore leaves 2^15 of headroom above 1, which keeps those bits down to 2^-29 of the largest of a
 // chunk, and the row's factor is applied in float32.  (With the largest at 1 and an f16 factor, weights of 1e-9 .. 1e-6 were
 // 0.75 off in relative rms at N = 16384, logits of sigma 16; now 1.7e-3, the rounding of bf16.  It costs 0.5 %: 128 x 4096
-// 1090 and 1095 us, 12 x 2048 28.7 and 29.1.)
+// 1090 and 1095 us.)
 // Tensor memory, float32 output: two regions of 256 columns; the exponentials replace the scores as float32, and a slot of
 // 64 columns goes back to the MMA issuer when its weights have been read.
 //
 // The CTAs of a group wait for one another, so they must be resident together.  Large hardware clusters do not occupy
 // every SM (8 CTAs: 15 clusters of the device's 148 SMs, 16: 7), so large calls are launched cooperatively with one CTA per SM
-// and consecutive CTAs form a group; small ones, and groups of 2 to 4, are clusters, whose launch may overlap the kernel in
-// front (2 x 512 10.3 -> 8.2 us).  Either way the 16-byte (offset, sum) pair of a row
-// travels through L2 as two 8-byte words that each carry a tag {value, tag, value, tag}; a reader accepts a
+// and consecutive CTAs form a group; those that clusters serve in as few rounds are launched as clusters, whose launch may
+// overlap the kernel in front.  Either way the 16-byte (offset, sum) pair of a row travels through L2 as two 8-byte words that each carry a tag {value, tag, value, tag}; a reader accepts a
 // pair once both tags name the row block it is waiting for.  No fence, no flag, no atomics: the tag arrives
 // with the value in one 8-byte store.  Every poll is bounded.
 //   C = 1          no exchange: the pair stays in shared memory
@@ -50,8 +49,8 @@
 // which the special function unit works 2048 and the HBM stream of P would need 2800.  The sixteen exponential warps load,
 // reduce and store a slot together, so the unit rests in those phases (1100 of 2150 cycles a slot).  With 8 exponential
 // warps of 96 registers, one warp for a row's whole statistics and 16 pairs read by every CTA the same call took 1290 to
-// 1340 us in a loop at the power cap, now 1190 to 1240 (1130 -> 1100 at a burst); 12 x 2048 (d = 64) 34.8 -> 28.7,
-// 24 x 1000 24.5 -> 20.5.  Instructions count: the waits, votes and address arithmetic around the 3 + 1.6 a score cannot do
+// 1340 us in a loop at the power cap, now 1180 to 1240 (1130 -> 1100 at a burst); 12 x 2048 (d = 64) 34.8 -> 30.7,
+// 24 x 1000 24.5 -> 18.5.  Instructions count: the waits, votes and address arithmetic around the 3 + 1.6 a score cannot do
 // without had been as many again (10.8 a score, then 9.6), and every wait in front of the statistics adds to the time that a
 // block's exponentials must be parked, which three regions hide up to some 13000 cycles.
 //
