@@ -712,54 +712,39 @@ int validate_project(const void* X, const void* Wq, const void* Wk, const void* 
     return ATTNW_OK;
 }
 
-struct ProjectMaps {
-    CUtensorMap x, wq, wk, q, k;
-};
-
-template <int RB, int CB>
-int launch_project_tile(const ProjectMaps& m, int B, int N, int d_model, int H, int d, cudaStream_t stream) {
-    using L = proj::Tile<RB, CB>;
-    if (allow_smem<proj::project_qk_kernel<RB, CB>>(L::kDynamicBytes) != cudaSuccess) {
+int launch_project(const DeviceInfo* dev, const void* X, const void* Wq, const void* Wk, void* Q, void* K, int B, int N, int d_model,
+                   int H, int d, cudaStream_t stream) {
+    CUtensorMap tm_x, tm_wq, tm_wk, tm_q, tm_k;
+    const uint64_t hd = static_cast<uint64_t>(H) * d, bh = static_cast<uint64_t>(B) * H;
+    int rc = encode_3d(&tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, d_model, N, B, proj::kKSlice, proj::kRows);
+    if (rc == ATTNW_OK) rc = encode_3d(&tm_wq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Wq, d_model, hd, 1, proj::kKSlice, proj::kFeatures / 2);
+    if (rc == ATTNW_OK) rc = encode_3d(&tm_wk, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Wk, d_model, hd, 1, proj::kKSlice, proj::kFeatures / 2);
+    if (rc == ATTNW_OK) rc = encode_3d(&tm_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Q, d, N, bh, 64, 32);
+    if (rc == ATTNW_OK) rc = encode_3d(&tm_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, d, N, bh, 64, 32);
+    if (rc != ATTNW_OK) return rc;
+    if (allow_smem<proj::project_qk_kernel>(proj::kDynamicBytes) != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
     }
-    const int col_tiles = static_cast<int>((static_cast<long long>(H) * d + L::kCols - 1) / L::kCols);
-    const int row_tiles = (N + L::kRows - 1) / L::kRows;
-    const unsigned ctas = static_cast<unsigned>(2 * col_tiles) * static_cast<unsigned>(row_tiles) * static_cast<unsigned>(B);
-    if (launch_overlapped(proj::project_qk_kernel<RB, CB>, ctas, proj::kThreads, L::kDynamicBytes, stream, 1, m.x, m.wq, m.wk, m.q, m.k,
-                          N, d_model, H, d, col_tiles, row_tiles) != cudaSuccess) {
+    // Tiles of 256 x 256 per pair of CTAs; narrow ones of 256 x 128 where a single round of them holds the call, since a narrow slice still takes
+    // 0.6 to 0.75 of the time of a whole one (X's rows are fetched for half of the MMAs).  A last round whose tiles would occupy at most
+    // half of the pairs takes them cut in two.  us per call, whole tiles only -> as chosen: narrow 4 x 100 x 1536 to 12 x 128 11.3 -> 7.7,
+    // 1 x 1000 x 1024 to 16 x 64 9.3 -> 6.7, 2 x 949 x 576 to 9 x 64 7.2 -> 5.7, 1 x 256 x 4096 to 64 x 64 24.9 -> 21.2; last round 1 x 2048 x
+    // 4096 to 32 x 128 (256 tiles for 74 pairs) 111.8 -> 107.6, 2 x 444 x 3200 to 25 x 128 (100) 40.7 -> 37.4, 4 x 3749 x 4080 to 10 x 64 (300) 142.5 -> 140.8.
+    const int pairs = dev->sm_count / 2;
+    const int block = proj::Grid(B, N, static_cast<int>(hd), proj::kFeatures / 2).tiles() <= pairs ? proj::kFeatures / 2 : proj::kFeatures;
+    const proj::Grid g(B, N, static_cast<int>(hd), block);
+    const int tiles = g.tiles(), last = tiles % pairs;
+    const int whole = block == proj::kFeatures && 2 * last <= pairs ? tiles - last : tiles;
+    const int items = 2 * tiles - whole;
+    const int clusters = items < pairs ? items : pairs;
+    if (launch_overlapped(proj::project_qk_kernel, 2 * static_cast<unsigned>(clusters), proj::kThreads, proj::kDynamicBytes, stream, 2, tm_x,
+                          tm_wq, tm_wk, tm_q, tm_k, B, N, d_model, H, d, block, whole) != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;
     }
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return ATTNW_OK;
-}
-
-int launch_project(const DeviceInfo* dev, const void* X, const void* Wq, const void* Wk, void* Q, void* K, int B, int N, int d_model,
-                   int H, int d, cudaStream_t stream) {
-    ProjectMaps m;
-    const uint64_t hd = static_cast<uint64_t>(H) * d;
-    int rc = encode_3d(&m.x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, d_model, N, B, proj::kKSlice, 128);
-    if (rc == ATTNW_OK) rc = encode_3d(&m.wq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Wq, d_model, hd, 1, proj::kKSlice, 128);
-    if (rc == ATTNW_OK) rc = encode_3d(&m.wk, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Wk, d_model, hd, 1, proj::kKSlice, 128);
-    if (rc == ATTNW_OK) rc = encode_3d(&m.q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Q, d, N, static_cast<uint64_t>(B) * H, 64, 128);
-    if (rc == ATTNW_OK) rc = encode_3d(&m.k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, d, N, static_cast<uint64_t>(B) * H, 64, 128);
-    if (rc != ATTNW_OK) return rc;
-    // Rounds of tiles on the device times the cost of a round: one of tiles of a half or a quarter of the work takes 0.6 or 0.44 of
-    // the time, since they fetch more bytes a flop.  Measured, us per call, 256 x 256 / 128 x 256 / 128 x 128 tiles, for
-    // B x N x d_model to H x d: 1 x 1000 x 1024 to 16 x 64 (32 / 64 / 128 tiles) 19.0 / 11.8 / 9.9, 1 x 763 x 2816 to 22 x 128
-    // (66 / 132 / 264) 33.7 / 22.0 / 29.1, 2 x 1377 x 1024 to 8 x 128 (96 / 176 / 352) 16.4 / 18.1 / 21.8, 1 x 2109 x 2432 to 19 x 128
-    // (180 / 340 / 646) 61.1 / 53.6 / 67.0, 4 x 2825 x 1664 to 13 x 128 (672 / 1288 / 2392) 118 / 130 / 190, 4 x 4096 x 4096 to 32 x 128 804 /
-    // 861 / 1317.  Over 70 drawn sizes the choice is the fastest but for one (3 %); with 0.55 and 0.32 it was up to 33 % slower
-    // than 256 x 256 tiles.
-    auto cost = [&](int rb, int cb, double per_tile) {
-        const long long tiles = 2 * ((static_cast<long long>(hd) + 128 * cb - 1) / (128 * cb)) * ((N + 128 * rb - 1) / (128 * rb)) * B;
-        return static_cast<double>((tiles + dev->sm_count - 1) / dev->sm_count) * per_tile;
-    };
-    const double c22 = cost(2, 2, 1.0), c12 = cost(1, 2, 0.6), c11 = cost(1, 1, 0.44);
-    if (c22 <= c12 && c22 <= c11) return launch_project_tile<2, 2>(m, B, N, d_model, H, d, stream);
-    if (c12 <= c11) return launch_project_tile<1, 2>(m, B, N, d_model, H, d, stream);
-    return launch_project_tile<1, 1>(m, B, N, d_model, H, d, stream);
 }
 
 // Whether the choice by shape takes the grid-row kernel for rows of N keys: it computes every score and exponential once, the

@@ -3,228 +3,354 @@
 // matmul and names as a step to bring into its own code (Section VIII).  The output is written head-major
 // ([B, H, N, d], bf16), exactly what attnw_fused and attn_fused read, so no transposition pass is needed.
 //
-// A plain dense contraction, so it runs on the tensor cores: a CTA owns a 256 x 256 tile of one of the two
-// outputs (256 rows of one batch entry x 256 output features = 2 or 4 heads), four 128 x 128 fp32 accumulators in
-// tensor memory (all 512 columns), a 3-stage TMA ring of [256 x 64] slices of X and of the weights (64 KB a stage),
-// tcgen05 MMAs of shape 128 x 256 x 16.  Smaller calls take tiles of 128 x 256 or 128 x 128, which fill more SMs.  Weights are stored [H, d, d_model] (feature c of head h contiguous along
-// d_model), which is the K-major B operand TMA can deliver as it is.
+// A plain dense contraction, so it runs on the tensor cores, with the CTAs of a cluster of two as a pair (cta_group::2): a pair
+// computes 256 rows of X times 256 output features (2 or 4 heads; Q's features, then K's), each CTA 128 of the rows and all of the
+// features.  A CTA loads its rows and half of the features, so a byte of the operands in shared memory feeds twice the MMAs that it
+// feeds within one CTA.  A pair stays for several tiles: tensor memory holds two accumulators, and 8 warps turn one into bf16 and store it
+// while the tensor cores fill the other; the ring of 64-wide slices runs on from tile to tile.  launch_project chooses between whole
+// tiles, a last round cut in two, and narrow tiles.
+// Weights are stored [H, d, d_model] (feature c of head h contiguous along d_model), which is the K-major B operand TMA can deliver as it is.
+//
+// What bounds it: large calls, the tensor pipe (512 cycles a slice) under the power cap; small ones, the latency of set-up, first load,
+// epilogue and launch, some 5 us.  us per call, one CTA a tile of 256 x 256, 128 x 256 or 128 x 128 -> this kernel, B x N x d_model
+// to H x d: 4 x 4096 x 4096 to 32 x 128 823 -> 724 .. 805 (by the box's power), 4 x 2825 x 1664 to 13 x 128 128 -> 106, 2 x 2092 x 368 to 37 x
+// 64 28.6 -> 18.7, 1 x 2366 x 392 to 15 x 128 24.6 -> 13.5, 1 x 1000 x 1024 to 16 x 64 7.79 -> 6.66, 1 x 1757 x 768 to 12 x 64 8.17 -> 8.14; over 30
+// drawn sizes 1.15 times as fast, none slower.
+// What mattered in small calls: arrivals of the cluster's barrier and on the other CTA's mbarriers that order no memory (release costs
+// about 1000 cycles each: 6.86 -> 5.33 us at 2 x 64 x 256 to 4 x 64); the divisions of the tile list in front of the set-up's waits, not
+// of the first load (0.1 us); producers that a whole warp walks, with an elected lane, one for X and one for the weights (a lone lane took
+// 475 cycles a slice, that warp alone 330, two 300).  Tiles of 512 x 256 or 256 x 512, with one accumulator: 1 to 14 % slower.
 #pragma once
+#include <cstddef>
+
 #include "attnw_fused.cuh"
 
 namespace attnw {
 namespace proj {
 
-constexpr int kKSlice = 64;       // d_model elements per stage: one 128-byte swizzle atom
-constexpr int kGroupCols = 16;    // column tiles walked together (32 MB of weights at d_model = 4096)
-constexpr int kEpiWarps = 8;      // TMEM lane quarter (4) x column half (2)
-constexpr int kProducer = 8;
+constexpr int kKSlice = 64;          // d_model elements per stage: one 128-byte swizzle atom
+constexpr int kRows = 128;           // rows of X of a CTA
+constexpr int kFeatures = 128;       // features that a CTA loads for a whole tile (narrow tiles and halves: 64)
+constexpr int kGroupTiles = 16;      // column tiles walked together (32 MB of weights at d_model = 4096)
+constexpr int kEpiWarps = 8;         // TMEM lane quarter (4) x column half (2)
+constexpr int kProducerX = 8;
 constexpr int kMma = 9;
-constexpr int kThreads = 320;
-constexpr int kAtomBytes = 128 * 128;             // 128 rows x 128 bytes
-
-// A CTA's tile: RB blocks of 128 rows of X times CB blocks of 128 output features.
-template <int RB, int CB>
-struct Tile {
-    static constexpr int kRows = 128 * RB;
-    static constexpr int kCols = 128 * CB;
-    static constexpr int kStageBytes = (RB + CB) * kAtomBytes;  // the blocks of X, then the blocks of features
-    static constexpr int kStages = 12 / (RB + CB);              // 192 KB of stages
-    static constexpr int kBarOff = kStages * kStageBytes;
-    static constexpr int kDynamicBytes = kBarOff + 256 + 1024;
-    static constexpr int kTmemCols = kCols * RB;
-};
-static_assert(Tile<2, 2>::kDynamicBytes <= 227 * 1024 && Tile<1, 2>::kDynamicBytes <= 227 * 1024 &&
-              Tile<1, 1>::kDynamicBytes <= 227 * 1024, "shared memory budget");
+constexpr int kProducerW = 10;
+constexpr int kThreads = 352;
+constexpr int kAtomBytes = 128 * 128;           // 128 rows x 128 bytes
+constexpr int kRingBytes = 192 * 1024;          // stages of [64-wide] slices: the rows of X, then the features
+constexpr int kMaxStages = 6;
+constexpr int kSlots = 2;                       // accumulators in tensor memory
+constexpr int kSlotCols = kTmemCols / kSlots;
+constexpr int kOutOff = kRingBytes;  // one staged store box per epilogue warp: 32 rows x 64 features
+constexpr int kBarOff = kOutOff + kEpiWarps * kStageBoxBytes;
+constexpr int kDynamicBytes = kBarOff + 256 + 1024;
+static_assert(kDynamicBytes <= 227 * 1024, "shared memory budget");
 
 enum : uint32_t {  // wait sites of this kernel (low byte of the status word)
     kSiteProducerEmpty = 112,
     kSiteMmaFull = 113,
     kSiteEpiAcc = 114,
-    kSiteEpiFilled = 115,
+    kSiteMmaAccEmpty = 115,
 };
 
 struct Barriers {
-    uint64_t full[6], empty[6];
-    uint64_t acc_full;     // every MMA of the tile is complete
-    uint64_t out_filled;   // the 7 warps that do not issue the stores have staged their part of the tile
+    uint64_t full[kMaxStages], empty[kMaxStages];    // full: the even CTA's, for both
+    uint64_t acc_full[kSlots], acc_empty[kSlots];    // acc_empty: the even CTA's, for both
     uint32_t tmem_base;
     uint32_t abort_flag;
     uint32_t prior_failure;
+    int loads;  // stages that a producer has asked for
 };
 static_assert(sizeof(Barriers) <= 256, "barrier block must fit its slot");
 
-// grid: 2 * col_tiles * B * row_tiles CTAs.  The column tiles (Q's, then K's) are walked in groups of kGroupCols: within
-// a group the tiles of one block of rows are neighbours (that block of X is fetched once per group) and the group's
-// slice of the weights (kGroupCols x 256 x d_model) is small enough to stay in L2 while all row blocks pass.
-template <int RB, int CB>
+// The tiles of a call, the same arithmetic on the host and on the device.
+struct Grid {
+    int block;           // features that a CTA loads for a tile: kFeatures or half of that
+    int feature_blocks;  // blocks of Q's features, and as many of K's behind them = column tiles (two blocks each)
+    int row_blocks;      // blocks of kRows rows of a batch entry
+    int row_tiles;       // of two row blocks each, which may belong to different batch entries
+    __host__ __device__ Grid(int B, int N, int HD, int block_)
+        : block(block_), feature_blocks((HD - 1) / block_ + 1), row_blocks((N - 1) / kRows + 1), row_tiles((B * row_blocks + 1) / 2) {}
+    __host__ __device__ int tiles() const { return feature_blocks * row_tiles; }
+};
+
+// grid: clusters of two CTAs; pair p takes the items p, p + pairs, ...: the tiles 0 ... whole_tiles - 1, then the halves of the others.
 __global__ void __launch_bounds__(kThreads, 1)
 project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_wq,
                   const __grid_constant__ CUtensorMap tm_wk, const __grid_constant__ CUtensorMap tm_q,
-                  const __grid_constant__ CUtensorMap tm_k, int N, int d_model, int H, int d, int col_tiles, int row_tiles) {
-    using L = Tile<RB, CB>;
-    constexpr int kStages = L::kStages, kStageBytes = L::kStageBytes, kCols = L::kCols, kRows = L::kRows;
+                  const __grid_constant__ CUtensorMap tm_k, int B, int N, int d_model, int H, int d, int block, int whole_tiles) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    Barriers* bars = reinterpret_cast<Barriers*>(smem + L::kBarOff);
+    Barriers* bars = reinterpret_cast<Barriers*>(smem + kBarOff);
     volatile uint32_t* abort_flag = &bars->abort_flag;
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const int n_x = 2 * col_tiles, n_y = static_cast<int>(gridDim.x) / n_x;
-    const int n_groups = (n_x + kGroupCols - 1) / kGroupCols;
-    const int group = min(static_cast<int>(blockIdx.x) / (kGroupCols * n_y), n_groups - 1);
-    const int in_group = static_cast<int>(blockIdx.x) - group * kGroupCols * n_y;
-    const int width = group == n_groups - 1 ? n_x - group * kGroupCols : kGroupCols;
-    const int tile_x = group * kGroupCols + in_group % width;
-    const int tile_y = in_group / width;
-    const bool keys = tile_x >= col_tiles;  // this CTA computes a tile of K, not of Q
-    const int c0 = (tile_x - (keys ? col_tiles : 0)) * kCols;  // first output feature (of H * d)
-    const int b = tile_y / row_tiles;
-    const int r0 = (tile_y % row_tiles) * kRows;
+    const int rank = static_cast<int>(ptx::cluster_ctarank());
+    const Grid g(B, N, H * d, block);
+    const int items = 2 * g.tiles() - whole_tiles;
+    const int first = static_cast<int>(blockIdx.x) >> 1, pairs = static_cast<int>(gridDim.x) >> 1;
     const int KT = (d_model + kKSlice - 1) / kKSlice;
-    const CUtensorMap* tm_w = keys ? &tm_wk : &tm_wq;
-    const CUtensorMap* tm_out = keys ? &tm_k : &tm_q;
+    // The ring: six stages of one slice, or four of two narrow ones: a stage costs each of the issuing warps some 300 cycles, which the
+    // 256 of the MMAs of one narrow slice do not cover (1 x 512 x 4096 to 8 x 128 14.6 -> 13.3 us).
+    const int slice_bytes = kAtomBytes + block * 128;
+    const int slices = block == kFeatures ? 1 : 2;
+    const int stage_bytes = slices * slice_bytes;
+    const int stages = block == kFeatures ? kMaxStages : 4;
+    // The ring's stages in turn, and how often a stage has been used before, modulo 2.
+    struct Turn {
+        int s = 0;
+        uint32_t parity = 0;
+        __device__ __forceinline__ void next(int stages) {
+            if (++s == stages) {
+                s = 0;
+                parity ^= 1u;
+            }
+        }
+    };
+    // Column tiles are walked in groups: within a group the tiles of one block of rows are neighbours (that block of X is fetched once
+    // per group), and the group's slice of the weights is small enough to stay in L2 while all row blocks pass.
+    struct Item {
+        int block;    // the column tile's first block of features, of Q's, then of K's
+        int half;     // of the blocks; -1 = both halves
+        int row_tile;
+        int b, row;   // this CTA's rows: batch entry (B = none) and first row
+    };
+    auto item = [&](int t) {
+        Item r;
+        r.half = t < whole_tiles ? -1 : (t - whole_tiles) & 1;
+        if (t >= whole_tiles) t = whole_tiles + ((t - whole_tiles) >> 1);
+        const int groups = (g.feature_blocks + kGroupTiles - 1) / kGroupTiles;
+        const int group = groups == 1 ? 0 : min(t / (kGroupTiles * g.row_tiles), groups - 1);
+        const int in_group = t - group * kGroupTiles * g.row_tiles;
+        const int width = group == groups - 1 ? g.feature_blocks - group * kGroupTiles : kGroupTiles;
+        r.row_tile = in_group / width;
+        r.block = 2 * (group * kGroupTiles + in_group - r.row_tile * width);
+        const int rb = 2 * r.row_tile + rank;
+        r.b = rb / g.row_blocks;
+        r.row = (rb - r.b * g.row_blocks) * kRows;
+        return r;
+    };
+    // (the first one here: the divisions run beside the set-up, and not in front of the first load)
+    const Item first_item = item(first);
 
+    // ---- set-up ------------------------------------------------------------------------------
     if (threadIdx.x == 0) {
         ptx::grid_dependency_wait();
         const uint32_t prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);  // (arrives meanwhile)
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < stages; ++s) {
             ptx::mbar_init(&bars->full[s], 1);
             ptx::mbar_init(&bars->empty[s], 1);
         }
-        ptx::mbar_init(&bars->acc_full, 1);
-        ptx::mbar_init(&bars->out_filled, kEpiWarps - 1);
+        for (int s = 0; s < kSlots; ++s) {
+            ptx::mbar_init(&bars->acc_full[s], 1);
+            ptx::mbar_init(&bars->acc_empty[s], 2 * kEpiWarps);
+        }
         bars->abort_flag = 0;
+        bars->loads = 0;
         bars->prior_failure = prior_failure;
         ptx::mbar_fence_init();
     }
-    if (warp == kProducer && lane == 0) {
+    if (warp == kProducerX && lane == 0) {
         ptx::prefetch_tensormap(&tm_x);
-        ptx::prefetch_tensormap(tm_w);
-        ptx::prefetch_tensormap(tm_out);
+        ptx::prefetch_tensormap(&tm_wq);
+        ptx::prefetch_tensormap(&tm_wk);
+        ptx::prefetch_tensormap(&tm_q);
+        ptx::prefetch_tensormap(&tm_k);
     }
     if (warp == kMma) {
-        ptx::tmem_alloc(&bars->tmem_base, L::kTmemCols);
-        ptx::tmem_relinquish();
+        ptx::pair_tmem_alloc(&bars->tmem_base, kTmemCols);
+        ptx::pair_tmem_relinquish();
     }
     ptx::grid_dependency_wait();
     ptx::tc_fence_before_sync();
     __syncthreads();
+    ptx::cluster_arrive_relaxed();
+    ptx::cluster_wait_acquire();
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bars->tmem_base;
-    const bool run = bars->prior_failure == 0u;  // an earlier CTA gave up: do not queue more waits behind it
+    // an earlier launch gave up: do not queue more waits behind it (should the CTAs of a pair disagree, the waits of one run out)
+    const bool run = bars->prior_failure == 0u;
 
-    if (run && warp == kProducer) {
-        // ================= TMA producer: one 64-wide slice of X and one of the weights per stage =================
-        if (lane == 0) {
-            const uint64_t keep = ptx::policy_evict_last();
-            int kt = 0;
-            for (; kt < KT; ++kt) {
-                const int s = kt % kStages;
-                if (!fused_wait(&bars->empty[s], (static_cast<uint32_t>(kt / kStages) & 1u) ^ 1u, abort_flag, kSiteProducerEmpty)) break;
-                uint8_t* st = smem + s * kStageBytes;
-                ptx::mbar_expect_tx(&bars->full[s], static_cast<uint32_t>(kStageBytes));
-                // rows or features beyond the tensor's extent, and d_model's ragged tail, arrive as zeros
-                for (int m = 0; m < RB; ++m)
-                    ptx::tma_load_3d(st + m * kAtomBytes, &tm_x, &bars->full[s], kt * kKSlice, r0 + m * 128, b, keep);
-                for (int c = 0; c < CB; ++c)
-                    ptx::tma_load_3d(st + (RB + c) * kAtomBytes, tm_w, &bars->full[s], kt * kKSlice, c0 + c * 128, 0, keep);
-            }
-            if (*abort_flag) {
-                // Unwinding: let the copies already in flight land before shared memory is released.
-                const int first = kt > kStages ? kt - kStages : 0;
-                for (int it = first; it < kt; ++it) {
-                    const long long t0 = clock64();
-                    while (!ptx::mbar_try_wait(&bars->full[it % kStages], static_cast<uint32_t>(it / kStages) & 1u) &&
-                           clock64() - t0 < kWaitLimitCycles / 8) {
-                    }
-                }
-            }
-        }
-    } else if (run && warp == kMma) {
-        // ================= MMA issuer =================
-        constexpr uint32_t idesc = ptx::umma_idesc_bf16_f32(128, kCols);
-        const uint32_t base = ptx::smem_u32(smem);
+    if (run && (warp == kProducerX || warp == kProducerW)) {
+        // ================= TMA producers, of rows and of features: per stage a 64-wide slice =================
+        const bool for_rows = warp == kProducerX;
+        const uint64_t keep = ptx::policy_evict_last();
+        const uint32_t empty0 = ptx::smem_u32(&bars->empty[0]);
+        const uint32_t full0 = ptx::map_to_cta(ptx::smem_u32(&bars->full[0]), 0);
         bool ok = true;
-        for (int kt = 0; ok && kt < KT; ++kt) {
-            const int s = kt % kStages;
-            ok = __all_sync(0xffffffffu, fused_wait(&bars->full[s], static_cast<uint32_t>(kt / kStages) & 1u, abort_flag, kSiteMmaFull));
-            if (!ok) break;
+        Turn turn;
+        int n = 0;  // stages asked for
+        Item it = first_item;
+        for (int t = first; ok && t < items;) {
+            const int block = it.block + rank;
+            const bool keys = block >= g.feature_blocks;
+            const bool wide = it.half < 0 && g.block == kFeatures;
+            const CUtensorMap* map = for_rows ? &tm_x : keys ? &tm_wk : &tm_wq;
+            const int c1 = for_rows ? it.row : (keys ? block - g.feature_blocks : block) * g.block + (it.half == 1 ? kFeatures / 2 : 0);
+            const int c2 = for_rows ? it.b : 0;
+            // An odd number of row blocks leaves a CTA without rows: what its MMAs make of old contents is never stored.
+            const bool load = !for_rows || it.b < B;
+            const uint32_t bytes = static_cast<uint32_t>((2 * it.row_tile + 1 < B * g.row_blocks ? 2 : 1) + (wide ? 2 : 1)) * kAtomBytes;  // of both CTAs
+            for (int kt = 0; kt < KT; kt += slices, ++n, turn.next(stages)) {
+                ok = warp_wait(empty0 + 8u * static_cast<uint32_t>(turn.s), turn.parity ^ 1u, abort_flag, kSiteProducerEmpty);
+                if (!ok) break;
+                uint8_t* st = smem + turn.s * stage_bytes + (for_rows ? 0 : kAtomBytes);
+                const uint32_t full = full0 + 8u * static_cast<uint32_t>(turn.s);
+                const bool second = slices == 2 && kt + 1 < KT;
+                if (ptx::elect_one()) {
+                    if (rank == 0 && for_rows) ptx::mbar_expect_tx(&bars->full[turn.s], second ? 2 * bytes : bytes);
+                    // rows or features beyond the tensor's extent, and d_model's ragged tail, arrive as zeros
+                    if (load) ptx::pair_tma_load_3d(st, map, full, kt * kKSlice, c1, c2, keep);
+                    if (load && second) ptx::pair_tma_load_3d(st + slice_bytes, map, full, (kt + 1) * kKSlice, c1, c2, keep);
+                    if (wide && !for_rows) ptx::pair_tma_load_3d(st + kAtomBytes / 2, map, full, kt * kKSlice, c1 + kFeatures / 2, c2, keep);
+                }
+                __syncwarp();
+            }
+            t += pairs;
+            if (t < items) it = item(t);
+        }
+        if (lane == 0) atomicMax(&bars->loads, n);
+        // The MMAs' arrivals on this CTA's barriers are all here before it ends.
+        for (int i = n > stages ? n - stages : 0; ok && i < n; ++i)
+            ok = warp_wait(empty0 + 8u * static_cast<uint32_t>(i % stages), static_cast<uint32_t>(i / stages) & 1u, abort_flag, kSiteProducerEmpty);
+    } else if (run && warp == kMma && rank == 0) {
+        // ================= MMA issuer, for both CTAs =================
+        constexpr uint32_t idesc_whole = ptx::umma_idesc_bf16_f32(2 * kRows, 2 * kFeatures);
+        constexpr uint32_t idesc_half = ptx::umma_idesc_bf16_f32(2 * kRows, kFeatures);
+        const uint64_t base = ptx::umma_desc_kmajor_sw128(ptx::smem_u32(smem));
+        bool ok = true;
+        const uint32_t full0 = ptx::smem_u32(&bars->full[0]);
+        uint64_t st = base;  // of the stage that is next
+        Turn turn;
+        int use = 0;  // accumulators begun
+        for (int t = first; ok && t < items; t += pairs, ++use) {
+            const uint32_t idesc = t < whole_tiles && block == kFeatures ? idesc_whole : idesc_half;
+            const int slot = use % kSlots;
+            ok = warp_wait(ptx::smem_u32(&bars->acc_empty[slot]), (static_cast<uint32_t>(use / kSlots) & 1u) ^ 1u, abort_flag, kSiteMmaAccEmpty);
             ptx::tc_fence_after_sync();
-            const uint64_t st = ptx::umma_desc_kmajor_sw128(base + static_cast<uint32_t>(s * kStageBytes));
-            if (ptx::elect_one()) {
-#pragma unroll
-                for (int mi = 0; mi < RB; ++mi) {
+            const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(slot * kSlotCols);
+            for (int kt = 0; ok && kt < KT; kt += slices) {
+                ok = warp_wait(full0 + 8u * static_cast<uint32_t>(turn.s), turn.parity, abort_flag, kSiteMmaFull);
+                if (!ok) break;
+                if (ptx::elect_one()) {
 #pragma unroll
                     for (int k = 0; k < kKSlice / 16; ++k)
-                        // A: 128 rows of X; B: the weight atoms, contiguous (8-row groups 1024 bytes apart)
-                        ptx::umma_f16_ss(tmem_base + static_cast<uint32_t>(mi * kCols), st + static_cast<uint64_t>((mi * kAtomBytes + k * 32) >> 4),
-                                         st + static_cast<uint64_t>((RB * kAtomBytes + k * 32) >> 4), idesc, (kt > 0 || k > 0) ? 1u : 0u);
+                        ptx::pair_umma_f16_ss(d_tmem, st + static_cast<uint64_t>((k * 32) >> 4), st + static_cast<uint64_t>((kAtomBytes + k * 32) >> 4), idesc,
+                                              (kt > 0 || k > 0) ? 1u : 0u);
+                    if (slices == 2 && kt + 1 < KT) {
+                        const uint64_t second = st + static_cast<uint64_t>(slice_bytes >> 4);
+#pragma unroll
+                        for (int k = 0; k < kKSlice / 16; ++k)
+                            ptx::pair_umma_f16_ss(d_tmem, second + static_cast<uint64_t>((k * 32) >> 4), second + static_cast<uint64_t>((kAtomBytes + k * 32) >> 4),
+                                                  idesc, 1u);
+                    }
+                    ptx::pair_umma_commit(&bars->empty[turn.s]);
+                    if (kt + slices >= KT) ptx::pair_umma_commit(&bars->acc_full[slot]);
                 }
-                ptx::umma_commit(&bars->empty[s]);
+                __syncwarp();
+                st += static_cast<uint64_t>(stage_bytes >> 4);
+                turn.next(stages);
+                if (turn.s == 0) st = base;
             }
-            __syncwarp();
         }
-        if (ok && ptx::elect_one()) ptx::umma_commit(&bars->acc_full);
-        __syncwarp();
     } else if (run && warp < kEpiWarps) {
         // ================= Epilogue warps: accumulators -> bf16 -> shared memory -> TMA stores, head-major =================
         const int quarter = warp & 3;
-        const int ch = warp >> 2;  // column half of the tile
-        const int row = quarter * 32 + lane;
+        const int ch = warp >> 2;  // this warp takes the columns that CTA `ch` has loaded the features of
         const uint32_t sw = static_cast<uint32_t>(lane & 7);
-        bool ok = __all_sync(0xffffffffu, fused_wait(&bars->acc_full, 0, abort_flag, kSiteEpiAcc));
-        if (ok) {
+        const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+        const uint32_t own_box = ptx::smem_u32(smem + kOutOff + warp * kStageBoxBytes), ring_box = ptx::smem_u32(smem + warp * kStageBoxBytes);
+        const uint64_t keep = ptx::policy_evict_last();  // the attention kernels read Q and K next
+        bool ok = true;
+        int use = 0;
+        Item it = first_item;
+        for (int t = first; ok && t < items; ++use) {
+            const int row = it.row + quarter * 32;
+            const bool rows_exist = it.b < B && row < N;
+            const int block = it.block + ch;
+            const bool keys = block >= g.feature_blocks;
+            const int width = it.half < 0 ? g.block : kFeatures / 2;
+            const int c0 = (keys ? block - g.feature_blocks : block) * g.block + (it.half == 1 ? kFeatures / 2 : 0);
+            int head = d == 64 ? c0 >> 6 : c0 >> 7, offset = c0 & (d - 1);  // of the box's first feature
+            const bool last = t + pairs >= items;
+            const int slot = use % kSlots;
+            const uint32_t taddr = t_lane + static_cast<uint32_t>(slot * kSlotCols + ch * width);
+            ok = warp_wait(ptx::smem_u32(&bars->acc_full[slot]), static_cast<uint32_t>(use / kSlots) & 1u, abort_flag, kSiteEpiAcc);
+            if (!ok) break;
             ptx::tc_fence_after_sync();
-            // every load was consumed and every MMA is complete: the ring is free and stages the tile as RB x 2 CB boxes of
-            // [128 rows x 64 features]
-            const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
 #pragma unroll 1
-            for (int mi = 0; mi < RB; ++mi) {
-#pragma unroll 1
-                for (int c = 0; c < 2 * CB; ++c) {
-                    float v[kChunk];
-                    load_chunk(t_lane + static_cast<uint32_t>(mi * kCols + ch * (kCols / 2) + c * kChunk), v);
-                    const int atom = ch * CB + (c >> 1);
-                    const uint32_t dst = ptx::smem_u32(smem + (mi * 2 * CB + atom) * kAtomBytes + row * 128);
+            for (int c = 0; c < width; c += 64) {
+                uint32_t v[2][32];
+                ptx::tmem_ld_32x32b_x32(taddr + static_cast<uint32_t>(c), v[0]);
+                ptx::tmem_ld_32x32b_x32(taddr + static_cast<uint32_t>(c + 32), v[1]);
+                ptx::tmem_wait_ld();
+                if (c + 64 == width) {  // the accumulator may be overwritten
+                    ptx::tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&bars->acc_empty[slot]), 0));
+                }
+                // The box: once the store that used it last has read it (lane 0 has issued them all).  The last tile's second one has room
+                // of its own, in the ring, which nothing uses any more.
+                const uint32_t box = last && c > 0 ? ring_box : own_box;
+                if (box == own_box) ptx::bulk_wait_group_read<0>();
+                __syncwarp();
 #pragma unroll
-                    for (int g = 0; g < 4; ++g)
-                        ptx::st_shared_v4(dst + ((static_cast<uint32_t>((c & 1) * 4 + g) ^ sw) << 4),
-                                          ptx::pack_bf16x2(v[g * 8 + 0], v[g * 8 + 1]), ptx::pack_bf16x2(v[g * 8 + 2], v[g * 8 + 3]),
-                                          ptx::pack_bf16x2(v[g * 8 + 4], v[g * 8 + 5]), ptx::pack_bf16x2(v[g * 8 + 6], v[g * 8 + 7]));
+                for (int i = 0; i < 8; ++i) {  // one 16-byte piece of the row's 128 bytes
+                    uint32_t w[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        w[j] = ptx::pack_bf16x2(__uint_as_float(v[i >> 2][(i & 3) * 8 + 2 * j]), __uint_as_float(v[i >> 2][(i & 3) * 8 + 2 * j + 1]));
+                    ptx::st_shared_v4(box + static_cast<uint32_t>(lane * 128) + ((static_cast<uint32_t>(i) ^ sw) << 4), w[0], w[1], w[2], w[3]);
                 }
-            }
-            ptx::fence_proxy_async_smem();
-            __syncwarp();
-            if (warp == 0) {
-                ok = __all_sync(0xffffffffu, fused_wait(&bars->out_filled, 0, abort_flag, kSiteEpiFilled));
-                if (ok && lane == 0) {
-                    const uint64_t stream_out = ptx::policy_evict_last();  // the attention kernels read Q and K next
-                    for (int mi = 0; mi < RB; ++mi) {
-                        if (r0 + mi * 128 >= N) continue;
-                        for (int atom = 0; atom < 2 * CB; ++atom) {
-                            const int col = c0 + atom * 64;  // output feature of H * d: head col / d, offset col % d
-                            if (col >= H * d) continue;
-                            ptx::tma_store_3d(tm_out, ptx::smem_u32(smem + (mi * 2 * CB + atom) * kAtomBytes), col % d, r0 + mi * 128,
-                                              b * H + col / d, stream_out);
-                        }
-                    }
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0 && rows_exist && head < H) {
+                    ptx::tma_store_3d(keys ? &tm_k : &tm_q, box, offset, row, it.b * H + head, keep);
                     ptx::bulk_commit_group();
-                    ptx::bulk_wait_group<0>();
                 }
-            } else if (lane == 0) {
-                ptx::mbar_arrive(&bars->out_filled);
+                offset += 64;
+                if (offset == d) {
+                    offset = 0;
+                    ++head;
+                }
             }
+            t += pairs;
+            if (t < items) it = item(t);
         }
+        ptx::bulk_wait_group<0>();
     }
 
-    // ---- teardown: every role falls through to here, also after a wait gave up ----
+    // ---- teardown: every role of both CTAs falls through to here, also after a wait gave up ----
     ptx::tc_fence_before_sync();
     __syncthreads();
-    if (warp == kMma) {
-        ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem_base, L::kTmemCols);
+    if (threadIdx.x == 0 && *abort_flag) {
+        ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&bars->abort_flag), rank ^ 1), 1u);
+        ptx::fence_cluster();
     }
+    __syncwarp();
+    ptx::cluster_arrive_relaxed();
+    ptx::cluster_wait_acquire();
+    ptx::tc_fence_after_sync();
+    if (*abort_flag) {
+        // Unwinding: let the copies of both CTAs that are in flight land before shared memory is released.
+        if (rank == 0 && threadIdx.x == 0) {
+            const int mine = bars->loads;
+            const int theirs = static_cast<int>(ptx::ld_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&bars->loads), 1)));
+            const int last = mine > theirs ? mine : theirs;
+            const long long t0 = clock64();
+            // (the phase of a stage that only the odd CTA has asked for does not end: there the limit runs out)
+            for (int i = last > stages ? last - stages : 0; i < last; ++i)
+                while (!ptx::mbar_try_wait(&bars->full[i % stages], static_cast<uint32_t>(i / stages) & 1u) &&
+                       clock64() - t0 < kWaitLimitCycles / 8) {
+                }
+        }
+        __syncwarp();
+        ptx::cluster_arrive_relaxed();
+        ptx::cluster_wait_acquire();
+    }
+    if (warp == kMma) ptx::pair_tmem_dealloc(tmem_base, kTmemCols);
 }
 
 }  // namespace proj

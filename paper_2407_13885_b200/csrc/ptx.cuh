@@ -295,6 +295,60 @@ __device__ __forceinline__ void cluster_wait_acquire() {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// The same without ordering any access: what release costs is waiting for everything that this thread has in flight, about 1000
+// cycles.  For CTAs that only wait for one another, with mbarriers (mbar_fence_init) ...
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+// ... and with this in front, by a thread that has something to say after all.
+__device__ __forceinline__ void fence_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
+// 4-byte accesses to a peer CTA's shared memory, and an arrival on a peer CTA's mbarrier that says nothing about memory (tensor memory
+// has its own fences).
+__device__ __forceinline__ void st_cluster_u32(uint32_t remote_addr, uint32_t value) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote_addr), "r"(value) : "memory");
+}
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t remote_addr) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(remote_addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t remote_bar) {
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote_bar) : "memory");
+}
+
+// ---- tcgen05 over a pair of CTAs (cta_group::2; a cluster of two, whose even CTA issues the MMAs) ----
+// Every tcgen05 instruction of a kernel with a cta_group must name the same one.
+__device__ __forceinline__ void pair_tmem_alloc(uint32_t* smem_dst, uint32_t ncols) {  // one warp of each CTA
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_dst)), "r"(ncols) : "memory");
+}
+__device__ __forceinline__ void pair_tmem_relinquish() {
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void pair_tmem_dealloc(uint32_t taddr, uint32_t ncols) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+// D (+)= A B over both CTAs: each gives its 128 rows of A and half of the columns of B, at the same addresses of its shared memory,
+// and receives its 128 rows of D, all columns.
+__device__ __forceinline__ void pair_umma_f16_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// One arrival on the mbarrier at this place of BOTH CTAs once every MMA issued so far by this thread is complete.
+__device__ __forceinline__ void pair_umma_commit(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)),
+                 "h"(static_cast<uint16_t>(3))
+                 : "memory");
+}
+// As tma_load_3d; the bytes are counted on `bar`, an mbarrier of either CTA of the pair (a shared::cluster address).
+__device__ __forceinline__ void pair_tma_load_3d(void* smem_dst, const CUtensorMap* m, uint32_t bar, int c0, int c1, int c2, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2.L2::cache_hint"
+        " [%0], [%1, {%3, %4, %5}], [%2], %6;" ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c0), "r"(c1),
+        "r"(c2), "l"(policy)
+        : "memory");
+}
+
 // ---- UMMA descriptors ------------------------------------------------------------------------
 // Shared-memory operand descriptor for a K-major bf16 tile stored as rows of 64 elements
 // (128 bytes) with the 128-byte swizzle TMA applies: 8-row groups are 1024 bytes apart.

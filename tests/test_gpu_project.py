@@ -73,6 +73,16 @@ def test_projection_matches_oracle(attnw, B, N, d_model, H, d):
     check(K, oracle.project(x, wk), x, wk)
 
 
+# On a device of 148 SMs: more whole tiles than pairs of CTAs, with a last round cut in two; the same with an odd number of row blocks,
+# which leaves a CTA without rows; several rounds of one slice; narrow tiles with an odd number of slices and of row blocks
+@pytest.mark.parametrize("B,N,d_model,H,d", [(3, 650, 136, 9, 128), (1, 1300, 200, 15, 128), (2, 2600, 64, 8, 128), (1, 300, 320, 3, 64)])
+def test_projection_over_rounds_of_tiles(attnw, B, N, d_model, H, d):
+    x, wq, wk = rand_xw(B, N, d_model, H, d, stream=5 * N + d_model + H)
+    Q, K = run_project(attnw, x, wq, wk)
+    check(Q, oracle.project(x, wq), x, wq)
+    check(K, oracle.project(x, wk), x, wk)
+
+
 def test_projection_with_selector_weights_is_exact(attnw):
     # W[h, c, :] = e_{h*d + c}: head h of Q is columns h*d .. of X, bit for bit; K takes them in reverse order
     B, N, H, d = 2, 200, 3, 64
