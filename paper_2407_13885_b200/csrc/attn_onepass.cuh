@@ -7,7 +7,8 @@
 // Per step j and unit q:
 //   MMA 1     S = Q K_j^T                         128 x 128 fp32 in tensor memory
 //   Softmax   two threads per row, 64 columns each: a thread takes its scores to registers (the buffer is handed back
-//             at once, so the next MMA 1 runs meanwhile); the two tell each other their maximum through shared memory;
+//             at once, so the next MMA 1 runs meanwhile); the two tell each other their maximum through shared memory; the units
+//             take turns at the exponentials;
 //             p = 2^(c s - mb) with the row's offset mb; l += sum p; P (bf16) becomes the A operand of MMA 2 in tensor memory
 //   MMA 2     O_q += P V_j                        128 x d fp32 in tensor memory; V_j as TMA delivers it
 //             ([128 keys x d], an MN-major B operand)
@@ -18,7 +19,7 @@
 // instead of 1.01 at 128 x 4096, d = 128: 88 bytes of spills, and the maximum is not what the unit waits for.)
 // What bounds it: in a loop of large calls, the power cap; at a burst, the chain of the Softmax warps' step (d = 128: 3100 cycles
 // of which the special function units and the tensor pipe need 2048 each).  Operand fetch from shared memory holds up
-// the tensor pipe, and the issuers' waits keep it idle (kTwoIssuers), so:
+// the tensor pipe, and the issuers' waits keep it idle (two_issuers), so:
 //   * P goes through tensor memory (through shared memory its port was busy 3072 of 4200 cycles a step): 128 x 4096, d = 64
 //     839 -> 801 us; d = 128 985 -> 941 at a burst, 1106 -> 1056 in a loop.  d = 64 has room for the scores of both units beside P
 //     and O.  d = 128 has one buffer of scores: the units are half a step apart and hold it only from MMA 1 until their
@@ -26,7 +27,10 @@
 //   * The two threads of a row exchange maxima (each read the other's scores too, which held the buffer longer), and the
 //     room of P's tiles makes the ring of K and V a stage longer: d = 128 941 -> 910 and 1057 -> 1027; d = 64 793 -> 768;
 //     12 x 1021, d = 64 13.0 -> 12.1.
-// Slower: the wait for the previous product put off until half of the weights are there (d = 64 780 -> 821 us, d = 128 no change);
+//   * The units take turns at the exponentials (turns), and units of one query tile have an issuing warp for the scores and one for the products
+//     (two_issuers): 12 x 1021, d = 64 11.9 -> 11.2, 3 x 12766 257 -> 236, 13 x 7115, d = 128 336 -> 318; 36 drawn sizes 1.035 times as fast.
+// Slower: the issuer asking for both barriers of a set of MMAs at once, and one election for MMAs and release (d = 128 977 -> 996 us, an
+// issuer that finds the second one not ready asks for the first again); the wait for the previous product put off until half of the weights are there (d = 64 780 -> 821 us, d = 128 no change);
 // one thread per row, 8 Softmax warps of 168 registers (d = 64 795 -> 1000: a lone warp of a scheduler gets half of
 // its special function unit); products before scores (780 -> 978); 1/8 or 1/4 of the exponentials by a polynomial of degree 5 on
 // the FMA pipes (d = 64 778 -> 776, 790; d = 128 965 -> 984, 1002 in a loop); CTAs that stay for several row blocks and store
@@ -43,8 +47,9 @@ namespace av1 {
 constexpr int kSmWarps = 16;      // Softmax warps: unit (2) x column half (2) x TMEM lane quarter (4)
 constexpr int kProducer = 16;
 constexpr int kMma = 17;
-constexpr int kMmaProduct = 18;   // kTwoIssuers: the products' issuer
+constexpr int kMmaProduct = 18;   // two_issuers: the products' issuer
 constexpr int kMaxCluster = 4;    // CTAs that share a query tile (of 8, 15 clusters fit, and a call that needs them has 16 tiles)
+constexpr int kPassAt = 4;        // of the 8 groups of 8 exponentials: behind which the other unit's turn begins
 constexpr float kLazy = 8.0f;     // the offset follows the maximum only when it has grown by more than this
 
 enum : uint32_t {  // wait sites of this kernel (low byte of the status word)
@@ -63,6 +68,9 @@ enum : uint32_t {  // wait sites of this kernel (low byte of the status word)
 
 constexpr int kUnitStats = 4 * kTile;
 
+// How the keys of a query tile are worked on.
+enum Mode { kWhole, kSplit, kCluster };
+
 template <int D>
 struct Smem {
     static constexpr int kAtoms = D / 64;
@@ -74,10 +82,17 @@ struct Smem {
     static constexpr bool kSharedS = D == 128;
     // A second warp issues the products: an issuer spends 200 to 550 cycles on the waits in front of each set of MMAs, 1360 of a
     // step's 3450 at d = 128, and nothing of the other kind was queued meanwhile.  128 x 4096 902 -> 856 us at a burst, 1012 -> 950
-    // in a loop; 12 x 2048 34.8 -> 32.4.  At d = 64 the MMAs take half as long and the exponentials set the pace: 780 us with
-    // one issuer, 811 with two (796 where the scores still keep the order).
-    static constexpr bool kTwoIssuers = D == 128;
-    static constexpr int kThreads = kTwoIssuers ? 608 : 576;
+    // in a loop; 12 x 2048 34.8 -> 32.4.  At d = 64 the MMAs take half as long: with two query tiles the exponentials set the pace
+    // (780 us with one issuer, 811 with two), but units of one query tile have K and V tiles of their own and twice the waits (12 x 1021 12.2 ->
+    // 11.2, 4 x 13233 302 -> 261).
+    static __host__ __device__ constexpr bool two_issuers(Mode m) { return D == 128 || m != kWhole; }
+    // The two units take turns at the exponentials.  The warps of a lane quarter, two of each unit, share a scheduler and its special function
+    // unit, and left alone they fall into step: all in their exponentials (twice as long), then all in their waits and maxima.  The turn
+    // passes when 5 of 8 groups of exponentials are issued: what is left of them covers the hand-over.  us per call without turns -> with
+    // them (behind 4, 6 or all groups): d = 64, 128 x 4096 756 -> 746 (785, 810, 872), 4 x 13233 274 -> 261; d = 128, 9 x 6108 175 -> 167, 3 x 13719
+    // 334 -> 314, 2 x 363 8.1 -> 7.6; not for two query tiles at d = 128, whose scores alternate anyway (956 -> 963).
+    static __host__ __device__ constexpr bool turns(Mode m) { return D == 64 || m != kWhole; }
+    static __host__ __device__ constexpr int threads(Mode m) { return two_issuers(m) ? 608 : 576; }
     static __host__ __device__ constexpr uint32_t s_col(int q) { return kSharedS ? 0u : static_cast<uint32_t>(q * 256); }
     static __host__ __device__ constexpr uint32_t p_col(int q) { return kSharedS ? 128u + static_cast<uint32_t>(q * 64) : static_cast<uint32_t>(q * 256 + 192); }
     static __host__ __device__ constexpr uint32_t o_col(int q) { return kSharedS ? 256u + static_cast<uint32_t>(q * 128) : static_cast<uint32_t>(q * 256 + 128); }
@@ -96,7 +111,7 @@ struct Barriers {
     uint64_t s_full[2], s_free[2];  // per unit: scores written / read into registers (8 warps)
     uint64_t p_full[2], p_free[2];  // per unit: P written (8 warps) / read by its MMAs
     uint64_t o_full[2];             // per unit: every product complete
-    uint64_t max_full[2][4];        // per unit and lane quarter: the maxima of both halves are in shared memory (2 warps)
+    uint64_t max_full[2][4];        // per unit and lane quarter, without turns: the maxima of both halves are in shared memory (2 warps)
     uint64_t l_full[2];             // per query tile: the row statistics of its warps are in shared memory
     uint64_t out_filled[2];
     uint32_t tmem_base;
@@ -123,16 +138,15 @@ __device__ __forceinline__ bool wait_in_place(uint64_t* bar, uint32_t parity, vo
     }
 }
 
-// How the keys of a query tile are worked on.
-enum Mode { kWhole, kSplit, kCluster };
-
 template <int D, Mode M>
-__global__ void __launch_bounds__(Smem<D>::kThreads, 1)
+__global__ void __launch_bounds__(Smem<D>::threads(M), 1)
 attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o, int N,
                     int row_blocks_per_head, float scale_log2e, __nv_bfloat16* O, int cluster_ctas) {
     using L = Smem<D>;
     constexpr bool split = M != kWhole;
+    constexpr bool two_issuers = L::two_issuers(M);
+    constexpr bool turns = L::turns(M);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     Barriers* bars = reinterpret_cast<Barriers*>(smem + L::kBarOff);
@@ -240,7 +254,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             }
         }
         __syncwarp();
-    } else if (run && (warp == kMma || (L::kTwoIssuers && warp == kMmaProduct))) {
+    } else if (run && (warp == kMma || (two_issuers && warp == kMmaProduct))) {
         // ================= MMA issuers (warp-uniform loops, one elected lane issues): of scores, of products, or of both =================
         constexpr uint32_t idesc_s = ptx::umma_idesc_bf16_f32(kTile, kTile);
         constexpr uint32_t idesc_o = ptx::umma_idesc_bf16_f32(kTile, D) | (1u << 16);  // B operand MN-major
@@ -297,7 +311,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         // The scores of step j + 1 first: the tensor pipe computes them while the row threads exponentiate step j.  The two
         // units alternate (with two issuers, because the scores take turns at their buffer) - scores of one, product of one, scores of the other, product of the other - which keeps their
         // row threads half a step apart (d = 64, 128 x 4096: 888 -> 841 us against both scores first).
-        if constexpr (L::kTwoIssuers) {
+        if constexpr (two_issuers) {
             const bool for_scores = warp == kMma;
             for (int j = -1; ok && j < steps[0]; ++j) {
                 for (int q = 0; ok && q < (split ? 2 : 1); ++q) {
@@ -386,9 +400,24 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         float l = 0.0f;         // sum of this thread's weights
         bool ok = true;
 
-        for (int j = 0; ok && j < steps[q]; ++j) {
-            ok = __all_sync(0xffffffffu, fused_wait(&bars->s_full[q], static_cast<uint32_t>(j) & 1u, abort_flag, kSiteSFull));
-            if (!ok) break;
+        const int my_steps = q == 0 ? steps[0] : steps[1], other_steps = q == 0 ? steps[1] : steps[0];
+        // turns: unit 0's step 0, unit 1's step 0, unit 0's step 1, ... of those that both units have; the barrier of a turn is the one that the
+        // two threads of a row exchange their maxima by.  Every warp takes part in all of them, also after a wait has given up.
+        const uint32_t turn_own = static_cast<uint32_t>(1 + q * 4 + quarter), turn_other = static_cast<uint32_t>(1 + (q ^ 1) * 4 + quarter);
+        const int behind = q == 0 ? 1 : 0;  // a step waits for the other unit's step so many before
+        auto take_turn = [&](int j) {
+            if (turns) ptx::named_sync(turn_own, j >= behind && j - behind < other_steps ? 128u : 64u);
+        };
+        auto pass_turn = [&](int j) {
+            if (turns && j + 1 - behind < other_steps) ptx::named_arrive(turn_other, 128u);
+        };
+        for (int j = 0; j < my_steps; ++j) {
+            if (ok) ok = warp_wait(bar_of(offsetof(Barriers, s_full), q), static_cast<uint32_t>(j) & 1u, abort_flag, kSiteSFull);
+            if (!ok) {
+                take_turn(j);
+                pass_turn(j);
+                continue;
+            }
             ptx::tc_fence_after_sync();
             const int valid = N - key_tile(j, q) * kTile;  // key columns of this tile that exist
             // ---- this thread's 64 scores into registers; the buffer goes back to the MMA issuer at once ----
@@ -426,22 +455,30 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             m0 = ptx::max3(fmaxf(m0, m1), m2, m3);
             const uint32_t place = static_cast<uint32_t>(j & 1) * (2 * kTile * 4);
             ptx::st_shared_f32(max_own + place, m0);
-            __syncwarp();
-            ptx::mbar_arrive_if(bar_of(offsetof(Barriers, max_full), q * 4 + quarter), lane0);
-            // P and O are free once the MMAs of the previous key tile are complete.  At d = 64 they are by now, as a rule, and the wait runs
-            // beside the other half's (128 x 4096 780 -> 763 us); at d = 128 they take longer than the maxima (976 -> 1022).
-            if constexpr (D == 64) {
-                ok = __all_sync(0xffffffffu, wait_in_place(&bars->p_free[q], (static_cast<uint32_t>(j) & 1u) ^ 1u, abort_flag, kSitePFree));
-                if (!ok) break;
+            // P and O are free once the MMAs of the previous key tile are complete: at d = 64, and where the units take turns, by now, as a
+            // rule, and the wait runs beside the other half's; two query tiles at d = 128 take longer than the maxima (976 -> 1022 us).
+            auto products_done = [&]() {
+                return static_cast<bool>(__all_sync(0xffffffffu, wait_in_place(&bars->p_free[q], (static_cast<uint32_t>(j) & 1u) ^ 1u, abort_flag, kSitePFree)));
+            };
+            if constexpr (turns) {
+                ok = products_done();
+                take_turn(j);
+                if (!ok) {
+                    pass_turn(j);
+                    continue;
+                }
+            } else {
+                __syncwarp();
+                ptx::mbar_arrive_if(bar_of(offsetof(Barriers, max_full), q * 4 + quarter), lane0);
+                ok = __all_sync(0xffffffffu, wait_in_place(&bars->max_full[q][quarter], static_cast<uint32_t>(j) & 1u, abort_flag, kSiteMaxFull));
+                if (!ok) continue;
             }
-            ok = __all_sync(0xffffffffu, wait_in_place(&bars->max_full[q][quarter], static_cast<uint32_t>(j) & 1u, abort_flag, kSiteMaxFull));
-            if (!ok) break;
             smax = ptx::max3(smax, m0, ptx::ld_shared_f32(max_other + place));
             const float mb_cand = fmaxf(smax * c2, -3.0e38f);
             const bool move = j == 0 || mb_cand - mb > kLazy;
-            if constexpr (D != 64) {
-                ok = __all_sync(0xffffffffu, wait_in_place(&bars->p_free[q], (static_cast<uint32_t>(j) & 1u) ^ 1u, abort_flag, kSitePFree));
-                if (!ok) break;
+            if constexpr (!turns) {
+                ok = products_done();
+                if (!ok) continue;
             }
             ptx::tc_fence_after_sync();
             uint32_t w[16];  // 32 keys of P on their way to tensor memory
@@ -485,6 +522,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 }
 #pragma unroll
                 for (int i = 0; i < 4; ++i) w[(g & 3) * 4 + i] = ptx::pack_bf16x2(p[2 * i], p[2 * i + 1]);
+                if (g == kPassAt) pass_turn(j);
                 if ((g & 3) == 3) ptx::tmem_st_32x32b_x16(p_own + static_cast<uint32_t>((g >> 2) * 16), w);
             }
             float a0, a1, a2, a3;
@@ -498,7 +536,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         }
 
         // ---- epilogue: O / l -> bf16 -> the query tile's shared memory -> TMA stores ----
-        if (split || steps[q] > 0) {  // (split: each unit has a step)
+        if (split || my_steps > 0) {  // (split: each unit has a step)
             // Two units of one query tile each finish alone.  Two units of the same query tile meet here: the four threads of a
             // row take D / 4 columns each of 2^(mb_0 - mb) O_0 + 2^(mb_1 - mb) O_1.
             const int u = split ? 0 : q;  // the barriers and the query tile this epilogue uses

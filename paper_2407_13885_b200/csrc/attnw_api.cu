@@ -605,7 +605,7 @@ int attn_max_clusters(DeviceInfo* dev, int ctas) {
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(av1::Smem<D>::kThreads, 1, 1);
+    cfg.blockDim = dim3(av1::Smem<D>::threads(av1::kCluster), 1, 1);
     cfg.gridDim = dim3(static_cast<unsigned>(ctas * dev->sm_count), 1, 1);
     cfg.dynamicSmemBytes = av1::Smem<D>::kDynamicBytes;
     cfg.attrs = attr;
@@ -663,7 +663,7 @@ int launch_attn_onepass(DeviceInfo* dev, const void* Q, const void* K, const voi
                   : mode == av1::kSplit ? av1::attn_onepass_kernel<D, av1::kSplit>
                                         : av1::attn_onepass_kernel<D, av1::kCluster>;
     if (allowed != cudaSuccess ||
-        launch_overlapped(kernel, static_cast<unsigned>(BH * row_blocks * ctas), L::kThreads, L::kDynamicBytes, stream, ctas, tm_q,
+        launch_overlapped(kernel, static_cast<unsigned>(BH * row_blocks * ctas), L::threads(mode), L::kDynamicBytes, stream, ctas, tm_q,
                           tm_k, tm_v, tm_o, N, row_blocks, scale_log2e, static_cast<__nv_bfloat16*>(O), ctas) != cudaSuccess) {
         (void)cudaGetLastError();
         return ATTNW_ERR_CUDA;

@@ -64,6 +64,12 @@ __device__ __forceinline__ void mbar_arrive_if(uint32_t bar, uint32_t pred) {
         : "memory");
 }
 
+// ---- named barriers of a CTA (1 ... 15) ---------------------------------------------------------
+// `threads` of whole warps; those that only announce themselves do not wait.  No limit can be set on the wait: every warp has to take part
+// in each use also after another wait has given up.
+__device__ __forceinline__ void named_sync(uint32_t id, uint32_t threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+__device__ __forceinline__ void named_arrive(uint32_t id, uint32_t threads) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+
 // ---- async-proxy fences and bulk groups --------------------------------------------------
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
