@@ -142,7 +142,7 @@ template <int D, Mode M>
 __global__ void __launch_bounds__(Smem<D>::threads(M), 1)
 attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o, int N,
-                    int row_blocks_per_head, float scale_log2e, __nv_bfloat16* O, int cluster_ctas) {
+                    int row_blocks_per_head, float scale_log2e, __nv_bfloat16* O, int cluster_ctas, int first_block) {
     using L = Smem<D>;
     constexpr bool split = M != kWhole;
     constexpr bool two_issuers = L::two_issuers(M);
@@ -158,7 +158,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     const int lane = threadIdx.x & 31;
     const int G = M == kCluster ? cluster_ctas : 1;  // CTAs that share a query tile
     const int rank = M == kCluster ? static_cast<int>(ptx::cluster_ctarank()) : 0;
-    const int block = static_cast<int>(blockIdx.x) / G;
+    const int block = first_block + static_cast<int>(blockIdx.x) / G;  // of those of all heads
     const int bh = block / row_blocks_per_head;
     const int row0 = (block % row_blocks_per_head) * (split ? kTile : kRowsPerCta);
     const int T = (N + kTile - 1) / kTile;  // key tiles
@@ -212,24 +212,36 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 
     if (run && warp == kProducer) {
         // ================= TMA producer: Q once, then the K and V tiles in the order the MMA issuer reads them =========
-        if (lane == 0) {
+        // Two query tiles at d = 128: the whole warp walks the list and an elected lane issues (a lone lane takes 300 cycles a tile: 2 x 97
+        // 6.4 -> 6.2 us).  Otherwise a lone lane (3 x 863, d = 64 10.06 us, the whole warp 10.16; 3 x 802, d = 128 11.05 and 11.15).
+        constexpr bool whole_warp = D == 128 && M == kWhole;
+        if (whole_warp || lane == 0) {
             const uint64_t keep = ptx::policy_evict_last();
+            auto issues = [&]() { return !whole_warp || ptx::elect_one(); };
             const int q_tiles = (!split && steps[1] > 0) ? 2 : 1;
-            ptx::mbar_expect_tx(&bars->q_full, static_cast<uint32_t>(q_tiles * L::kTileBytes));
-            for (int q = 0; q < q_tiles; ++q)
-                for (int a = 0; a < L::kAtoms; ++a)
-                    ptx::tma_load_3d(smem + L::kQOff + q * L::kTileBytes + a * L::kAtomBytes, &tm_q, &bars->q_full, a * 64,
-                                     row0 + q * kTile, bh, keep);
+            if (issues()) {
+                ptx::mbar_expect_tx(&bars->q_full, static_cast<uint32_t>(q_tiles * L::kTileBytes));
+                for (int q = 0; q < q_tiles; ++q)
+                    for (int a = 0; a < L::kAtoms; ++a)
+                        ptx::tma_load_3d(smem + L::kQOff + q * L::kTileBytes + a * L::kAtomBytes, &tm_q, &bars->q_full, a * 64,
+                                         row0 + q * kTile, bh, keep);
+            }
+            if (whole_warp) __syncwarp();
             int n = 0;
             bool ok = true;
             auto load = [&](const CUtensorMap* map, int kt) {
                 if (!ok) return;
                 const int s = n % kStages;
-                ok = fused_wait(&bars->k_empty[s], (static_cast<uint32_t>(n / kStages) & 1u) ^ 1u, abort_flag, kSiteProducerEmpty);
+                const uint32_t parity = (static_cast<uint32_t>(n / kStages) & 1u) ^ 1u;
+                ok = whole_warp ? warp_wait(bar_of(offsetof(Barriers, k_empty), s), parity, abort_flag, kSiteProducerEmpty)
+                                : fused_wait(&bars->k_empty[s], parity, abort_flag, kSiteProducerEmpty);
                 if (!ok) return;
-                ptx::mbar_expect_tx(&bars->k_full[s], static_cast<uint32_t>(L::kTileBytes));
-                for (int a = 0; a < L::kAtoms; ++a)
-                    ptx::tma_load_3d(smem + stage_offset(n % kStages) + a * L::kAtomBytes, map, &bars->k_full[s], a * 64, kt * kTile, bh, keep);
+                if (issues()) {
+                    ptx::mbar_expect_tx(&bars->k_full[s], static_cast<uint32_t>(L::kTileBytes));
+                    for (int a = 0; a < L::kAtoms; ++a)
+                        ptx::tma_load_3d(smem + stage_offset(s) + a * L::kAtomBytes, map, &bars->k_full[s], a * 64, kt * kTile, bh, keep);
+                }
+                if (whole_warp) __syncwarp();
                 ++n;
             };
             const int lists = split ? 2 : 1;  // units that have key tiles of their own
@@ -239,7 +251,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                     if (j >= 0 && j < steps[q]) load(&tm_v, key_tile(j, q));
                 }
             }
-            if (*abort_flag) {
+            if (*abort_flag && lane == 0) {
                 // Unwinding: let the copies already in flight land before shared memory is released.
                 const int first = n > kStages ? n - kStages : 0;
                 for (int it = first; it < n; ++it) {

@@ -629,46 +629,76 @@ int launch_attn_onepass(DeviceInfo* dev, const void* Q, const void* K, const voi
     if (rc == ATTNW_OK) rc = encode_3d(&tm_o, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, O, D, N, BH, 64, kTile);
     if (rc != ATTNW_OK) return rc;
     // Two query tiles per CTA; or one whose even and odd key tiles are worked on side by side; or one for a cluster of 2 or 4
-    // CTAs.  Chosen by the rounds of key tiles on the device (about 2 us each) plus what a round of CTAs costs besides: 1.5 of
-    // them for set-up and epilogue, 2 more for a cluster's merge.  us per call, one CTA -> cluster: 1 x 4744 (d = 64)
-    // 43.5 -> 28.5, 1 x 9260 (d = 128) 85.6 -> 53.6, 4 x 2155 24.2 -> 19.8, 3 x 824 11.9 -> 10.8, 1 x 1000 13.3 -> 13.2.
-    const long long tiles = (N + kTile - 1) / kTile, pairs = (tiles + 1) / 2;
+    // CTAs.  Chosen by the rounds of key tiles on the device (about 1.6 us each at d = 64, 1.9 at d = 128, and there a tenth more where the units
+    // have key tiles of their own) plus what a round of CTAs costs besides: 2.5 of them for its begin, set-up and epilogue, 2 more for a cluster's
+    // merge.  us per call, one CTA -> cluster: 1 x 4744 (d = 64) 43.5 -> 28.5, 1 x 9260 (d = 128) 85.6 -> 53.6, 4 x 2155 24.2 ->
+    // 19.8, 3 x 824 11.9 -> 10.8, 1 x 1000 13.3 -> 13.2.
+    // Or full rounds of CTAs first, and the query tiles that are left spread over the device by a second launch.  One launch -> two:
+    // 2 x 10215 (d = 64, 160 query tiles) 129 -> 104, 3 x 13719 (d = 128) 312 -> 258, 22 x 1940 (d = 64) 51 -> 45, 5 x 4607 (d = 64) 65 -> 56, 19 x
+    // 10023 (d = 128) 1058 -> 954, 114 x 692 (d = 128) 48.7 -> 46.5; 9 x 2487 (d = 128) 37.9 -> 39.1, not taken.
+    const long long tiles = (N + kTile - 1) / kTile, pairs = (tiles + 1) / 2, all = BH * tiles;
+    const int sms = dev->sm_count;
+    struct Part {
+        av1::Mode mode;
+        int ctas;         // per query tile (kWhole: per pair of query tiles)
+        long long first;  // query tile (pair of them) of all heads that the part begins with, and how many it has
+        long long count;
+        double cost;
+    };
     auto waves = [](long long work, long long at_once) { return static_cast<double>((work + at_once - 1) / at_once); };
-    av1::Mode mode = av1::kWhole;
-    int ctas = 1;  // per row block
-    double best = waves(BH * pairs, dev->sm_count) * (static_cast<double>(tiles) + 1.5);
-    if (tiles > 1 && BH * tiles <= INT_MAX) {
-        const double cost = waves(BH * tiles, dev->sm_count) * (static_cast<double>(pairs) + 1.5);
-        if (cost * 1.05 < best) {
-            best = cost;
-            mode = av1::kSplit;
-        }
-        for (int g = 2; g <= av1::kMaxCluster && 2 * g <= tiles && BH * tiles * g <= INT_MAX; g *= 2) {
+    const double whole_round = static_cast<double>(tiles) + 2.5, own = D == 128 ? 1.1 : 1.0, split_round = (static_cast<double>(pairs) + 2.5) * own;
+    auto best_part = [&](long long first_tile) {  // for the query tiles from there on, each by a CTA or a cluster
+        const long long n = all - first_tile;
+        Part p{av1::kSplit, 1, first_tile, n, waves(n, sms) * split_round};
+        for (int g = 2; g <= av1::kMaxCluster && 2 * g <= tiles && all * g <= INT_MAX; g *= 2) {
             const int clusters = attn_max_clusters<D>(dev, g);
             if (clusters < 1) break;
-            const double c = waves(BH * tiles, clusters) * (static_cast<double>((tiles + 2 * g - 1) / (2 * g)) + 3.5);
-            if (c * 1.05 < best) {
-                best = c;
-                mode = av1::kCluster;
-                ctas = g;
+            const double c = waves(n, clusters) * (static_cast<double>((tiles + 2 * g - 1) / (2 * g)) + 4.5) * own;
+            if (c * 1.05 < p.cost) p = {av1::kCluster, g, first_tile, n, c};
+        }
+        return p;
+    };
+    Part parts[2] = {{av1::kWhole, 1, 0, BH * pairs, waves(BH * pairs, sms) * whole_round}, {}};
+    int n_parts = 1;
+    double best = parts[0].cost;
+    if (tiles > 1 && all <= INT_MAX) {
+        const Part one = best_part(0);
+        if (one.cost * 1.05 < best) {
+            parts[0] = one;
+            best = one.cost;
+        }
+        for (const av1::Mode mode : {av1::kWhole, av1::kSplit}) {
+            const long long units = mode == av1::kWhole ? BH * pairs : all, full = units / sms * sms;
+            if (full == 0 || full == units) continue;
+            const double front = static_cast<double>(full / sms) * (mode == av1::kWhole ? whole_round : split_round);
+            const Part rest = best_part(mode == av1::kWhole ? full / pairs * tiles + 2 * (full % pairs) : full);
+            const double cost = front + rest.cost + 0.5;
+            if (cost * 1.03 < best) {
+                parts[0] = {mode, 1, 0, full, front};
+                parts[1] = rest;
+                n_parts = 2;
+                best = cost;
             }
         }
     }
-    const int row_blocks = static_cast<int>(mode == av1::kWhole ? pairs : tiles);
     const float scale_log2e = static_cast<float>(static_cast<double>(scale) * 1.4426950408889634074);
-    const cudaError_t allowed = mode == av1::kWhole   ? allow_smem<av1::attn_onepass_kernel<D, av1::kWhole>>(L::kDynamicBytes)
-                                : mode == av1::kSplit ? allow_smem<av1::attn_onepass_kernel<D, av1::kSplit>>(L::kDynamicBytes)
-                                                      : allow_smem<av1::attn_onepass_kernel<D, av1::kCluster>>(L::kDynamicBytes);
-    auto kernel = mode == av1::kWhole   ? av1::attn_onepass_kernel<D, av1::kWhole>
-                  : mode == av1::kSplit ? av1::attn_onepass_kernel<D, av1::kSplit>
-                                        : av1::attn_onepass_kernel<D, av1::kCluster>;
-    if (allowed != cudaSuccess ||
-        launch_overlapped(kernel, static_cast<unsigned>(BH * row_blocks * ctas), L::threads(mode), L::kDynamicBytes, stream, ctas, tm_q,
-                          tm_k, tm_v, tm_o, N, row_blocks, scale_log2e, static_cast<__nv_bfloat16*>(O), ctas) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return ATTNW_ERR_CUDA;
+    for (int i = 0; i < n_parts; ++i) {
+        const Part& p = parts[i];
+        const cudaError_t allowed = p.mode == av1::kWhole   ? allow_smem<av1::attn_onepass_kernel<D, av1::kWhole>>(L::kDynamicBytes)
+                                    : p.mode == av1::kSplit ? allow_smem<av1::attn_onepass_kernel<D, av1::kSplit>>(L::kDynamicBytes)
+                                                            : allow_smem<av1::attn_onepass_kernel<D, av1::kCluster>>(L::kDynamicBytes);
+        auto kernel = p.mode == av1::kWhole   ? av1::attn_onepass_kernel<D, av1::kWhole>
+                      : p.mode == av1::kSplit ? av1::attn_onepass_kernel<D, av1::kSplit>
+                                              : av1::attn_onepass_kernel<D, av1::kCluster>;
+        if (allowed != cudaSuccess ||
+            launch_overlapped(kernel, static_cast<unsigned>(p.count * p.ctas), L::threads(p.mode), L::kDynamicBytes, stream, p.ctas, tm_q, tm_k,
+                              tm_v, tm_o, N, static_cast<int>(p.mode == av1::kWhole ? pairs : tiles), scale_log2e, static_cast<__nv_bfloat16*>(O),
+                              p.ctas, static_cast<int>(p.first)) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return ATTNW_ERR_CUDA;
+        }
+        g_launches.fetch_add(1, std::memory_order_relaxed);
     }
-    g_launches.fetch_add(1, std::memory_order_relaxed);
     return ATTNW_OK;
 }
 

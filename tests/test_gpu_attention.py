@@ -194,3 +194,15 @@ def test_attention_of_many_query_tiles(attnw, B, H, N, d):
     for _ in range(2):
         got = run_attn(attnw, q, k, v, scale).double().cpu().numpy().reshape(ref.shape)
         assert np.all(np.abs(got - ref) <= tolerance_map(q, k, v, scale, ref))
+
+
+# On a device of 148 SMs these are two launches, across heads, with a ragged last tile: a round of CTAs with two query tiles each, then clusters of 2;
+# two rounds of them, then CTAs with one query tile each; a round of those, then clusters of 4
+@pytest.mark.parametrize("B,H,N,d", [(1, 22, 1940, 64), (2, 57, 692, 128), (1, 10, 1940, 64)])
+def test_attention_in_two_parts(attnw, B, H, N, d):
+    q, k = small_fused_inputs(B, H, N, d, sigma=2.0, stream=N + d + 41)
+    v = rand_v(B, H, N, d, stream=N + d + 43)
+    scale = float(np.float32(1.0 / math.sqrt(d)))
+    ref = oracle.attn(q, k, v, scale)
+    got = run_attn(attnw, q, k, v, scale).double().cpu().numpy().reshape(ref.shape)
+    assert np.all(np.abs(got - ref) <= tolerance_map(q, k, v, scale, ref))
