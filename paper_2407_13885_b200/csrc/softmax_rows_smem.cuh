@@ -91,8 +91,8 @@ softmax_rows_smem_kernel(const float* S, OutT* P, long long rows, long long cols
     __syncthreads();
     // A CTA that sees an earlier failure still takes part in every cluster barrier below, without touching memory.
     bool ok = ctl->prior_failure == 0u;
-    if (C > 1) {  // peers' control blocks are initialised before anyone writes into them
-        ptx::cluster_arrive_release();
+    if (C > 1) {  // peers' control blocks are initialised before anyone writes into them (nothing that they read later)
+        ptx::cluster_arrive_relaxed();
         ptx::cluster_wait_acquire();
     }
 
@@ -170,7 +170,7 @@ softmax_rows_smem_kernel(const float* S, OutT* P, long long rows, long long cols
         __syncthreads();                // the slice is free for the next row's copy
     }
     if (C > 1) {  // no CTA leaves while a peer may still write into its control block
-        ptx::cluster_arrive_release();
+        ptx::cluster_arrive_relaxed();
         ptx::cluster_wait_acquire();
     }
 }
@@ -276,16 +276,19 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
     ptx::grid_dependency_wait();
     __syncthreads();
     bool ok = ctl->prior_failure == 0u;
-    if (C > 1) {  // every CTA of the cluster runs before anyone writes into a peer
-        ptx::cluster_arrive_release();
-        ptx::cluster_wait_acquire();
-    }
     auto issue = [&](long long row) {  // one lane: this warp's piece of `row` -> shared memory
         ptx::mbar_expect_tx(&ctl->full[warp], bytes);
         ptx::bulk_load_1d(ptx::smem_u32(x + v0), reinterpret_cast<const float4*>(S + row * cols + c0) + v0, bytes,
                           &ctl->full[warp]);
     };
     if (ok && lane == 0 && bytes > 0 && cluster < rows) issue(cluster);
+    // Every CTA of the cluster runs, with its barriers in place, before anyone writes into a peer.  This barrier and the last one order no
+    // memory but the barriers' begin (mbar_fence_init): with release, which waits for everything in flight, 12 x 183144 took 6.7 us (now 5.6), 2 x 29664 5.8 (4.9).
+    __syncwarp();
+    if (C > 1) {
+        ptx::cluster_arrive_relaxed();
+        ptx::cluster_wait_acquire();
+    }
 
     // Where a wait gives up, the copy of this warp's next piece that is in flight has to land first (the warps that wait for this
     // one's pair give up as well).
@@ -395,7 +398,7 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
         }
     }
     if (C > 1) {  // no CTA leaves while a peer may still write into its control block
-        ptx::cluster_arrive_release();
+        ptx::cluster_arrive_relaxed();
         ptx::cluster_wait_acquire();
     }
     if (!ok) {
