@@ -966,8 +966,9 @@ int rows_entry(const void* S, void* P, long long rows, long long cols, void* str
     if (variant == 1 && cols > srs::kMaxCols) return ATTNW_ERR_UNSUPPORTED;
     // Longer rows can be kept in the shared memory of a CTA or of a cluster (caching form).  By default that is done
     // where it is the faster way (measured): from 8192 columns on - there the register tier needs a whole CTA of 1024
-    // threads per row and stops overlapping rows - with one CTA, or a cluster of two up to 32768 columns; beyond, the
-    // cluster barrier of every row costs more than the second read (from L2) of the two-read kernel.
+    // threads per row and stops overlapping rows - with one CTA, or a cluster of two up to 32768 columns; beyond, the two-read kernel and
+    // the registers of a cluster are ahead (us, default / a cluster of two, bfloat16 6000 x 36864 241 / 252, 5000 x 45000 229 / 248; float32 308 / 298,
+    // 291 / 293, 100 x 36864 6.9 / 8.9; larger clusters 1.3 to 1.9 times the default).
     const int smem_ctas = cols > kSoftmaxRowsSmemTierMinCols ? srs::cluster_ctas_for(cols) : 0;
     const bool smem_default = smem_ctas == 1 || (smem_ctas == 2 && cols <= kSoftmaxRowsRegTierMaxCols);
     if ((variant == 0 && smem_default) || (variant == 1 && smem_ctas >= 1)) {

@@ -268,10 +268,7 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t smem_addr, uint32_t rank
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
     return r;
 }
-// 4-byte store into a peer CTA's shared memory (made visible by the cluster barrier that follows).
-__device__ __forceinline__ void st_cluster_f32(uint32_t remote_addr, float value) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote_addr), "f"(value) : "memory");
-}
+// 16-byte store into a peer CTA's shared memory (made visible by the cluster barrier that follows).
 __device__ __forceinline__ void st_cluster_v4(uint32_t remote_addr, float a, float b, float c, float d) {
     asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(remote_addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }

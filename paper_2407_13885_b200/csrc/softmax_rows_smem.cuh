@@ -9,6 +9,7 @@
 // maximum m_c; pass 2: e = 2^((x - m_c) log2 e) written back to shared memory, the slice's sum l_c; ONE exchange of
 // the pairs (m_c, l_c); M = max m_c, L = sum l_c 2^((m_c - M) log2 e); pass 3: e * 2^((m_c - M) log2 e) / L -> P
 // (coalesced streaming stores).
+// What bounds it: HBM, from 24577 columns on 97 % of the copy rate with bfloat16 and many rows, 88 to 95 % with float32.
 #pragma once
 #include "attnw_fused.cuh"
 #include "launch.cuh"
@@ -27,12 +28,15 @@ constexpr int kSliceMaxCols = 24576;                 // 96 KB of float32 per CTA
 constexpr int kMaxCluster = 16;
 constexpr long long kMaxCols = static_cast<long long>(kSliceMaxCols) * kMaxCluster;  // 393216
 constexpr uint32_t kPieceBytes = 16384;              // one bulk copy instruction
-constexpr uint32_t kSiteRowLoad = 120;               // wait site (low byte of the status word)
+constexpr uint32_t kSiteRowLoad = 120;               // wait sites (low byte of the status word)
+constexpr uint32_t kSiteRowExchange = 123;
+constexpr long long kLatePairCycles = 1ll << 17;     // some 70 us
 
 struct Control {
     uint64_t full;                 // the slice of the current row has landed
     float red[kWarps];             // block reduction
-    float xch[2][2][kMaxCluster];  // [row parity][0: local maxima, 1: local sums] of every CTA of the cluster
+    uint64_t pairs_in[2];          // by row parity: the (maximum, sum) pairs of every CTA of the cluster have arrived
+    float2 xch[2][kMaxCluster];    // [row parity][CTA]
     uint32_t abort_flag;
     uint32_t prior_failure;
 };
@@ -43,6 +47,14 @@ static_assert(sizeof(Control) <= kControlBytes, "control block must fit its slot
 __device__ __noinline__ void drain_copy(uint32_t bar, uint32_t parity) {
     const long long t0 = clock64();
     while (!ptx::mbar_try_wait(bar, parity) && clock64() - t0 < kWaitLimitCycles / 8) {
+    }
+}
+
+// Pairs that peers sent to a CTA that did not wait for them: the cluster's last barrier does not order them, but no more are sent behind
+// it, and the last ones arrive within microseconds.
+__device__ __noinline__ void wait_for_late_pairs() {
+    const long long t0 = clock64();
+    while (clock64() - t0 < kLatePairCycles) {
     }
 }
 
@@ -83,76 +95,78 @@ softmax_rows_smem_kernel(const float* S, OutT* P, long long rows, long long cols
         ptx::grid_dependency_wait();
         const uint32_t prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);  // (arrives meanwhile)
         ptx::mbar_init(&ctl->full, 1);
+        for (int i = 0; i < 2; ++i) ptx::mbar_init(&ctl->pairs_in[i], 1);
         ctl->abort_flag = 0;
         ctl->prior_failure = prior_failure;
         ptx::mbar_fence_init();
     }
     ptx::grid_dependency_wait();
     __syncthreads();
-    // A CTA that sees an earlier failure still takes part in every cluster barrier below, without touching memory.
     bool ok = ctl->prior_failure == 0u;
-    if (C > 1) {  // peers' control blocks are initialised before anyone writes into them (nothing that they read later)
+    if (C > 1) {  // every CTA of the cluster runs, with its barriers in place, before anyone writes into a peer
         ptx::cluster_arrive_relaxed();
         ptx::cluster_wait_acquire();
     }
 
     uint32_t it = 0;
-    for (long long row = cluster; row < rows; row += n_clusters, ++it) {
+    const long long end = ok ? rows : 0;
+    for (long long row = cluster; row < end; row += n_clusters, ++it) {
         const float* src = S + row * cols + c0;
-        if (ok && threadIdx.x == 0 && n > 0) {
+        if (threadIdx.x == 0 && n > 0) {
             const uint32_t bytes = static_cast<uint32_t>(n) * 4u;
             ptx::mbar_expect_tx(&ctl->full, bytes);
             for (uint32_t off = 0; off < bytes; off += kPieceBytes)
                 ptx::bulk_load_1d(ptx::smem_u32(x) + off, reinterpret_cast<const uint8_t*>(src) + off,
                                   bytes - off < kPieceBytes ? bytes - off : kPieceBytes, &ctl->full);
         }
-        if (ok && n > 0 && !fused_wait(&ctl->full, it & 1u, abort_flag, kSiteRowLoad)) {
+        if (n > 0 && !fused_wait(&ctl->full, it & 1u, abort_flag, kSiteRowLoad)) {
             drain_copy(ptx::smem_u32(&ctl->full), it & 1u);
             ok = false;
         }
-        ok = __syncthreads_and(ok);  // all or none of the CTA goes on
+        ok = __syncthreads_and(ok);  // all or none of the CTA goes on, also after a wait for pairs that gave up
+        if (!ok) break;
 
         // ---- pass 1: maximum of the slice ----
         float m = -INFINITY;
-        if (ok)
-            for (int i = threadIdx.x; i < nvec; i += NT) {
-                const float4 v = reinterpret_cast<const float4*>(x)[i];
-                m = fmaxf(m, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
-            }
+        for (int i = threadIdx.x; i < nvec; i += NT) {
+            const float4 v = reinterpret_cast<const float4*>(x)[i];
+            m = fmaxf(m, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+        }
         m = block_reduce<true, NT>(m, ctl->red);
         const float mc = (m > -INFINITY) ? m : 0.0f;  // an empty slice (or a failure upstream): keeps inf - inf out
 
         // ---- pass 2: exponentials relative to the slice's maximum (kept in shared memory), their sum ----
         float l = 0.0f;
-        if (ok)
-            for (int i = threadIdx.x; i < nvec; i += NT) {
-                float4 v = reinterpret_cast<float4*>(x)[i];
-                // (x - m) first: the difference is exact near the maximum, so a constant row gives exactly 1
-                v.x = sr_ex2((v.x - mc) * kLog2e);
-                v.y = sr_ex2((v.y - mc) * kLog2e);
-                v.z = sr_ex2((v.z - mc) * kLog2e);
-                v.w = sr_ex2((v.w - mc) * kLog2e);
-                reinterpret_cast<float4*>(x)[i] = v;
-                l += (v.x + v.y) + (v.z + v.w);
-            }
+        for (int i = threadIdx.x; i < nvec; i += NT) {
+            float4 v = reinterpret_cast<float4*>(x)[i];
+            // (x - m) first: the difference is exact near the maximum, so a constant row gives exactly 1
+            v.x = sr_ex2((v.x - mc) * kLog2e);
+            v.y = sr_ex2((v.y - mc) * kLog2e);
+            v.z = sr_ex2((v.z - mc) * kLog2e);
+            v.w = sr_ex2((v.w - mc) * kLog2e);
+            reinterpret_cast<float4*>(x)[i] = v;
+            l += (v.x + v.y) + (v.z + v.w);
+        }
         l = block_reduce<false, NT>(l, ctl->red);
 
         // ---- one exchange of (maximum, sum) across the cluster; the row's maximum and sum; this slice's factor ----
         float factor;
         if (C > 1) {
-            const uint32_t par = it & 1u;  // two sets of slots: a fast CTA's next row does not overwrite what a slow one reads
-            if (threadIdx.x < static_cast<unsigned>(C)) {
-                ptx::st_cluster_f32(ptx::map_to_cta(ptx::smem_u32(&ctl->xch[par][0][rank]), threadIdx.x), m);
-                ptx::st_cluster_f32(ptx::map_to_cta(ptx::smem_u32(&ctl->xch[par][1][rank]), threadIdx.x), l);
-            }
-            ptx::cluster_arrive_release();
-            ptx::cluster_wait_acquire();
-            float M = ctl->xch[par][0][0];
-            for (int c = 1; c < C; ++c) M = fmaxf(M, ctl->xch[par][0][c]);
+            // By stores that complete bytes on the receiver's mbarrier (with the cluster's barrier, whose release waits for everything in flight:
+            // 8192 x 32768 280 -> 253 us, 300 x 32768 16.3 -> 14.6, 2 x 29664 4.9 -> 4.5).  Two sets of slots, by row parity: a pair of row r + 2 is written only after every pair of row r + 1 has been received, which
+            // the others sent after reading those of row r.
+            const uint32_t par = it & 1u;
+            if (threadIdx.x < static_cast<unsigned>(C))
+                ptx::st_async_b64(ptx::map_to_cta(ptx::smem_u32(&ctl->xch[par][rank]), threadIdx.x), ptx::pack2(m, l),
+                                  ptx::map_to_cta(ptx::smem_u32(&ctl->pairs_in[par]), threadIdx.x));
+            if (threadIdx.x == 0) ptx::mbar_expect_tx(&ctl->pairs_in[par], static_cast<uint32_t>(C) * 8u);
+            ok = fused_wait(&ctl->pairs_in[par], (it >> 1) & 1u, abort_flag, kSiteRowExchange);
+            float M = ctl->xch[par][0].x;
+            for (int c = 1; c < C; ++c) M = fmaxf(M, ctl->xch[par][c].x);
             if (!(M > -INFINITY)) M = 0.0f;
             float L = 0.0f;
             for (int c = 0; c < C; ++c)  // the same order in every CTA; an empty slice has sum 0 and maximum -inf
-                L += ctl->xch[par][1][c] * sr_ex2((ctl->xch[par][0][c] - M) * kLog2e);
+                L += ctl->xch[par][c].y * sr_ex2((ctl->xch[par][c].x - M) * kLog2e);
             factor = sr_ex2((mc - M) * kLog2e) / L;
         } else {
             factor = 1.0f / l;
@@ -172,6 +186,7 @@ softmax_rows_smem_kernel(const float* S, OutT* P, long long rows, long long cols
     if (C > 1) {  // no CTA leaves while a peer may still write into its control block
         ptx::cluster_arrive_relaxed();
         ptx::cluster_wait_acquire();
+        if (!ok) wait_for_late_pairs();
     }
 }
 
@@ -189,7 +204,11 @@ inline cudaError_t launch_nt(const float* S, OutT* P, long long rows, long long 
     const size_t smem = kControlBytes + static_cast<size_t>(slice_cols) * 4;
     const cudaError_t e = allow_smem<softmax_rows_smem_kernel<OutT, NT>>(kControlBytes + kSliceMaxCols * 4, true);
     if (e != cudaSuccess) return e;
-    const long long per_sm = NT == 256 ? (smem * 4 <= 224 * 1024 ? 4 : 3) : 2;
+    // Four CTAs of 256 threads on an SM where they fit, but three for many float32 rows: there fewer rows in flight keep the stream of HBM
+    // smoother.  us, four / three: 14000 x 12000 237 / 214, 16000 x 10240 229 / 214, 9000 x 24580 300 / 286, 6000 x 26000 222 / 203, 2000 x 25000 72.8 /
+    // 70.9; few rounds of rows or short slices want four: 2500 x 13000 47.3 / 47.4, 1000 x 14000 20.4 / 21.5, 20000 x 8200 203 / 218.
+    const bool many_f32 = sizeof(OutT) == 4 && slice_cols >= 10240 && rows * C >= 27ll * sm_count;
+    const long long per_sm = NT == 256 ? (smem * 4 <= 224 * 1024 && !many_f32 ? 4 : 3) : 2;
     long long n_clusters = (per_sm * sm_count) / C;  // CTAs that fit at once
     if (n_clusters < 1) n_clusters = 1;
     if (n_clusters > rows) n_clusters = rows;
@@ -225,7 +244,6 @@ constexpr int kRcSliceMaxCols = kRcThreads * kRcVecPerThread * 4;               
 constexpr long long kRcMaxCols = static_cast<long long>(kRcSliceMaxCols) * kMaxCluster;  // 262144
 constexpr uint32_t kSiteRcRowLoad = 121;
 constexpr uint32_t kSiteRcExchange = 122;
-constexpr long long kLatePairCycles = 1ll << 17;  // some 70 us
 
 struct RcControl {
     uint64_t full[kRcThreads / 32];  // one per warp: its piece of the current row has landed
@@ -401,13 +419,7 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
         ptx::cluster_arrive_relaxed();
         ptx::cluster_wait_acquire();
     }
-    if (!ok) {
-        // Pairs that peers sent to a CTA that did not wait for them: the barrier does not order them, but no more are sent behind
-        // it, and the last ones arrive within microseconds.
-        const long long t0 = clock64();
-        while (clock64() - t0 < kLatePairCycles) {
-        }
-    }
+    if (!ok) wait_for_late_pairs();
 }
 
 inline int rc_cluster_ctas_for(long long cols) {  // any size up to 16, not only powers of two
