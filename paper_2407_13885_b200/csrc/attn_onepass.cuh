@@ -64,6 +64,7 @@ enum : uint32_t {  // wait sites of this kernel (low byte of the status word)
     kSiteOutFilled = 104,
     kSiteLFull = 105,
     kSiteMaxFull = 106,
+    kSitePairsIn = 107,
 };
 
 constexpr int kUnitStats = 4 * kTile;
@@ -99,7 +100,8 @@ struct Smem {
     static constexpr int kQOff = 0;                            // two query tiles; split: one, and one more stage of the ring
     static constexpr int kKOff = kQOff + 2 * kTileBytes;
     static constexpr int kStatOff = kKOff + kStages * kTileBytes;  // per unit: maxima, float [2 steps][2 halves][128 rows]; at the end sums and offset
-    static constexpr int kBarOff = kStatOff + 2 * kUnitStats * 4;
+    static constexpr int kPairOff = kStatOff + 2 * kUnitStats * 4;  // clusters: float2 [CTA][128 rows], (offset, sum) of each CTA's part
+    static constexpr int kBarOff = kPairOff + kMaxCluster * kTile * 8;
     static constexpr int kBytes = kBarOff + 512;
     static constexpr int kDynamicBytes = kBytes + 1024;
 };
@@ -114,6 +116,7 @@ struct Barriers {
     uint64_t max_full[2][4];        // per unit and lane quarter, without turns: the maxima of both halves are in shared memory (2 warps)
     uint64_t l_full[2];             // per query tile: the row statistics of its warps are in shared memory
     uint64_t out_filled[2];
+    uint64_t pairs_in;              // clusters: the pairs of every CTA have arrived
     uint32_t tmem_base;
     uint32_t abort_flag;
     uint32_t prior_failure;
@@ -189,6 +192,10 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             ptx::mbar_init(&bars->l_full[q], split ? 16 : 8);
             ptx::mbar_init(&bars->out_filled[q], split ? 15 : 7);
         }
+        if constexpr (M == kCluster) {
+            ptx::mbar_init(&bars->pairs_in, 1);
+            ptx::mbar_expect_tx(&bars->pairs_in, static_cast<uint32_t>(G * kTile * 8));
+        }
         bars->abort_flag = 0;
         bars->prior_failure = prior_failure;
         ptx::mbar_fence_init();
@@ -206,6 +213,10 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     ptx::grid_dependency_wait();
     ptx::tc_fence_before_sync();
     __syncthreads();
+    if constexpr (M == kCluster) {  // every CTA runs, with its barriers in place, before anyone writes into a peer
+        ptx::cluster_arrive_relaxed();
+        ptx::cluster_wait_acquire();
+    }
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bars->tmem_base;
     const bool run = bars->prior_failure == 0u;  // an earlier CTA gave up: do not queue more waits behind it
@@ -564,28 +575,31 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 ok = warp_wait(bar_of(offsetof(Barriers, l_full), u), 0, abort_flag, kSiteLFull);
             }
             if constexpr (M == kCluster) {
-                // The CTAs of a cluster have worked on other key tiles of the same query tile.  Each leaves its rows' (offset, sum) in
-                // its shared memory; after the cluster's barrier every thread knows its row's global ones, scales its
-                // part of O and sends it to the CTA that owns the row (128 / G rows each); after another barrier the
-                // owners add the G parts, in the order of the CTAs, and write O.
-                float2* pairs = reinterpret_cast<float2*>(smem + L::kKOff + 4096);
-                const uint32_t parts = ptx::smem_u32(smem + L::kKOff + 8192);  // float [G CTAs][128 / G rows][D], 16-byte pieces XOR-swizzled by row
+                // The CTAs of a cluster have worked on other key tiles of the same query tile.  Each sends its rows' (offset, sum) to all; with
+                // them every thread knows its row's global ones, scales its part of O and sends it to the CTA that owns the row (128 / G
+                // rows each); after the cluster's barrier the owners add the G parts, in the order of the CTAs, and write O.  The pairs complete
+                // bytes on their readers' mbarriers: with a barrier of the cluster there too 2 x 1798, d = 128 took 13.3 us (now 12.9), 1 x 2500 14.5 (14.25); the parts by such stores were slower (1 x 2500, d =
+                // 128 14.5 -> 15.4 us).
                 const int my_rows = kTile / G;
                 const float l_own = ok ? l + stats[(half ^ 1) * kTile + row] : 1.0f;
                 const float mb_other = ok ? *mb_peer : 0.0f;
                 if (ok && q == 0 && half == 0) {
                     const float top = fmaxf(mb, mb_other);
-                    pairs[row] = make_float2(top, l_own * ptx::ex2_approx(mb - top) + (l_peer[0] + l_peer[kTile]) * ptx::ex2_approx(mb_other - top));
+                    const uint64_t pair = ptx::pack2(top, l_own * ptx::ex2_approx(mb - top) + (l_peer[0] + l_peer[kTile]) * ptx::ex2_approx(mb_other - top));
+                    for (int g = 0; g < G; ++g)
+                        ptx::st_async_b64(ptx::map_to_cta(ptx::smem_u32(smem + L::kPairOff + (rank * kTile + row) * 8), static_cast<uint32_t>(g)), pair,
+                                          ptx::map_to_cta(ptx::smem_u32(&bars->pairs_in), static_cast<uint32_t>(g)));
                 }
                 __syncwarp();
-                ptx::cluster_arrive_release();
-                ptx::cluster_wait_acquire();
+                if (ok) ok = warp_wait(bar_of(offsetof(Barriers, pairs_in), 0), 0, abort_flag, kSitePairsIn);
                 if (ok) {
+                    // (every CTA has sent its pairs behind its last product: the rings of all are free)
+                    const float2* pairs = reinterpret_cast<const float2*>(smem + L::kPairOff) + row;
                     float2 pair[kMaxCluster];
                     float top = -3.0e38f, sum = 0.0f;
 #pragma unroll
                     for (int g = 0; g < kMaxCluster; ++g) {
-                        pair[g] = ptx::ld_cluster_v2(ptx::map_to_cta(ptx::smem_u32(pairs + row), static_cast<uint32_t>(g < G ? g : 0)));
+                        pair[g] = pairs[(g < G ? g : 0) * kTile];
                         top = fmaxf(top, pair[g].x);
                     }
 #pragma unroll
@@ -595,8 +609,9 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                     ptx::tc_fence_after_sync();
                     const uint32_t o_unit = t_quarter + L::o_col(q);
                     const uint32_t o_peer = t_quarter + L::o_col(q ^ 1);
-                    const uint32_t dst = ptx::map_to_cta(parts + static_cast<uint32_t>((rank * my_rows + row % my_rows) * D * 4),
-                                                         static_cast<uint32_t>(row / my_rows));
+                    // float [G CTAs][128 / G rows][D], 16-byte pieces XOR-swizzled by row
+                    const uint32_t owner = static_cast<uint32_t>(row / my_rows);
+                    const uint32_t dst = ptx::map_to_cta(ptx::smem_u32(smem + L::kKOff) + static_cast<uint32_t>((rank * my_rows + row % my_rows) * D * 4), owner);
                     const int col0 = (q * 2 + half) * (D / 4);
 #pragma unroll 1
                     for (int c = col0; c < col0 + D / 4; c += 16) {
@@ -625,7 +640,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                         if (at >= N) continue;
                         float v[8] = {};
                         for (int g = 0; g < G; ++g) {
-                            const float4* src = reinterpret_cast<const float4*>(smem + L::kKOff + 8192) + (g * my_rows + r) * (D / 4);
+                            const float4* src = reinterpret_cast<const float4*>(smem + L::kKOff) + (g * my_rows + r) * (D / 4);
                             const float4 a = src[(2 * piece) ^ (r & 7)], b = src[(2 * piece + 1) ^ (r & 7)];
                             v[0] += a.x, v[1] += a.y, v[2] += a.z, v[3] += a.w;
                             v[4] += b.x, v[5] += b.y, v[6] += b.z, v[7] += b.w;
@@ -702,10 +717,8 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     }
 
     if constexpr (M == kCluster) {
-        if (!run || warp >= kSmWarps) {  // the Softmax warps' two barriers
+        if (!run || warp >= kSmWarps) {  // the Softmax warps' barrier, behind which no CTA writes into a peer
             __syncwarp();
-            ptx::cluster_arrive_release();
-            ptx::cluster_wait_acquire();
             ptx::cluster_arrive_release();
             ptx::cluster_wait_acquire();
         }
@@ -713,6 +726,9 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     // ---- teardown: every role falls through to here, also after a wait gave up ----
     ptx::tc_fence_before_sync();
     __syncthreads();
+    if constexpr (M == kCluster) {
+        if (*abort_flag || !run) wait_for_late_stores();
+    }
     if (warp == kMma) {
         ptx::tc_fence_after_sync();
         ptx::tmem_dealloc(tmem_base, kTmemCols);

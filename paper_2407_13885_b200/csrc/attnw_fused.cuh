@@ -160,6 +160,15 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
     return warp_wait_slow(bar, parity, abort_flag, site);
 }
 
+// Values that peers sent (st.async) to a CTA that, after a wait gave up, did not wait for them: the cluster's last barrier does not order
+// them, but no more are sent behind it, and the last ones arrive within microseconds.
+constexpr long long kLateStoreCycles = 1ll << 17;  // some 70 us
+__device__ __noinline__ void wait_for_late_stores() {
+    const long long t0 = clock64();
+    while (clock64() - t0 < kLateStoreCycles) {
+    }
+}
+
 // One thread's 32 consecutive columns of a score tile (TMEM lane = row).
 __device__ __forceinline__ void load_chunk(uint32_t taddr, float (&s)[kChunk]) {
     uint32_t r[32];

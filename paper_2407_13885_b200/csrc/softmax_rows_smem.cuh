@@ -30,7 +30,6 @@ constexpr long long kMaxCols = static_cast<long long>(kSliceMaxCols) * kMaxClust
 constexpr uint32_t kPieceBytes = 16384;              // one bulk copy instruction
 constexpr uint32_t kSiteRowLoad = 120;               // wait sites (low byte of the status word)
 constexpr uint32_t kSiteRowExchange = 123;
-constexpr long long kLatePairCycles = 1ll << 17;     // some 70 us
 
 struct Control {
     uint64_t full;                 // the slice of the current row has landed
@@ -47,14 +46,6 @@ static_assert(sizeof(Control) <= kControlBytes, "control block must fit its slot
 __device__ __noinline__ void drain_copy(uint32_t bar, uint32_t parity) {
     const long long t0 = clock64();
     while (!ptx::mbar_try_wait(bar, parity) && clock64() - t0 < kWaitLimitCycles / 8) {
-    }
-}
-
-// Pairs that peers sent to a CTA that did not wait for them: the cluster's last barrier does not order them, but no more are sent behind
-// it, and the last ones arrive within microseconds.
-__device__ __noinline__ void wait_for_late_pairs() {
-    const long long t0 = clock64();
-    while (clock64() - t0 < kLatePairCycles) {
     }
 }
 
@@ -186,7 +177,7 @@ softmax_rows_smem_kernel(const float* S, OutT* P, long long rows, long long cols
     if (C > 1) {  // no CTA leaves while a peer may still write into its control block
         ptx::cluster_arrive_relaxed();
         ptx::cluster_wait_acquire();
-        if (!ok) wait_for_late_pairs();
+        if (!ok) wait_for_late_stores();
     }
 }
 
@@ -419,7 +410,7 @@ softmax_rows_regcluster_kernel(const float* S, OutT* P, long long rows, long lon
         ptx::cluster_arrive_relaxed();
         ptx::cluster_wait_acquire();
     }
-    if (!ok) wait_for_late_pairs();
+    if (!ok) wait_for_late_stores();
 }
 
 inline int rc_cluster_ctas_for(long long cols) {  // any size up to 16, not only powers of two
