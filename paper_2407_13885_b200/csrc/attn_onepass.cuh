@@ -119,7 +119,6 @@ struct Barriers {
     uint64_t pairs_in;              // clusters: the pairs of every CTA have arrived
     uint32_t tmem_base;
     uint32_t abort_flag;
-    uint32_t prior_failure;
 };
 static_assert(sizeof(Barriers) <= 512, "barrier block must fit its slot");
 
@@ -175,8 +174,6 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 
     // ---- set-up ------------------------------------------------------------------------------
     if (threadIdx.x == 0) {
-        ptx::grid_dependency_wait();
-        const uint32_t prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);  // (arrives meanwhile)
         ptx::mbar_init(&bars->q_full, 1);
         for (int s = 0; s < 7; ++s) {
             ptx::mbar_init(&bars->k_full[s], 1);
@@ -197,7 +194,6 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             ptx::mbar_expect_tx(&bars->pairs_in, static_cast<uint32_t>(G * kTile * 8));
         }
         bars->abort_flag = 0;
-        bars->prior_failure = prior_failure;
         ptx::mbar_fence_init();
     }
     if (warp == kProducer && lane == 0) {
@@ -219,9 +215,9 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     }
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bars->tmem_base;
-    const bool run = bars->prior_failure == 0u;  // an earlier CTA gave up: do not queue more waits behind it
+    int loads = 0;  // producer: ring entries asked for
 
-    if (run && warp == kProducer) {
+    if (warp == kProducer) {
         // ================= TMA producer: Q once, then the K and V tiles in the order the MMA issuer reads them =========
         // Two query tiles at d = 128: the whole warp walks the list and an elected lane issues (a lone lane takes 300 cycles a tile: 2 x 97
         // 6.4 -> 6.2 us).  Otherwise a lone lane (3 x 863, d = 64 10.06 us, the whole warp 10.16; 3 x 802, d = 128 11.05 and 11.15).
@@ -262,27 +258,22 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                     if (j >= 0 && j < steps[q]) load(&tm_v, key_tile(j, q));
                 }
             }
-            if (*abort_flag && lane == 0) {
-                // Unwinding: let the copies already in flight land before shared memory is released.
-                const int first = n > kStages ? n - kStages : 0;
-                for (int it = first; it < n; ++it) {
-                    const long long t0 = clock64();
-                    while (!ptx::mbar_try_wait(&bars->k_full[it % kStages], static_cast<uint32_t>(it / kStages) & 1u) &&
-                           clock64() - t0 < kWaitLimitCycles / 8) {
-                    }
-                }
-                const long long t0 = clock64();
-                while (!ptx::mbar_try_wait(&bars->q_full, 0) && clock64() - t0 < kWaitLimitCycles / 8) {
-                }
-            }
+            loads = n;
         }
         __syncwarp();
-    } else if (run && (warp == kMma || (two_issuers && warp == kMmaProduct))) {
+    } else if (warp == kMma || (two_issuers && warp == kMmaProduct)) {
         // ================= MMA issuers (warp-uniform loops, one elected lane issues): of scores, of products, or of both =================
         constexpr uint32_t idesc_s = ptx::umma_idesc_bf16_f32(kTile, kTile);
         constexpr uint32_t idesc_o = ptx::umma_idesc_bf16_f32(kTile, D) | (1u << 16);  // B operand MN-major
         const uint32_t base = ptx::smem_u32(smem);
+        // Did an earlier launch give up?  Then this one computes and writes nothing: looked at in front of the first MMA, when it has
+        // arrived beside the first loads (in front of the set-up's barrier: 3 x 128 5.04 us, now 4.91; 7 x 64, d = 128 6.10, 5.93; 12 x 1021 11.2, 11.1).
+        const uint32_t prior_failure = *reinterpret_cast<volatile unsigned int*>(&g_attnw_status);
         bool ok = warp_wait(bar_of(offsetof(Barriers, q_full), 0), 0, abort_flag, kSiteMmaQ);
+        if (__any_sync(0xffffffffu, prior_failure != 0u)) {
+            *abort_flag = 1;
+            ok = false;
+        }
         int n = 0;            // next ring entry, in step with the producer
         auto arrived = [&]() {
             ok = ok && warp_wait(bar_of(offsetof(Barriers, k_full), n % kStages), static_cast<uint32_t>(n / kStages) & 1u, abort_flag, kSiteMmaKFull);
@@ -400,7 +391,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 }
             }
         }
-    } else if (run && warp < kSmWarps) {
+    } else if (warp < kSmWarps) {
         // ================= Softmax warps: two threads per query row, 64 key columns of a tile each =================
         const int q = warp >> 3;
         const int half = (warp >> 2) & 1;
@@ -717,7 +708,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     }
 
     if constexpr (M == kCluster) {
-        if (!run || warp >= kSmWarps) {  // the Softmax warps' barrier, behind which no CTA writes into a peer
+        if (warp >= kSmWarps) {  // the Softmax warps' barrier, behind which no CTA writes into a peer
             __syncwarp();
             ptx::cluster_arrive_release();
             ptx::cluster_wait_acquire();
@@ -726,8 +717,18 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     // ---- teardown: every role falls through to here, also after a wait gave up ----
     ptx::tc_fence_before_sync();
     __syncthreads();
-    if constexpr (M == kCluster) {
-        if (*abort_flag || !run) wait_for_late_stores();
+    if (*abort_flag) {
+        if constexpr (M == kCluster) wait_for_late_stores();
+        // Unwinding: let the copies already in flight land before shared memory is released.
+        if (warp == kProducer && lane == 0) {
+            const long long t0 = clock64();
+            for (int it = loads > kStages ? loads - kStages : 0; it < loads; ++it)
+                while (!ptx::mbar_try_wait(&bars->k_full[it % kStages], static_cast<uint32_t>(it / kStages) & 1u) &&
+                       clock64() - t0 < kWaitLimitCycles / 8) {
+                }
+            while (!ptx::mbar_try_wait(&bars->q_full, 0) && clock64() - t0 < kWaitLimitCycles / 8) {
+            }
+        }
     }
     if (warp == kMma) {
         ptx::tc_fence_after_sync();

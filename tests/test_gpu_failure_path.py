@@ -91,3 +91,17 @@ def test_selftest_rejects_limits_out_of_range(attnw):
             attnw.selftest_wait_timeout(bad)
         assert e.value.code == 2
     assert attnw.query_status() == 0
+
+
+@pytest.mark.parametrize("n", [100, 600, 2500])  # one CTA a pair of query tiles, a query tile; a cluster a query tile
+def test_attention_behind_a_failure_writes_nothing(attnw, n):
+    q = torch.randn(1, 1, n, 64, device="cuda").to(torch.bfloat16)
+    out = torch.full((1, 1, n, 64), float("nan"), dtype=torch.bfloat16, device="cuda")
+    attnw.selftest_wait_timeout(200_000)
+    attnw.attn_fused(q, q, q, 0.125, O=out)
+    torch.cuda.synchronize()
+    assert bool(torch.isnan(out).all())
+    assert attnw.query_status() == SELFTEST_SITE
+    attnw.attn_fused(q, q, q, 0.125, O=out)
+    torch.cuda.synchronize()
+    assert not bool(torch.isnan(out).any()) and attnw.query_status() == 0
