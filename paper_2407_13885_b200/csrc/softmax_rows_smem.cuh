@@ -100,49 +100,49 @@ softmax_rows_smem_kernel(const float* S, OutT* P, long long rows, long long cols
     }
 
     uint32_t it = 0;
-    const long long end = ok ? rows : 0;
-    for (long long row = cluster; row < end; row += n_clusters, ++it) {
+    for (long long row = cluster; row < rows; row += n_clusters, ++it) {
         const float* src = S + row * cols + c0;
-        if (threadIdx.x == 0 && n > 0) {
+        if (ok && threadIdx.x == 0 && n > 0) {
             const uint32_t bytes = static_cast<uint32_t>(n) * 4u;
             ptx::mbar_expect_tx(&ctl->full, bytes);
             for (uint32_t off = 0; off < bytes; off += kPieceBytes)
                 ptx::bulk_load_1d(ptx::smem_u32(x) + off, reinterpret_cast<const uint8_t*>(src) + off,
                                   bytes - off < kPieceBytes ? bytes - off : kPieceBytes, &ctl->full);
         }
-        if (n > 0 && !fused_wait(&ctl->full, it & 1u, abort_flag, kSiteRowLoad)) {
+        if (ok && n > 0 && !fused_wait(&ctl->full, it & 1u, abort_flag, kSiteRowLoad)) {
             drain_copy(ptx::smem_u32(&ctl->full), it & 1u);
             ok = false;
         }
         ok = __syncthreads_and(ok);  // all or none of the CTA goes on, also after a wait for pairs that gave up
-        if (!ok) break;
 
         // ---- pass 1: maximum of the slice ----
         float m = -INFINITY;
-        for (int i = threadIdx.x; i < nvec; i += NT) {
-            const float4 v = reinterpret_cast<const float4*>(x)[i];
-            m = fmaxf(m, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
-        }
+        if (ok)
+            for (int i = threadIdx.x; i < nvec; i += NT) {
+                const float4 v = reinterpret_cast<const float4*>(x)[i];
+                m = fmaxf(m, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+            }
         m = block_reduce<true, NT>(m, ctl->red);
         const float mc = (m > -INFINITY) ? m : 0.0f;  // an empty slice (or a failure upstream): keeps inf - inf out
 
         // ---- pass 2: exponentials relative to the slice's maximum (kept in shared memory), their sum ----
         float l = 0.0f;
-        for (int i = threadIdx.x; i < nvec; i += NT) {
-            float4 v = reinterpret_cast<float4*>(x)[i];
-            // (x - m) first: the difference is exact near the maximum, so a constant row gives exactly 1
-            v.x = sr_ex2((v.x - mc) * kLog2e);
-            v.y = sr_ex2((v.y - mc) * kLog2e);
-            v.z = sr_ex2((v.z - mc) * kLog2e);
-            v.w = sr_ex2((v.w - mc) * kLog2e);
-            reinterpret_cast<float4*>(x)[i] = v;
-            l += (v.x + v.y) + (v.z + v.w);
-        }
+        if (ok)
+            for (int i = threadIdx.x; i < nvec; i += NT) {
+                float4 v = reinterpret_cast<float4*>(x)[i];
+                // (x - m) first: the difference is exact near the maximum, so a constant row gives exactly 1
+                v.x = sr_ex2((v.x - mc) * kLog2e);
+                v.y = sr_ex2((v.y - mc) * kLog2e);
+                v.z = sr_ex2((v.z - mc) * kLog2e);
+                v.w = sr_ex2((v.w - mc) * kLog2e);
+                reinterpret_cast<float4*>(x)[i] = v;
+                l += (v.x + v.y) + (v.z + v.w);
+            }
         l = block_reduce<false, NT>(l, ctl->red);
 
         // ---- one exchange of (maximum, sum) across the cluster; the row's maximum and sum; this slice's factor ----
-        float factor;
-        if (C > 1) {
+        float factor = 0.0f;
+        if (C > 1 && ok) {  // (a CTA that has given up sends nothing)
             // By stores that complete bytes on the receiver's mbarrier (with the cluster's barrier, whose release waits for everything in flight:
             // 8192 x 32768 280 -> 253 us, 300 x 32768 16.3 -> 14.6, 2 x 29664 4.9 -> 4.5).  Two sets of slots, by row parity: a pair of row r + 2 is written only after every pair of row r + 1 has been received, which
             // the others sent after reading those of row r.
@@ -159,7 +159,7 @@ softmax_rows_smem_kernel(const float* S, OutT* P, long long rows, long long cols
             for (int c = 0; c < C; ++c)  // the same order in every CTA; an empty slice has sum 0 and maximum -inf
                 L += ctl->xch[par][c].y * sr_ex2((ctl->xch[par][c].x - M) * kLog2e);
             factor = sr_ex2((mc - M) * kLog2e) / L;
-        } else {
+        } else if (C == 1) {
             factor = 1.0f / l;
         }
 
