@@ -759,7 +759,7 @@ int launch_project(const DeviceInfo* dev, const void* X, const void* Wq, const v
     // Tiles of 256 x 256 per pair of CTAs; narrow ones of 256 x 128 where a single round of them holds the call, since a narrow slice still takes
     // 0.6 to 0.75 of the time of a whole one (X's rows are fetched for half of the MMAs).  A last round whose tiles would occupy at most
     // half of the pairs takes them cut in two.  us per call, whole tiles only -> as chosen: narrow 4 x 100 x 1536 to 12 x 128 11.3 -> 7.7,
-    // 1 x 1000 x 1024 to 16 x 64 9.3 -> 6.7, 2 x 949 x 576 to 9 x 64 7.2 -> 5.7, 1 x 256 x 4096 to 64 x 64 24.9 -> 21.2; last round 1 x 2048 x
+    // 1 x 1000 x 1024 to 16 x 64 9.3 -> 6.7, 2 x 949 x 576 to 9 x 64 7.2 -> 5.7, 1 x 256 x 4096 to 64 x 64 24.9 -> 21.2; tiles cut in two 1 x 2048 x
     // 4096 to 32 x 128 (256 tiles for 74 pairs) 111.8 -> 107.6, 2 x 444 x 3200 to 25 x 128 (100) 40.7 -> 37.4, 4 x 3749 x 4080 to 10 x 64 (300) 142.5 -> 140.8.
     const int pairs = dev->sm_count / 2;
     const int block = proj::Grid(B, N, static_cast<int>(hd), proj::kFeatures / 2).tiles() <= pairs ? proj::kFeatures / 2 : proj::kFeatures;
