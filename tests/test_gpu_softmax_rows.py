@@ -181,3 +181,16 @@ def test_chain_reads_what_the_kernel_in_front_wrote(attnw, rows, cols):
         torch.cuda.synchronize()
         assert attnw.query_status() == 0
         assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+# Several rows a cluster of two, so that both sets of exchange slots are used again (slices of up to 14300 and of up to 16384 columns, an uneven
+# last slice), and many float32 rows of one CTA each
+@pytest.mark.parametrize("rows,cols,dtype", [(1500, 24580, torch.bfloat16), (1300, 32768, torch.float32), (2100, 24580, torch.float32), (4100, 10244, torch.float32)])
+def test_many_rows_in_shared_memory(attnw, rows, cols, dtype):
+    S = inputs.normal_f32(11, rows * 151 + cols, rows * cols, 3.0).reshape(rows, cols)
+    raw, P, g = guarded_empty((rows, cols), dtype)
+    attnw.softmax_rows(torch.from_numpy(S).cuda(), P=P)
+    torch.cuda.synchronize()
+    assert_guards_intact(raw, g)
+    assert_close_to_oracle(P, oracle.softmax_rows(S), f"rows={rows} cols={cols}")
+    assert attnw.query_status() == 0
