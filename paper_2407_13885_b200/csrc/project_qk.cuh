@@ -75,6 +75,10 @@ struct Grid {
     __host__ __device__ int tiles() const { return feature_blocks * row_tiles; }
 };
 
+// Whether the accumulator of item t is filled again by the same pair.  Only then does anyone wait for its release, and only then may the odd
+// CTA send one: the even CTA might have ended before an arrival that nothing waits for.
+__host__ __device__ constexpr bool accumulator_comes_again(int t, int pairs, int items) { return items - t > kSlots * pairs; }
+
 // grid: clusters of two CTAs; pair p takes the items p, p + pairs, ...: the tiles 0 ... whole_tiles - 1, then the halves of the others.
 __global__ void __launch_bounds__(kThreads, 1)
 project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_wq,
@@ -286,7 +290,7 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 ptx::tmem_ld_32x32b_x32(taddr + static_cast<uint32_t>(c), v[0]);
                 ptx::tmem_ld_32x32b_x32(taddr + static_cast<uint32_t>(c + 32), v[1]);
                 ptx::tmem_wait_ld();
-                if (c + 64 == width) {  // the accumulator may be overwritten
+                if (c + 64 == width && accumulator_comes_again(t, pairs, items)) {  // it may be overwritten
                     ptx::tc_fence_before_sync();
                     __syncwarp();
                     if (lane == 0) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&bars->acc_empty[slot]), 0));
