@@ -160,8 +160,8 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
     return warp_wait_slow(bar, parity, abort_flag, site);
 }
 
-// Values that peers sent (st.async) to a CTA that, after a wait gave up, did not wait for them: the cluster's last barrier does not order
-// them, but no more are sent behind it, and the last ones arrive within microseconds.
+// Values (st.async) and arrivals that peers sent to a CTA that, after a wait gave up, did not wait for them: the cluster's last barrier does
+// not order them, but no more are sent behind it, and the last ones arrive within microseconds.
 constexpr long long kLateStoreCycles = 1ll << 17;  // some 70 us
 __device__ __noinline__ void wait_for_late_stores() {
     const long long t0 = clock64();

@@ -60,7 +60,8 @@ struct Barriers {
     uint32_t tmem_base;
     uint32_t abort_flag;
     uint32_t prior_failure;
-    int loads;  // stages that a producer has asked for
+    uint32_t peer_ran;  // written by the other CTA when it unwinds
+    int loads;          // stages that a producer has asked for
 };
 static_assert(sizeof(Barriers) <= 256, "barrier block must fit its slot");
 
@@ -151,7 +152,8 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             ptx::mbar_init(&bars->acc_full[s], 1);
             ptx::mbar_init(&bars->acc_empty[s], 2 * kEpiWarps);
         }
-        bars->abort_flag = 0;
+        bars->abort_flag = prior_failure;
+        bars->peer_ran = 0;
         bars->loads = 0;
         bars->prior_failure = prior_failure;
         ptx::mbar_fence_init();
@@ -174,7 +176,8 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     ptx::cluster_wait_acquire();
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bars->tmem_base;
-    // an earlier launch gave up: do not queue more waits behind it (should the CTAs of a pair disagree, the waits of one run out)
+    // An earlier launch gave up: do not queue more waits behind it.  Should the word be cleared between the two CTAs' looks at it, the one that
+    // has seen it tells the other in the teardown, where nothing is stored yet: each tile needs both CTAs' loads and the even one's MMAs.
     const bool run = bars->prior_failure == 0u;
 
     if (run && (warp == kProducerX || warp == kProducerW)) {
@@ -331,6 +334,7 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     __syncthreads();
     if (threadIdx.x == 0 && *abort_flag) {
         ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&bars->abort_flag), rank ^ 1), 1u);
+        if (run) ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&bars->peer_ran), rank ^ 1), 1u);
         ptx::fence_cluster();
     }
     __syncwarp();
@@ -338,7 +342,9 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     ptx::cluster_wait_acquire();
     ptx::tc_fence_after_sync();
     if (*abort_flag) {
-        // Unwinding: let the copies of both CTAs that are in flight land before shared memory is released.
+        // Unwinding: let the MMAs of the pair and the arrivals on either CTA that nobody has waited for come to their end, and the copies of both
+        // CTAs land, before shared and tensor memory are released.
+        if (run || bars->peer_ran) wait_for_late_stores();
         if (rank == 0 && threadIdx.x == 0) {
             const int mine = bars->loads;
             const int theirs = static_cast<int>(ptx::ld_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&bars->loads), 1)));

@@ -105,3 +105,19 @@ def test_attention_behind_a_failure_writes_nothing(attnw, n):
     attnw.attn_fused(q, q, q, 0.125, O=out)
     torch.cuda.synchronize()
     assert not bool(torch.isnan(out).any()) and attnw.query_status() == 0
+
+
+# narrow tiles, an odd CTA without rows; several rounds of tiles
+@pytest.mark.parametrize("B,N,d_model,H,d", [(1, 100, 72, 3, 64), (2, 2600, 64, 8, 128)])
+def test_projection_behind_a_failure_writes_nothing(attnw, B, N, d_model, H, d):
+    x = torch.randn(B, N, d_model, device="cuda").to(torch.bfloat16)
+    w = torch.randn(H, d, d_model, device="cuda").to(torch.bfloat16)
+    Q, K = (torch.full((B, H, N, d), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    attnw.selftest_wait_timeout(200_000)
+    attnw.project_qk(x, w, w, Q=Q, K=K)
+    torch.cuda.synchronize()
+    assert bool(torch.isnan(Q).all()) and bool(torch.isnan(K).all())
+    assert attnw.query_status() == SELFTEST_SITE  # the launch has not given up on a wait of its own
+    attnw.project_qk(x, w, w, Q=Q, K=K)
+    torch.cuda.synchronize()
+    assert not bool(torch.isnan(Q).any()) and torch.equal(Q, K) and attnw.query_status() == 0
