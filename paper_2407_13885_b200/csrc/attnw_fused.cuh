@@ -169,6 +169,13 @@ __device__ __noinline__ void wait_for_late_stores() {
     }
 }
 
+// Each CTA of a cluster looks at the status word for itself, and another stream's query may clear it in between.  One that has seen a failure,
+// or has given up, and will send nothing more tells its peers, which wait for it in front of their stores: they give up as well, and no second
+// failure is recorded.  Only when every CTA of the cluster runs.
+__device__ __noinline__ void tell_peers(uint32_t* abort_flag, int ctas) {
+    for (int c = 0; c < ctas; ++c) ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(abort_flag), static_cast<uint32_t>(c)), 1u);
+}
+
 // One thread's 32 consecutive columns of a score tile (TMEM lane = row).
 __device__ __forceinline__ void load_chunk(uint32_t taddr, float (&s)[kChunk]) {
     uint32_t r[32];

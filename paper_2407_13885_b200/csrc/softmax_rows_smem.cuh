@@ -144,8 +144,8 @@ softmax_rows_smem_kernel(const float* S, OutT* P, long long rows, long long cols
         float factor = 0.0f;
         if (C > 1 && ok) {  // (a CTA that has given up sends nothing)
             // By stores that complete bytes on the receiver's mbarrier (with the cluster's barrier, whose release waits for everything in flight:
-            // 8192 x 32768 280 -> 253 us, 300 x 32768 16.3 -> 14.6, 2 x 29664 4.9 -> 4.5).  Two sets of slots, by row parity: a pair of row r + 2 is written only after every pair of row r + 1 has been received, which
-            // the others sent after reading those of row r.
+            // 8192 x 32768 280 -> 253 us, 300 x 32768 16.3 -> 14.6, 2 x 29664 4.9 -> 4.5).  Two sets of slots, by row parity: a pair of row
+            // r + 2 is written only after every pair of row r + 1 has been received, which the others sent after reading those of row r.
             const uint32_t par = it & 1u;
             if (threadIdx.x < static_cast<unsigned>(C))
                 ptx::st_async_b64(ptx::map_to_cta(ptx::smem_u32(&ctl->xch[par][rank]), threadIdx.x), ptx::pack2(m, l),
@@ -175,6 +175,8 @@ softmax_rows_smem_kernel(const float* S, OutT* P, long long rows, long long cols
         __syncthreads();                // the slice is free for the next row's copy
     }
     if (C > 1) {  // no CTA leaves while a peer may still write into its control block
+        if (!ok) tell_peers(&ctl->abort_flag, C);
+        __syncwarp();
         ptx::cluster_arrive_relaxed();
         ptx::cluster_wait_acquire();
         if (!ok) wait_for_late_stores();

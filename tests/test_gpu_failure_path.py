@@ -121,3 +121,19 @@ def test_projection_behind_a_failure_writes_nothing(attnw, B, N, d_model, H, d):
     attnw.project_qk(x, w, w, Q=Q, K=K)
     torch.cuda.synchronize()
     assert not bool(torch.isnan(Q).any()) and torch.equal(Q, K) and attnw.query_status() == 0
+
+
+# a cluster of two a row: one row; several rows a cluster
+@pytest.mark.parametrize("rows,cols", [(1, 24580), (700, 32768)])
+def test_rows_of_two_ctas_behind_a_failure_write_nothing(attnw, rows, cols):
+    S = torch.randn(rows, cols, device="cuda")
+    P = torch.full((rows, cols), float("nan"), device="cuda")
+    attnw.selftest_wait_timeout(200_000)
+    attnw.softmax_rows(S, P=P)
+    torch.cuda.synchronize()
+    assert bool(torch.isnan(P).all())
+    assert attnw.query_status() == SELFTEST_SITE  # the launch has not given up on a wait of its own
+    attnw.softmax_rows(S, P=P)
+    torch.cuda.synchronize()
+    assert attnw.query_status() == 0
+    assert float((P - torch.softmax(S, 1)).abs().max()) <= 2e-6  # the largest weights are below 0.1: some 20 roundings
