@@ -273,6 +273,7 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         if (__any_sync(0xffffffffu, prior_failure != 0u)) {
             *abort_flag = 1;
             ok = false;
+            if constexpr (M == kCluster) tell_peers(&bars->abort_flag, G);
         }
         int n = 0;            // next ring entry, in step with the producer
         auto arrived = [&]() {
