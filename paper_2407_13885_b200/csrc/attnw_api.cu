@@ -635,7 +635,11 @@ int launch_attn_onepass(DeviceInfo* dev, const void* Q, const void* K, const voi
     // 19.8, 3 x 824 11.9 -> 10.8, 1 x 1000 13.3 -> 13.2.
     // Or full rounds of CTAs first, and the query tiles that are left spread over the device by a second launch.  One launch -> two:
     // 2 x 10215 (d = 64, 160 query tiles) 129 -> 104, 3 x 13719 (d = 128) 312 -> 258, 22 x 1940 (d = 64) 51 -> 45, 5 x 4607 (d = 64) 65 -> 56, 19 x
-    // 10023 (d = 128) 1058 -> 954, 114 x 692 (d = 128) 48.7 -> 46.5; 9 x 2487 (d = 128) 37.9 -> 39.1, not taken.
+    // 10023 (d = 128) 1058 -> 954, 114 x 692 (d = 128) 48.7 -> 46.5; 9 x 2487 (d = 128) 37.9 -> 39.1, not taken.  The second launch counts as 0.75
+    // key tiles, and has to give 4 percent, or 8 where the number of query tiles is odd: a head's last CTA has one query tile then, and the rounds of one
+    // launch overlap better than they are counted (not taken: 150 x 384, d = 64 22.2 / 23.8, 150 x 640 40.1 / 43.4, 9 x 3000 45.9 / 49.9, 300 x 500, d = 128
+    // 63.1 / 65.3).  Of 836 sizes near full rounds, each measured both ways, none is more than 0.5 percent behind the better one launch; with 0.5 and 3
+    // percent for all 29 were by more than 1.5, up to 8.
     const long long tiles = (N + kTile - 1) / kTile, pairs = (tiles + 1) / 2, all = BH * tiles;
     const int sms = dev->sm_count;
     struct Part {
@@ -672,8 +676,8 @@ int launch_attn_onepass(DeviceInfo* dev, const void* Q, const void* K, const voi
             if (full == 0 || full == units) continue;
             const double front = static_cast<double>(full / sms) * (mode == av1::kWhole ? whole_round : split_round);
             const Part rest = best_part(mode == av1::kWhole ? full / pairs * tiles + 2 * (full % pairs) : full);
-            const double cost = front + rest.cost + 0.5;
-            if (cost * 1.03 < best) {
+            const double cost = front + rest.cost + 0.75;
+            if (cost * (tiles % 2 == 0 ? 1.04 : 1.08) < best) {
                 parts[0] = {mode, 1, 0, full, front};
                 parts[1] = rest;
                 n_parts = 2;
