@@ -67,9 +67,11 @@ __device__ __forceinline__ float block_reduce(float v, float* red) {
 
 // grid: n_clusters * C CTAs in clusters of C; cluster i takes rows i, i + n_clusters, ...; slice_cols columns per CTA
 // (a multiple of 4; the last CTA's slice may be shorter or empty).
-template <typename OutT, int NT>
+// kClusters = false: C is 1, known to the compiler.
+template <typename OutT, int NT, bool kClusters>
 __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 2)
-softmax_rows_smem_kernel(const float* S, OutT* P, long long rows, long long cols, int slice_cols, int C) {
+softmax_rows_smem_kernel(const float* S, OutT* P, long long rows, long long cols, int slice_cols, int cluster_ctas) {
+    const int C = kClusters ? cluster_ctas : 1;
     extern __shared__ __align__(16) uint8_t srs_smem[];
     Control* ctl = reinterpret_cast<Control*>(srs_smem);
     float* x = reinterpret_cast<float*>(srs_smem + kControlBytes);
@@ -191,11 +193,11 @@ inline int cluster_ctas_for(long long cols) {
     return c;
 }
 
-template <typename OutT, int NT>
+template <typename OutT, int NT, bool kClusters>
 inline cudaError_t launch_nt(const float* S, OutT* P, long long rows, long long cols, int sm_count, int C, int slice_cols,
                              cudaStream_t stream) {
     const size_t smem = kControlBytes + static_cast<size_t>(slice_cols) * 4;
-    const cudaError_t e = allow_smem<softmax_rows_smem_kernel<OutT, NT>>(kControlBytes + kSliceMaxCols * 4, true);
+    const cudaError_t e = allow_smem<softmax_rows_smem_kernel<OutT, NT, kClusters>>(kControlBytes + kSliceMaxCols * 4, true);
     if (e != cudaSuccess) return e;
     // Four CTAs of 256 threads on an SM where they fit, but three for many float32 rows: there fewer rows in flight keep the stream of HBM
     // smoother.  us, four / three: 14000 x 12000 237 / 214, 16000 x 10240 229 / 214, 9000 x 24580 300 / 286, 6000 x 26000 222 / 203, 2000 x 25000 72.8 /
@@ -205,7 +207,7 @@ inline cudaError_t launch_nt(const float* S, OutT* P, long long rows, long long 
     long long n_clusters = (per_sm * sm_count) / C;  // CTAs that fit at once
     if (n_clusters < 1) n_clusters = 1;
     if (n_clusters > rows) n_clusters = rows;
-    return launch_overlapped(softmax_rows_smem_kernel<OutT, NT>, static_cast<unsigned>(n_clusters * C), NT, smem, stream, C, S, P,
+    return launch_overlapped(softmax_rows_smem_kernel<OutT, NT, kClusters>, static_cast<unsigned>(n_clusters * C), NT, smem, stream, C, S, P,
                              rows, cols, slice_cols, C);
 }
 
@@ -214,8 +216,15 @@ inline cudaError_t launch(const float* S, OutT* P, long long rows, long long col
     const int C = cluster_ctas_for(cols);
     if (C == 0) return cudaErrorInvalidValue;
     const int slice_cols = static_cast<int>(((cols / 4 + C - 1) / C) * 4);
-    if (slice_cols <= 16384) return launch_nt<OutT, 256>(S, P, rows, cols, sm_count, C, slice_cols, stream);
-    return launch_nt<OutT, 512>(S, P, rows, cols, sm_count, C, slice_cols, stream);
+    // One CTA a row: the kernel without the cluster's part for up to two rows an SM (one where a CTA has 512 threads), whose CTAs have a row each: 1 x
+    // 12000 float32 4.24 -> 4.00 us, 20 x 24576 6.20 -> 5.83, 148 x 16384 bfloat16 4.50 -> 4.41.  Many rows are slower with it, 900 x 14000 15.0 -> 16.3,
+    // 1250 x 10240 14.6 -> 16.0, 4000 x 12000 48.0 -> 49.5.
+    const bool few = C == 1 && rows <= (slice_cols <= 16384 ? 2 : 1) * sm_count;
+    if (slice_cols <= 16384)
+        return few ? launch_nt<OutT, 256, false>(S, P, rows, cols, sm_count, C, slice_cols, stream)
+                   : launch_nt<OutT, 256, true>(S, P, rows, cols, sm_count, C, slice_cols, stream);
+    return few ? launch_nt<OutT, 512, false>(S, P, rows, cols, sm_count, C, slice_cols, stream)
+               : launch_nt<OutT, 512, true>(S, P, rows, cols, sm_count, C, slice_cols, stream);
 }
 
 

@@ -194,3 +194,16 @@ def test_many_rows_in_shared_memory(attnw, rows, cols, dtype):
     assert_guards_intact(raw, g)
     assert_close_to_oracle(P, oracle.softmax_rows(S), f"rows={rows} cols={cols}")
     assert attnw.query_status() == 0
+
+
+# One CTA a row: on a device of 148 SMs the last count of rows that takes the kernel of its own for few rows, and the first that does not
+@pytest.mark.parametrize("rows,cols", [(296, 8196), (297, 16384), (148, 16388), (149, 24576)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_few_rows_in_shared_memory(attnw, rows, cols, dtype):
+    S = inputs.normal_f32(11, rows * 157 + cols, rows * cols, 3.0).reshape(rows, cols)
+    raw, P, g = guarded_empty((rows, cols), dtype)
+    attnw.softmax_rows(torch.from_numpy(S).cuda(), P=P)
+    torch.cuda.synchronize()
+    assert_guards_intact(raw, g)
+    assert_close_to_oracle(P, oracle.softmax_rows(S), f"rows={rows} cols={cols}")
+    assert attnw.query_status() == 0
