@@ -8,7 +8,7 @@
 // features.  A CTA loads its rows and half of the features, so a byte of the operands in shared memory feeds twice the MMAs that it
 // feeds within one CTA.  A pair stays for several tiles: tensor memory holds two accumulators, and 8 warps turn one into bf16 and store it
 // while the tensor cores fill the other; the ring of 64-wide slices runs on from tile to tile.  launch_project chooses between whole
-// tiles, a last round cut in two, and narrow tiles.
+// tiles, a last round cut in two, and narrow tiles, by pairs or (small calls that pairs only hold up) by single CTAs.
 // Weights are stored [H, d, d_model] (feature c of head h contiguous along d_model), which is the K-major B operand TMA can deliver as it is.
 //
 // What bounds it: large calls, the tensor pipe (512 cycles a slice) under the power cap; small ones, the latency of set-up, first load,
@@ -70,9 +70,9 @@ struct Grid {
     int block;           // features that a CTA loads for a tile: kFeatures or half of that
     int feature_blocks;  // blocks of Q's features, and as many of K's behind them = column tiles (two blocks each)
     int row_blocks;      // blocks of kRows rows of a batch entry
-    int row_tiles;       // of two row blocks each, which may belong to different batch entries
-    __host__ __device__ Grid(int B, int N, int HD, int block_)
-        : block(block_), feature_blocks((HD - 1) / block_ + 1), row_blocks((N - 1) / kRows + 1), row_tiles((B * row_blocks + 1) / 2) {}
+    int row_tiles;       // of a row block for each CTA; they may belong to different batch entries
+    __host__ __device__ Grid(int B, int N, int HD, int block_, int ctas)
+        : block(block_), feature_blocks((HD - 1) / block_ + 1), row_blocks((N - 1) / kRows + 1), row_tiles((B * row_blocks + ctas - 1) / ctas) {}
     __host__ __device__ int tiles() const { return feature_blocks * row_tiles; }
 };
 
@@ -81,6 +81,8 @@ struct Grid {
 __host__ __device__ constexpr bool accumulator_comes_again(int t, int pairs, int items) { return items - t > kSlots * pairs; }
 
 // grid: clusters of two CTAs; pair p takes the items p, p + pairs, ...: the tiles 0 ... whole_tiles - 1, then the halves of the others.
+// kPair = false: single CTAs, each in the place of a pair, with narrow tiles of kRows rows and both blocks of features.
+template <bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
 project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_wq,
                   const __grid_constant__ CUtensorMap tm_wk, const __grid_constant__ CUtensorMap tm_q,
@@ -92,17 +94,18 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const int rank = static_cast<int>(ptx::cluster_ctarank());
-    const Grid g(B, N, H * d, block);
+    constexpr int kCtas = kPair ? 2 : 1;
+    const int rank = kPair ? static_cast<int>(ptx::cluster_ctarank()) : 0;
+    const Grid g(B, N, H * d, block, kCtas);
     const int items = 2 * g.tiles() - whole_tiles;
-    const int first = static_cast<int>(blockIdx.x) >> 1, pairs = static_cast<int>(gridDim.x) >> 1;
+    const int first = static_cast<int>(blockIdx.x) / kCtas, pairs = static_cast<int>(gridDim.x) / kCtas;
     const int KT = (d_model + kKSlice - 1) / kKSlice;
-    // The ring: six stages of one slice, or four of two narrow ones: a stage costs each of the issuing warps some 300 cycles, which the
+    // The ring: six stages of one slice, or four (single CTAs: three) of two narrow ones: a stage costs each of the issuing warps some 300 cycles, which the
     // 256 of the MMAs of one narrow slice do not cover (1 x 512 x 4096 to 8 x 128 14.6 -> 13.3 us).
-    const int slice_bytes = kAtomBytes + block * 128;
+    const int slice_bytes = kAtomBytes + (kPair ? block : kFeatures) * 128;
     const int slices = block == kFeatures ? 1 : 2;
     const int stage_bytes = slices * slice_bytes;
-    const int stages = block == kFeatures ? kMaxStages : 4;
+    const int stages = !kPair ? 3 : block == kFeatures ? kMaxStages : 4;
     // The ring's stages in turn, and how often a stage has been used before, modulo 2.
     struct Turn {
         int s = 0;
@@ -132,7 +135,7 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         const int width = group == groups - 1 ? g.feature_blocks - group * kGroupTiles : kGroupTiles;
         r.row_tile = in_group / width;
         r.block = 2 * (group * kGroupTiles + in_group - r.row_tile * width);
-        const int rb = 2 * r.row_tile + rank;
+        const int rb = kCtas * r.row_tile + rank;
         r.b = rb / g.row_blocks;
         r.row = (rb - r.b * g.row_blocks) * kRows;
         return r;
@@ -150,7 +153,7 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         }
         for (int s = 0; s < kSlots; ++s) {
             ptx::mbar_init(&bars->acc_full[s], 1);
-            ptx::mbar_init(&bars->acc_empty[s], 2 * kEpiWarps);
+            ptx::mbar_init(&bars->acc_empty[s], kCtas * kEpiWarps);
         }
         bars->abort_flag = prior_failure;
         bars->peer_ran = 0;
@@ -166,14 +169,21 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         ptx::prefetch_tensormap(&tm_k);
     }
     if (warp == kMma) {
-        ptx::pair_tmem_alloc(&bars->tmem_base, kTmemCols);
-        ptx::pair_tmem_relinquish();
+        if constexpr (kPair) {
+            ptx::pair_tmem_alloc(&bars->tmem_base, kTmemCols);
+            ptx::pair_tmem_relinquish();
+        } else {
+            ptx::tmem_alloc(&bars->tmem_base, kTmemCols);
+            ptx::tmem_relinquish();
+        }
     }
     ptx::grid_dependency_wait();
     ptx::tc_fence_before_sync();
     __syncthreads();
-    ptx::cluster_arrive_relaxed();
-    ptx::cluster_wait_acquire();
+    if constexpr (kPair) {
+        ptx::cluster_arrive_relaxed();
+        ptx::cluster_wait_acquire();
+    }
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bars->tmem_base;
     // An earlier launch gave up: do not queue more waits behind it.  Should the word be cleared between the two CTAs' looks at it, the one that
@@ -185,7 +195,7 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         const bool for_rows = warp == kProducerX;
         const uint64_t keep = ptx::policy_evict_last();
         const uint32_t empty0 = ptx::smem_u32(&bars->empty[0]);
-        const uint32_t full0 = ptx::map_to_cta(ptx::smem_u32(&bars->full[0]), 0);
+        const uint32_t full0 = kPair ? ptx::map_to_cta(ptx::smem_u32(&bars->full[0]), 0) : ptx::smem_u32(&bars->full[0]);
         bool ok = true;
         Turn turn;
         int n = 0;  // stages asked for
@@ -193,13 +203,17 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         for (int t = first; ok && t < items;) {
             const int block = it.block + rank;
             const bool keys = block >= g.feature_blocks;
-            const bool wide = it.half < 0 && g.block == kFeatures;
+            const bool wide = kPair && it.half < 0 && g.block == kFeatures;
             const CUtensorMap* map = for_rows ? &tm_x : keys ? &tm_wk : &tm_wq;
+            // a single CTA loads the column tile's second block too
+            const bool keys2 = it.block + 1 >= g.feature_blocks;
+            const int c1_2 = (keys2 ? it.block + 1 - g.feature_blocks : it.block + 1) * g.block;
             const int c1 = for_rows ? it.row : (keys ? block - g.feature_blocks : block) * g.block + (it.half == 1 ? kFeatures / 2 : 0);
             const int c2 = for_rows ? it.b : 0;
             // An odd number of row blocks leaves a CTA without rows: what its MMAs make of old contents is never stored.
             const bool load = !for_rows || it.b < B;
-            const uint32_t bytes = static_cast<uint32_t>((2 * it.row_tile + 1 < B * g.row_blocks ? 2 : 1) + (wide ? 2 : 1)) * kAtomBytes;  // of both CTAs
+            const uint32_t bytes = !kPair ? 2 * kAtomBytes
+                                          : static_cast<uint32_t>((2 * it.row_tile + 1 < B * g.row_blocks ? 2 : 1) + (wide ? 2 : 1)) * kAtomBytes;  // of both CTAs
             for (int kt = 0; kt < KT; kt += slices, ++n, turn.next(stages)) {
                 ok = warp_wait(empty0 + 8u * static_cast<uint32_t>(turn.s), turn.parity ^ 1u, abort_flag, kSiteProducerEmpty);
                 if (!ok) break;
@@ -209,9 +223,17 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 if (ptx::elect_one()) {
                     if (rank == 0 && for_rows) ptx::mbar_expect_tx(&bars->full[turn.s], second ? 2 * bytes : bytes);
                     // rows or features beyond the tensor's extent, and d_model's ragged tail, arrive as zeros
-                    if (load) ptx::pair_tma_load_3d(st, map, full, kt * kKSlice, c1, c2, keep);
-                    if (load && second) ptx::pair_tma_load_3d(st + slice_bytes, map, full, (kt + 1) * kKSlice, c1, c2, keep);
-                    if (wide && !for_rows) ptx::pair_tma_load_3d(st + kAtomBytes / 2, map, full, kt * kKSlice, c1 + kFeatures / 2, c2, keep);
+                    if constexpr (kPair) {
+                        if (load) ptx::pair_tma_load_3d(st, map, full, kt * kKSlice, c1, c2, keep);
+                        if (load && second) ptx::pair_tma_load_3d(st + slice_bytes, map, full, (kt + 1) * kKSlice, c1, c2, keep);
+                        if (wide && !for_rows) ptx::pair_tma_load_3d(st + kAtomBytes / 2, map, full, kt * kKSlice, c1 + kFeatures / 2, c2, keep);
+                    } else {
+                        for (int i = 0; i < (second ? 2 : 1); ++i) {
+                            ptx::tma_load_3d(st + i * slice_bytes, map, &bars->full[turn.s], (kt + i) * kKSlice, c1, c2, keep);
+                            if (!for_rows)
+                                ptx::tma_load_3d(st + i * slice_bytes + kAtomBytes / 2, keys2 ? &tm_wk : &tm_wq, &bars->full[turn.s], (kt + i) * kKSlice, c1_2, 0, keep);
+                        }
+                    }
                 }
                 __syncwarp();
             }
@@ -224,8 +246,20 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             ok = warp_wait(empty0 + 8u * static_cast<uint32_t>(i % stages), static_cast<uint32_t>(i / stages) & 1u, abort_flag, kSiteProducerEmpty);
     } else if (run && warp == kMma && rank == 0) {
         // ================= MMA issuer, for both CTAs =================
-        constexpr uint32_t idesc_whole = ptx::umma_idesc_bf16_f32(2 * kRows, 2 * kFeatures);
-        constexpr uint32_t idesc_half = ptx::umma_idesc_bf16_f32(2 * kRows, kFeatures);
+        constexpr uint32_t idesc_whole = ptx::umma_idesc_bf16_f32(kCtas * kRows, 2 * kFeatures);
+        constexpr uint32_t idesc_half = ptx::umma_idesc_bf16_f32(kCtas * kRows, kFeatures);
+        auto mma = [](uint32_t to, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+            if constexpr (kPair)
+                ptx::pair_umma_f16_ss(to, a, b, idesc, accumulate);
+            else
+                ptx::umma_f16_ss(to, a, b, idesc, accumulate);
+        };
+        auto commit = [](uint64_t* bar) {
+            if constexpr (kPair)
+                ptx::pair_umma_commit(bar);
+            else
+                ptx::umma_commit(bar);
+        };
         const uint64_t base = ptx::umma_desc_kmajor_sw128(ptx::smem_u32(smem));
         bool ok = true;
         const uint32_t full0 = ptx::smem_u32(&bars->full[0]);
@@ -244,17 +278,16 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 if (ptx::elect_one()) {
 #pragma unroll
                     for (int k = 0; k < kKSlice / 16; ++k)
-                        ptx::pair_umma_f16_ss(d_tmem, st + static_cast<uint64_t>((k * 32) >> 4), st + static_cast<uint64_t>((kAtomBytes + k * 32) >> 4), idesc,
-                                              (kt > 0 || k > 0) ? 1u : 0u);
+                        mma(d_tmem, st + static_cast<uint64_t>((k * 32) >> 4), st + static_cast<uint64_t>((kAtomBytes + k * 32) >> 4), idesc,
+                            (kt > 0 || k > 0) ? 1u : 0u);
                     if (slices == 2 && kt + 1 < KT) {
                         const uint64_t second = st + static_cast<uint64_t>(slice_bytes >> 4);
 #pragma unroll
                         for (int k = 0; k < kKSlice / 16; ++k)
-                            ptx::pair_umma_f16_ss(d_tmem, second + static_cast<uint64_t>((k * 32) >> 4), second + static_cast<uint64_t>((kAtomBytes + k * 32) >> 4),
-                                                  idesc, 1u);
+                            mma(d_tmem, second + static_cast<uint64_t>((k * 32) >> 4), second + static_cast<uint64_t>((kAtomBytes + k * 32) >> 4), idesc, 1u);
                     }
-                    ptx::pair_umma_commit(&bars->empty[turn.s]);
-                    if (kt + slices >= KT) ptx::pair_umma_commit(&bars->acc_full[slot]);
+                    commit(&bars->empty[turn.s]);
+                    if (kt + slices >= KT) commit(&bars->acc_full[slot]);
                 }
                 __syncwarp();
                 st += static_cast<uint64_t>(stage_bytes >> 4);
@@ -296,7 +329,12 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 if (c + 64 == width && accumulator_comes_again(t, pairs, items)) {  // it may be overwritten
                     ptx::tc_fence_before_sync();
                     __syncwarp();
-                    if (lane == 0) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&bars->acc_empty[slot]), 0));
+                    if (lane == 0) {
+                        if constexpr (kPair)
+                            ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&bars->acc_empty[slot]), 0));
+                        else
+                            ptx::mbar_arrive(&bars->acc_empty[slot]);
+                    }
                 }
                 // The box: once the store that used it last has read it (lane 0 has issued them all).  The last tile's second one has room
                 // of its own, in the ring, which nothing uses any more.
@@ -332,14 +370,16 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     // ---- teardown: every role of both CTAs falls through to here, also after a wait gave up ----
     ptx::tc_fence_before_sync();
     __syncthreads();
-    if (threadIdx.x == 0 && *abort_flag) {
-        ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&bars->abort_flag), rank ^ 1), 1u);
-        if (run) ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&bars->peer_ran), rank ^ 1), 1u);
-        ptx::fence_cluster();
+    if constexpr (kPair) {
+        if (threadIdx.x == 0 && *abort_flag) {
+            ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&bars->abort_flag), rank ^ 1), 1u);
+            if (run) ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&bars->peer_ran), rank ^ 1), 1u);
+            ptx::fence_cluster();
+        }
+        __syncwarp();
+        ptx::cluster_arrive_relaxed();
+        ptx::cluster_wait_acquire();
     }
-    __syncwarp();
-    ptx::cluster_arrive_relaxed();
-    ptx::cluster_wait_acquire();
     ptx::tc_fence_after_sync();
     if (*abort_flag) {
         // Unwinding: let the MMAs of the pair and the arrivals on either CTA that nobody has waited for come to their end, and the copies of both
@@ -347,20 +387,29 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         if (run || bars->peer_ran) wait_for_late_stores();
         if (rank == 0 && threadIdx.x == 0) {
             const int mine = bars->loads;
-            const int theirs = static_cast<int>(ptx::ld_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&bars->loads), 1)));
+            const int theirs = kPair ? static_cast<int>(ptx::ld_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&bars->loads), 1))) : 0;
             const int last = mine > theirs ? mine : theirs;
             const long long t0 = clock64();
-            // (the phase of a stage that only the odd CTA has asked for does not end: there the limit runs out)
+            // (the phase of a stage that only one of the producers has asked for does not end: there the limit runs out)
             for (int i = last > stages ? last - stages : 0; i < last; ++i)
                 while (!ptx::mbar_try_wait(&bars->full[i % stages], static_cast<uint32_t>(i / stages) & 1u) &&
                        clock64() - t0 < kWaitLimitCycles / 8) {
                 }
         }
         __syncwarp();
-        ptx::cluster_arrive_relaxed();
-        ptx::cluster_wait_acquire();
+        if constexpr (kPair) {
+            ptx::cluster_arrive_relaxed();
+            ptx::cluster_wait_acquire();
+        } else {
+            __syncthreads();
+        }
     }
-    if (warp == kMma) ptx::pair_tmem_dealloc(tmem_base, kTmemCols);
+    if (warp == kMma) {
+        if constexpr (kPair)
+            ptx::pair_tmem_dealloc(tmem_base, kTmemCols);
+        else
+            ptx::tmem_dealloc(tmem_base, kTmemCols);
+    }
 }
 
 }  // namespace proj

@@ -83,6 +83,16 @@ def test_projection_over_rounds_of_tiles(attnw, B, N, d_model, H, d):
     check(K, oracle.project(x, wk), x, wk)
 
 
+# On a device of 148 SMs.  Single CTAs: one slice, four with a ragged last one, and a column tile that is half Q's and half K's; several rounds of the ring with an odd number of
+# slices, where pairs would leave SMs idle; the most tiles that they take, and one more.  Pairs: the first number of slices beyond, and an X that is too small
+@pytest.mark.parametrize("B,N,d_model,H,d", [(1, 5, 8, 1, 64), (2, 130, 200, 5, 64), (1, 300, 680, 39, 64), (1, 128, 256, 74, 128), (1, 128, 256, 149, 64), (2, 130, 264, 5, 64), (1, 20, 712, 80, 64)])
+def test_projection_by_single_ctas_and_pairs(attnw, B, N, d_model, H, d):
+    x, wq, wk = rand_xw(B, N, d_model, H, d, stream=11 * N + d_model + H)
+    Q, K = run_project(attnw, x, wq, wk)
+    check(Q, oracle.project(x, wq), x, wq)
+    check(K, oracle.project(x, wk), x, wk)
+
+
 def test_projection_with_selector_weights_is_exact(attnw):
     # W[h, c, :] = e_{h*d + c}: head h of Q is columns h*d .. of X, bit for bit; K takes them in reverse order
     B, N, H, d = 2, 200, 3, 64
