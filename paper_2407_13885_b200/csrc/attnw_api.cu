@@ -773,21 +773,25 @@ int launch_project(const DeviceInfo* dev, const void* X, const void* Wq, const v
     // and end cost it 0.2 to 0.4 us - or as many rows by pairs would not be one round (an odd number of row blocks, most often one or three: whole tiles
     // leave half of the SMs idle then).  us per call, pairs -> single CTAs: 2 x 64 x 256 to 4 x 64 4.70 -> 4.52, 1 x 128 x 64 to 8 x 64 4.27 -> 3.96, 1 x
     // 384 x 64 to 40 x 64 5.03 -> 4.02, 1 x 300 x 1024 to 40 x 64 9.68 -> 7.39, 1 x 128 x 2048 to 96 x 64 15.2 -> 12.2, 1 x 600 x 4096 to 28 x 64 23.4 -> 18.3; but 1 x
-    // 1000 x 512 to 16 x 64 5.53 -> 5.61, 1 x 1000 x 4096 to 16 x 64 14.8 -> 17.3 (a pair fetches 24 KB a slice, not 32), and an X below 128 KB, which all CTAs read from
-    // few places of L2, wants fewer readers: 1 x 8 x 4096 to 80 x 64 24.1 -> 32.4, 1 x 16 x 4096 23.5 -> 20.7.
-    constexpr int kNarrow = proj::kFeatures / 2;
-    const int singles = proj::Grid(B, N, static_cast<int>(hd), kNarrow, 1).tiles(), pairs = dev->sm_count / 2;
-    const bool narrow = proj::Grid(B, N, static_cast<int>(hd), kNarrow, 2).tiles() <= pairs;
-    if (singles <= dev->sm_count && (d_model <= 256 || (!narrow && static_cast<long long>(B) * N * d_model >= 65536)))
-        return launch(std::false_type{}, singles, kNarrow, singles);
+    // 1000 x 512 to 16 x 64 5.53 -> 5.61, 1 x 1000 x 4096 to 16 x 64 14.8 -> 17.3 (a pair fetches 24 KB a slice, not 32), and a few rows of X, which all CTAs read from
+    // the same places of L2, want fewer readers: 1 x 8 x 4096 to 80 x 64 24.1 -> 32.4, 1 x 16 x 4096 23.5 -> 20.7.
+    // The same with tiles of 128 x 256, where pairs need a second round for what single CTAs do in one: 1 x 300 x 768 to 40 x 128 10.4 -> 8.4,
+    // 1 x 1400 x 2048 to 13 x 128 22.6 -> 15.7, 1 x 128 x 768 to 80 x 128 12.3 -> 8.4, 1 x 64 x 4096 to 148 x 128 58.2 -> 53.4.
+    constexpr int kNarrow = proj::kFeatures / 2, kWide = proj::kFeatures;
+    auto tiles_of = [&](int block, int ctas) { return proj::Grid(B, N, static_cast<int>(hd), block, ctas).tiles(); };
+    const int sms = dev->sm_count, pairs = sms / 2;
+    const bool narrow = tiles_of(kNarrow, 2) <= pairs, shared_x = d_model > 512 && static_cast<long long>(B) * N < 64 && static_cast<long long>(B) * N * d_model < 65536;
+    if (tiles_of(kNarrow, 1) <= sms && (d_model <= 256 || (!narrow && !shared_x)))
+        return launch(std::false_type{}, tiles_of(kNarrow, 1), kNarrow, tiles_of(kNarrow, 1));
+    if (tiles_of(kWide, 1) <= sms && tiles_of(kWide, 2) > pairs && !shared_x) return launch(std::false_type{}, tiles_of(kWide, 1), kWide, tiles_of(kWide, 1));
     // Tiles of 256 x 256 per pair of CTAs; narrow ones of 256 x 128 where a single round of them holds the call, since a narrow slice still takes
     // 0.6 to 0.75 of the time of a whole one (X's rows are fetched for half of the MMAs).  A last round whose tiles would occupy at most
     // half of the pairs takes them cut in two.  us per call, whole tiles only -> as chosen: narrow 4 x 100 x 1536 to 12 x 128 11.3 -> 7.7,
     // 1 x 1000 x 1024 to 16 x 64 9.3 -> 6.7, 2 x 949 x 576 to 9 x 64 7.2 -> 5.7, 1 x 256 x 4096 to 64 x 64 24.9 -> 21.2; tiles cut in two 1 x 2048 x
     // 4096 to 32 x 128 (256 tiles for 74 pairs) 111.8 -> 107.6, 2 x 444 x 3200 to 25 x 128 (100) 40.7 -> 37.4, 4 x 3749 x 4080 to 10 x 64 (300) 142.5 -> 140.8.
-    const int block = narrow ? kNarrow : proj::kFeatures;
-    const int tiles = proj::Grid(B, N, static_cast<int>(hd), block, 2).tiles(), last = tiles % pairs;
-    const int whole = block == proj::kFeatures && 2 * last <= pairs ? tiles - last : tiles;
+    const int block = narrow ? kNarrow : kWide;
+    const int tiles = tiles_of(block, 2), last = tiles % pairs;
+    const int whole = block == kWide && 2 * last <= pairs ? tiles - last : tiles;
     const int items = 2 * tiles - whole;
     return launch(std::true_type{}, items < pairs ? items : pairs, block, whole);
 }

@@ -81,7 +81,7 @@ struct Grid {
 __host__ __device__ constexpr bool accumulator_comes_again(int t, int pairs, int items) { return items - t > kSlots * pairs; }
 
 // grid: clusters of two CTAs; pair p takes the items p, p + pairs, ...: the tiles 0 ... whole_tiles - 1, then the halves of the others.
-// kPair = false: single CTAs, each in the place of a pair, with narrow tiles of kRows rows and both blocks of features.
+// kPair = false: single CTAs, each in the place of a pair, with tiles of kRows rows and both blocks of features.
 template <bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
 project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_wq,
@@ -100,12 +100,12 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     const int items = 2 * g.tiles() - whole_tiles;
     const int first = static_cast<int>(blockIdx.x) / kCtas, pairs = static_cast<int>(gridDim.x) / kCtas;
     const int KT = (d_model + kKSlice - 1) / kKSlice;
-    // The ring: six stages of one slice, or four (single CTAs: three) of two narrow ones: a stage costs each of the issuing warps some 300 cycles, which the
+    // The ring: six stages of one slice, or four of two narrow ones (single CTAs, with all features: four and three): a stage costs each of the issuing warps some 300 cycles, which the
     // 256 of the MMAs of one narrow slice do not cover (1 x 512 x 4096 to 8 x 128 14.6 -> 13.3 us).
-    const int slice_bytes = kAtomBytes + (kPair ? block : kFeatures) * 128;
+    const int slice_bytes = kAtomBytes + (kPair ? block : 2 * block) * 128;
     const int slices = block == kFeatures ? 1 : 2;
     const int stage_bytes = slices * slice_bytes;
-    const int stages = !kPair ? 3 : block == kFeatures ? kMaxStages : 4;
+    const int stages = kPair ? (block == kFeatures ? kMaxStages : 4) : (block == kFeatures ? 4 : 3);  // kRingBytes of them
     // The ring's stages in turn, and how often a stage has been used before, modulo 2.
     struct Turn {
         int s = 0;
@@ -212,7 +212,7 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             const int c2 = for_rows ? it.b : 0;
             // An odd number of row blocks leaves a CTA without rows: what its MMAs make of old contents is never stored.
             const bool load = !for_rows || it.b < B;
-            const uint32_t bytes = !kPair ? 2 * kAtomBytes
+            const uint32_t bytes = !kPair ? static_cast<uint32_t>(slice_bytes)
                                           : static_cast<uint32_t>((2 * it.row_tile + 1 < B * g.row_blocks ? 2 : 1) + (wide ? 2 : 1)) * kAtomBytes;  // of both CTAs
             for (int kt = 0; kt < KT; kt += slices, ++n, turn.next(stages)) {
                 ok = warp_wait(empty0 + 8u * static_cast<uint32_t>(turn.s), turn.parity ^ 1u, abort_flag, kSiteProducerEmpty);
@@ -229,9 +229,16 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                         if (wide && !for_rows) ptx::pair_tma_load_3d(st + kAtomBytes / 2, map, full, kt * kKSlice, c1 + kFeatures / 2, c2, keep);
                     } else {
                         for (int i = 0; i < (second ? 2 : 1); ++i) {
-                            ptx::tma_load_3d(st + i * slice_bytes, map, &bars->full[turn.s], (kt + i) * kKSlice, c1, c2, keep);
-                            if (!for_rows)
-                                ptx::tma_load_3d(st + i * slice_bytes + kAtomBytes / 2, keys2 ? &tm_wk : &tm_wq, &bars->full[turn.s], (kt + i) * kKSlice, c1_2, 0, keep);
+                            uint8_t* to = st + i * slice_bytes;
+                            const int c0 = (kt + i) * kKSlice;
+                            if (for_rows) {
+                                ptx::tma_load_3d(to, map, &bars->full[turn.s], c0, c1, c2, keep);
+                            } else {
+                                for (int f = 0; f < g.block; f += kFeatures / 2) {
+                                    ptx::tma_load_3d(to + f * 128, map, &bars->full[turn.s], c0, c1 + f, 0, keep);
+                                    ptx::tma_load_3d(to + (g.block + f) * 128, keys2 ? &tm_wk : &tm_wq, &bars->full[turn.s], c0, c1_2 + f, 0, keep);
+                                }
+                            }
                         }
                     }
                 }

@@ -84,8 +84,9 @@ def test_projection_over_rounds_of_tiles(attnw, B, N, d_model, H, d):
 
 
 # On a device of 148 SMs.  Single CTAs: one slice, four with a ragged last one, and a column tile that is half Q's and half K's; several rounds of the ring with an odd number of
-# slices, where pairs would leave SMs idle; the most tiles that they take, and one more.  Pairs: the first number of slices beyond, and an X that is too small
-@pytest.mark.parametrize("B,N,d_model,H,d", [(1, 5, 8, 1, 64), (2, 130, 200, 5, 64), (1, 300, 680, 39, 64), (1, 128, 256, 74, 128), (1, 128, 256, 149, 64), (2, 130, 264, 5, 64), (1, 20, 712, 80, 64)])
+# slices, where pairs would leave SMs idle; the most tiles that they take, and one more; tiles of 128 x 256
+# with a ragged column tile.  Pairs: the first number of slices beyond, and an X that is too small
+@pytest.mark.parametrize("B,N,d_model,H,d", [(1, 5, 8, 1, 64), (2, 130, 200, 5, 64), (1, 300, 680, 39, 64), (1, 128, 256, 74, 128), (1, 128, 256, 149, 64), (1, 300, 328, 77, 64), (3, 90, 264, 48, 128), (2, 130, 264, 5, 64), (1, 20, 712, 80, 64)])
 def test_projection_by_single_ctas_and_pairs(attnw, B, N, d_model, H, d):
     x, wq, wk = rand_xw(B, N, d_model, H, d, stream=11 * N + d_model + H)
     Q, K = run_project(attnw, x, wq, wk)
