@@ -324,8 +324,9 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             __syncwarp();
         };
         // The scores of step j + 1 first: the tensor pipe computes them while the row threads exponentiate step j.  The two
-        // units alternate (with two issuers, because the scores take turns at their buffer) - scores of one, product of one, scores of the other, product of the other - which keeps their
-        // row threads half a step apart (d = 64, 128 x 4096: 888 -> 841 us against both scores first).
+        // units alternate (with two issuers, because the scores take turns at their buffer) - scores of one, product of one, scores of
+        // the other, product of the other - which keeps their row threads half a step apart (d = 64, 128 x 4096: 888 -> 841 us against
+        // both scores first).
         if constexpr (two_issuers) {
             const bool for_scores = warp == kMma;
             for (int j = -1; ok && j < steps[0]; ++j) {
@@ -353,42 +354,28 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 }
             }
         } else {
+            static_assert(two_issuers || !split, "one issuer: two query tiles");
             for (int j = -1; ok && j < steps[0]; ++j) {
-                if (split) {
-                    for (int q = 0; q < 2; ++q) {
-                        if (ok && j + 1 < steps[q]) {
-                            arrived();
-                            scores(q, j + 1);
-                            release();
-                        }
-                        if (ok && j >= 0 && j < steps[q]) {
-                            arrived();
-                            product(q, j);
-                            release();
-                        }
-                    }
-                } else {
-                    const bool next = j + 1 < T;
-                    const int k_entry = n, v_entry = next ? n + 1 : n;  // K of step j + 1, V of step j
-                    if (next) {
-                        arrived();
-                        scores(0, j + 1);
-                    }
+                const bool next = j + 1 < T;
+                const int k_entry = n, v_entry = next ? n + 1 : n;  // K of step j + 1, V of step j
+                if (next) {
+                    arrived();
+                    scores(0, j + 1);
+                }
+                n = v_entry;
+                if (ok && j >= 0) {
+                    arrived();
+                    product(0, j);
+                }
+                if (ok && next) {
+                    n = k_entry;
+                    if (steps[1] > 0) scores(1, j + 1);
+                    release();
+                }
+                if (ok && j >= 0) {
                     n = v_entry;
-                    if (ok && j >= 0) {
-                        arrived();
-                        product(0, j);
-                    }
-                    if (ok && next) {
-                        n = k_entry;
-                        if (steps[1] > 0) scores(1, j + 1);
-                        release();
-                    }
-                    if (ok && j >= 0) {
-                        n = v_entry;
-                        if (steps[1] > 0) product(1, j);
-                        release();
-                    }
+                    if (steps[1] > 0) product(1, j);
+                    release();
                 }
             }
         }
@@ -570,8 +557,8 @@ attn_onepass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 // The CTAs of a cluster have worked on other key tiles of the same query tile.  Each sends its rows' (offset, sum) to all; with
                 // them every thread knows its row's global ones, scales its part of O and sends it to the CTA that owns the row (128 / G
                 // rows each); after the cluster's barrier the owners add the G parts, in the order of the CTAs, and write O.  The pairs complete
-                // bytes on their readers' mbarriers: with a barrier of the cluster there too 2 x 1798, d = 128 took 13.3 us (now 12.9), 1 x 2500 14.5 (14.25); the parts by such stores were slower (1 x 2500, d =
-                // 128 14.5 -> 15.4 us).
+                // bytes on their readers' mbarriers: with a barrier of the cluster there too 2 x 1798, d = 128 took 13.3 us (now 12.9), 1 x 2500
+                // 14.5 (14.25); the parts by such stores were slower (1 x 2500, d = 128 14.5 -> 15.4 us).
                 const int my_rows = kTile / G;
                 const float l_own = ok ? l + stats[(half ^ 1) * kTile + row] : 1.0f;
                 const float mb_other = ok ? *mb_peer : 0.0f;
