@@ -61,7 +61,7 @@ def check(got: torch.Tensor, ref: np.ndarray, x, w):
 # a single row, more than one batch entry
 SHAPES = [(1, 256, 64, 2, 128), (1, 128, 128, 1, 64), (2, 300, 192, 3, 64), (1, 1, 64, 1, 128), (1, 520, 328, 5, 64),
           (2, 77, 72, 1, 128), (1, 1024, 512, 4, 128), (3, 130, 256, 6, 64), (1, 257, 8, 2, 64),
-          # tiles of 256 x 256 and of 128 x 256 on a device of 148 SMs, with a last tile that is partly empty (the others: 128 x 128)
+          # whole tiles by pairs of CTAs on a device of 148 SMs, with a last tile that is partly empty (the others: narrow ones, up to d_model = 256 by single CTAs)
           (2, 469, 136, 60, 64), (1, 3872, 72, 7, 64)]
 
 
@@ -74,8 +74,9 @@ def test_projection_matches_oracle(attnw, B, N, d_model, H, d):
 
 
 # On a device of 148 SMs: more whole tiles than pairs of CTAs, with a last round cut in two; the same with an odd number of row blocks,
-# which leaves a CTA without rows; several rounds of one slice; narrow tiles with an odd number of slices and of row blocks
-@pytest.mark.parametrize("B,N,d_model,H,d", [(3, 650, 136, 9, 128), (1, 1300, 200, 15, 128), (2, 2600, 64, 8, 128), (1, 300, 320, 3, 64)])
+# which leaves a CTA without rows; several rounds of one slice; narrow tiles with an odd number of slices and of row blocks; tiles cut in two with
+# heads of 64 and an odd number of them: the second half of a last block has no features
+@pytest.mark.parametrize("B,N,d_model,H,d", [(3, 650, 136, 9, 128), (1, 1300, 200, 15, 128), (2, 2600, 64, 8, 128), (1, 300, 320, 3, 64), (1, 1500, 264, 25, 64)])
 def test_projection_over_rounds_of_tiles(attnw, B, N, d_model, H, d):
     x, wq, wk = rand_xw(B, N, d_model, H, d, stream=5 * N + d_model + H)
     Q, K = run_project(attnw, x, wq, wk)
