@@ -3,7 +3,7 @@
  *
  * C ABI of libattnw.so.  The operations, each a hand-written CUDA kernel:
  *
- *   attn_fused     the whole of Attention(Q, K, V) = softmax(Q K^T / sqrt(d_k)) V of Section IV in one kernel
+ *   attn_fused     the whole of Attention(Q, K, V) = softmax(Q K^T / sqrt(d_k)) V of Section IV, scores and weights on chip
  *   attnw_fused*   matmul + scaling + Softmax in one kernel; scores never reach HBM
  *                  (the fused kernel of Section VII of "Attention in SRAM on Tenstorrent
  *                  Grayskull"; the product is Attention's softmax(QK^T/sqrt(d_k)) of Section IV).
@@ -90,8 +90,9 @@ int attnw_fused_noalloc(const void* Q, const void* K, void* P, int B, int H, int
 
 /*
  * attn_fused: O[b,h,i,c] = sum_j P[b,h,i,j] * V[b,h,j,c] with P as defined for attnw_fused - Attention(Q, K, V) of
- * Section IV, the product with V that Section VIII leaves as future work - in one kernel; neither the scores nor the
- * weights reach HBM.
+ * Section IV, the product with V that Section VIII leaves as future work; neither the scores nor the weights reach HBM.
+ * One launch, or two of the same kernel on parts of the rows (attnw_launch_count counts them); if the second cannot be launched the
+ * call returns ATTNW_ERR_CUDA while the first is already writing its part of O.
  *
  *   Q, K, V  device, bfloat16, [B, H, N, d]                    (read only)
  *   O        device, bfloat16, [B, H, N, d]; every element is written exactly once; must not overlap Q, K or V
@@ -214,13 +215,14 @@ int attnw_host_release(void);
  * that launch is then undefined.
  * The word is STICKY: while it is non-zero, every later launch of the tensor-core kernels (attnw_fused*, attn_fused,
  * attnw_project_qk) and of the shared-memory and cluster tiers of softmax_rows* (rows of 8193 to 262144 columns, but
- * for those that are read twice) returns at once WITHOUT WRITING ITS OUTPUT - the
+ * for those that are read twice) ends after its set-up and first loads WITHOUT WRITING ITS OUTPUT - the
  * call itself still returns ATTNW_OK, since it only enqueues - so that no work piles up behind a device that has
  * stopped making progress.  The register and streaming tiers of softmax_rows* have no waits and ignore the word.
  * attnw_query_status() synchronises `stream`, stores the word in *device_status (0 = no failure; otherwise
  * 0x80000000 | an implementation code naming the wait that gave up), clears it, and returns ATTNW_OK or
  * ATTNW_ERR_TIMEOUT; after it has returned ATTNW_ERR_TIMEOUT, launches work again.  attnw_fused_host and
- * softmax_rows_host read and clear the word themselves before they return.
+ * softmax_rows_host read and clear the word themselves before they return.  The word is looked at by each block of a launch: one
+ * that runs on another stream while it is cleared may write a part of its output, so wait for those streams first.
  */
 int attnw_query_status(void* stream, unsigned int* device_status);
 

@@ -629,18 +629,18 @@ int launch_attn_onepass(DeviceInfo* dev, const void* Q, const void* K, const voi
     if (rc == ATTNW_OK) rc = encode_3d(&tm_v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, V, D, N, BH, 64, kTile);
     if (rc == ATTNW_OK) rc = encode_3d(&tm_o, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, O, D, N, BH, 64, kTile);
     if (rc != ATTNW_OK) return rc;
-    // Two query tiles per CTA; or one whose even and odd key tiles are worked on side by side; or one for a cluster of 2 or 4
-    // CTAs.  Chosen by the rounds of key tiles on the device (about 1.6 us each at d = 64, 1.9 at d = 128, and there a tenth more where the units
-    // have key tiles of their own) plus what a round of CTAs costs besides: 2.5 of them for its begin, set-up and epilogue, 2 more for a cluster's
-    // merge.  us per call, one CTA -> cluster: 1 x 4744 (d = 64) 43.5 -> 28.5, 1 x 9260 (d = 128) 85.6 -> 53.6, 4 x 2155 24.2 ->
-    // 19.8, 3 x 824 11.9 -> 10.8, 1 x 1000 13.3 -> 13.2.
-    // Or full rounds of CTAs first, and the query tiles that are left spread over the device by a second launch.  One launch -> two:
-    // 2 x 10215 (d = 64, 160 query tiles) 129 -> 104, 3 x 13719 (d = 128) 312 -> 258, 22 x 1940 (d = 64) 51 -> 45, 5 x 4607 (d = 64) 65 -> 56, 19 x
-    // 10023 (d = 128) 1058 -> 954, 114 x 692 (d = 128) 48.7 -> 46.5; 9 x 2487 (d = 128) 37.9 -> 39.1, not taken.  The second launch counts as 0.75
-    // key tiles, and has to give 4 percent, or 8 where the number of query tiles is odd: a head's last CTA has one query tile then, and the rounds of one
-    // launch overlap better than they are counted (not taken: 150 x 384, d = 64 22.2 / 23.8, 150 x 640 40.1 / 43.4, 9 x 3000 45.9 / 49.9, 300 x 500, d = 128
-    // 63.1 / 65.3).  Of 836 sizes near full rounds, each measured both ways, none is more than 0.5 percent behind the better one launch; with 0.5 and 3
-    // percent for all 29 were by more than 1.5, up to 8.
+    // Two query tiles per CTA; or one whose even and odd key tiles are worked on side by side; or one for a cluster of 2 or 4 CTAs.  Chosen by
+    // the rounds of key tiles on the device (about 1.6 us each at d = 64, 1.9 at d = 128, and there a tenth more where the units have key tiles
+    // of their own) plus what a round of CTAs costs besides: 2.5 of them for its begin, set-up and epilogue, 2 more for a cluster's merge.  us
+    // per call, one CTA -> cluster: 1 x 4744 (d = 64) 43.5 -> 28.5, 1 x 9260 (d = 128) 85.6 -> 53.6, 4 x 2155 24.2 -> 19.8, 3 x 824 11.9 ->
+    // 10.8, 1 x 1000 13.3 -> 13.2.
+    // Or full rounds of CTAs first, and the query tiles that are left spread over the device by a second launch.
+    // One launch -> two: 2 x 10215 (d = 64, 160 query tiles) 129 -> 104, 3 x 13719 (d = 128) 312 -> 258, 22 x 1940 (d = 64) 51 -> 45, 5 x 4607
+    // (d = 64) 65 -> 56, 19 x 10023 (d = 128) 1058 -> 954, 114 x 692 (d = 128) 48.7 -> 46.5; 9 x 2487 (d = 128) 37.9 -> 39.1, not taken.  The
+    // second launch counts as 0.75 key tiles, and has to give 4 percent, or 8 where the number of query tiles is odd: a head's last CTA has one
+    // query tile then, and the rounds of one launch overlap better than they are counted (not taken: 150 x 384, d = 64 22.2 / 23.8, 150 x 640
+    // 40.1 / 43.4, 9 x 3000 45.9 / 49.9, 300 x 500, d = 128 63.1 / 65.3).  Of 836 sizes near full rounds, each measured both ways, none is more
+    // than 0.5 percent behind the better one launch; with 0.5 and 3 percent for all 29 were by more than 1.5, up to 8.
     const long long tiles = (N + kTile - 1) / kTile, pairs = (tiles + 1) / 2, all = BH * tiles;
     const int sms = dev->sm_count;
     struct Part {
@@ -769,14 +769,15 @@ int launch_project(const DeviceInfo* dev, const void* X, const void* Wq, const v
         g_launches.fetch_add(1, std::memory_order_relaxed);
         return ATTNW_OK;
     };
-    // One CTA a tile of 128 x 128, without a partner, where one round of them holds the call and either a few slices are all there is - a pair's set-up
-    // and end cost it 0.2 to 0.4 us - or as many rows by pairs would not be one round (an odd number of row blocks, most often one or three: whole tiles
-    // leave half of the SMs idle then).  us per call, pairs -> single CTAs: 2 x 64 x 256 to 4 x 64 4.70 -> 4.52, 1 x 128 x 64 to 8 x 64 4.27 -> 3.96, 1 x
-    // 384 x 64 to 40 x 64 5.03 -> 4.02, 1 x 300 x 1024 to 40 x 64 9.68 -> 7.39, 1 x 128 x 2048 to 96 x 64 15.2 -> 12.2, 1 x 600 x 4096 to 28 x 64 23.4 -> 18.3; but 1 x
-    // 1000 x 512 to 16 x 64 5.53 -> 5.61, 1 x 1000 x 4096 to 16 x 64 14.8 -> 17.3 (a pair fetches 24 KB a slice, not 32), and a few rows of X, which all CTAs read from
-    // the same places of L2, want fewer readers: 1 x 8 x 4096 to 80 x 64 24.1 -> 32.4, 1 x 16 x 4096 23.5 -> 20.7.
-    // The same with tiles of 128 x 256, where pairs need a second round for what single CTAs do in one: 1 x 300 x 768 to 40 x 128 10.4 -> 8.4,
-    // 1 x 1400 x 2048 to 13 x 128 22.6 -> 15.7, 1 x 128 x 768 to 80 x 128 12.3 -> 8.4, 1 x 64 x 4096 to 148 x 128 58.2 -> 53.4.
+    // One CTA a tile of 128 x 128, without a partner, where one round of them holds the call and either a few slices are all there is - a pair's
+    // set-up and end cost it 0.2 to 0.4 us - or narrow tiles by pairs would not be one round (an odd number of row blocks, most often one or three:
+    // whole tiles leave half of the SMs idle then).  us per call, pairs -> single CTAs: 2 x 64 x 256 to 4 x 64 4.70 -> 4.52, 1 x 128 x 64 to 8 x 64
+    // 4.27 -> 3.96, 1 x 384 x 64 to 40 x 64 5.03 -> 4.02, 1 x 300 x 1024 to 40 x 64 9.68 -> 7.39, 1 x 128 x 2048 to 96 x 64 15.2 -> 12.2, 1 x 600 x
+    // 4096 to 28 x 64 23.4 -> 18.3; but 1 x 1000 x 512 to 16 x 64 5.53 -> 5.61, 1 x 1000 x 4096 to 16 x 64 14.8 -> 17.3 (a pair fetches 24 KB a
+    // slice, not 32), and a few rows of X, which all CTAs read from the same places of L2, want fewer readers: 1 x 8 x 4096 to 80 x 64 24.1 -> 32.4,
+    // 1 x 16 x 4096 23.5 -> 20.7.
+    // The same with tiles of 128 x 256, where pairs need a second round for what single CTAs do in one: 1 x 300 x 768 to 40 x 128 10.4 -> 8.4, 1 x
+    // 1400 x 2048 to 13 x 128 22.6 -> 15.7, 1 x 128 x 768 to 80 x 128 12.3 -> 8.4, 1 x 64 x 4096 to 148 x 128 58.2 -> 53.4.
     constexpr int kNarrow = proj::kFeatures / 2, kWide = proj::kFeatures;
     auto tiles_of = [&](int block, int ctas) { return proj::Grid(B, N, static_cast<int>(hd), block, ctas).tiles(); };
     const int sms = dev->sm_count, pairs = sms / 2;

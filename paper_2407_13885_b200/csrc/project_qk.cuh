@@ -14,8 +14,8 @@
 // What bounds it: large calls, the tensor pipe (512 cycles a slice) under the power cap; small ones, the latency of set-up, first load,
 // epilogue and launch, some 5 us.  us per call, one CTA a tile of 256 x 256, 128 x 256 or 128 x 128 -> this kernel, B x N x d_model
 // to H x d: 4 x 4096 x 4096 to 32 x 128 823 -> 724 .. 805 (by the box's power), 4 x 2825 x 1664 to 13 x 128 128 -> 106, 2 x 2092 x 368 to 37 x
-// 64 28.6 -> 18.7, 1 x 2366 x 392 to 15 x 128 24.6 -> 13.5, 1 x 1000 x 1024 to 16 x 64 7.79 -> 6.66, 1 x 1757 x 768 to 12 x 64 8.17 -> 8.14; over 30
-// drawn sizes 1.15 times as fast, none slower.
+// 64 28.6 -> 18.7, 1 x 2366 x 392 to 15 x 128 24.6 -> 13.5, 1 x 1000 x 1024 to 16 x 64 7.79 -> 6.66, 1 x 1757 x 768 to 12 x 64 8.17 -> 8.14; 547
+// sizes, most of few tiles, together with the single CTAs 1.13 times as fast; behind: one head of 64 features, by 0.2 us (1 x 512 x 64 3.54 -> 3.75).
 // What mattered in small calls: arrivals of the cluster's barrier and on the other CTA's mbarriers that order no memory (release costs
 // about 1000 cycles each: 6.86 -> 5.33 us at 2 x 64 x 256 to 4 x 64); the divisions of the tile list in front of the set-up's waits, not
 // of the first load (0.1 us); producers that a whole warp walks, with an elected lane, one for X and one for the weights (a lone lane took
@@ -100,8 +100,8 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     const int items = 2 * g.tiles() - whole_tiles;
     const int first = static_cast<int>(blockIdx.x) / kCtas, pairs = static_cast<int>(gridDim.x) / kCtas;
     const int KT = (d_model + kKSlice - 1) / kKSlice;
-    // The ring: six stages of one slice, or four of two narrow ones (single CTAs, with all features: four and three): a stage costs each of the issuing warps some 300 cycles, which the
-    // 256 of the MMAs of one narrow slice do not cover (1 x 512 x 4096 to 8 x 128 14.6 -> 13.3 us).
+    // The ring: six stages of one slice, or four of two narrow ones (single CTAs, with all features: four and three): a stage costs each of the
+    // issuing warps some 300 cycles, which the 256 of the MMAs of one narrow slice do not cover (1 x 512 x 4096 to 8 x 128 14.6 -> 13.3 us).
     const int slice_bytes = kAtomBytes + (kPair ? block : 2 * block) * 128;
     const int slices = block == kFeatures ? 1 : 2;
     const int stage_bytes = slices * slice_bytes;

@@ -1,7 +1,8 @@
 // Thin inline-PTX wrappers for sm_100a: mbarrier, TMA (cp.async.bulk.tensor), tcgen05
 // (TMEM allocation, MMA, commit, load), proxy fences and a few packed-math instructions.
-// Every wait in here is bounded: it gives up after a time limit and reports failure so the
-// caller can unwind, free TMEM and return instead of hanging the device.
+// The waits on mbarriers are single tries: their callers bound them, report failure, unwind, free
+// TMEM and return instead of hanging the device.  Barriers of a CTA or a cluster have no limit: each warp takes part in them
+// also after a bounded wait of its own has given up, so they end too.
 #pragma once
 #include <cstdint>
 #include <cuda.h>

@@ -201,7 +201,8 @@ inline cudaError_t launch_nt(const float* S, OutT* P, long long rows, long long 
     if (e != cudaSuccess) return e;
     // Four CTAs of 256 threads on an SM where they fit, but three for many float32 rows: there fewer rows in flight keep the stream of HBM
     // smoother.  us, four / three: 14000 x 12000 237 / 214, 16000 x 10240 229 / 214, 9000 x 24580 300 / 286, 6000 x 26000 222 / 203, 2000 x 25000 72.8 /
-    // 70.9; few rounds of rows or short slices want four: 2500 x 13000 47.3 / 47.4, 1000 x 14000 20.4 / 21.5, 20000 x 8200 203 / 218.
+    // 70.9; few rounds of rows or short slices want four: 2500 x 13000 47.3 / 47.4, 1000 x 14000 20.4 / 21.5, 20000 x 8200 203 / 218.  Rows an SM, times
+    // as fast with three: 10 0.91 to 1.00, 13 0.96 to 1.00, 16 0.99 to 1.04, 18 0.99 to 1.01, 22 0.98 to 1.07, 27 0.99 to 1.08, 40 0.99 to 1.12.
     const bool many_f32 = sizeof(OutT) == 4 && slice_cols >= 10240 && rows * C >= 27ll * sm_count;
     const long long per_sm = NT == 256 ? (smem * 4 <= 224 * 1024 && !many_f32 ? 4 : 3) : 2;
     long long n_clusters = (per_sm * sm_count) / C;  // CTAs that fit at once
