@@ -174,6 +174,7 @@ __device__ __noinline__ void wait_for_late_stores() {
 // failure is recorded.  Only when every CTA of the cluster runs.
 __device__ __noinline__ void tell_peers(uint32_t* abort_flag, int ctas) {
     for (int c = 0; c < ctas; ++c) ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(abort_flag), static_cast<uint32_t>(c)), 1u);
+    ptx::fence_cluster();  // before the cluster's last barrier, behind which a peer may end
 }
 
 // One thread's 32 consecutive columns of a score tile (TMEM lane = row).

@@ -305,7 +305,7 @@ project_qk_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     } else if (run && warp < kEpiWarps) {
         // ================= Epilogue warps: accumulators -> bf16 -> shared memory -> TMA stores, head-major =================
         const int quarter = warp & 3;
-        const int ch = warp >> 2;  // this warp takes the columns that CTA `ch` has loaded the features of
+        const int ch = warp >> 2;  // this warp takes the columns of the item's block `ch` of features (a pair: those that CTA `ch` has loaded)
         const uint32_t sw = static_cast<uint32_t>(lane & 7);
         const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
         const uint32_t own_box = ptx::smem_u32(smem + kOutOff + warp * kStageBoxBytes), ring_box = ptx::smem_u32(smem + warp * kStageBoxBytes);
